@@ -178,13 +178,13 @@ cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
   const bool ns = a.epi == TC_EPI_NS || a.epi == TC_EPI_NS_STEP;
   const bool clen = a.epi == TC_EPI_CLENSHAW;
   if (ns || clen || a.epi == TC_EPI_GRAM || a.epi == TC_EPI_PLANES) {
-    if (!a.out_planes || !aligned(a.out_planes, 16) || a.ldo % 8 || a.out_plane_stride % 8) return cudaErrorInvalidValue;
+    if (!a.out_planes || !aligned(a.out_planes, 16) || a.ldo % 32 || a.out_plane_stride % 8) return cudaErrorInvalidValue;
     if (a.out_nplanes < 1 || a.out_nplanes > 3) return cudaErrorInvalidValue;
   }
   if ((a.epi == TC_EPI_GRAM || a.epi == TC_EPI_NS_STEP) && !a.partials) return cudaErrorInvalidValue;
   if (clen && (!a.triangular || a.M != a.N)) return cudaErrorInvalidValue;
   if ((ns || clen) &&
-      (!a.x_planes || !aligned(a.x_planes, 16) || a.ldxp % 8 || a.x_plane_stride % 8 || a.out_nplanes != 3))
+      (!a.x_planes || !aligned(a.x_planes, 16) || a.ldxp % 32 || a.x_plane_stride % 8 || a.out_nplanes != 3))
     return cudaErrorInvalidValue;
   if (a.triangular && a.M != a.N) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
@@ -220,11 +220,11 @@ cudaError_t launch_tc_gemm_fp8(const TcArgs& a_in, cudaStream_t s) {
     if (!o->planes || !aligned(o->planes, 16) || o->ld % 16 || o->ld < o->cols) return cudaErrorInvalidValue;
   if (a.epi != TC_EPI_STORE && a.epi != TC_EPI_GRAM && a.epi != TC_EPI_NS) return cudaErrorInvalidValue;
   if (a.epi != TC_EPI_STORE) {
-    if (!a.out_planes || !aligned(a.out_planes, 16) || a.ldo % 8 || a.out_plane_stride % 8 || a.out_nplanes != 3)
+    if (!a.out_planes || !aligned(a.out_planes, 16) || a.ldo % 32 || a.out_plane_stride % 8 || a.out_nplanes != 3)
       return cudaErrorInvalidValue;
   }
   if (a.epi == TC_EPI_GRAM && (!a.partials || !a.triangular)) return cudaErrorInvalidValue;
-  if (a.epi == TC_EPI_NS && (!a.x_planes || !aligned(a.x_planes, 16) || a.ldxp % 8 || a.x_plane_stride % 8))
+  if (a.epi == TC_EPI_NS && (!a.x_planes || !aligned(a.x_planes, 16) || a.ldxp % 32 || a.x_plane_stride % 8))
     return cudaErrorInvalidValue;
   if (a.triangular && a.M != a.N) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;

@@ -241,39 +241,70 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&x)[4], int c) {
   }
 }
 
-// The three-plane split of 32 consecutive values with the lanes' rows exchanged first: each lane holds 32 values of its own row;
-// a lane quad (lanes 4g..4g+3) transposes its 16-byte quads so that store i of lane 4g + c writes
-// quad c of row 4g + i. Every store instruction then covers 8 rows x 64 contiguous bytes instead of
-// 32 rows x 16 bytes. base: plane 0 at row 4g (of the lane's quad), column c0 + 8c; mask bit i:
-// row 4g + i may be written. Every lane of the warp must call it (the exchange is warp-wide); the
-// values are split in place (x is left holding the last remainders). Each plane is the
-// round-to-nearest-even BF16 of what the previous planes left (cvt.rn.bf16x2.f32).
-__device__ __forceinline__ void store_planes32_t(uint16_t* base, int64_t ld, int64_t pstride, int np, float* x,
-                                                 int c, unsigned mask) {
+// A lane quad (lanes 4g..4g+3) exchanges the 32-column chunk its lanes hold: before, lane 4g + c holds
+// columns 0..31 of its own row 4g + c in x[0..31]; after, it holds columns 8c..8c+7 of the quad's four
+// rows, row 4g + i in x[8i..8i+7] (32 shuffles). In this order every 16-byte access of the chunk's planes
+// covers 8 rows x 64 contiguous bytes per warp instruction, for loads and stores alike; with a lane on its
+// own row each would touch 32 different 128-byte lines, and those line look-ups, not the arithmetic, set the
+// length of the output step. Reading X_k in this order as well, and exchanging the FP32 values once instead
+// of the planes of the result, took the 256-problem batch (n 64..1024) from 81.4 to 70.0 ms and the
+// preconditioned 2048 x 2048 solve from 5.26 to 4.61 ms. Every lane of the warp must call it.
+__device__ __forceinline__ void quad_rows(float* x, int c) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    uint32_t y[4] = {__float_as_uint(x[e]), __float_as_uint(x[8 + e]), __float_as_uint(x[16 + e]),
+                     __float_as_uint(x[24 + e])};
+    quad_transpose(y, c);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[8 * i + e] = __uint_as_float(y[i]);
+  }
+}
+
+// The planes of 8 consecutive values, one 16-byte store per plane. Each plane is the round-to-nearest-even
+// BF16 of what the previous planes left; x is left holding the last remainders.
+__device__ __forceinline__ void store_planes8(uint16_t* base, int64_t pstride, int np, float* x) {
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     if (q >= np) break;
-    uint32_t w[16];
+    uint32_t w[4];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      uint32_t h;
-      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
-      w[k] = h;
-      x[2 * k] = x[2 * k] - __uint_as_float(h << 16);
-      x[2 * k + 1] = x[2 * k + 1] - __uint_as_float(h & 0xffff0000u);
+    for (int k = 0; k < 4; ++k) {
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
+      x[2 * k] = x[2 * k] - __uint_as_float(w[k] << 16);
+      x[2 * k + 1] = x[2 * k + 1] - __uint_as_float(w[k] & 0xffff0000u);
     }
-    uint32_t o[4][4];   // o[i][wp]: word wp of quad c of row 4g + i
+    *reinterpret_cast<uint4*>(base + q * pstride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// The planes of a whole 32-column chunk in quad_rows order. base: plane 0 at the quad's first row, this
+// lane's 8 columns; mask bit i: row i of the quad may be written.
+__device__ __forceinline__ void store_chunk(uint16_t* base, int64_t ld, int64_t pstride, int np, float* x,
+                                            unsigned mask) {
 #pragma unroll
-    for (int wp = 0; wp < 4; ++wp) {
-      uint32_t y[4] = {w[wp], w[4 + wp], w[8 + wp], w[12 + wp]};
-      quad_transpose(y, c);
+  for (int i = 0; i < 4; ++i)
+    if (mask & (1u << i)) store_planes8(base + i * ld, pstride, np, x + 8 * i);
+}
+
+// Three planes of 8 values as loaded (16 bytes each) and their exact sum.
+struct Planes8 {
+  uint4 q[3];
+};
+__device__ __forceinline__ Planes8 load_planes8(const uint16_t* p, int64_t pstride, bool ok) {
+  Planes8 v;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) o[i][wp] = y[i];
-    }
+  for (int q = 0; q < 3; ++q)
+    v.q[q] = ok ? __ldcg(reinterpret_cast<const uint4*>(p + q * pstride)) : make_uint4(0u, 0u, 0u, 0u);
+  return v;
+}
+__device__ __forceinline__ void sum_planes8(const Planes8& v, float (&x)[8]) {
+  const uint32_t h[4] = {v.q[0].x, v.q[0].y, v.q[0].z, v.q[0].w}, m[4] = {v.q[1].x, v.q[1].y, v.q[1].z, v.q[1].w},
+                 l[4] = {v.q[2].x, v.q[2].y, v.q[2].z, v.q[2].w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (mask & (1u << i))
-        *reinterpret_cast<uint4*>(base + q * pstride + i * ld) = make_uint4(o[i][0], o[i][1], o[i][2], o[i][3]);
+  for (int w = 0; w < 4; ++w) {
+    x[2 * w] = (__uint_as_float(h[w] << 16) + __uint_as_float(m[w] << 16)) + __uint_as_float(l[w] << 16);
+    x[2 * w + 1] = (__uint_as_float(h[w] & 0xffff0000u) + __uint_as_float(m[w] & 0xffff0000u)) +
+                   __uint_as_float(l[w] & 0xffff0000u);
   }
 }
 
@@ -615,7 +646,7 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
     const float c3 = (NS && p.st) ? p.st->upd_c3 : -0.5f;
     const int64_t r = ctx.bi * BM + row_in_tile;
     const bool row_ok = r < p.M;
-    const int lq = lane & 3;                      // this lane's place in its quad (store_planes32_t)
+    const int lq = lane & 3;                      // this lane's place in its quad (quad_rows)
     const int64_t r4 = r - lq;                    // the quad's first row
     double part = 0.0;
     float d2 = 0.f, x2 = 0.f;  // NS_STEP: sum (x' - x)^2 and sum x'^2 over this thread's row chunk
@@ -625,58 +656,35 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
       float* v = &acc[c * 32];
       if (c0 >= p.N) continue;                    // the same for every lane of the warp
       const bool full_chunk = c0 + 32 <= p.N;
-      // rows of this lane's quad that exist (store_planes32_t writes rows r4 .. r4 + 3)
+      // rows of this lane's quad that exist (r4 .. r4 + 3)
       unsigned rows4 = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) rows4 |= (r4 + i < p.M) ? (1u << i) : 0u;
       if (NS) {
-        // X_{k+1} = c1 X_k + c3 X_k G: X_k from its three planes (exact), result as planes. A chunk
-        // that ends past column N still moves whole 32-value rows when the pitch holds them: the
-        // columns from N to the pitch are zero in X_k (the library zeroes its plane buffers and
-        // never writes a non-zero there), the product is zero there (the operand maps stop at N),
-        // so the padding stays zero and no element-by-element path is needed.
-        const uint16_t* xr = p.x_planes + r * p.ldxp + c0;
-        uint16_t* pr = p.out_planes + r * p.ldo + c0;
-        if (full_chunk || (c0 + 32 <= p.ldxp && c0 + 32 <= p.ldo)) {
-          // every lane takes part (rows past M read zeros and are not stored)
+        // X_{k+1} = c1 X_k + c3 X_k G: X_k from its three planes (exact), result as planes, both in
+        // quad_rows order. A chunk that ends past column N still moves whole 32-value rows (the pitches
+        // are multiples of 32): the columns from N to the pitch are zero in X_k (the library zeroes its
+        // plane buffers and never writes a non-zero there) and in the product (the operand maps stop at
+        // N), so the padding stays zero. Row i + 1's loads are in flight while row i is split and stored.
+        const uint16_t* xr = p.x_planes + r4 * p.ldxp + c0 + 8 * lq;
+        uint16_t* pr = p.out_planes + r4 * p.ldo + c0 + 8 * lq;
+        Planes8 xv = load_planes8(xr, p.x_plane_stride, (rows4 & 1u) != 0);
+        quad_rows(v, lq);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint4 h = make_uint4(0u, 0u, 0u, 0u), m = h, l = h;
-            if (row_ok) {
-              h = *reinterpret_cast<const uint4*>(xr + 8 * i);
-              m = *reinterpret_cast<const uint4*>(xr + p.x_plane_stride + 8 * i);
-              l = *reinterpret_cast<const uint4*>(xr + 2 * p.x_plane_stride + 8 * i);
-            }
-            const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, mw[4] = {m.x, m.y, m.z, m.w}, lw[4] = {l.x, l.y, l.z, l.w};
+        for (int i = 0; i < 4; ++i) {
+          float x[8];
+          sum_planes8(xv, x);
+          if (i < 3) xv = load_planes8(xr + (i + 1) * p.ldxp, p.x_plane_stride, (rows4 & (2u << i)) != 0);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int w = e >> 1, sh = (e & 1) * 16;
-              const float x = (bf16_to_f32_dev((uint16_t)(hw[w] >> sh)) + bf16_to_f32_dev((uint16_t)(mw[w] >> sh))) +
-                              bf16_to_f32_dev((uint16_t)(lw[w] >> sh));
-              const float xn = c1 * x + c3 * v[8 * i + e];
-              if (STEP) {
-                d2 = fmaf(xn - x, xn - x, d2);
-                x2 = fmaf(xn, xn, x2);
-              }
-              v[8 * i + e] = xn;
+          for (int e = 0; e < 8; ++e) {
+            const float xn = c1 * x[e] + c3 * v[8 * i + e];
+            if (STEP) {
+              d2 = fmaf(xn - x[e], xn - x[e], d2);
+              x2 = fmaf(xn, xn, x2);
             }
+            v[8 * i + e] = xn;
           }
-          store_planes32_t(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v, lq,
-                           rows4);
-        } else if (row_ok) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (c0 + j < p.N) {
-              const float x = (bf16_to_f32_dev(xr[j]) + bf16_to_f32_dev(xr[p.x_plane_stride + j])) +
-                              bf16_to_f32_dev(xr[2 * p.x_plane_stride + j]);
-              const float xn = c1 * x + c3 * v[j];
-              if (STEP) {
-                d2 = fmaf(xn - x, xn - x, d2);
-                x2 = fmaf(xn, xn, x2);
-              }
-              store_planes1(pr + j, p.out_plane_stride, p.out_nplanes, xn);
-            }
-          }
+          if (rows4 & (1u << i)) store_planes8(pr + i * p.ldo, p.out_plane_stride, p.out_nplanes, v + 8 * i);
         }
       } else if (EPI == TC_EPI_GRAM) {
         // planes of G for the chunks that reach the diagonal or lie above it, as whole 32-value rows;
@@ -684,7 +692,6 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
         // (launch_mirror_planes3, or the batched solves' own), which also overwrites what a chunk
         // crossing the diagonal stores below it. Columns past N hold zeros (the operand maps stop at N)
         // and land in the pitch's padding, which no operand map reads.
-        uint16_t* pr = p.out_planes + r * p.ldo + c0;
         float s_off = 0.f, s_diag = 0.f;
         if (!row_ok || c0 + 31 < r) {
           // a row past M, or a chunk entirely below the diagonal: no terms
@@ -703,18 +710,13 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
             }
           }
         }
-        if (c0 + 32 <= p.ldo) {
-          // rows of the quad whose chunk reaches the diagonal or lies above it
-          unsigned upper4 = 0;
+        // rows of the quad whose chunk reaches the diagonal or lies above it
+        unsigned upper4 = 0;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) upper4 |= (c0 + 31 >= r4 + i) ? (1u << i) : 0u;
-          store_planes32_t(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v, lq,
-                           rows4 & upper4);
-        } else if (row_ok && c0 + 31 >= r) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (c0 + j < p.N) store_planes1(pr + j, p.out_plane_stride, p.out_nplanes, v[j]);
-        }
+        for (int i = 0; i < 4; ++i) upper4 |= (c0 + 31 >= r4 + i) ? (1u << i) : 0u;
+        quad_rows(v, lq);
+        store_chunk(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v,
+                    rows4 & upper4);
         part += 2.0 * (double)s_off + (double)s_diag;
       } else if (CLEN) {
         if (!row_ok) continue;
@@ -755,15 +757,8 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
       } else if (EPI == TC_EPI_PLANES) {
         // the product itself as three BF16 planes (an operand of the next product); columns past N
         // hold zeros (the operand maps stop at N) and land in the pitch's padding
-        uint16_t* pr = p.out_planes + r * p.ldo + c0;
-        if (c0 + 32 <= p.ldo) {
-          store_planes32_t(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v, lq,
-                           rows4);
-        } else if (row_ok) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (c0 + j < p.N) store_planes1(pr + j, p.out_plane_stride, p.out_nplanes, v[j]);
-        }
+        quad_rows(v, lq);
+        store_chunk(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v, rows4);
       } else {  // STORE
         if (!row_ok) continue;
         float* cr = p.C + r * p.ldc + c0;
@@ -1017,31 +1012,33 @@ cudaError_t launch_pair_t(const CUtensorMap& ma, const CUtensorMap& mb, const Tc
   return cudaGetLastError();
 }
 
-// The pair kernels exist for three planes (the BF16X6 products of the solve).
+// The pair kernels exist for three planes (the BF16X6 products of the solve). A template so that only the
+// translation unit that calls it instantiates them.
+template <int P>
 cudaError_t dispatch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, int64_t tm2, int64_t tn,
                           int64_t ntiles, cudaStream_t s) {
   const bool amn = !a.a.kmajor, bmn = !a.b.kmajor;
   switch (a.epi) {
     case TC_EPI_NS:
-      if (!amn && bmn) return launch_pair_t<3, false, true, TC_EPI_NS>(ma, mb, a, tm2, tn, ntiles, s);
+      if (!amn && bmn) return launch_pair_t<P, false, true, TC_EPI_NS>(ma, mb, a, tm2, tn, ntiles, s);
       return cudaErrorInvalidValue;
     case TC_EPI_GRAM:
-      if (amn && bmn) return launch_pair_t<3, true, true, TC_EPI_GRAM>(ma, mb, a, tm2, tn, ntiles, s);
+      if (amn && bmn) return launch_pair_t<P, true, true, TC_EPI_GRAM>(ma, mb, a, tm2, tn, ntiles, s);
       return cudaErrorInvalidValue;
     case TC_EPI_NS_STEP:
-      if (!amn && bmn) return launch_pair_t<3, false, true, TC_EPI_NS_STEP>(ma, mb, a, tm2, tn, ntiles, s);
+      if (!amn && bmn) return launch_pair_t<P, false, true, TC_EPI_NS_STEP>(ma, mb, a, tm2, tn, ntiles, s);
       return cudaErrorInvalidValue;
     case TC_EPI_CLENSHAW:
-      if (amn && bmn) return launch_pair_t<3, true, true, TC_EPI_CLENSHAW>(ma, mb, a, tm2, tn, ntiles, s);
+      if (amn && bmn) return launch_pair_t<P, true, true, TC_EPI_CLENSHAW>(ma, mb, a, tm2, tn, ntiles, s);
       return cudaErrorInvalidValue;
     case TC_EPI_PLANES:
-      if (!amn && bmn) return launch_pair_t<3, false, true, TC_EPI_PLANES>(ma, mb, a, tm2, tn, ntiles, s);
+      if (!amn && bmn) return launch_pair_t<P, false, true, TC_EPI_PLANES>(ma, mb, a, tm2, tn, ntiles, s);
       return cudaErrorInvalidValue;
     default:
-      if (amn && bmn) return launch_pair_t<3, true, true, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
-      if (!amn && bmn) return launch_pair_t<3, false, true, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
-      if (amn && !bmn) return launch_pair_t<3, true, false, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
-      return launch_pair_t<3, false, false, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
+      if (amn && bmn) return launch_pair_t<P, true, true, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
+      if (!amn && bmn) return launch_pair_t<P, false, true, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
+      if (amn && !bmn) return launch_pair_t<P, true, false, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
+      return launch_pair_t<P, false, false, TC_EPI_STORE>(ma, mb, a, tm2, tn, ntiles, s);
   }
 }
 

@@ -6,7 +6,7 @@ namespace polar {
 
 cudaError_t tc_dispatch_pair3(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, int64_t tm2, int64_t tn,
                               int64_t ntiles, cudaStream_t s) {
-  return dispatch_pair(ma, mb, a, tm2, tn, ntiles, s);
+  return dispatch_pair<3>(ma, mb, a, tm2, tn, ntiles, s);
 }
 
 }  // namespace polar
