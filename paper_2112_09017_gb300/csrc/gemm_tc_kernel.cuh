@@ -22,7 +22,7 @@
 // Structure (one CTA per SM, persistent over output tiles of 128 x 256; or CTA pairs, below):
 //   warp 0      TMA producer: cp.async.bulk.tensor 3-D loads (columns, rows,
 //               planes) into a ring of shared-memory stages, mbarrier tx count
-//   warp 1      TMEM allocator and MMA issuer: tcgen05.mma kind::f16 M128 N256
+//   warp 1      TMEM allocator and MMA issuer (one elected lane): tcgen05.mma kind::f16 M128 N256
 //               K16 into two alternating 256-column slice buffers; commits free
 //               the stage and publish the slice
 //   warps 2..9  epilogue: two warps per TMEM lane quarter, 128 columns each;
@@ -130,7 +130,7 @@ __host__ __device__ constexpr int pass_b(int np, int i) {
        : ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 3 ? 1 : 0;
 }
 
-__host__ __device__ __forceinline__ int passes_for(int planes) { return planes == 1 ? 1 : (planes == 2 ? 3 : 6); }
+__host__ __device__ constexpr int passes_for(int planes) { return planes == 1 ? 1 : (planes == 2 ? 3 : 6); }
 
 // ---------------------------------------------------------------- tile schedule
 
@@ -260,18 +260,36 @@ __device__ __forceinline__ void quad_rows(float* x, int c) {
   }
 }
 
+// Two FP32 operations per instruction (round-to-nearest each).
+__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 c, a, b;\n\t"
+      "mov.b64 {%0, %1}, c;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 sub_x2(float2 a, float2 b) { return add_x2(a, make_float2(-b.x, -b.y)); }
+
+// The two BF16 values of a word as floats.
+__device__ __forceinline__ float2 bf16_pair(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
 // The planes of 8 consecutive values, one 16-byte store per plane. Each plane is the round-to-nearest-even
-// BF16 of what the previous planes left; x is left holding the last remainders.
-__device__ __forceinline__ void store_planes8(uint16_t* base, int64_t pstride, int np, float* x) {
+// BF16 of what the previous planes left.
+__device__ __forceinline__ void store_planes8(uint16_t* base, int64_t pstride, int np, const float* x) {
+  float2 r[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r[k] = make_float2(x[2 * k], x[2 * k + 1]);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     if (q >= np) break;
     uint32_t w[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
-      x[2 * k] = x[2 * k] - __uint_as_float(w[k] << 16);
-      x[2 * k + 1] = x[2 * k + 1] - __uint_as_float(w[k] & 0xffff0000u);
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(r[k].y), "f"(r[k].x));
+      r[k] = sub_x2(r[k], bf16_pair(w[k]));
     }
     *reinterpret_cast<uint4*>(base + q * pstride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -302,9 +320,9 @@ __device__ __forceinline__ void sum_planes8(const Planes8& v, float (&x)[8]) {
                  l[4] = {v.q[2].x, v.q[2].y, v.q[2].z, v.q[2].w};
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    x[2 * w] = (__uint_as_float(h[w] << 16) + __uint_as_float(m[w] << 16)) + __uint_as_float(l[w] << 16);
-    x[2 * w + 1] = (__uint_as_float(h[w] & 0xffff0000u) + __uint_as_float(m[w] & 0xffff0000u)) +
-                   __uint_as_float(l[w] & 0xffff0000u);
+    const float2 t = add_x2(add_x2(bf16_pair(h[w]), bf16_pair(m[w])), bf16_pair(l[w]));
+    x[2 * w] = t.x;
+    x[2 * w + 1] = t.y;
   }
 }
 
@@ -466,39 +484,50 @@ __device__ __noinline__ void role_producer(const Src& src, uint32_t smem_base, B
     if (armed & (1u << s2)) mbar_drain(br.full0 + 8 * s2, (armed_phase >> s2) & 1u);
 }
 
-// The NP-plane passes on one k-stage: descriptors are the stage-0 bases plus
-// compile-time offsets (the start-address field is the low 14 bits, address / 16).
-// FP8: the stage's 128 K-elements as four K = 32 MMAs on E4M3 codes (32 bytes of every row each).
-template <int TN>
-__device__ __forceinline__ void issue_stage_f8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t first_acc) {
-  constexpr uint32_t idesc = make_idesc_f8(TN);
-#pragma unroll
-  for (int kk = 0; kk < 4; ++kk)
-    tc_mma_f8(d_tmem, a_desc + ((kk * 32) >> 4), b_desc + ((kk * 32) >> 4), idesc, kk == 0 ? first_acc : 1u);
-}
-
-template <int P, bool A_MN, bool B_MN, int NP, int TN = BN, int CG = 1>
-__device__ __forceinline__ void issue_stage(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t first_acc) {
+// MMAs LO .. HI-1 of one k-stage's NP-plane passes (two K = 16 MMAs per pass): descriptors are the stage-0
+// bases plus compile-time offsets (the start-address field is the low 14 bits, address / 16).
+template <int P, bool A_MN, bool B_MN, int NP, int TN, int CG, int LO, int HI>
+__device__ __forceinline__ void issue_range(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t first_acc) {
   constexpr uint32_t idesc = make_idesc(A_MN, B_MN, TN, BM * CG);
   constexpr uint32_t B_PL = (TN / CG) * BK * 2;
 #pragma unroll
-  for (int ps = 0; ps < passes_for(NP); ++ps) {
-#pragma unroll
-    for (int kk = 0; kk < BK / 16; ++kk) {
-      const uint32_t aoff = A_MN ? pass_a(NP, ps) * MN_CHUNK + kk * 2048 : pass_a(NP, ps) * A_PLANE + kk * 32;
-      const uint32_t boff = B_MN ? pass_b(NP, ps) * MN_CHUNK + kk * 2048 : pass_b(NP, ps) * B_PL + kk * 32;
-      const uint32_t acc = (ps == 0 && kk == 0) ? first_acc : 1u;
-      if (CG == 2) tc_mma_pair(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
-      else tc_mma(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
-    }
+  for (int i = LO; i < HI; ++i) {
+    const int ps = i / (BK / 16), kk = i % (BK / 16);
+    const uint32_t aoff = A_MN ? pass_a(NP, ps) * MN_CHUNK + kk * 2048 : pass_a(NP, ps) * A_PLANE + kk * 32;
+    const uint32_t boff = B_MN ? pass_b(NP, ps) * MN_CHUNK + kk * 2048 : pass_b(NP, ps) * B_PL + kk * 32;
+    const uint32_t acc = i == 0 ? first_acc : 1u;
+    if (CG == 2) tc_mma_pair(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
+    else tc_mma(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
   }
 }
 
+// First (HALF = 0) or second half of a k-stage's MMAs. FP8: the stage's 128 K-elements as four K = 32 MMAs
+// on E4M3 codes (32 bytes of every row each).
+template <int P, bool A_MN, bool B_MN, int NP, int TN, int CG, int HALF>
+__device__ __forceinline__ void issue_half(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t first_acc) {
+  if constexpr (P == FP8) {
+    constexpr uint32_t idesc = make_idesc_f8(TN);
+#pragma unroll
+    for (int kk = 2 * HALF; kk < 2 * HALF + 2; ++kk)
+      tc_mma_f8(d_tmem, a_desc + ((kk * 32) >> 4), b_desc + ((kk * 32) >> 4), idesc, kk == 0 ? first_acc : 1u);
+  } else {
+    constexpr int N = passes_for(NP) * (BK / 16), MID = N / 2;
+    issue_range<P, A_MN, B_MN, NP, TN, CG, HALF ? MID : 0, HALF ? N : MID>(d_tmem, a_desc, b_desc, first_acc);
+  }
+}
+
+// The whole warp runs the loop and one elected lane issues: the descriptors then stay in uniform registers.
+// A wait costs about 250 cycles even when its phase has completed, because it cannot pass the MMAs queued
+// before it, and only about three MMAs queue up; so a stage's barriers are tested between the halves of the
+// stage before it, and waited for after it where they were not complete. Measured alone (a stage of twelve MMAs with both waits and commits, one SM): 1735 cycles with
+// one lane waiting ahead of every stage and 1562 in this form for 256-wide tiles, whose MMAs take 1560;
+// 1212 and 839 for 128-wide ones (790); 1202 and 681 for 64-wide ones (595).
 template <int P, bool A_MN, bool B_MN, int TN, int CG, class Src>
 __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32_t tmem_base, Bars br,
                                       volatile int* abort_flag, int pu) {
   using C = Cfg<P, TN, CG>;
   constexpr int S = C::STAGES;
+  const bool issuer = elect_one();
   // FP8 operands: K-major rows of 128 bytes, 128-byte swizzle, 8-row groups of 1024 bytes
   const uint64_t a_desc0 = P == FP8 ? smem_desc(smem_base, 16, 1024, 2)
                          : A_MN ? smem_desc(smem_base, P * MN_CHUNK, 1024, 2)
@@ -514,49 +543,74 @@ __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32
   uint32_t gphase[2] = {0u, 0u};
   int64_t ntile = 0;
   bool ok = true;
+  auto half = [&](int h, uint32_t d_tmem, uint64_t soff, uint32_t first_acc) {
+    if (!issuer) return;
+    const uint64_t a = a_desc0 + soff, b = b_desc0 + soff;
+    if (pu == P || P == FP8) {
+      if (h == 0) issue_half<P, A_MN, B_MN, (P == FP8 ? 1 : P), TN, CG, 0>(d_tmem, a, b, first_acc);
+      else issue_half<P, A_MN, B_MN, (P == FP8 ? 1 : P), TN, CG, 1>(d_tmem, a, b, first_acc);
+    } else if (pu == 2) {
+      if (h == 0) issue_half<P, A_MN, B_MN, (P == 3 ? 2 : 1), TN, CG, 0>(d_tmem, a, b, first_acc);
+      else issue_half<P, A_MN, B_MN, (P == 3 ? 2 : 1), TN, CG, 1>(d_tmem, a, b, first_acc);
+    } else {
+      if (h == 0) issue_half<P, A_MN, B_MN, 1, TN, CG, 0>(d_tmem, a, b, first_acc);
+      else issue_half<P, A_MN, B_MN, 1, TN, CG, 1>(d_tmem, a, b, first_acc);
+    }
+  };
   for (int64_t t = src.t0; t < src.ntiles && ok; t += src.dt) {
     TileCtx c;
     if (!src.get(t, c)) continue;
     const int grp = TN == BN ? 0 : (int)(ntile++ & 1);
-    int& buf = gbuf[grp];
-    uint32_t& buf_phase = gphase[grp];
+    int buf = gbuf[grp];
+    uint32_t buf_phase = gphase[grp];
     int kin = 0;  // k-stage index within the current slice
-    for (int64_t kb = 0; kb < c.nk; ++kb) {
-      // c.sl k-stages into a fresh slice buffer, then published to the epilogue
-      const bool slice_start = kin == 0;
+    // c.sl k-stages into a fresh slice buffer, then published to the epilogue
+    ok = mbar_wait_warp(br.tempty0 + 8 * (2 * grp + buf), buf_phase ^ 1u, abort_flag) &&
+         mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag);
+    for (int64_t kb = 0; kb < c.nk && ok; ++kb) {
       const bool slice_end = kin == c.sl - 1 || kb == c.nk - 1;
       const int bslot = 2 * grp + buf;
-      if (slice_start && !mbar_wait(br.tempty0 + 8 * bslot, buf_phase ^ 1u, abort_flag)) { ok = false; break; }
-      if (!mbar_wait(br.full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
-      tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(bslot * TN);
       const uint64_t soff = (uint64_t)((stage * C::STAGE_BYTES) >> 4);
-      const uint32_t first_acc = slice_start ? 0u : 1u;
-      if constexpr (P == FP8) {
-        issue_stage_f8<TN>(d_tmem, a_desc0 + soff, b_desc0 + soff, first_acc);
-      } else {
-        if (pu == P) issue_stage<P, A_MN, B_MN, P, TN, CG>(d_tmem, a_desc0 + soff, b_desc0 + soff, first_acc);
-        else if (pu == 2)
-          issue_stage<P, A_MN, B_MN, (P >= 2 ? 2 : P), TN, CG>(d_tmem, a_desc0 + soff, b_desc0 + soff, first_acc);
-        else issue_stage<P, A_MN, B_MN, 1, TN, CG>(d_tmem, a_desc0 + soff, b_desc0 + soff, first_acc);
-      }
-      // the stage is free in both CTAs of a pair, the slice is ready in both CTAs' TMEM
-      if (CG == 2) tc_commit_pair(br.empty0 + 8 * stage, 3);
-      else tc_commit(br.empty0 + 8 * stage);
+      const uint32_t first_acc = kin == 0 ? 0u : 1u;
+      tc_fence_after();
+      half(0, d_tmem, soff, first_acc);
+      // the next stage of this tile, and its slice's buffer
+      const int this_stage = stage;
+      if (++stage == S) { stage = 0; phase ^= 1u; }
       if (slice_end) {
-        if (CG == 2) tc_commit_pair(br.tfull0 + 8 * bslot, 3);
-        else tc_commit(br.tfull0 + 8 * bslot);
         if (++buf == 2) { buf = 0; buf_phase ^= 1u; }
         kin = 0;
       } else {
         ++kin;
       }
-      if (++stage == S) { stage = 0; phase ^= 1u; }
+      const bool more = kb + 1 < c.nk;
+      const uint32_t full = br.full0 + 8 * stage, tempty = br.tempty0 + 8 * (2 * grp + buf);
+      const bool full_ok = !more || mbar_peek_warp(full, phase);
+      const bool tempty_ok = !more || !slice_end || mbar_peek_warp(tempty, buf_phase ^ 1u);
+      half(1, d_tmem, soff, 1u);
+      // the stage is free in both CTAs of a pair, the slice is ready in both CTAs' TMEM
+      if (issuer) {
+        if (CG == 2) tc_commit_pair(br.empty0 + 8 * this_stage, 3);
+        else tc_commit(br.empty0 + 8 * this_stage);
+        if (slice_end) {
+          if (CG == 2) tc_commit_pair(br.tfull0 + 8 * bslot, 3);
+          else tc_commit(br.tfull0 + 8 * bslot);
+        }
+      }
+      __syncwarp();
+      if (!full_ok) ok = mbar_wait_warp(full, phase, abort_flag);
+      if (!tempty_ok) ok = ok && mbar_wait_warp(tempty, buf_phase ^ 1u, abort_flag);
     }
+    gbuf[grp] = buf;
+    gphase[grp] = buf_phase;
   }
   // every MMA issued so far completes before TMEM is released
-  if (CG == 2) tc_commit_pair(br.drain, 1);
-  else tc_commit(br.drain);
+  if (issuer) {
+    if (CG == 2) tc_commit_pair(br.drain, 1);
+    else tc_commit(br.drain);
+  }
+  __syncwarp();
   mbar_drain(br.drain, 0);
 }
 
@@ -870,7 +924,7 @@ __device__ __forceinline__ void tc_body(const Src& src, DevState* st, int* err_w
   if (warp == 0) {
     if (lane == 0) role_producer<P, A_MN, B_MN, TN, CG>(src, smem_base, br, abort_flag, withhold);
   } else if (warp == 1) {
-    if (lane == 0 && (CG == 1 || cluster_rank() == 0)) {   // a pair's MMAs come from its even CTA
+    if (CG == 1 || cluster_rank() == 0) {   // a pair's MMAs come from its even CTA
       const int pu = planes_dyn ? min(max(*planes_dyn, 1), P) : P;
       role_mma<P, A_MN, B_MN, TN, CG>(src, smem_base, tmem_base, br, abort_flag, pu);
     }
