@@ -1,0 +1,576 @@
+// Persistent cooperative kernels: a whole chain of split-BF16 tensor-core products (three planes, six
+// passes) in one launch, for sizes at which a product is one or two waves of small tiles. The chain's
+// products depend on each other through global memory, so a grid barrier separates them; what it replaces
+// per product is a kernel launch, the set-up of barriers, TMEM and descriptors, and the small kernels
+// between the products (residual and stop rule, mirror).
+//
+// The product itself is that of gemm_tc_kernel.cuh: TMA producer, one MMA-issuing thread, eight epilogue
+// warps that promote every 64-deep k-slice into FP32 registers with round-to-nearest, the same passes in
+// the same order. What differs is the tile: 128 x TN with TN = 64 or 128, all eight epilogue warps on one
+// tile (TN / 2 columns each), so that a matrix of a few hundred rows spreads over the chip and the output
+// step of a tile is short. G is kept as its upper triangle only: a k-block of the update's B operand below
+// the triangle is read from the mirrored place as a K-major operand, above it as an MN-major one.
+//
+// The blocks wait on one another, so the launch is cooperative (every block resident, or an error), and
+// every wait is bounded: a grid barrier that expires raises the block's abort flag like an mbarrier that
+// expires, the block leaves, and the others leave when their own waits expire.
+#pragma once
+
+#include "gemm_tc_kernel.cuh"
+
+namespace polar {
+namespace {
+
+constexpr int CO_P = 3;
+constexpr int CO_THREADS = NTHREADS + 32;   // one warp more, for what must not hold up the products: the stop test
+constexpr int CO_WARPS = CO_THREADS / 32;
+constexpr int CO_CTL_WARP = CO_WARPS - 1;
+
+template <int TN>
+struct CoCfg {
+  // A stage holds SUB k-blocks of 32: with 64-wide tiles two, because the twelve short MMAs of one do not
+  // cover the waits and commits of a stage (measured at 512 x 512: about 940 cycles per k-block against 595
+  // of products).
+  static constexpr int SUB = TN == 64 ? 2 : 1;
+  static constexpr int STAGES = TN == 64 ? 3 : 4;          // 72 or 48 KiB each
+  static constexpr uint32_t A_BYTES = CO_P * A_PLANE;      // of one k-block
+  static constexpr uint32_t B_BYTES = CO_P * TN * BK * 2;
+  static constexpr uint32_t KB_BYTES = A_BYTES + B_BYTES;
+  static constexpr uint32_t STAGE_BYTES = SUB * KB_BYTES;
+  static constexpr int BKS = SUB * BK;                     // K of one stage
+  static constexpr int NBUF = 4;                           // TMEM slice buffers of TN columns
+  static constexpr uint32_t TCOLS = NBUF * TN;
+  static constexpr int CW = TN / 2;                        // columns of one epilogue warp
+  static constexpr int SLICE = 64 / BKS;                   // stages per promoted slice
+};
+
+// Shared control block, behind the stages.
+struct CoCtl {
+  uint64_t bars[2 * 6 + 2 * 4 + 1];
+  double red[CO_WARPS];
+  uint32_t tmem;
+  int abort;
+  int status;              // of the last stop test
+};
+
+template <int TN>
+constexpr size_t co_smem() { return (size_t)CoCfg<TN>::STAGES * CoCfg<TN>::STAGE_BYTES + sizeof(CoCtl) + 1024; }
+
+// Words of the grid barrier in device memory; both zero between launches (the last block to leave
+// resets them).
+struct CoBar {
+  unsigned int count, left;
+};
+
+// What a role carries from one product to the next.
+struct CoPipe {
+  int stage = 0;
+  uint32_t phase = 0;
+  int buf = 0;
+  uint32_t buf_phase = 0;
+};
+
+struct CoCtx {
+  CoCtl* ctl;
+  uint8_t* smem;             // 1024-byte aligned, the stages
+  uint32_t smem_base, tmem;
+  Bars br;
+  CoBar* bar;
+  unsigned int target;       // arrivals the next grid barrier waits for
+  int warp, lane;
+  volatile int* abort_flag;
+};
+
+// One product of a chain: tiles of 128 x TN, rectangular (column by column) or the upper triangle's.
+struct CoTiles {
+  int tm, tn, ntiles, tri;
+};
+
+template <int TN>
+__host__ __device__ inline CoTiles co_tiles(int64_t M, int64_t N, bool tri) {
+  CoTiles t;
+  t.tm = (int)((M + BM - 1) / BM);
+  t.tn = (int)((N + TN - 1) / TN);
+  t.tri = tri ? 1 : 0;
+  if (!tri) t.ntiles = t.tm * t.tn;
+  else if (TN == 128) t.ntiles = t.tn * (t.tn + 1) / 2;
+  else t.ntiles = (t.tn / 2) * (t.tn / 2 + 1) + (t.tn & 1) * (t.tn / 2 + 1);
+  return t;
+}
+
+template <int TN>
+__device__ __forceinline__ void co_coords(const CoTiles& c, int t, int& bi, int& bj) {
+  if (!c.tri) {
+    bj = t / c.tm;
+    bi = t - bj * c.tm;
+  } else if (TN == 128) {   // column bj holds bj + 1 tiles
+    int j = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while (j > 0 && j * (j + 1) / 2 > t) --j;
+    while ((j + 1) * (j + 2) / 2 <= t) ++j;
+    bj = j;
+    bi = t - j * (j + 1) / 2;
+  } else {                  // columns 2j and 2j + 1 hold j + 1 tiles each
+    int j = (int)((sqrtf(4.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while (j > 0 && j * (j + 1) > t) --j;
+    while ((j + 1) * (j + 2) <= t) ++j;
+    const int r = t - j * (j + 1);
+    bj = 2 * j + (r > j ? 1 : 0);
+    bi = r > j ? r - j - 1 : r;
+  }
+}
+
+// First k of the B operand that a column tile at n0 reads from the mirrored place: the rows above it were
+// stored by the upper triangle's tiles (whole 128-row tiles that hold an entry on or above the diagonal).
+template <int TN>
+__device__ __forceinline__ int co_mirror_from(int n0) { return 128 * ((n0 + TN - 1) / 128 + 1); }
+
+// ------------------------------------------------------------------ set-up, grid barrier, teardown
+
+template <int TN>
+__device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, CoBar* bar) {
+  using C = CoCfg<TN>;
+  CoCtx x;
+  x.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  x.ctl = reinterpret_cast<CoCtl*>(x.smem + C::STAGES * C::STAGE_BYTES);
+  x.smem_base = smem_u32(x.smem);
+  x.br.full0 = smem_u32(&x.ctl->bars[0]);
+  x.br.empty0 = smem_u32(&x.ctl->bars[C::STAGES]);
+  x.br.tfull0 = smem_u32(&x.ctl->bars[2 * C::STAGES]);
+  x.br.tempty0 = smem_u32(&x.ctl->bars[2 * C::STAGES + C::NBUF]);
+  x.br.drain = smem_u32(&x.ctl->bars[2 * C::STAGES + 2 * C::NBUF]);
+  x.bar = bar;
+  x.target = 0;
+  x.warp = threadIdx.x >> 5;
+  x.lane = threadIdx.x & 31;
+  x.abort_flag = reinterpret_cast<volatile int*>(&x.ctl->abort);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::STAGES; ++s) {
+      mbar_init(x.br.full0 + 8 * s, 1);
+      mbar_init(x.br.empty0 + 8 * s, 1);
+    }
+    for (int b = 0; b < C::NBUF; ++b) {
+      mbar_init(x.br.tfull0 + 8 * b, 1);
+      mbar_init(x.br.tempty0 + 8 * b, EPI_WARPS);
+    }
+    mbar_init(x.br.drain, 1);
+    x.ctl->abort = 0;
+    x.ctl->status = ST_RUNNING;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (x.warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&x.ctl->tmem)),
+                 "r"(C::TCOLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  x.tmem = *reinterpret_cast<volatile uint32_t*>(&x.ctl->tmem);
+  return x;
+}
+
+// Orders what the last grid barrier made visible to this thread before the copies (the async proxy) that it
+// issues from here on.
+__device__ __forceinline__ void co_fence_proxy() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+// s + e = a + b exactly (Knuth's two-sum): the sums of a product's tiles go through FP32 pairs, because a
+// chain of FP64 additions takes longer than the rest of the output step on this part.
+__device__ __forceinline__ void two_sum(float2& s, float2 b) {
+  const float t = s.x + b.x, bb = t - s.x;
+  const float e = (s.x - (t - bb)) + (b.x - bb);
+  s = make_float2(t, s.y + (b.y + e));
+}
+
+// Grid barrier: every block's global writes before it are visible after it. False when it expired or the
+// block had aborted. Must be reached by all threads of the block.
+__device__ __forceinline__ bool co_grid_sync(CoCtx& x) {
+  __syncthreads();
+  x.target += gridDim.x;
+  if (threadIdx.x == 0 && !*x.abort_flag && gridDim.x > 1) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&x.bar->count) : "memory");
+    const uint64_t t0 = gtime();
+    for (uint32_t i = 1;; ++i) {
+      unsigned int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&x.bar->count) : "memory");
+      if (v >= x.target) break;
+      if ((i & 63u) == 0 && gtime() - t0 > 2 * WAIT_LIMIT_NS) {
+        *x.abort_flag = 1;
+        break;
+      }
+    }
+  }
+  __syncthreads();
+  return !*x.abort_flag;
+}
+
+// Leaves the kernel: every thread of the block, after its last product. Reports an expired wait.
+template <int TN>
+__device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st) {
+  if (x.warp == 1 && x.lane == 0) {   // every MMA issued has completed before TMEM is released
+    tc_commit(x.br.drain);
+    mbar_drain(x.br.drain, 0);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (*x.abort_flag) {
+      atomicOr(&st->err_flags, 1u);
+      st->status = ST_TIMEOUT;
+    }
+    __threadfence();
+    if (atomicAdd(&x.bar->left, 1u) == gridDim.x - 1) {
+      x.bar->count = 0;
+      x.bar->left = 0;
+    }
+  }
+  if (x.warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(x.tmem), "r"(CoCfg<TN>::TCOLS)
+                 : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ the roles of one product
+//
+// All in line, so that what they carry stays in registers: the grid barrier's acquire empties L1, and a
+// context kept in local memory for calls was read back from L2 at the start of every product.
+
+// mbt: the mirrored (K-major) map of B for SYM, whose upper triangle alone is stored.
+template <int TN, bool A_MN, bool SYM>
+__device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, const CUtensorMap* ma, const CUtensorMap* mb,
+                                         const CUtensorMap* mbt, CoTiles ct, int K, int withhold) {
+  using C = CoCfg<TN>;
+  if (withhold) return;   // test hook: no copies are issued, the consumers' bounded waits expire
+  co_fence_proxy();
+  int stage = pp.stage;
+  uint32_t phase = pp.phase;
+  bool ok = true;
+  uint32_t armed = 0, armed_phase = 0;
+  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
+    int bi, bj;
+    co_coords<TN>(ct, t, bi, bj);
+    const int m0 = bi * BM, n0 = bj * TN;
+    const int km = SYM ? co_mirror_from<TN>(n0) : 0x7fffffff;
+    for (int k0 = 0; k0 < K; k0 += C::BKS) {
+      if (!mbar_wait(x.br.empty0 + 8 * stage, phase ^ 1u, x.abort_flag)) { ok = false; break; }
+      const uint32_t fb = x.br.full0 + 8 * stage;
+      mbar_expect_tx(fb, C::SUB == 2 && k0 + BK < K ? 2 * C::KB_BYTES : C::KB_BYTES);
+      armed |= 1u << stage;
+      armed_phase = (armed_phase & ~(1u << stage)) | (phase << stage);
+#pragma unroll
+      for (int s = 0; s < C::SUB; ++s) {
+        const int k = k0 + s * BK;
+        if (s > 0 && k >= K) break;
+        const uint32_t a_dst = x.smem_base + stage * C::STAGE_BYTES + s * C::KB_BYTES, b_dst = a_dst + C::A_BYTES;
+        if (A_MN) {
+#pragma unroll
+          for (int cc = 0; cc < BM / 64; ++cc) tma_load_3d(a_dst + cc * CO_P * MN_CHUNK, ma, fb, m0 + 64 * cc, k, 0);
+        } else {
+          tma_load_3d(a_dst, ma, fb, k, m0, 0);
+        }
+        if (k < km) {
+#pragma unroll
+          for (int cc = 0; cc < TN / 64; ++cc) tma_load_3d(b_dst + cc * CO_P * MN_CHUNK, mb, fb, n0 + 64 * cc, k, 0);
+        } else {
+          tma_load_3d(b_dst, mbt, fb, k, n0, 0);
+        }
+      }
+      if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+    }
+  }
+  pp.stage = stage;
+  pp.phase = phase;
+  // every copy this thread started lands before the block can leave (another role may have aborted)
+  for (int s = 0; s < C::STAGES; ++s)
+    if (armed & (1u << s)) mbar_drain(x.br.full0 + 8 * s, (armed_phase >> s) & 1u);
+}
+
+// The whole warp runs the loop and one elected lane issues, a stage's waits between the halves of the stage
+// before it (see role_mma; with four slice buffers the wait for one is rarely a real one).
+template <int TN, bool A_MN, bool SYM>
+__device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, CoTiles ct, int K) {
+  using C = CoCfg<TN>;
+  const bool issuer = elect_one();
+  const uint64_t a0 = A_MN ? smem_desc(x.smem_base, CO_P * MN_CHUNK, 1024, 2)
+                           : smem_desc(x.smem_base, 16, KM_SBO, KM_SWZ);
+  const uint64_t bm0 = smem_desc(x.smem_base + C::A_BYTES, CO_P * MN_CHUNK, 1024, 2);
+  const uint64_t bk0 = smem_desc(x.smem_base + C::A_BYTES, 16, KM_SBO, KM_SWZ);
+  const Bars br = x.br;
+  volatile int* abort_flag = x.abort_flag;
+  const uint32_t tmem = x.tmem;
+  int stage = pp.stage, buf = pp.buf;
+  uint32_t phase = pp.phase, buf_phase = pp.buf_phase;
+  bool ok = true;
+  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
+    int bi, bj;
+    co_coords<TN>(ct, t, bi, bj);
+    const int km = SYM ? co_mirror_from<TN>(bj * TN) : 0x7fffffff;
+    int kin = 0;
+    ok = mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag) &&
+         mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag);
+    for (int k0 = 0; k0 < K && ok; k0 += C::BKS) {
+      const bool last = kin == C::SLICE - 1 || k0 + C::BKS >= K;
+      const uint32_t d = tmem + (uint32_t)(buf * TN), acc = kin == 0 ? 0u : 1u;
+      const uint64_t so = (uint64_t)((stage * C::STAGE_BYTES) >> 4);
+      const int this_stage = stage, this_buf = buf;
+      const bool two = C::SUB == 2 && k0 + BK < K;   // the stage's second k-block exists
+      tc_fence_after();
+      if (issuer) {
+        // km and the stages are multiples of 64: a stage lies on one side of it
+        if (k0 < km) {
+          issue_half<CO_P, A_MN, true, CO_P, TN, 1, 0>(d, a0 + so, bm0 + so, acc);
+          if (two) issue_half<CO_P, A_MN, true, CO_P, TN, 1, 1>(d, a0 + so, bm0 + so, 1u);
+        } else {
+          issue_half<CO_P, A_MN, false, CO_P, TN, 1, 0>(d, a0 + so, bk0 + so, acc);
+          if (two) issue_half<CO_P, A_MN, false, CO_P, TN, 1, 1>(d, a0 + so, bk0 + so, 1u);
+        }
+      }
+      if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+      if (last) {
+        if (++buf == C::NBUF) { buf = 0; buf_phase ^= 1u; }
+        kin = 0;
+      } else {
+        ++kin;
+      }
+      if (k0 + C::BKS < K)
+        ok = mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag) &&
+             (!last || mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag));
+      if (issuer) {
+        const uint64_t so2 = so + (two ? (uint64_t)(C::KB_BYTES >> 4) : 0u);
+        if (k0 < km) {
+          if (two) issue_half<CO_P, A_MN, true, CO_P, TN, 1, 0>(d, a0 + so2, bm0 + so2, 1u);
+          issue_half<CO_P, A_MN, true, CO_P, TN, 1, 1>(d, a0 + so2, bm0 + so2, 1u);
+        } else {
+          if (two) issue_half<CO_P, A_MN, false, CO_P, TN, 1, 0>(d, a0 + so2, bk0 + so2, 1u);
+          issue_half<CO_P, A_MN, false, CO_P, TN, 1, 1>(d, a0 + so2, bk0 + so2, 1u);
+        }
+        tc_commit(br.empty0 + 8 * this_stage);
+        if (last) tc_commit(br.tfull0 + 8 * this_buf);
+      }
+      __syncwarp();
+    }
+  }
+  pp.stage = stage;
+  pp.phase = phase;
+  pp.buf = buf;
+  pp.buf_phase = buf_phase;
+}
+
+// What the output step of a product needs.
+struct CoEpi {
+  int M, N;
+  const uint16_t* x;         // NS, NS_STEP: three planes of X_k; CLENSHAW: of Z
+  int64_t ldx, xs;
+  uint16_t* out;             // planes (every kind but STORE)
+  int64_t ldo, os;
+  float* C;                  // STORE
+  int64_t ldc;
+  float c1, c3;              // NS: c1 X + c3 acc; CLENSHAW: c3 acc + c1 Z + diag I
+  float diag;
+  float2* part;              // GRAM: per epilogue warp of every block; NS_STEP: two each
+};
+
+// Sums over each warp's tiles, as unevaluated pairs hi + lo, go to e.part: GRAM ||G - I||_F^2; NS_STEP
+// ||X' - X||^2 and ||X'||^2.
+template <int TN, int EPI>
+__device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const CoEpi& e, CoTiles ct, int K) {
+  using C = CoCfg<TN>;
+  constexpr int CW = C::CW, NCH = CW / 32;
+  constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP, STEP = EPI == TC_EPI_NS_STEP;
+  constexpr bool READS_X = NS || EPI == TC_EPI_CLENSHAW;
+  const int q = x.warp & 3, half = (x.warp - 2) >> 2, lane = x.lane, lq = lane & 3;
+  const uint32_t t_lane = x.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * CW);
+  const int nslices = (K + 63) / 64;
+  int buf = pp.buf;
+  uint32_t buf_phase = pp.buf_phase;
+  float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
+  bool ok = true;
+  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
+    int bi, bj;
+    co_coords<TN>(ct, t, bi, bj);
+    const int r = bi * BM + q * 32 + lane, r4 = r - lq;
+    const int cb = bj * TN + half * CW;
+    unsigned rows4 = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) rows4 |= (r4 + i < e.M) ? (1u << i) : 0u;
+    // one chunk per warp: X_k's planes are read while the products run
+    Planes8 pre[4];
+    if (READS_X && NCH == 1 && cb < e.N) {
+      const uint16_t* xr = e.x + r4 * e.ldx + cb + 8 * lq;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) pre[i] = load_planes8(xr + i * e.ldx, e.xs, (rows4 & (1u << i)) != 0);
+    }
+    float acc[CW];
+#pragma unroll
+    for (int i = 0; i < CW; ++i) acc[i] = 0.0f;
+    for (int sl = 0; sl < nslices; ++sl) {
+      if (!mbar_wait(x.br.tfull0 + 8 * buf, buf_phase, x.abort_flag)) { ok = false; break; }
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < CW / 16; ++c) {
+        float v[16];
+        tmem_ld16(t_lane + (uint32_t)(buf * TN + c * 16), v);
+        add16_packed(&acc[c * 16], v);   // round-to-nearest promotion
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(x.br.tempty0 + 8 * buf);
+      if (++buf == C::NBUF) { buf = 0; buf_phase ^= 1u; }
+    }
+    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+    float d2 = 0.f, x2 = 0.f;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+      const int c0 = cb + 32 * c;
+      float* v = &acc[32 * c];
+      if (c0 >= e.N) continue;                       // the same for every lane of the warp
+      if (EPI == TC_EPI_GRAM) {
+        // residual terms: twice the squares above the diagonal, (g - 1)^2 on it (columns past N hold zeros)
+        if (r < e.M && c0 + 31 >= r) {
+          float s4[4] = {0.f, 0.f, 0.f, 0.f};
+          if (c0 > r) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) s4[j & 3] = fmaf(v[j], v[j], s4[j & 3]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s4[j] *= 2.0f;
+          } else {
+            const int d = r - c0;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float g = j == d ? v[j] - 1.0f : v[j], w = j < d ? 0.0f : j == d ? 1.0f : 2.0f;
+              s4[j & 3] = fmaf(w * g, g, s4[j & 3]);
+            }
+          }
+          two_sum(sum0, make_float2((s4[0] + s4[1]) + (s4[2] + s4[3]), 0.f));
+        }
+      }
+      quad_rows(v, lq);
+      if (EPI == TC_EPI_GRAM || EPI == TC_EPI_PLANES) {
+        // columns past N hold zeros (the operand maps stop at N) and land in the pitch's padding
+        store_chunk(e.out + r4 * e.ldo + c0 + 8 * lq, e.ldo, e.os, 3, v, rows4);
+      } else if (READS_X) {
+        const uint16_t* xr = e.x + r4 * e.ldx + c0 + 8 * lq;
+        uint16_t* pr = e.out + r4 * e.ldo + c0 + 8 * lq;
+        Planes8 xv;
+        if (NCH > 1) xv = load_planes8(xr, e.xs, (rows4 & 1u) != 0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float xo[8];
+          if (NCH == 1) {
+            sum_planes8(pre[i], xo);
+          } else {
+            sum_planes8(xv, xo);
+            if (i < 3) xv = load_planes8(xr + (i + 1) * e.ldx, e.xs, (rows4 & (2u << i)) != 0);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            if (NS) {
+              const float xn = e.c1 * xo[j] + e.c3 * v[8 * i + j];
+              if (STEP) {
+                d2 = fmaf(xn - xo[j], xn - xo[j], d2);
+                x2 = fmaf(xn, xn, x2);
+              }
+              v[8 * i + j] = xn;
+            } else {
+              float o = fmaf(e.c3, v[8 * i + j], e.c1 * xo[j]);
+              if (r4 + i == c0 + 8 * lq + j) o += e.diag;
+              v[8 * i + j] = o;
+            }
+          }
+          if (rows4 & (1u << i)) store_planes8(pr + i * e.ldo, e.os, 3, v + 8 * i);
+        }
+      } else {   // STORE (the pitch is a multiple of 4: whole 16-byte groups up to it)
+        float* cr = e.C + r4 * e.ldc + c0 + 8 * lq;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (!(rows4 & (1u << i))) continue;
+          if (c0 + 8 * lq < e.ldc)
+            *reinterpret_cast<float4*>(cr + i * e.ldc) = make_float4(v[8 * i], v[8 * i + 1], v[8 * i + 2], v[8 * i + 3]);
+          if (c0 + 8 * lq + 4 < e.ldc)
+            *reinterpret_cast<float4*>(cr + i * e.ldc + 4) =
+                make_float4(v[8 * i + 4], v[8 * i + 5], v[8 * i + 6], v[8 * i + 7]);
+        }
+      }
+    }
+    if (STEP) {
+      two_sum(sum0, make_float2(d2, 0.f));
+      two_sum(sum1, make_float2(x2, 0.f));
+    }
+  }
+  pp.buf = buf;
+  pp.buf_phase = buf_phase;
+  if (EPI == TC_EPI_GRAM || STEP) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
+      if (STEP)
+        two_sum(sum1, make_float2(__shfl_xor_sync(0xffffffffu, sum1.x, o), __shfl_xor_sync(0xffffffffu, sum1.y, o)));
+    }
+    if (lane == 0) {
+      float2* dst = e.part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + x.warp - 2);
+      __stcg(dst, sum0);
+      if (STEP) __stcg(dst + 1, sum1);
+    }
+  }
+}
+
+// Sum of n doubles in device memory in a fixed order, by one warp (every lane gets it).
+__device__ __forceinline__ double co_warp_sum(const double* p, int n, int stride, int lane) {
+  double v = 0.0;
+  for (int i = lane; i < n; i += 32) v += __ldcg(p + (size_t)i * stride);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The same of unevaluated pairs; the lanes' sums stay pairs until the end (see two_sum).
+__device__ __forceinline__ double co_warp_sum2(const float2* p, int n, int stride, int lane) {
+  float2 v = make_float2(0.f, 0.f);
+  for (int i = lane; i < n; i += 32) two_sum(v, __ldcg(p + (size_t)i * stride));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    two_sum(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)));
+  return (double)v.x + (double)v.y;
+}
+
+// Block sum of one double per thread (valid in thread 0).
+__device__ __forceinline__ double co_block_sum(CoCtx& x, double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if (x.lane == 0) x.ctl->red[x.warp] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < CO_WARPS; ++w) t += x.ctl->red[w];
+  return t;
+}
+
+// 8 consecutive values of a float32 row, `n` of them existing (zeros beyond), 16-byte loads when vec.
+__device__ __forceinline__ void co_load8(const float* p, int n, bool vec, float (&v)[8]) {
+  if (vec && n >= 8) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = j < n ? __ldg(p + j) : 0.0f;
+  }
+}
+
+// The reverse for stores.
+__device__ __forceinline__ void co_store8(float* p, int n, bool vec, const float (&v)[8]) {
+  if (vec && n >= 8) {
+    reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < n) p[j] = v[j];
+  }
+}
+
+}  // namespace
+}  // namespace polar

@@ -1,0 +1,328 @@
+// One polar solve in one cooperative launch (Sec. III.D, Eq. NewtonSchulz, Algorithm 1), for matrices whose
+// products are one or two waves of 128 x 64 or 128 x 128 tiles; the pieces are in coop_kernel.cuh.
+//
+//   ||A||_F | X_0 = A / ||A||_F and the planes of A | per step: Gram | update | ... | U^T A | U, H
+//
+// with a grid barrier at every bar. The update of step k runs before its stop test is known (each block
+// evaluates the test in a warp of its own, from the same partials in the same order, while the products run): when the test
+// stops the iteration at X_k, the update has written the other buffer and is ignored.
+#include <math.h>
+
+#include <algorithm>
+#include <new>
+
+#include "coop_kernel.cuh"
+
+namespace polar {
+namespace {
+
+struct CoSolve {
+  CUtensorMap xmn[2], xk[2], gmn, gk, amn;   // X_k as MN-major and K-major operand, G, mirrored G, A
+  const float* A;
+  int64_t lda;
+  float* U;
+  int64_t ldu;
+  float* H;
+  int64_t ldh;
+  uint16_t* xp[2];
+  uint16_t* gp;
+  uint16_t* ap;
+  float* C;
+  int64_t ldc, ldp, xps, gps;
+  double* partials;                          // one per block, two per block at the end
+  float2* part2;                             // residual sums, EPI_WARPS per block
+  DevState* st;
+  int m, n;
+  double v_tol, stag2, v_floor;              // the stop rule on squares: n tol^2, stagnation^2, n stag_floor^2
+  int n_pre, max_iter;
+  float pre_c1, pre_c3;                      // update coefficients of the first n_pre steps
+  double inv_sqrt_n;
+  int withhold;
+};
+
+// The stop rule of step k on v = ||G - I||_F^2 = n r^2 against squared thresholds: r <= tol is
+// v <= n tol^2 and r > s r_{k-2} is v > s^2 v_{k-2}.
+__device__ __forceinline__ int co_stop_status(const CoSolve& p, int k, double v, double v_km2) {
+  const bool testing = k >= p.n_pre;
+  if (!isfinite(v)) return ST_NONFINITE;
+  if (testing && v <= p.v_tol) return ST_CONVERGED;
+  if (testing && k >= p.n_pre + 2 && v > p.stag2 * v_km2 && v < p.v_floor) return ST_NOT_CONVERGED;
+  if (k >= p.max_iter) return ST_NOT_CONVERGED;
+  return ST_RUNNING;
+}
+
+template <int TN>
+__global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_constant__ CoSolve p) {
+  extern __shared__ uint8_t co_raw[];
+  CoCtx x = co_setup<TN>(co_raw, reinterpret_cast<CoBar*>(&p.st->bar));
+  const int m = p.m, n = p.n, tid = threadIdx.x, nthr = CO_THREADS;
+  const int gtid = blockIdx.x * nthr + tid, gthr = gridDim.x * nthr;
+  const bool vec_a = (reinterpret_cast<uintptr_t>(p.A) & 15u) == 0 && p.lda % 4 == 0;
+  const bool vec_u = (reinterpret_cast<uintptr_t>(p.U) & 15u) == 0 && p.ldu % 4 == 0;
+  const int c8n = (n + 7) / 8;
+  DevState* st = p.st;
+  CoPipe pipe;
+  bool run = true;
+  // ---- ||A||_F, float64 sums in a fixed order
+  {
+    double acc = 0.0;
+    for (int u = gtid; u < m * c8n; u += gthr) {
+      const int r = u / c8n, c = (u - r * c8n) * 8;
+      float v[8];
+      co_load8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc = fma((double)v[j], (double)v[j], acc);
+    }
+    const double t = co_block_sum(x, acc);
+    if (tid == 0) p.partials[blockIdx.x] = t;
+    run = co_grid_sync(x);
+  }
+  if (run) {
+    const double nrm = sqrt(co_warp_sum(p.partials, gridDim.x, 1, x.lane));
+    const bool good = isfinite(nrm) && nrm > 0.0;
+    if (gtid == 0) {
+      st->normA = nrm;
+      st->inv_sqrt_n = p.inv_sqrt_n;
+      st->iters = 0;
+      st->hist_len = 0;
+      st->err_flags = 0;
+      st->planes_next = CO_P;
+      st->fp8_on = 0;
+      st->sym_err = 0.0;
+      st->status = good ? ST_RUNNING : ST_NONFINITE;
+    }
+    run = good;            // the same in every block
+    if (run) {
+      // ---- X_0 = A / ||A||_F and A as planes; columns from n to the next multiple of 8 are zeros
+      const float s = (float)nrm;
+      for (int u = gtid; u < m * c8n; u += gthr) {
+        const int r = u / c8n, c = (u - r * c8n) * 8;
+        float v[8], y[8];
+        co_load8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) y[j] = __fdiv_rn(v[j], s);
+        const int64_t o = (int64_t)r * p.ldp + c;
+        store_planes8(p.xp[0] + o, p.xps, 3, y);
+        store_planes8(p.ap + o, p.xps, 3, v);
+      }
+      run = co_grid_sync(x);
+    }
+  }
+  // ---- the iteration
+  const CoTiles tg = co_tiles<TN>(n, n, true), tu = co_tiles<TN>(m, n, false);
+  double v_km1 = 0.0, v_km2 = 0.0;   // the control warp's last two residual sums
+  int it = 0, status = ST_TIMEOUT;
+  for (int k = 0; run; ++k) {
+    const int b = k & 1;
+    // Gram of X_k: the upper triangle's tiles, and this block's part of ||G - I||_F^2
+    if (x.warp == 0) {
+      if (x.lane == 0) co_producer<TN, true, false>(x, pipe, &p.xmn[b], &p.xmn[b], nullptr, tg, m, p.withhold);
+    } else if (x.warp == 1) {
+      co_mma<TN, true, false>(x, pipe, tg, m);
+    } else if (x.warp < CO_CTL_WARP) {
+      CoEpi e{};
+      e.M = n; e.N = n;
+      e.out = p.gp; e.ldo = p.ldp; e.os = p.gps;
+      e.part = p.part2;
+      co_epilogue<TN, TC_EPI_GRAM>(x, pipe, e, tg, m);
+    }
+    run = co_grid_sync(x);
+    if (!run) break;
+    // the update, and beside it the stop test of X_k and its record
+    if (k < p.max_iter) {
+      if (x.warp == 0) {
+        if (x.lane == 0) co_producer<TN, false, true>(x, pipe, &p.xk[b], &p.gmn, &p.gk, tu, n, p.withhold);
+      } else if (x.warp == 1) {
+        co_mma<TN, false, true>(x, pipe, tu, n);
+      } else if (x.warp < CO_CTL_WARP) {
+        CoEpi e{};
+        e.M = m; e.N = n;
+        e.x = p.xp[b]; e.ldx = p.ldp; e.xs = p.xps;
+        e.out = p.xp[b ^ 1]; e.ldo = p.ldp; e.os = p.xps;
+        e.c1 = k < p.n_pre ? p.pre_c1 : 1.5f;
+        e.c3 = k < p.n_pre ? p.pre_c3 : -0.5f;
+        co_epilogue<TN, TC_EPI_NS>(x, pipe, e, tu, n);
+      }
+    }
+    if (x.warp == CO_CTL_WARP) {
+      const double v = co_warp_sum2(p.part2, gridDim.x * EPI_WARPS, 1, x.lane);
+      const int s = co_stop_status(p, k, v, v_km2);
+      v_km2 = v_km1;
+      v_km1 = v;
+      if (x.lane == 0) {
+        x.ctl->status = s;
+        if (blockIdx.x == 0) {
+          st->res_hist[k] = sqrt(v) * p.inv_sqrt_n;   // k <= max_iter < POLAR_HIST
+          st->planes_hist[k] = (unsigned char)CO_P;
+          st->hist_len = k + 1;
+          st->iters = k;
+          st->status = s;
+        }
+      }
+    }
+    run = co_grid_sync(x);
+    if (!run) break;
+    status = *reinterpret_cast<volatile int*>(&x.ctl->status);
+    it = k;
+    if (status != ST_RUNNING) break;
+  }
+  // ---- C = U^T A, then U and H = (C + C^T) / 2
+  if (run && (status == ST_CONVERGED || status == ST_NOT_CONVERGED)) {
+    const CoTiles th = co_tiles<TN>(n, n, false);
+    if (x.warp == 0) {
+      if (x.lane == 0) co_producer<TN, true, false>(x, pipe, &p.xmn[it & 1], &p.amn, nullptr, th, m, p.withhold);
+    } else if (x.warp == 1) {
+      co_mma<TN, true, false>(x, pipe, th, m);
+    } else if (x.warp < CO_CTL_WARP) {
+      CoEpi e{};
+      e.M = n; e.N = n;
+      e.C = p.C; e.ldc = p.ldc;
+      co_epilogue<TN, TC_EPI_STORE>(x, pipe, e, th, m);
+    }
+    run = co_grid_sync(x);
+    if (run) {
+      const uint16_t* X = p.xp[it & 1];
+      for (int u = gtid; u < m * c8n; u += gthr) {
+        const int r = u / c8n, c = (u - r * c8n) * 8;
+        float v[8];
+        sum_planes8(load_planes8(X + (int64_t)r * p.ldp + c, p.xps, true), v);
+        co_store8(p.U + (int64_t)r * p.ldu + c, n - c, vec_u, v);
+      }
+      // H by pairs of 32 x 32 tiles (bi <= bj) through shared memory (the stages are idle)
+      float* ta = reinterpret_cast<float*>(x.smem);
+      float* tb = ta + 32 * 33;
+      const int nt = (n + 31) / 32, npair = nt * (nt + 1) / 2;
+      double skew = 0.0, full = 0.0;
+      for (int t = blockIdx.x; t < npair; t += gridDim.x) {
+        int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while (bj > 0 && bj * (bj + 1) / 2 > t) --bj;
+        while ((bj + 1) * (bj + 2) / 2 <= t) ++bj;
+        const int bi = t - bj * (bj + 1) / 2, i0 = bi * 32, j0 = bj * 32;
+        __syncthreads();
+        for (int u = tid; u < 1024; u += nthr) {
+          const int yy = u >> 5, xx = u & 31;
+          ta[yy * 33 + xx] = (i0 + yy < n && j0 + xx < n) ? __ldcg(p.C + (int64_t)(i0 + yy) * p.ldc + j0 + xx) : 0.0f;
+          tb[yy * 33 + xx] = (j0 + yy < n && i0 + xx < n) ? __ldcg(p.C + (int64_t)(j0 + yy) * p.ldc + i0 + xx) : 0.0f;
+        }
+        __syncthreads();
+        for (int u = tid; u < 1024; u += nthr) {
+          const int yy = u >> 5, xx = u & 31;
+          if (i0 + yy < n && j0 + xx < n) {   // C(i, j) and C(j, i) of the upper tile's entry
+            const float c = ta[yy * 33 + xx], ct = tb[xx * 33 + yy];
+            p.H[(int64_t)(i0 + yy) * p.ldh + j0 + xx] = 0.5f * (c + ct);
+            const double d = 0.5 * ((double)c - (double)ct), w = bi < bj ? 2.0 : 1.0;
+            skew = fma(w * d, d, skew);
+            full = fma((double)c, (double)c, full);
+            if (bi < bj) full = fma((double)ct, (double)ct, full);
+          }
+          if (bi < bj && j0 + yy < n && i0 + xx < n)
+            p.H[(int64_t)(j0 + yy) * p.ldh + i0 + xx] = 0.5f * (tb[yy * 33 + xx] + ta[xx * 33 + yy]);
+        }
+      }
+      const double s1 = co_block_sum(x, skew);
+      const double s2 = co_block_sum(x, full);
+      if (tid == 0) {
+        p.partials[2 * blockIdx.x] = s1;
+        p.partials[2 * blockIdx.x + 1] = s2;
+      }
+      run = co_grid_sync(x);
+      if (run && blockIdx.x == 0 && x.warp == 0) {
+        const double a = co_warp_sum(p.partials, gridDim.x, 2, x.lane);
+        const double c = co_warp_sum(p.partials + 1, gridDim.x, 2, x.lane);
+        if (x.lane == 0) st->sym_err = c > 0.0 ? sqrt(a / c) : 0.0;
+      }
+    }
+  }
+  co_teardown<TN>(x, st);
+}
+
+template <int TN>
+cudaError_t co_prepare() {
+  return cudaFuncSetAttribute(co_solve_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)co_smem<TN>());
+}
+
+template <int TN>
+cudaError_t co_launch(const CoSolve& p, int grid, cudaStream_t s) {
+  void* args[] = {const_cast<CoSolve*>(&p)};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(co_solve_kernel<TN>), dim3((unsigned)grid),
+                                     dim3(CO_THREADS), args, co_smem<TN>(), s);
+}
+
+}  // namespace
+
+struct CoopSolve {
+  CoSolve p;
+  int tn, grid;
+};
+
+// Width of the chain's tiles for products of m x n, or 0 where the separate launches are faster. A 64-wide
+// tile takes about 5/9 of a 128-wide one's time, so it is taken while it does not need more waves than that
+// makes up for. One launch against separate ones, per solve at kappa 100: 96 x 64 202 against 915 us, 512^2
+// 503 against 1713, 1024^2 827 against 2411, 2048^2 (two waves of 128-wide tiles) 2637 against 4063, 8192 x
+// 512 3370 against 6016. Beyond two waves the separate launches' 256-wide tiles and CTA pairs take over: a
+// wave's length then hides what a launch costs.
+int coop_tile_n(int64_t m, int64_t n, int sms) {
+  const int64_t t64 = co_tiles<64>(m, n, false).ntiles, t128 = co_tiles<128>(m, n, false).ntiles;
+  const int64_t w64 = (t64 + sms - 1) / sms, w128 = (t128 + sms - 1) / sms;
+  if (m * n > (int64_t)1 << 24 || w128 > 2) return 0;
+  return w64 * 5 <= w128 * 9 ? 64 : 128;
+}
+
+CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {
+  const int tn = coop_tile_n(m, n, sms);
+  if (!tn) return nullptr;
+  CoopSolve* c = new (std::nothrow) CoopSolve();
+  if (!c) return nullptr;
+  c->tn = tn;
+  // enough blocks for the larger product's tiles, and for the passes over A
+  const int64_t tiles = tn == 64 ? co_tiles<64>(m, n, false).ntiles : co_tiles<128>(m, n, false).ntiles;
+  int64_t grid = std::max<int64_t>(tiles, (m * n + 8191) / 8192);
+  grid = std::min<int64_t>(grid, std::min<int64_t>(sms, b.nparts / 2));
+  c->grid = (int)std::max<int64_t>(grid, 1);
+  if (8 * c->grid > b.nparts && (size_t)8 * c->grid * 8 > (size_t)n * b.ldc * 4) c->grid = std::max(1, b.nparts / 8);
+  CoSolve& p = c->p;
+  TcOperand x[2], g, a;
+  for (int i = 0; i < 2; ++i) {
+    x[i].planes = b.xp[i]; x[i].rows = m; x[i].cols = n; x[i].ld = b.ldp; x[i].plane_stride = b.xps;
+    p.xp[i] = b.xp[i];
+  }
+  g = x[0];
+  g.planes = b.gp; g.rows = n; g.plane_stride = b.gps;
+  a = x[0];
+  a.planes = b.ap;
+  bool ok = tc_make_map(&p.gmn, g, CO_P, true, 0) && tc_make_map(&p.gk, g, CO_P, false, tn) &&
+            tc_make_map(&p.amn, a, CO_P, true, 0);
+  for (int i = 0; i < 2; ++i)
+    ok = ok && tc_make_map(&p.xmn[i], x[i], CO_P, true, 0) && tc_make_map(&p.xk[i], x[i], CO_P, false, BM);
+  ok = ok && (tn == 64 ? co_prepare<64>() : co_prepare<128>()) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    delete c;
+    return nullptr;
+  }
+  p.gp = b.gp; p.ap = b.ap; p.C = b.C; p.ldc = b.ldc; p.ldp = b.ldp; p.xps = b.xps; p.gps = b.gps;
+  p.partials = b.partials; p.st = b.st;
+  // the residual sums take C's place (written only after the iteration) where the partials are too few
+  p.part2 = 8 * c->grid <= b.nparts ? reinterpret_cast<float2*>(b.partials) : reinterpret_cast<float2*>(b.C);
+  p.m = (int)m; p.n = (int)n;
+  p.inv_sqrt_n = 1.0 / sqrt((double)n);
+  return c;
+}
+
+void coop_solve_destroy(CoopSolve* c) { delete c; }
+
+cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
+                              const StopRule& rule, cudaStream_t s) {
+  CoSolve& p = c->p;
+  p.A = A; p.lda = lda; p.U = U; p.ldu = ldu; p.H = H; p.ldh = ldh;
+  p.v_tol = rule.tol * rule.tol * (double)p.n;
+  p.stag2 = rule.stagnation * rule.stagnation;
+  p.v_floor = rule.stag_floor * rule.stag_floor * (double)p.n;
+  p.n_pre = rule.n_pre;
+  p.max_iter = rule.max_iter;
+  update_coeffs(rule, 0, p.pre_c1, p.pre_c3);   // of the preconditioning steps, where there are any
+  p.withhold = tc_withhold();
+  return c->tn == 64 ? co_launch<64>(p, c->grid, s) : co_launch<128>(p, c->grid, s);
+}
+
+}  // namespace polar

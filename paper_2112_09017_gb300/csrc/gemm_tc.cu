@@ -109,6 +109,10 @@ cudaError_t tc_take_error(cudaStream_t s, unsigned int* out) {
   return cudaStreamSynchronize(s);
 }
 
+bool tc_make_map(void* map, const TcOperand& op, int nplanes, bool mn_major, int mn_box) {
+  return make_map(static_cast<CUtensorMap*>(map), op, nplanes, mn_major, mn_box);
+}
+
 bool tc_available() {
   int dev = 0, major = 0, minor = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
@@ -117,14 +121,21 @@ bool tc_available() {
   return major == 10 && minor == 3 && encode_fn() != nullptr;
 }
 
+// POLAR_TC_CTA_PAIR in the environment: 0 or 1, or -1 when it names neither form.
+int forced_pair_mode() {
+  const char* e = getenv("POLAR_TC_CTA_PAIR");
+  return (e && (e[0] == '0' || e[0] == '1')) ? e[0] - '0' : -1;
+}
+
+bool tc_forced_form() { return forced_pair_mode() >= 0; }
+
 // Whether a launch of `planes`-plane products runs as CTA pairs: three planes (the pair kernels'
 // instantiations) and at least one 256 x 256 pair tile for every pair of SMs, so that the pairs'
 // halved shared-memory operand traffic is not paid for with idle SMs. POLAR_TC_CTA_PAIR in the
 // environment overrides the size rule: 0 never, 1 whenever the planes allow it.
 bool use_pair(int planes, int64_t M, int64_t N, bool tri) {
   if (planes != 3) return false;
-  const char* e = getenv("POLAR_TC_CTA_PAIR");
-  const int mode = (e && (e[0] == '0' || e[0] == '1')) ? e[0] - '0' : -1;
+  const int mode = forced_pair_mode();
   if (mode >= 0) return mode == 1;
   const int64_t tm2 = (M + 2 * BM - 1) / (2 * BM), tn = (N + BN - 1) / BN;
   const int64_t tiles = tri ? pair_tri_tiles(tn) : tm2 * tn;
@@ -161,7 +172,7 @@ int default_slice_stages(int planes) {
 // Test hook for the bounded waits: with POLAR_TEST_WITHHOLD_TMA=1 in the environment
 // the producer issues no copies, so the consumers' waits expire after about one
 // second and the launch reports a timeout instead of computing.
-int withhold_tma() {
+int tc_withhold() {
   const char* e = getenv("POLAR_TEST_WITHHOLD_TMA");
   return (e && e[0] == '1') ? 1 : 0;
 }
@@ -169,7 +180,7 @@ int withhold_tma() {
 cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
   TcArgs a = a_in;
   if (a.slice_stages <= 0) a.slice_stages = default_slice_stages(a.nplanes);
-  a.withhold_tma = withhold_tma();
+  a.withhold_tma = tc_withhold();
   if (!a.st && !a.err_out) a.err_out = default_error_word();
   if (a.nplanes < 1 || a.nplanes > 3 || a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
   const TcOperand* ops[2] = {&a.a, &a.b};
@@ -209,7 +220,7 @@ cudaError_t launch_tc_gemm_fp8(const TcArgs& a_in, cudaStream_t s) {
   a.slice_stages = 1;                 // one 128-K block per slice: its scale is applied at the promotion
   if (a.a_uni && a.b_uni && a.fp8_run <= 0) a.fp8_run = 8;   // tiles under one scale: 1024 K per slice
   if (!a.a_uni || !a.b_uni) a.a_uni = a.b_uni = nullptr;
-  a.withhold_tma = withhold_tma();
+  a.withhold_tma = tc_withhold();
   if (!a.st && !a.err_out) a.err_out = default_error_word();
   if (a.M <= 0 || a.N <= 0 || a.K <= 0 || !a.a_exp || !a.b_exp || a.lde_a < (a.K + 127) / 128 ||
       a.lde_b < (a.K + 127) / 128)
@@ -249,7 +260,7 @@ cudaError_t launch_tc_gemm_grouped(const TcGroupLaunch& g_in, cudaStream_t s) {
   TcGroupLaunch g = g_in;
   if (g.nplanes < 1 || g.nplanes > 3 || !g.tiles || !g.entries) return cudaErrorInvalidValue;
   if (g.slice_stages <= 0) g.slice_stages = default_slice_stages(g.nplanes);
-  g.withhold_tma = withhold_tma();
+  g.withhold_tma = tc_withhold();
   switch (g.nplanes) {
     case 1: return tc_dispatch_grouped1(g, s);
     case 2: return tc_dispatch_grouped2(g, s);

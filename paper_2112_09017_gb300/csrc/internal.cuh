@@ -28,7 +28,10 @@ struct DevState {
   unsigned int err_flags;// device error bits (timeouts)
   int fp8_on;            // FP8 schedule: 1 while the products take E4M3-quantized operands
   float upd_c1, upd_c3;  // the next update is X <- upd_c1 X + upd_c3 X G
-  double ring[4];        // r_k at slot k % 4 (stagnation test beyond the history)
+  union {
+    double ring[4];      // r_k at slot k % 4 (stagnation test beyond the history)
+    struct { unsigned int count, left; } bar;   // a plan solved in one cooperative launch: its grid barrier
+  };
   double sym_err;        // ||skew(U^T A)||_F / ||U^T A||_F
   double res_hist[POLAR_HIST];
   unsigned char planes_hist[POLAR_HIST];
@@ -238,6 +241,31 @@ bool tc_make_entry_maps(TcGroupEntry* entry);
 int tc_gram_partials(int64_t n, int planes);
 int tc_gram_partials_max(int64_t n);
 bool tc_available();
+
+// Tensor map of one stage's box of an operand's planes: 64 columns x 32 rows for MN-major operands, 32
+// columns x mn_box rows for K-major ones.
+bool tc_make_map(void* map, const TcOperand& op, int nplanes, bool mn_major, int mn_box);
+int tc_withhold();                                // test hook: 1 when producers are to issue no copies
+bool tc_forced_form();                            // the environment names the single-CTA or the CTA-pair form
+
+// ---------------------------------------------------------------------------------
+// One solve in one cooperative launch (coop_solve.cu), for sizes whose products are one or two waves of
+// small tiles, three planes. The buffers are the plan's.
+struct CoopBuffers {
+  uint16_t* xp[2];
+  uint16_t* gp;
+  uint16_t* ap;
+  float* C;
+  int64_t ldc, ldp, xps, gps;
+  double* partials;
+  int nparts;
+  DevState* st;           // st->bar zero before the first launch
+};
+struct CoopSolve;
+CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms);   // null: not for this size
+void coop_solve_destroy(CoopSolve* c);
+cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
+                              const StopRule& rule, cudaStream_t s);
 
 // Host helpers defined in polar_api.cu and shared with the other entry points.
 bool device_is_sm103(int* sms = nullptr);         // the current device is an sm_103 GPU

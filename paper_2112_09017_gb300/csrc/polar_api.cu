@@ -140,6 +140,7 @@ struct polar_plan_s {
   struct Prof { cudaEvent_t a, b; int kind, k; };  // kind 0: Gram, 1: update
   std::vector<Prof> prof;
   size_t prof_used = 0;
+  CoopSolve* coop = nullptr;             // the whole solve in one cooperative launch (chosen at creation)
   // batched
   int count = 0;
   BatchedPlan* bp = nullptr;
@@ -229,6 +230,8 @@ polar_status_t plan_alloc(polar_plan_s* p, size_t bytes, void** out) {
 void plan_free(polar_plan_s* p) {
   for (void* a : p->allocs) cudaFree(a);
   p->allocs.clear();
+  coop_solve_destroy(p->coop);
+  p->coop = nullptr;
   if (p->st_host) cudaFreeHost(p->st_host);
   if (p->ev_start) cudaEventDestroy(p->ev_start);
   if (p->ev_stop) cudaEventDestroy(p->ev_stop);
@@ -318,6 +321,15 @@ polar_status_t plan_setup(polar_plan_s* p) {
   CK(cudaEventCreate(&p->ev_start));
   CK(cudaEventCreate(&p->ev_stop));
   for (auto& e : p->ev_chunk) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  // Small and medium six-pass solves run as one cooperative launch, unless their launches are to be timed
+  // one by one, may be more than the residual history holds, or are to take a named tile form.
+  if (p->prec == POLAR_BF16X6 && !p->opt.profile && p->opt.max_iter < POLAR_HIST && !tc_forced_form()) {
+    CoopBuffers b{};
+    b.xp[0] = p->Xp[0]; b.xp[1] = p->Xp[1]; b.gp = p->Gp; b.ap = p->Ap; b.C = p->G;
+    b.ldc = p->ldg; b.ldp = p->ldp; b.xps = p->xps; b.gps = p->gps;
+    b.partials = p->partials; b.nparts = p->nparts; b.st = p->st;
+    p->coop = coop_solve_create(b, m, n, p->sms);
+  }
   return POLAR_OK;
 }
 
@@ -502,6 +514,45 @@ cudaError_t enqueue_update_tc(polar_plan_s* p, int k, const StopRule& rule, cuda
   return prof_end(p, pi, s);
 }
 
+// The caller's record of a finished solve, from the state it left on the device.
+void fill_info(const polar_plan_s* p, const DevState& h, polar_status_t ret, float ms, int n_pre, polar_info_t* info) {
+  memset(info, 0, sizeof(*info));
+  info->status = ret;
+  info->normA_F = h.normA;
+  info->prec = p->prec;
+  info->iters = h.iters;
+  info->hist_len = h.hist_len;
+  memcpy(info->res_hist, h.res_hist, sizeof(h.res_hist));
+  memcpy(info->planes_hist, h.planes_hist, sizeof(h.planes_hist));
+  if (ret != POLAR_OK && ret != POLAR_NOT_CONVERGED) return;
+  const int it = h.iters;
+  info->residual = (it < POLAR_HIST && it < h.hist_len) ? h.res_hist[it] : h.ring[it & 3];
+  info->sym_err = h.sym_err;
+  info->ms_total = ms;
+  info->launches = p->launches;
+  info->n_precond = std::min(n_pre, it);
+}
+
+// The solve as one cooperative launch; the device decides when it stops, so the host waits once.
+polar_status_t run_coop(polar_plan_s* p, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
+                        const StopRule& rule, polar_info_t* info, cudaStream_t s) {
+  CK(coop_solve_launch(p->coop, A, lda, U, ldu, H, ldh, rule, s));
+  p->launches = 1;
+  CK(cudaEventRecord(p->ev_stop, s));
+  CK(cudaMemcpyAsync(p->st_host, p->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  float ms = 0.f;
+  CK(cudaEventElapsedTime(&ms, p->ev_start, p->ev_stop));
+  const DevState& h = *p->st_host;
+  const polar_status_t ret = h.err_flags || h.status == ST_TIMEOUT ? POLAR_ETIMEOUT
+                             : h.status == ST_CONVERGED            ? POLAR_OK
+                             : h.status == ST_NOT_CONVERGED        ? POLAR_NOT_CONVERGED
+                             : h.status == ST_NONFINITE            ? POLAR_ENONFINITE
+                                                                   : POLAR_ECUDA;
+  if (info) fill_info(p, h, ret, ms, rule.n_pre, info);
+  return ret;
+}
+
 polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U, int64_t ldu, float* H,
                           int64_t ldh, double tol, polar_info_t* info, cudaStream_t s) {
   const int64_t m = p->m, n = p->n;
@@ -510,6 +561,7 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
   p->launches = 0;
   p->prof_used = 0;
   CK(cudaEventRecord(p->ev_start, s));
+  if (p->coop) return run_coop(p, A, lda, U, ldu, H, ldh, rule, info, s);
   // ||A||_F and X_0 = A / ||A||_F (+ planes of X_0)
   int fb = frob_partials_blocks(m, n);
   CK(launch_frob_partials(A, m, n, lda, p->partials, fb, s));
@@ -555,16 +607,10 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
   if (status == ST_NONFINITE || status == ST_TIMEOUT || status == ST_RUNNING) {
     CK(cudaEventRecord(p->ev_stop, s));
     CK(cudaEventSynchronize(p->ev_stop));
-    if (info) {
-      memset(info, 0, sizeof(*info));
-      info->status = status == ST_NONFINITE ? POLAR_ENONFINITE : status == ST_TIMEOUT ? POLAR_ETIMEOUT : POLAR_ECUDA;
-      info->normA_F = h.normA;
-      info->prec = p->prec;
-      info->iters = h.iters;
-      info->hist_len = h.hist_len;
-      memcpy(info->res_hist, h.res_hist, sizeof(h.res_hist));
-      memcpy(info->planes_hist, h.planes_hist, sizeof(h.planes_hist));
-    }
+    if (info)
+      fill_info(p, h,
+                status == ST_NONFINITE ? POLAR_ENONFINITE : status == ST_TIMEOUT ? POLAR_ETIMEOUT : POLAR_ECUDA, 0.f,
+                rule.n_pre, info);
     return status == ST_NONFINITE ? POLAR_ENONFINITE : status == ST_TIMEOUT ? POLAR_ETIMEOUT : POLAR_ECUDA;
   }
   const int it = h.iters;
@@ -608,17 +654,7 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
                        : status == ST_NOT_CONVERGED ? POLAR_NOT_CONVERGED
                        : POLAR_ETIMEOUT;
   if (info) {
-    memset(info, 0, sizeof(*info));
-    info->status = ret;
-    info->iters = it;
-    info->prec = p->prec;
-    info->hist_len = h.hist_len;
-    info->residual = (it < POLAR_HIST && it < h.hist_len) ? h.res_hist[it] : h.ring[it & 3];
-    info->normA_F = h.normA;
-    info->sym_err = h.sym_err;
-    info->ms_total = ms;
-    info->launches = p->launches;
-    info->n_precond = std::min(rule.n_pre, it);
+    fill_info(p, h, ret, ms, rule.n_pre, info);
     for (size_t i = 0; i < p->prof_used; ++i) {
       const auto& pr = p->prof[i];
       if ((pr.kind == 0 && pr.k > it) || (pr.kind == 1 && pr.k >= it)) continue;  // launches after the stop
@@ -627,8 +663,6 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
       if (pr.kind == 0) { info->ms_gram += t; info->n_gram++; }
       else { info->ms_update += t; info->n_update++; }
     }
-    memcpy(info->res_hist, h.res_hist, sizeof(h.res_hist));
-    memcpy(info->planes_hist, h.planes_hist, sizeof(h.planes_hist));
   }
   return ret;
 }
