@@ -250,8 +250,9 @@ POLAR_API polar_status_t polar_split_bf16(const float* X, int64_t count, int pla
  * ||X' - X||_F / ||X'||_F <= u 2^k after update k (u = 2^-24: the paper's doubling tolerance), or
  * max_iter (<= 0 means 100) updates. The doubling tolerance ends the loop within ~25 updates, so for
  * ill-conditioned A (kappa >~ 1e2) the result is an approximate inverse. prec: BF16X6, BF16X3 or BF16
- * (products on the tensor cores with the same promotion as polar_run); FP32 -> ENOTSUP. Device pointers;
- * allocates its workspace for the call and returns after the result is in X. *iters (updates applied)
+ * (products on the tensor cores with the same promotion as polar_run); FP32 -> ENOTSUP. Device pointers.
+ * Its workspace is a library-owned block of at most 512 MiB kept between calls (one per device; concurrent
+ * calls get their own), or, when that does not fit, allocated for the call; returns after the result is in X. *iters (updates applied)
  * and *delta (the last relative change) may be NULL. Returns OK, NOT_CONVERGED (max_iter reached),
  * ENONFINITE (A zero or non-finite), EINVAL, ENOMEM, ENOTSUP or ECUDA.
  * Paper: Sec. III.D, Algorithm 2. */
@@ -278,7 +279,7 @@ POLAR_API polar_status_t polar_chebyshev_fit(const double* g, int degree, double
  * Only the upper triangle of A (lda >= n) is read; F (ldf >= n) is written in full and is exactly
  * symmetric. A and F are device pointers, coef host memory (degree + 1 finite values, rounded to
  * float32 where they enter the device arithmetic). prec: BF16X6, BF16X3 or BF16; FP32 -> ENOTSUP.
- * Allocates its workspace for the call and returns after F is written. Returns OK, EINVAL, ENOMEM,
+ * Workspace as polar_ns_inverse; returns after F is written. Returns OK, EINVAL, ENOMEM,
  * ENOTSUP, ETIMEOUT or ECUDA. Paper: Sec. III.D, the matrix-function paragraph after Algorithm 2. */
 POLAR_API polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda, double a, double b,
                                          const double* coef, int degree, float* F, int64_t ldf, int prec,

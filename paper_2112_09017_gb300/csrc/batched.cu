@@ -302,10 +302,7 @@ namespace {
 polar_status_t b_alloc(BatchedPlan* b, size_t bytes, void** out) {
   if (b->opt.ws_limit && b->ws_bytes + bytes > b->opt.ws_limit) return POLAR_ENOMEM;
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return POLAR_ENOMEM;
-  }
+  if (device_alloc(&p, bytes) != cudaSuccess) return POLAR_ENOMEM;
   b->allocs.push_back(p);
   b->ws_bytes += bytes;
   *out = p;

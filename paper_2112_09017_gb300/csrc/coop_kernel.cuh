@@ -25,6 +25,7 @@ constexpr int CO_P = 3;
 constexpr int CO_THREADS = NTHREADS + 32;   // one warp more, for what must not hold up the products: the stop test
 constexpr int CO_WARPS = CO_THREADS / 32;
 constexpr int CO_CTL_WARP = CO_WARPS - 1;
+constexpr int CO_EPI_NORM = 16;             // beside the TcEpi kinds: no output, ||C||_F^2 of a symmetric product
 
 template <int TN>
 struct CoCfg {
@@ -370,10 +371,11 @@ struct CoEpi {
   float c1, c3;              // NS: c1 X + c3 acc; CLENSHAW: c3 acc + c1 Z + diag I
   float diag;
   float2* part;              // GRAM: per epilogue warp of every block; NS_STEP: two each
+  double* norm;              // NORM: per epilogue warp of every block
 };
 
 // Sums over each warp's tiles, as unevaluated pairs hi + lo, go to e.part: GRAM ||G - I||_F^2; NS_STEP
-// ||X' - X||^2 and ||X'||^2.
+// ||X' - X||^2 and ||X'||^2. NORM's go to e.norm, in float64 (entries of any magnitude).
 template <int TN, int EPI>
 __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const CoEpi& e, CoTiles ct, int K) {
   using C = CoCfg<TN>;
@@ -386,6 +388,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
   int buf = pp.buf;
   uint32_t buf_phase = pp.buf_phase;
   float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
+  double norm = 0.0;
   bool ok = true;
   for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
     int bi, bj;
@@ -446,6 +449,19 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
           two_sum(sum0, make_float2((s4[0] + s4[1]) + (s4[2] + s4[3]), 0.f));
         }
       }
+      if (EPI == CO_EPI_NORM) {   // twice the squares above the diagonal, the squares on it
+        if (r < e.M && c0 + 31 >= r) {
+          double on = 0.0, off = 0.0;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const double g = (double)v[j];
+            if (c0 + j > r) off = fma(g, g, off);
+            else if (c0 + j == r) on = g * g;
+          }
+          norm += 2.0 * off + on;
+        }
+        continue;
+      }
       quad_rows(v, lq);
       if (EPI == TC_EPI_GRAM || EPI == TC_EPI_PLANES) {
         // columns past N hold zeros (the operand maps stop at N) and land in the pitch's padding
@@ -501,6 +517,11 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
   }
   pp.buf = buf;
   pp.buf_phase = buf_phase;
+  if (EPI == CO_EPI_NORM) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
+    if (lane == 0) __stcg(e.norm + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
+  }
   if (EPI == TC_EPI_GRAM || STEP) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

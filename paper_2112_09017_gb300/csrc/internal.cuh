@@ -267,7 +267,36 @@ void coop_solve_destroy(CoopSolve* c);
 cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                               const StopRule& rule, cudaStream_t s);
 
+// The inverse and the Chebyshev function in one cooperative launch (coop_funcs.cu), three planes. The
+// caller provides the plane buffers (no initial contents needed) and a state whose barrier words are zero.
+int coop_tile_n(int64_t m, int64_t n, int sms);   // tile width for products of up to m x n; 0: not for this size
+constexpr int COOP_MAX_DEGREE = 511;
+struct CoopInverseArgs {
+  const float* A; int64_t rows, cols, lda;
+  float* X; int64_t ldx;
+  uint16_t* ap; int64_t lpa, sa;                  // planes of A
+  uint16_t* xp[2]; int64_t lpx, sx;               // of X_k (cols x rows, pitch lpx)
+  uint16_t* pp; int64_t sp;                       // of A X_k (rows x rows, pitch lpx)
+  double* sums;                                   // coop_inverse_sums(sms) bytes
+  DevState* st;                                   // iters, sym_err (the last delta), status
+  int max_iter;
+};
+size_t coop_inverse_sums(int sms);
+cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaStream_t s);
+struct CoopChebArgs {
+  const float* A; int64_t n, lda;
+  float* F; int64_t ldf;
+  uint16_t* tp; uint16_t* bp[3]; int64_t ldp, sp;
+  double am, bm;
+  const double* coef;                             // host
+  int degree;                                     // 2 .. COOP_MAX_DEGREE
+  DevState* st;
+};
+cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_t s);
+
 // Host helpers defined in polar_api.cu and shared with the other entry points.
+cudaError_t device_alloc(void** p, size_t bytes); // cudaMalloc; when it fails, again without the block kept
+                                                  // between calls
 bool device_is_sm103(int* sms = nullptr);         // the current device is an sm_103 GPU
 int resolve_precision(int prec, int64_t n);       // POLAR_AUTO -> BF16X6 for n >= 256, FP32 below
 int product_planes(int prec);                     // BF16 planes of a product mode (0: FP32 or not a product mode)

@@ -77,19 +77,109 @@ polar_status_t scratch_get(size_t bytes, void** out) {
       s.ptr = nullptr;
       s.bytes = 0;
     }
-    if (cudaMalloc(&s.ptr, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return POLAR_ENOMEM;
-    }
+    if (device_alloc(&s.ptr, bytes) != cudaSuccess) return POLAR_ENOMEM;
     s.bytes = bytes;
   }
   *out = s.ptr;
   return POLAR_OK;
 }
 
+// Workspace of the calls that own one only while they run (polar_ns_inverse, polar_chebyshev): one block
+// per device is kept between calls, up to kKeepBytes, because cudaMalloc, cudaMallocHost and their frees
+// cost such a call 0.3 to 1 ms, as much as the work of a matrix of a few hundred rows. A call takes the
+// block out (another thread's call then allocates its own) and puts it back after its stream has been
+// waited for, so no two calls ever share it; an allocation that fails in this library frees it first.
+constexpr size_t kKeepBytes = (size_t)512 << 20;
+
+struct CallBlock {
+  void* dev = nullptr;
+  size_t bytes = 0;
+  DevState* host = nullptr;   // pinned
+};
+struct KeptBlock {
+  std::mutex mu;
+  CallBlock b;
+};
+KeptBlock g_kept[64];
+
+void block_free(CallBlock& b) {
+  if (b.dev) cudaFree(b.dev);
+  if (b.host) cudaFreeHost(b.host);
+  b = CallBlock();
+}
+
+// Frees the current device's kept block; false when there was none.
+bool kept_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  std::lock_guard<std::mutex> lk(g_kept[dev].mu);
+  if (!g_kept[dev].b.dev) return false;
+  block_free(g_kept[dev].b);
+  return true;
+}
+
+// A call's workspace: taken in the constructor's place by get(), put back (or freed) on every way out.
+class CallWorkspace {
+ public:
+  explicit CallWorkspace(cudaStream_t s) : s_(s) {}
+  ~CallWorkspace() {
+    if (!b_.dev) return;
+    cudaStreamSynchronize(s_);
+    if (dev_ < 64 && b_.bytes <= kKeepBytes) {
+      std::lock_guard<std::mutex> lk(g_kept[dev_].mu);
+      if (!g_kept[dev_].b.dev) {
+        g_kept[dev_].b = b_;
+        return;
+      }
+    }
+    block_free(b_);
+  }
+  CallWorkspace(const CallWorkspace&) = delete;
+  CallWorkspace& operator=(const CallWorkspace&) = delete;
+  polar_status_t get(size_t bytes) {
+    CK(cudaGetDevice(&dev_));
+    if (dev_ < 0 || dev_ >= 64) return POLAR_ECUDA;
+    {
+      std::lock_guard<std::mutex> lk(g_kept[dev_].mu);
+      if (g_kept[dev_].b.bytes >= bytes) {
+        b_ = g_kept[dev_].b;
+        g_kept[dev_].b = CallBlock();
+      }
+    }
+    if (b_.dev) return POLAR_OK;
+    kept_trim();   // too small for this call: the larger block takes its place
+    if (device_alloc(&b_.dev, bytes) != cudaSuccess) { b_ = CallBlock(); return POLAR_ENOMEM; }
+    b_.bytes = bytes;
+    if (cudaMallocHost((void**)&b_.host, sizeof(DevState)) != cudaSuccess) {
+      cudaGetLastError();
+      block_free(b_);
+      return POLAR_ENOMEM;
+    }
+    return POLAR_OK;
+  }
+  uint8_t* dev() const { return static_cast<uint8_t*>(b_.dev); }
+  DevState* host() const { return b_.host; }
+
+ private:
+  cudaStream_t s_;
+  int dev_ = 0;
+  CallBlock b_;
+};
+
 }  // namespace
 
 namespace polar {
+// cudaMalloc, once more without the kept block when it fails.
+cudaError_t device_alloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();
+  if (!kept_trim()) return e;
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 bool device_is_sm103(int* sms) { return device_ok(sms); }
 int resolve_precision(int prec, int64_t n) { return prec == POLAR_AUTO ? (n >= 256 ? POLAR_BF16X6 : POLAR_FP32) : prec; }
 int product_planes(int prec) {
@@ -217,10 +307,7 @@ int resolve_prec(int prec, int64_t n) { return polar::resolve_precision(prec, n)
 polar_status_t plan_alloc(polar_plan_s* p, size_t bytes, void** out) {
   if (p->opt.ws_limit && p->ws_bytes + bytes > p->opt.ws_limit) return POLAR_ENOMEM;
   void* ptr = nullptr;
-  if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return POLAR_ENOMEM;
-  }
+  if (device_alloc(&ptr, bytes) != cudaSuccess) return POLAR_ENOMEM;
   p->allocs.push_back(ptr);
   p->ws_bytes += bytes;
   *out = ptr;
@@ -533,10 +620,20 @@ void fill_info(const polar_plan_s* p, const DevState& h, polar_status_t ret, flo
   info->n_precond = std::min(n_pre, it);
 }
 
+polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
+                          double tol, polar_info_t* info, cudaStream_t s);
+
 // The solve as one cooperative launch; the device decides when it stops, so the host waits once.
 polar_status_t run_coop(polar_plan_s* p, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                         const StopRule& rule, polar_info_t* info, cudaStream_t s) {
-  CK(coop_solve_launch(p->coop, A, lda, U, ldu, H, ldh, rule, s));
+  const cudaError_t le = coop_solve_launch(p->coop, A, lda, U, ldu, H, ldh, rule, s);
+  if (le == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs to this process than the device has
+    cudaGetLastError();
+    coop_solve_destroy(p->coop);
+    p->coop = nullptr;
+    return run_single(p, A, lda, U, ldu, H, ldh, rule.tol, info, s);
+  }
+  CK(le);
   p->launches = 1;
   CK(cudaEventRecord(p->ev_stop, s));
   CK(cudaMemcpyAsync(p->st_host, p->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
@@ -981,7 +1078,8 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   if (prec == POLAR_AUTO) prec = POLAR_BF16X6;
   const int P = planes_of(prec);
   if (prec == POLAR_SCHED_BF16_THEN_X3 || P == 0) return prec == POLAR_FP32 ? POLAR_ENOTSUP : POLAR_EINVAL;
-  if (!device_ok()) { cudaGetLastError(); return POLAR_ECUDA; }
+  int sms = 0;
+  if (!device_ok(&sms)) { cudaGetLastError(); return POLAR_ECUDA; }
   if (!tc_available()) return POLAR_ENOTSUP;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t N = rows, M = cols;
@@ -998,20 +1096,49 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   const size_t o_a = take((size_t)P * sa * 2), o_x0 = take((size_t)3 * sx * 2), o_x1 = take((size_t)3 * sx * 2),
                o_p = take((size_t)3 * sp * 2), o_c = take((size_t)M * ldc * 4),
                o_part = take((size_t)std::max<int64_t>(2 * npairs, fb) * 8), o_st = take(sizeof(DevState));
-  void* ws = nullptr;
-  if (cudaMalloc(&ws, off) != cudaSuccess) { cudaGetLastError(); return POLAR_ENOMEM; }
-  int* status_host = nullptr;
+  const size_t o_sums = take(coop_inverse_sums(sms));
+  CallWorkspace call(s);
+  polar_status_t wr = call.get(off);
+  if (wr != POLAR_OK) return wr;
+  uint8_t* w = call.dev();
+  // small and medium matrices: the whole iteration in one cooperative launch
+  const int tn = prec == POLAR_BF16X6 && !tc_forced_form() ? coop_tile_n(N, N, sms) : 0;
+  if (tn) {
+    DevState* st = (DevState*)(w + o_st);
+    if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
+    CoopInverseArgs c{};
+    c.A = A; c.rows = rows; c.cols = cols; c.lda = lda; c.X = X; c.ldx = ldx;
+    c.ap = (uint16_t*)(w + o_a); c.lpa = lpa; c.sa = sa;
+    c.xp[0] = (uint16_t*)(w + o_x0); c.xp[1] = (uint16_t*)(w + o_x1); c.lpx = lpx; c.sx = sx;
+    c.pp = (uint16_t*)(w + o_p); c.sp = sp;
+    c.sums = (double*)(w + o_sums);
+    c.st = st;
+    c.max_iter = max_iter;
+    const cudaError_t e = coop_inverse_launch(c, tn, sms, s);
+    if (e == cudaSuccess) {
+      if (cudaMemcpyAsync(call.host(), st, sizeof(DevState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaGetLastError();
+        return POLAR_ECUDA;
+      }
+      const DevState& h = *call.host();
+      if (h.err_flags || h.status == ST_TIMEOUT) return POLAR_ETIMEOUT;
+      if (h.status == ST_NONFINITE) return POLAR_ENONFINITE;
+      if (iters) *iters = h.iters;
+      if (delta) *delta = h.sym_err;
+      return h.status == ST_CONVERGED ? POLAR_OK : POLAR_NOT_CONVERGED;
+    }
+    cudaGetLastError();
+    if (e != cudaErrorCooperativeLaunchTooLarge) return POLAR_ECUDA;   // else: the separate launches
+  }
+  int* status_host = reinterpret_cast<int*>(call.host());
   cudaEvent_t ev[2] = {nullptr, nullptr};
-  if (cudaMallocHost(&status_host, 2 * sizeof(int)) != cudaSuccess ||
-      cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) != cudaSuccess ||
+  if (cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     for (auto e : ev) if (e) cudaEventDestroy(e);
-    if (status_host) cudaFreeHost(status_host);
-    cudaFree(ws);
     return POLAR_ENOMEM;
   }
-  uint8_t* w = (uint8_t*)ws;
   uint16_t* ap = (uint16_t*)(w + o_a);
   uint16_t* xp[2] = {(uint16_t*)(w + o_x0), (uint16_t*)(w + o_x1)};
   uint16_t* pp = (uint16_t*)(w + o_p);
@@ -1021,7 +1148,7 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   polar_status_t ret = POLAR_ECUDA;
   DevState h;
   do {
-    if (cudaMemsetAsync(ws, 0, off, s) != cudaSuccess) break;
+    if (cudaMemsetAsync(w, 0, off, s) != cudaSuccess) break;
     // a = ||A A^T||_F = ||A^T A||_F: the Gram of A's columns on the tensor cores, mirrored, its norm
     if (launch_scale_split(A, lda, N, M, nullptr, false, nullptr, 0, ap, lpa, sa, P, s) != cudaSuccess) break;
     TcArgs g{};
@@ -1094,8 +1221,6 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   } while (0);
   cudaStreamSynchronize(s);
   for (auto e : ev) cudaEventDestroy(e);
-  cudaFreeHost(status_host);
-  cudaFree(ws);
   if (ret == POLAR_ECUDA) cudaGetLastError();
   return ret;
 }
@@ -1132,7 +1257,8 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
   if (prec == POLAR_AUTO) prec = POLAR_BF16X6;
   const int P = planes_of(prec);
   if (prec == POLAR_SCHED_BF16_THEN_X3 || P == 0) return prec == POLAR_FP32 ? POLAR_ENOTSUP : POLAR_EINVAL;
-  if (!device_ok()) { cudaGetLastError(); return POLAR_ECUDA; }
+  int sms = 0;
+  if (!device_ok(&sms)) { cudaGetLastError(); return POLAR_ECUDA; }
   if (!tc_available()) return POLAR_ENOTSUP;
   cudaStream_t s = (cudaStream_t)stream;
   const double am = 2.0 / (b - a), bm = -(a + b) / (b - a);   // T = am A + bm I
@@ -1143,15 +1269,39 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
   const size_t o_t = take((size_t)P * sp * 2), o_b0 = take((size_t)3 * sp * 2), o_b1 = take((size_t)3 * sp * 2),
                o_b2 = take((size_t)3 * sp * 2), o_st = take(sizeof(DevState));
-  void* ws = nullptr;
-  if (cudaMalloc(&ws, off) != cudaSuccess) { cudaGetLastError(); return POLAR_ENOMEM; }
-  uint8_t* w = (uint8_t*)ws;
+  CallWorkspace call(s);
+  polar_status_t wr = call.get(off);
+  if (wr != POLAR_OK) return wr;
+  uint8_t* w = call.dev();
   uint16_t* tp = (uint16_t*)(w + o_t);
   uint16_t* bk[3] = {(uint16_t*)(w + o_b0), (uint16_t*)(w + o_b1), (uint16_t*)(w + o_b2)};
   DevState* st = (DevState*)(w + o_st);
+  // small and medium matrices: every step in one cooperative launch
+  const int tn = prec == POLAR_BF16X6 && degree >= 2 && degree <= COOP_MAX_DEGREE && !tc_forced_form()
+                     ? coop_tile_n(n, n, sms) : 0;
+  if (tn) {
+    if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
+    CoopChebArgs c{};
+    c.A = A; c.n = n; c.lda = lda; c.F = F; c.ldf = ldf;
+    c.tp = tp; c.ldp = ldp; c.sp = sp;
+    for (int i = 0; i < 3; ++i) c.bp[i] = bk[i];
+    c.am = am; c.bm = bm; c.coef = coef; c.degree = degree;
+    c.st = st;
+    const cudaError_t e = coop_cheb_launch(c, tn, sms, s);
+    if (e == cudaSuccess) {
+      if (cudaMemcpyAsync(call.host(), st, sizeof(DevState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaGetLastError();
+        return POLAR_ECUDA;
+      }
+      return call.host()->err_flags || call.host()->status == ST_TIMEOUT ? POLAR_ETIMEOUT : POLAR_OK;
+    }
+    cudaGetLastError();
+    if (e != cudaErrorCooperativeLaunchTooLarge) return POLAR_ECUDA;   // else: the separate launches
+  }
   polar_status_t ret = POLAR_ECUDA;
   do {
-    if (cudaMemsetAsync(ws, 0, off, s) != cudaSuccess) break;   // also status = RUNNING
+    if (cudaMemsetAsync(w, 0, off, s) != cudaSuccess) break;   // also status = RUNNING
     bool ok = true;
     if (degree <= 1) {
       // F = c_0 I + c_1 T: no product
@@ -1187,7 +1337,6 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
     ret = (h.err_flags || h.status == ST_TIMEOUT) ? POLAR_ETIMEOUT : POLAR_OK;
   } while (0);
   cudaStreamSynchronize(s);
-  cudaFree(ws);
   if (ret == POLAR_ECUDA) cudaGetLastError();
   return ret;
 }

@@ -81,3 +81,76 @@ def test_coop_statuses_and_reuse(lib):
     assert i3["status"] == lib.POLAR_NOT_CONVERGED and i3["iters"] == 5 and len(i3["res_hist"]) == 6
     assert i3["res_hist"] == i1["res_hist"][:6]
     assert bool(torch.isfinite(U3).all()) and bool(torch.isfinite(H3).all())
+
+
+# sizes of the inverse's and the Chebyshev function's dispatch and tiles that their own tests do not reach:
+# 64- and 128-wide tiles over the whole chip, two waves, the separate launches beyond
+@pytest.mark.parametrize("m,n", [(1001, 1001), (1300, 1250), (2100, 700), (2400, 2300)], ids=lambda v: str(v))
+def test_coop_inverse_matches_separate_launches(lib, monkeypatch, m, n):
+    import torch
+    a = torch.from_numpy(synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 0.2), m)).cuda()
+    big = torch.full((n + 2, m + 7), 9.0, device="cuda")
+    X = big[1:n + 1, 3:m + 3]                       # strided, unaligned rows
+    out = lib.polar_ns_inverse(a, X)
+    monkeypatch.setenv("POLAR_TC_CTA_PAIR", "0")    # names a form: the separate launches
+    Y = torch.empty((n, m), device="cuda")
+    ref = lib.polar_ns_inverse(a, Y)
+    assert out["status"] == ref["status"] == lib.POLAR_OK and out["iters"] == ref["iters"]
+    # delta is a ratio of rounded sums over the last, small step
+    assert out["delta"] == pytest.approx(ref["delta"], rel=1e-2, abs=1e-7)
+    assert float(torch.linalg.matrix_norm(X - Y) / torch.linalg.matrix_norm(Y)) <= 2e-6
+    xa = X.double() @ a.double()
+    assert float(torch.linalg.matrix_norm(xa - torch.eye(n, device="cuda", dtype=torch.float64))) <= 1e-5 * math.sqrt(n)
+    X.fill_(9.0)
+    assert bool(torch.all(big == 9.0))
+
+
+@pytest.mark.parametrize("n,d", [(1000, 9), (1450, 4), (1536, 3), (2300, 3)])
+def test_coop_chebyshev_matches_separate_launches(lib, monkeypatch, n, d):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, _ = torch.linalg.qr(torch.randn(n, n, device="cuda", dtype=torch.float64, generator=g))
+    lam = torch.linspace(-1.0, 1.0, n, device="cuda", dtype=torch.float64)
+    a = ((q * lam) @ q.T).float()
+    coef = [0.3 / (k + 1.0) for k in range(d + 1)]
+    F = torch.empty((n, n), device="cuda")
+    lib.polar_chebyshev(a, F, -1.0, 1.0, coef)
+    monkeypatch.setenv("POLAR_TC_CTA_PAIR", "0")
+    G = torch.empty((n, n), device="cuda")
+    lib.polar_chebyshev(a, G, -1.0, 1.0, coef)
+    assert torch.equal(F, F.T)
+    # d - 1 steps of float32-grade products in either form (2e-6: the bound of the form's own test)
+    assert float(torch.linalg.matrix_norm(F - G) / torch.linalg.matrix_norm(G)) <= 2e-6
+
+
+def test_kept_workspace_is_not_shared_between_threads(lib):
+    """Concurrent calls of different sizes on streams of their own, after calls that left a block behind:
+    each gets the result it gets alone."""
+    import threading
+
+    import torch
+    mats = [torch.from_numpy(synth.matrix_with_spectrum(n, n, synth.logspace_spectrum(n, 0.3), n)).cuda()
+            for n in (150, 260, 400)]
+    want = []
+    for a in mats:
+        X = torch.empty_like(a)
+        lib.polar_ns_inverse(a, X)
+        want.append(X)
+    torch.cuda.synchronize()
+    errs = []
+
+    def work(i):
+        s = torch.cuda.Stream()
+        for _ in range(4):
+            X = torch.empty_like(mats[i])
+            s.wait_stream(torch.cuda.default_stream())
+            lib.polar_ns_inverse(mats[i], X, stream=s)
+            if not torch.equal(X, want[i]):
+                errs.append(i)
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(3)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not errs
