@@ -33,7 +33,7 @@ struct CoInverse {
 template <int TN>
 __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_constant__ CoInverse p) {
   extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, reinterpret_cast<CoBar*>(&p.st->bar));
+  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
   const int N = p.rows, M = p.cols, tid = threadIdx.x;
   const int gtid = blockIdx.x * CO_THREADS + tid, gthr = gridDim.x * CO_THREADS;
   DevState* st = p.st;
@@ -208,7 +208,7 @@ __device__ __forceinline__ void co_put(uint16_t* P, int64_t ld, int64_t ps, int 
 template <int TN>
 __global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_constant__ CoCheb p) {
   extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, reinterpret_cast<CoBar*>(&p.st->bar));
+  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
   const int n = p.n, d = p.degree, tid = threadIdx.x;
   const int nt = (n + 31) / 32, npair = nt * (nt + 1) / 2;
   CoPipe pipe;

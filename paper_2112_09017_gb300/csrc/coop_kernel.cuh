@@ -16,6 +16,7 @@
 // expires, the block leaves, and the others leave when their own waits expire.
 #pragma once
 
+#include "coop_barrier.cuh"
 #include "gemm_tc_kernel.cuh"
 
 namespace polar {
@@ -57,12 +58,6 @@ struct CoCtl {
 template <int TN>
 constexpr size_t co_smem() { return (size_t)CoCfg<TN>::STAGES * CoCfg<TN>::STAGE_BYTES + sizeof(CoCtl) + 1024; }
 
-// Words of the grid barrier in device memory; both zero between launches (the last block to leave
-// resets them).
-struct CoBar {
-  unsigned int count, left;
-};
-
 // What a role carries from one product to the next.
 struct CoPipe {
   int stage = 0;
@@ -76,8 +71,7 @@ struct CoCtx {
   uint8_t* smem;             // 1024-byte aligned, the stages
   uint32_t smem_base, tmem;
   Bars br;
-  CoBar* bar;
-  unsigned int target;       // arrivals the next grid barrier waits for
+  GridBarrier bar;
   int warp, lane;
   volatile int* abort_flag;
 };
@@ -128,19 +122,17 @@ __device__ __forceinline__ int co_mirror_from(int n0) { return 128 * ((n0 + TN -
 // ------------------------------------------------------------------ set-up, grid barrier, teardown
 
 template <int TN>
-__device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, CoBar* bar) {
+__device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
   using C = CoCfg<TN>;
-  CoCtx x;
-  x.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  x.ctl = reinterpret_cast<CoCtl*>(x.smem + C::STAGES * C::STAGE_BYTES);
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  CoCtl* ctl = reinterpret_cast<CoCtl*>(smem + C::STAGES * C::STAGE_BYTES);
+  CoCtx x{ctl, smem, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort)};
   x.smem_base = smem_u32(x.smem);
   x.br.full0 = smem_u32(&x.ctl->bars[0]);
   x.br.empty0 = smem_u32(&x.ctl->bars[C::STAGES]);
   x.br.tfull0 = smem_u32(&x.ctl->bars[2 * C::STAGES]);
   x.br.tempty0 = smem_u32(&x.ctl->bars[2 * C::STAGES + C::NBUF]);
   x.br.drain = smem_u32(&x.ctl->bars[2 * C::STAGES + 2 * C::NBUF]);
-  x.bar = bar;
-  x.target = 0;
   x.warp = threadIdx.x >> 5;
   x.lane = threadIdx.x & 31;
   x.abort_flag = reinterpret_cast<volatile int*>(&x.ctl->abort);
@@ -184,27 +176,7 @@ __device__ __forceinline__ void two_sum(float2& s, float2 b) {
   s = make_float2(t, s.y + (b.y + e));
 }
 
-// Grid barrier: every block's global writes before it are visible after it. False when it expired or the
-// block had aborted. Must be reached by all threads of the block.
-__device__ __forceinline__ bool co_grid_sync(CoCtx& x) {
-  __syncthreads();
-  x.target += gridDim.x;
-  if (threadIdx.x == 0 && !*x.abort_flag && gridDim.x > 1) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&x.bar->count) : "memory");
-    const uint64_t t0 = gtime();
-    for (uint32_t i = 1;; ++i) {
-      unsigned int v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&x.bar->count) : "memory");
-      if (v >= x.target) break;
-      if ((i & 63u) == 0 && gtime() - t0 > 2 * WAIT_LIMIT_NS) {
-        *x.abort_flag = 1;
-        break;
-      }
-    }
-  }
-  __syncthreads();
-  return !*x.abort_flag;
-}
+__device__ __forceinline__ bool co_grid_sync(CoCtx& x) { return x.bar.sync(); }
 
 // Leaves the kernel: every thread of the block, after its last product. Reports an expired wait.
 template <int TN>
@@ -215,17 +187,11 @@ __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st) {
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (*x.abort_flag) {
-      atomicOr(&st->err_flags, 1u);
-      st->status = ST_TIMEOUT;
-    }
-    __threadfence();
-    if (atomicAdd(&x.bar->left, 1u) == gridDim.x - 1) {
-      x.bar->count = 0;
-      x.bar->left = 0;
-    }
+  if (threadIdx.x == 0 && *x.abort_flag) {
+    atomicOr(&st->err_flags, 1u);
+    st->status = ST_TIMEOUT;
   }
+  x.bar.leave();
   if (x.warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(x.tmem), "r"(CoCfg<TN>::TCOLS)

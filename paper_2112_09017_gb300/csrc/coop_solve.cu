@@ -54,7 +54,7 @@ __device__ __forceinline__ int co_stop_status(const CoSolve& p, int k, double v,
 template <int TN>
 __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_constant__ CoSolve p) {
   extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, reinterpret_cast<CoBar*>(&p.st->bar));
+  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
   const int m = p.m, n = p.n, tid = threadIdx.x, nthr = CO_THREADS;
   const int gtid = blockIdx.x * nthr + tid, gthr = gridDim.x * nthr;
   const bool vec_a = (reinterpret_cast<uintptr_t>(p.A) & 15u) == 0 && p.lda % 4 == 0;

@@ -10,7 +10,12 @@
 // shared-memory buffers with register prefetch of the next k-slice. Each
 // 16-wide k-slice is summed into a fresh register tile before it is added to
 // the running sums (blocked summation).
+#include <math.h>
+
+#include <algorithm>
+
 #include "internal.cuh"
+#include "simt_small.cuh"
 
 namespace polar {
 
@@ -242,6 +247,70 @@ __global__ void __launch_bounds__(NT) simt_gemm_kernel(SimtArgs p, bool vec_a, b
   }
 }
 
+// C = alpha op(A) op(B) + beta C in 32 x 32 tiles, one per block (simt_small.cuh).
+template <bool AK, bool BK_>
+__global__ void __launch_bounds__(SS_THREADS) simt_small_kernel(SimtArgs p, bool vec_a, bool vec_b) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SsSmem& sm = *reinterpret_cast<SsSmem*>(smem_raw);
+  const int tm = (int)((p.M + SS_T - 1) / SS_T);
+  int bi, bj;
+  if (p.triangular) {   // the upper triangle, column by column
+    const int t = (int)blockIdx.x;
+    int j = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while (j > 0 && (int64_t)j * (j + 1) / 2 > t) --j;
+    while ((int64_t)(j + 1) * (j + 2) / 2 <= t) ++j;
+    bj = j;
+    bi = (int)(t - (int64_t)j * (j + 1) / 2);
+  } else {
+    bj = (int)blockIdx.x / tm;
+    bi = (int)blockIdx.x - bj * tm;
+  }
+  const SsOperand a{p.A, p.lda, (int)p.M, vec_a}, b{p.B, p.ldb, (int)p.N, vec_b};
+  ss_tile<AK, BK_>(sm, a, b, bi * SS_T, bj * SS_T, (int)p.K);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int rr = (threadIdx.x >> 5) + 16 * h, cc = threadIdx.x & 31;
+    const int64_t r = (int64_t)bi * SS_T + rr, c = (int64_t)bj * SS_T + cc;
+    if (r < p.M && c < p.N) {
+      float* dst = p.C + r * p.ldc + c;
+      const float v = ss_sum(sm, rr, cc);
+      *dst = p.alpha * v + (p.beta != 0.0f ? p.beta * *dst : 0.0f);
+    }
+  }
+}
+
+int simt_sms() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
+
+// 32 x 32 tiles where they finish first: an SM does about 60 of its 128 FMAs a cycle on them and 80 on 128 x
+// 128 tiles, but those come in whole waves of one tile per SM.
+bool use_small(const SimtArgs& a, int64_t tiles128) {
+  const int64_t lim = (int64_t)1 << 30;
+  if (a.K < 1 || a.M > lim || a.N > lim || a.K > lim) return false;
+  const int64_t tm = (a.M + SS_T - 1) / SS_T, tn = (a.N + SS_T - 1) / SS_T;
+  const int64_t t32 = a.triangular ? tn * (tn + 1) / 2 : tm * tn;
+  if (t32 > lim) return false;
+  const int64_t sms = simt_sms();
+  const double big = (double)((tiles128 + sms - 1) / sms) * BM * BN / 80.0;
+  const double small = std::max(1.0, (double)t32 / sms) * SS_T * SS_T / 60.0;
+  return small < big;
+}
+
+cudaError_t launch_small(const SimtArgs& a, bool vec_a, bool vec_b, cudaStream_t s) {
+  const int64_t tm = (a.M + SS_T - 1) / SS_T, tn = (a.N + SS_T - 1) / SS_T;
+  const unsigned grid = (unsigned)(a.triangular ? tn * (tn + 1) / 2 : tm * tn);
+  auto k = a.a_kmajor ? (a.b_kmajor ? simt_small_kernel<true, true> : simt_small_kernel<true, false>)
+                      : (a.b_kmajor ? simt_small_kernel<false, true> : simt_small_kernel<false, false>);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsSmem));
+  if (e != cudaSuccess) return e;
+  k<<<grid, SS_THREADS, sizeof(SsSmem), s>>>(a, vec_a, vec_b);
+  return cudaGetLastError();
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -259,6 +328,7 @@ cudaError_t launch_simt_gemm(const SimtArgs& a, int epi, cudaStream_t s) {
   const bool vec_b = aligned16(a.B) && (a.ldb % 4 == 0);
   const bool vec_c = aligned16(a.C) && (a.ldc % 4 == 0) &&
                      (epi != SIMT_EPI_NS || (aligned16(a.Xold) && a.ldx % 4 == 0));
+  if (epi == SIMT_EPI_STORE && !a.st && use_small(a, tiles)) return launch_small(a, vec_a, vec_b, s);
   const size_t smem = sizeof(Smem);
   cudaError_t e = cudaSuccess;
   switch (epi) {

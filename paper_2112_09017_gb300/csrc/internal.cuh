@@ -267,6 +267,22 @@ void coop_solve_destroy(CoopSolve* c);
 cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                               const StopRule& rule, cudaStream_t s);
 
+// The same for the plain form (coop_fp32.cu): 32 x 32 tiles on the SIMT cores.
+struct CoopFp32Buffers {
+  float* x[2];
+  int64_t ldx;            // multiple of 4
+  float* G;
+  int64_t ldg;            // multiple of 4
+  double* partials;
+  int nparts;
+  DevState* st;
+};
+struct CoopFp32;
+CoopFp32* coop_fp32_create(const CoopFp32Buffers& b, int64_t m, int64_t n, int sms);
+void coop_fp32_destroy(CoopFp32* c);
+cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
+                             const StopRule& rule, cudaStream_t s);
+
 // The inverse and the Chebyshev function in one cooperative launch (coop_funcs.cu), three planes. The
 // caller provides the plane buffers (no initial contents needed) and a state whose barrier words are zero.
 int coop_tile_n(int64_t m, int64_t n, int sms);   // tile width for products of up to m x n; 0: not for this size

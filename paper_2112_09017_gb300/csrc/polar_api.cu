@@ -230,7 +230,8 @@ struct polar_plan_s {
   struct Prof { cudaEvent_t a, b; int kind, k; };  // kind 0: Gram, 1: update
   std::vector<Prof> prof;
   size_t prof_used = 0;
-  CoopSolve* coop = nullptr;             // the whole solve in one cooperative launch (chosen at creation)
+  CoopSolve* coop = nullptr;             // the whole solve in one cooperative launch (chosen at creation),
+  CoopFp32* coop32 = nullptr;            // or its plain form
   // batched
   int count = 0;
   BatchedPlan* bp = nullptr;
@@ -319,6 +320,8 @@ void plan_free(polar_plan_s* p) {
   p->allocs.clear();
   coop_solve_destroy(p->coop);
   p->coop = nullptr;
+  coop_fp32_destroy(p->coop32);
+  p->coop32 = nullptr;
   if (p->st_host) cudaFreeHost(p->st_host);
   if (p->ev_start) cudaEventDestroy(p->ev_start);
   if (p->ev_stop) cudaEventDestroy(p->ev_stop);
@@ -408,9 +411,17 @@ polar_status_t plan_setup(polar_plan_s* p) {
   CK(cudaEventCreate(&p->ev_start));
   CK(cudaEventCreate(&p->ev_stop));
   for (auto& e : p->ev_chunk) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  // Small and medium six-pass solves run as one cooperative launch, unless their launches are to be timed
-  // one by one, may be more than the residual history holds, or are to take a named tile form.
-  if (p->prec == POLAR_BF16X6 && !p->opt.profile && p->opt.max_iter < POLAR_HIST && !tc_forced_form()) {
+  // Small and medium solves run as one cooperative launch, unless their launches are to be timed one by one,
+  // may be more than the residual history holds, or are to take a named tile form.
+  const bool one_launch = !p->opt.profile && p->opt.max_iter < POLAR_HIST;
+  if (one_launch && p->prec == POLAR_FP32) {
+    CoopFp32Buffers b{};
+    b.x[0] = p->X[0]; b.x[1] = p->X[1]; b.ldx = p->ldx;
+    b.G = p->G; b.ldg = p->ldg;
+    b.partials = p->partials; b.nparts = p->nparts; b.st = p->st;
+    p->coop32 = coop_fp32_create(b, m, n, p->sms);
+  }
+  if (one_launch && p->prec == POLAR_BF16X6 && !tc_forced_form()) {
     CoopBuffers b{};
     b.xp[0] = p->Xp[0]; b.xp[1] = p->Xp[1]; b.gp = p->Gp; b.ap = p->Ap; b.C = p->G;
     b.ldc = p->ldg; b.ldp = p->ldp; b.xps = p->xps; b.gps = p->gps;
@@ -626,11 +637,14 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
 // The solve as one cooperative launch; the device decides when it stops, so the host waits once.
 polar_status_t run_coop(polar_plan_s* p, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                         const StopRule& rule, polar_info_t* info, cudaStream_t s) {
-  const cudaError_t le = coop_solve_launch(p->coop, A, lda, U, ldu, H, ldh, rule, s);
+  const cudaError_t le = p->coop ? coop_solve_launch(p->coop, A, lda, U, ldu, H, ldh, rule, s)
+                                 : coop_fp32_launch(p->coop32, A, lda, U, ldu, H, ldh, rule, s);
   if (le == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs to this process than the device has
     cudaGetLastError();
     coop_solve_destroy(p->coop);
+    coop_fp32_destroy(p->coop32);
     p->coop = nullptr;
+    p->coop32 = nullptr;
     return run_single(p, A, lda, U, ldu, H, ldh, rule.tol, info, s);
   }
   CK(le);
@@ -658,7 +672,7 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
   p->launches = 0;
   p->prof_used = 0;
   CK(cudaEventRecord(p->ev_start, s));
-  if (p->coop) return run_coop(p, A, lda, U, ldu, H, ldh, rule, info, s);
+  if (p->coop || p->coop32) return run_coop(p, A, lda, U, ldu, H, ldh, rule, info, s);
   // ||A||_F and X_0 = A / ||A||_F (+ planes of X_0)
   int fb = frob_partials_blocks(m, n);
   CK(launch_frob_partials(A, m, n, lda, p->partials, fb, s));

@@ -14,10 +14,10 @@ from .gpu_util import metrics, to_np
 pytestmark = pytest.mark.gpu
 
 
-def _solve(lib, a, **kw):
+def _solve(lib, a, prec="bf16x6", **kw):
     import torch
     m, n = a.shape
-    plan = lib.Plan(m, n, prec="bf16x6", **kw)
+    plan = lib.Plan(m, n, prec=prec, **kw)
     U, H, info = plan(torch.from_numpy(a).cuda(), raw_status=True)
     plan.close()
     return to_np(U), to_np(H), info
@@ -30,13 +30,19 @@ SIZES = [(1, 1), (32, 31), (64, 64), (128, 65), (129, 128), (130, 129), (192, 19
          (2500, 33), (1000, 996), (1300, 1290), (2100, 2050), (2400, 2304)]
 
 
-@pytest.mark.parametrize("m,n", SIZES, ids=lambda v: str(v))
-def test_coop_solve_matches_oracle_and_separate_launches(lib, m, n):
+# the plain form's 32 x 32 tiles: edges, remainders of the 64-deep chunks, the largest of its dispatch
+SIZES32 = [(1, 1), (31, 31), (33, 32), (64, 33), (65, 64), (300, 200), (130, 129), (3000, 40), (1000, 990),
+           (1700, 1650)]
+
+
+@pytest.mark.parametrize("prec,m,n", [("bf16x6", *s) for s in SIZES] + [("fp32", *s) for s in SIZES32],
+                         ids=lambda v: str(v))
+def test_coop_solve_matches_oracle_and_separate_launches(lib, prec, m, n):
     kappa = 50.0
     a = synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 1.0 / kappa), 40 + n)
-    U, H, info = _solve(lib, a)
+    U, H, info = _solve(lib, a, prec)
     # a residual history that may not hold every step sends a plan to the separate launches
-    U2, H2, info2 = _solve(lib, a, max_iter=lib.POLAR_HIST + 10)
+    U2, H2, info2 = _solve(lib, a, prec, max_iter=lib.POLAR_HIST + 10)
     assert info["status"] == info2["status"] == lib.POLAR_OK
     assert info["iters"] == info2["iters"]
     assert info["launches"] == 1 or info["launches"] == info2["launches"]
@@ -55,13 +61,14 @@ def test_coop_solve_matches_oracle_and_separate_launches(lib, m, n):
         assert met["fwd"] <= 1e-7 * kappa, met
 
 
-def test_coop_statuses_and_reuse(lib):
+@pytest.mark.parametrize("prec", ["bf16x6", "fp32"])
+def test_coop_statuses_and_reuse(lib, prec):
     """Zero and non-finite input leave U and H untouched, max_iter returns the last iterate, and the same
     plan solves again afterwards, bit for bit the same twice."""
     import torch
     m, n = 300, 260
     a = torch.from_numpy(synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 1e-2), 3)).cuda()
-    plan = lib.Plan(m, n, prec="bf16x6", max_iter=20)
+    plan = lib.Plan(m, n, prec=prec, max_iter=20)
     U = torch.full((m, n), 7.0, device="cuda")
     H = torch.full((n, n), 7.0, device="cuda")
     bad = a.clone()
@@ -75,12 +82,41 @@ def test_coop_statuses_and_reuse(lib):
     assert i1["status"] == lib.POLAR_OK and i1["res_hist"] == i2["res_hist"]
     assert torch.equal(U1, U2) and torch.equal(H1, H2)
     plan.close()
-    plan = lib.Plan(m, n, prec="bf16x6", max_iter=5)
+    plan = lib.Plan(m, n, prec=prec, max_iter=5)
     U3, H3, i3 = plan(a, raw_status=True)
     plan.close()
     assert i3["status"] == lib.POLAR_NOT_CONVERGED and i3["iters"] == 5 and len(i3["res_hist"]) == 6
     assert i3["res_hist"] == i1["res_hist"][:6]
     assert bool(torch.isfinite(U3).all()) and bool(torch.isfinite(H3).all())
+
+
+@pytest.mark.parametrize("ta", [False, True])
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("M,N,K,off", [(31, 33, 1, 0), (32, 64, 64, 0), (100, 700, 130, 1), (700, 40, 129, 0),
+                                       (1100, 1000, 65, 1)], ids=lambda v: str(v))
+def test_fp32_products_in_small_tiles(lib, ta, tb, M, N, K, off):
+    """Both storage orders of both operands, tile and chunk remainders, aligned rows and rows that are not
+    (a view one element into a wider matrix), with C read and written in place."""
+    import torch
+
+    from .gpu_util import gemm_bound
+    rng = np.random.default_rng(M + N + K)
+    a = rng.standard_normal((K, M) if ta else (M, K)).astype(np.float32)
+    b = rng.standard_normal((N, K) if tb else (K, N)).astype(np.float32)
+    c = rng.standard_normal((M, N)).astype(np.float32)
+
+    def view(x):
+        big = torch.full((x.shape[0] + 1, x.shape[1] + 3 * off), float("nan"), device="cuda")
+        v = big[:x.shape[0], off:off + x.shape[1]]
+        v.copy_(torch.from_numpy(x))
+        return v
+
+    C = torch.from_numpy(c).cuda()
+    lib.polar_gemm(view(a), view(b), C, ta, tb, 0.75, -1.25, lib.POLAR_FP32)
+    A64 = (a.T if ta else a).astype(np.float64)
+    B64 = (b.T if tb else b).astype(np.float64)
+    err = np.abs(to_np(C).astype(np.float64) - (0.75 * A64 @ B64 - 1.25 * c.astype(np.float64)))
+    assert np.all(err <= gemm_bound(np.abs(A64), np.abs(B64), K, np.abs(c), 0.75, -1.25))
 
 
 # sizes of the inverse's and the Chebyshev function's dispatch and tiles that their own tests do not reach:
