@@ -1,5 +1,5 @@
 // The Newton-Schulz inverse (Algorithm 2) and the Chebyshev matrix function (Clenshaw summation), each as one
-// cooperative launch, for matrices whose products are one or two waves of 128 x 64 or 128 x 128 tiles; the
+// cooperative launch, for matrices whose products are a few waves of 128 x 64 or 128 x 128 tiles; the
 // pieces are in coop_kernel.cuh. What bounds them there is what bounds the solve: with separate launches a
 // 1001 x 1001 product ran as 32 tiles of 128 x 256 (56 us, and 145 us for a Clenshaw step at 1536 with its
 // mirrored two-byte stores); here it is 128 tiles, and a Clenshaw step stores only the upper triangle.

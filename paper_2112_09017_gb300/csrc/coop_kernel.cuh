@@ -1,5 +1,5 @@
 // Persistent cooperative kernels: a whole chain of split-BF16 tensor-core products (three planes, six
-// passes) in one launch, for sizes at which a product is one or two waves of small tiles. The chain's
+// passes) in one launch, for sizes at which a product is a few waves of small tiles. The chain's
 // products depend on each other through global memory, so a grid barrier separates them; what it replaces
 // per product is a kernel launch, the set-up of barriers, TMEM and descriptors, and the small kernels
 // between the products (residual and stop rule, mirror).

@@ -1,5 +1,5 @@
 // One polar solve in one cooperative launch (Sec. III.D, Eq. NewtonSchulz, Algorithm 1), for matrices whose
-// products are one or two waves of 128 x 64 or 128 x 128 tiles; the pieces are in coop_kernel.cuh.
+// products are a few waves of 128 x 64 or 128 x 128 tiles; the pieces are in coop_kernel.cuh.
 //
 //   ||A||_F | X_0 = A / ||A||_F and the planes of A | per step: Gram | update | ... | U^T A | U, H
 //
@@ -255,21 +255,35 @@ struct CoopSolve {
   int tn, grid;
 };
 
-// Width of the chain's tiles for products of m x n, or 0 where the separate launches are faster. A 64-wide
-// tile takes about 5/9 of a 128-wide one's time, so it is taken while it does not need more waves than that
-// makes up for. One launch against separate ones, per solve at kappa 100: 96 x 64 202 against 915 us, 512^2
-// 503 against 1713, 1024^2 827 against 2411, 2048^2 (two waves of 128-wide tiles) 2637 against 4063, 8192 x
-// 512 3370 against 6016. Beyond two waves the separate launches' 256-wide tiles and CTA pairs take over: a
-// wave's length then hides what a launch costs.
-int coop_tile_n(int64_t m, int64_t n, int sms) {
-  const int64_t t64 = co_tiles<64>(m, n, false).ntiles, t128 = co_tiles<128>(m, n, false).ntiles;
-  const int64_t w64 = (t64 + sms - 1) / sms, w128 = (t128 + sms - 1) / sms;
-  if (m * n > (int64_t)1 << 24 || w128 > 2) return 0;
-  return w64 * 5 <= w128 * 9 ? 64 : 128;
+// Cycles of a chain's products with tiles of one width: whole waves, a k-block of 32 costing about 820 cycles
+// with 64-wide tiles and 950 with 128-wide ones (measured inside the solve; the MMAs alone take 595 and 790),
+// a tile's output step about 4000 and 7000. Waves: the most of any product.
+template <int TN>
+static double co_cost(const CoopProduct* p, int count, int sms, int64_t* waves) {
+  double c = 0.0;
+  *waves = 0;
+  for (int i = 0; i < count; ++i) {
+    const int64_t w = ((int64_t)co_tiles<TN>(p[i].M, p[i].N, p[i].tri).ntiles + sms - 1) / sms;
+    c += (double)w * ((double)((p[i].K + BK - 1) / BK) * (TN == 64 ? 820.0 : 950.0) + (TN == 64 ? 4000.0 : 7000.0));
+    *waves = std::max(*waves, w);
+  }
+  return c;
+}
+
+// One launch against separate ones, per step at kappa 100: 512^2 23 against 84 us, 1024^2 36 against 111, 2048^2
+// 113 against 174, 3072^2 326 against 445, 8192 x 2048 (7 waves of 128-wide tiles) 415 against 563, 4096^2 (7)
+// 805 against 838; 8192^2 (27 waves) 6782 against 5700, where the CTA pairs' 256 x 256 tiles read a third less
+// from L2. So the line lies at eight waves.
+int coop_tile_n(const CoopProduct* p, int count, int sms) {
+  int64_t w64, w128;
+  const double c64 = co_cost<64>(p, count, sms, &w64), c128 = co_cost<128>(p, count, sms, &w128);
+  if (w128 > 8) return 0;
+  return c64 <= c128 ? 64 : 128;
 }
 
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {
-  const int tn = coop_tile_n(m, n, sms);
+  const CoopProduct prod[2] = {{n, n, m, true}, {m, n, n, false}};
+  const int tn = coop_tile_n(prod, 2, sms);
   if (!tn) return nullptr;
   CoopSolve* c = new (std::nothrow) CoopSolve();
   if (!c) return nullptr;

@@ -249,8 +249,8 @@ int tc_withhold();                                // test hook: 1 when producers
 bool tc_forced_form();                            // the environment names the single-CTA or the CTA-pair form
 
 // ---------------------------------------------------------------------------------
-// One solve in one cooperative launch (coop_solve.cu), for sizes whose products are one or two waves of
-// small tiles, three planes. The buffers are the plan's.
+// One solve in one cooperative launch (coop_solve.cu), for sizes whose products are a few waves of small
+// tiles, three planes. The buffers are the plan's.
 struct CoopBuffers {
   uint16_t* xp[2];
   uint16_t* gp;
@@ -285,7 +285,11 @@ cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U,
 
 // The inverse and the Chebyshev function in one cooperative launch (coop_funcs.cu), three planes. The
 // caller provides the plane buffers (no initial contents needed) and a state whose barrier words are zero.
-int coop_tile_n(int64_t m, int64_t n, int sms);   // tile width for products of up to m x n; 0: not for this size
+struct CoopProduct {
+  int64_t M, N, K;
+  bool tri;                                       // only the upper triangle's tiles
+};
+int coop_tile_n(const CoopProduct* p, int count, int sms);   // tile width of a chain; 0: not for these sizes
 constexpr int COOP_MAX_DEGREE = 511;
 struct CoopInverseArgs {
   const float* A; int64_t rows, cols, lda;

@@ -1116,7 +1116,8 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   if (wr != POLAR_OK) return wr;
   uint8_t* w = call.dev();
   // small and medium matrices: the whole iteration in one cooperative launch
-  const int tn = prec == POLAR_BF16X6 && !tc_forced_form() ? coop_tile_n(N, N, sms) : 0;
+  const CoopProduct prod[2] = {{N, N, M, false}, {M, N, N, false}};
+  const int tn = prec == POLAR_BF16X6 && !tc_forced_form() ? coop_tile_n(prod, 2, sms) : 0;
   if (tn) {
     DevState* st = (DevState*)(w + o_st);
     if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
@@ -1291,8 +1292,9 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
   uint16_t* bk[3] = {(uint16_t*)(w + o_b0), (uint16_t*)(w + o_b1), (uint16_t*)(w + o_b2)};
   DevState* st = (DevState*)(w + o_st);
   // small and medium matrices: every step in one cooperative launch
+  const CoopProduct prod = {n, n, n, true};
   const int tn = prec == POLAR_BF16X6 && degree >= 2 && degree <= COOP_MAX_DEGREE && !tc_forced_form()
-                     ? coop_tile_n(n, n, sms) : 0;
+                     ? coop_tile_n(&prod, 1, sms) : 0;
   if (tn) {
     if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
     CoopChebArgs c{};
