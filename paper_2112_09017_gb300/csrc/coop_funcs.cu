@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
     for (int u = gtid; u < N * c8; u += gthr) {
       const int r = u / c8, c = (u - r * c8) * 8;
       float v[8];
-      co_load8(p.A + (int64_t)r * p.lda + c, M - c, vec, v);
+      load_row8(p.A + (int64_t)r * p.lda + c, M - c, vec, v);
       store_planes8(p.ap + (int64_t)r * p.lpa + c, p.sa, 3, v);
     }
     if (gtid == 0) {
@@ -62,14 +62,15 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
   if (run) {
     const CoTiles t = co_tiles<TN>(M, M, true);
     if (x.warp == 0) {
-      if (x.lane == 0) co_producer<TN, true, false>(x, pipe, &p.amn, &p.amn, nullptr, t, N, p.withhold);
+      if (x.lane == 0)
+        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.amn, &p.amn, nullptr, t, N), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, true, false>(x, pipe, t, N);
+      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, t, N));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = M; e.N = M;
       e.norm = p.norm;
-      co_epilogue<TN, CO_EPI_NORM>(x, pipe, e, t, N);
+      co_epilogue<TN, CO_EPI_NORM>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, t, N, &e));
     }
     run = co_grid_sync(x);
   }
@@ -116,14 +117,15 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
   for (; run; ++k) {
     const int b = k & 1;
     if (x.warp == 0) {
-      if (x.lane == 0) co_producer<TN, false, false>(x, pipe, &p.ak, &p.xmn[b], nullptr, ta, M, p.withhold);
+      if (x.lane == 0)
+        co_producer<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(&p.ak, &p.xmn[b], nullptr, ta, M), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, false, false>(x, pipe, ta, M);
+      co_mma<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, ta, M));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = N; e.N = N;
       e.out = p.pp; e.ldo = p.lpx; e.os = p.sp;
-      co_epilogue<TN, TC_EPI_PLANES>(x, pipe, e, ta, M);
+      co_epilogue<TN, TC_EPI_PLANES>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, ta, M, &e));
     } else if (k > 0) {
       // Algorithm 2's test after update k - 1: ||X' - X||_F / ||X'||_F against u 2^(k-1), u = 2^-24
       const double sd = co_warp_sum2(p.part, gridDim.x * EPI_WARPS, 2, x.lane);
@@ -151,9 +153,10 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
     else status = ST_RUNNING;
     if (status != ST_RUNNING) break;
     if (x.warp == 0) {
-      if (x.lane == 0) co_producer<TN, false, false>(x, pipe, &p.xk[b], &p.pmn, nullptr, tu, N, p.withhold);
+      if (x.lane == 0)
+        co_producer<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(&p.xk[b], &p.pmn, nullptr, tu, N), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, false, false>(x, pipe, tu, N);
+      co_mma<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, N));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = M; e.N = N;
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
       e.out = p.xp[b ^ 1]; e.ldo = p.lpx; e.os = p.sx;
       e.c1 = 2.0f; e.c3 = -1.0f;
       e.part = p.part;
-      co_epilogue<TN, TC_EPI_NS_STEP>(x, pipe, e, tu, N);
+      co_epilogue<TN, TC_EPI_NS_STEP>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, N, &e));
     }
     run = co_grid_sync(x);
   }
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
       const int r = u / c8, c = (u - r * c8) * 8;
       float v[8];
       sum_planes8(load_planes8(X + (int64_t)r * p.lpx + c, p.sx, true), v);
-      co_store8(p.X + (int64_t)r * p.ldx + c, N - c, vec, v);
+      store_row8(p.X + (int64_t)r * p.ldx + c, N - c, vec, v);
     }
   }
   co_teardown<TN>(x, st);
@@ -254,9 +257,9 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_con
   for (int k = d - 2; k >= 0 && run; --k) {
     if (x.warp == 0) {
       if (x.lane == 0)
-        co_producer<TN, true, true>(x, pipe, &p.tmn, &p.bmn[(k + 1) % 3], &p.bk[(k + 1) % 3], tt, n, p.withhold);
+        co_producer<TN, CO_P, true, true>(x, pipe, CoChainSrc<TN>(&p.tmn, &p.bmn[(k + 1) % 3], &p.bk[(k + 1) % 3], tt, n), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, true, true>(x, pipe, tt, n);
+      co_mma<TN, CO_P, true, true>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tt, n));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = n; e.N = n;
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_con
       e.c1 = -1.0f;
       e.c3 = k > 0 ? 2.0f : 1.0f;
       e.diag = p.coef[k];
-      co_epilogue<TN, TC_EPI_CLENSHAW>(x, pipe, e, tt, n);
+      co_epilogue<TN, TC_EPI_CLENSHAW>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tt, n, &e));
     }
     run = co_grid_sync(x);
   }

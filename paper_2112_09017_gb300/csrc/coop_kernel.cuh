@@ -22,21 +22,21 @@
 namespace polar {
 namespace {
 
-constexpr int CO_P = 3;
+constexpr int CO_P = 3;                     // planes of the chains (the batched ones take 1, 2 or 3)
 constexpr int CO_THREADS = NTHREADS + 32;   // one warp more, for what must not hold up the products: the stop test
 constexpr int CO_WARPS = CO_THREADS / 32;
 constexpr int CO_CTL_WARP = CO_WARPS - 1;
 constexpr int CO_EPI_NORM = 16;             // beside the TcEpi kinds: no output, ||C||_F^2 of a symmetric product
 
-template <int TN>
+template <int TN, int P = CO_P>
 struct CoCfg {
   // A stage holds SUB k-blocks of 32: with 64-wide tiles two, because the twelve short MMAs of one do not
   // cover the waits and commits of a stage (measured at 512 x 512: about 940 cycles per k-block against 595
   // of products).
   static constexpr int SUB = TN == 64 ? 2 : 1;
   static constexpr int STAGES = TN == 64 ? 3 : 4;          // 72 or 48 KiB each
-  static constexpr uint32_t A_BYTES = CO_P * A_PLANE;      // of one k-block
-  static constexpr uint32_t B_BYTES = CO_P * TN * BK * 2;
+  static constexpr uint32_t A_BYTES = P * A_PLANE;         // of one k-block
+  static constexpr uint32_t B_BYTES = P * TN * BK * 2;
   static constexpr uint32_t KB_BYTES = A_BYTES + B_BYTES;
   static constexpr uint32_t STAGE_BYTES = SUB * KB_BYTES;
   static constexpr int BKS = SUB * BK;                     // K of one stage
@@ -55,8 +55,10 @@ struct CoCtl {
   int status;              // of the last stop test
 };
 
-template <int TN>
-constexpr size_t co_smem() { return (size_t)CoCfg<TN>::STAGES * CoCfg<TN>::STAGE_BYTES + sizeof(CoCtl) + 1024; }
+template <int TN, int P = CO_P>
+constexpr size_t co_smem() {
+  return (size_t)CoCfg<TN, P>::STAGES * CoCfg<TN, P>::STAGE_BYTES + sizeof(CoCtl) + 1024;
+}
 
 // What a role carries from one product to the next.
 struct CoPipe {
@@ -114,6 +116,42 @@ __device__ __forceinline__ void co_coords(const CoTiles& c, int t, int& bi, int&
   }
 }
 
+// What the roles need of one tile: its operand maps, place, K, and stages per promoted slice.
+struct CoTile {
+  const CUtensorMap* ma;
+  const CUtensorMap* mb;
+  const CUtensorMap* mbt;    // the mirrored (K-major) map of a B whose upper triangle alone is stored
+  int bi, bj, K;
+  int slice;                 // k-blocks of 32 per promoted slice
+};
+
+struct CoEpi;
+
+// Tiles of one product of a chain: this block's are blockIdx.x, blockIdx.x + gridDim.x, ...
+template <int TN>
+struct CoChainSrc {
+  static constexpr bool TABLE = false;
+  const CUtensorMap *ma, *mb, *mbt;
+  CoTiles ct;
+  int K;
+  const CoEpi* e;
+  int t;
+  __device__ __forceinline__ CoChainSrc(const CUtensorMap* a, const CUtensorMap* b, const CUtensorMap* bt, CoTiles c,
+                                        int k, const CoEpi* ep = nullptr)
+      : ma(a), mb(b), mbt(bt), ct(c), K(k), e(ep), t((int)blockIdx.x) {}
+  __device__ __forceinline__ bool next(CoTile& c) {
+    if (t >= ct.ntiles) return false;
+    co_coords<TN>(ct, t, c.bi, c.bj);
+    t += (int)gridDim.x;
+    c.ma = ma; c.mb = mb; c.mbt = mbt;
+    c.K = K;
+    c.slice = 64 / BK;
+    return true;
+  }
+  __device__ __forceinline__ void poke(bool) {}
+  __device__ __forceinline__ const CoEpi& epi(const CoTile&) { return *e; }
+};
+
 // First k of the B operand that a column tile at n0 reads from the mirrored place: the rows above it were
 // stored by the upper triangle's tiles (whole 128-row tiles that hold an entry on or above the diagonal).
 template <int TN>
@@ -121,9 +159,9 @@ __device__ __forceinline__ int co_mirror_from(int n0) { return 128 * ((n0 + TN -
 
 // ------------------------------------------------------------------ set-up, grid barrier, teardown
 
-template <int TN>
+template <int TN, int P = CO_P>
 __device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
-  using C = CoCfg<TN>;
+  using C = CoCfg<TN, P>;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   CoCtl* ctl = reinterpret_cast<CoCtl*>(smem + C::STAGES * C::STAGE_BYTES);
   CoCtx x{ctl, smem, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort)};
@@ -168,19 +206,11 @@ __device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
 // issues from here on.
 __device__ __forceinline__ void co_fence_proxy() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
-// s + e = a + b exactly (Knuth's two-sum): the sums of a product's tiles go through FP32 pairs, because a
-// chain of FP64 additions takes longer than the rest of the output step on this part.
-__device__ __forceinline__ void two_sum(float2& s, float2 b) {
-  const float t = s.x + b.x, bb = t - s.x;
-  const float e = (s.x - (t - bb)) + (b.x - bb);
-  s = make_float2(t, s.y + (b.y + e));
-}
-
 __device__ __forceinline__ bool co_grid_sync(CoCtx& x) { return x.bar.sync(); }
 
 // Leaves the kernel: every thread of the block, after its last product. Reports an expired wait.
 template <int TN>
-__device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st) {
+__device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st, int* err_word = nullptr) {
   if (x.warp == 1 && x.lane == 0) {   // every MMA issued has completed before TMEM is released
     tc_commit(x.br.drain);
     mbar_drain(x.br.drain, 0);
@@ -188,8 +218,11 @@ __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st) {
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *x.abort_flag) {
-    atomicOr(&st->err_flags, 1u);
-    st->status = ST_TIMEOUT;
+    if (err_word) atomicOr(err_word, 1);
+    if (st) {
+      atomicOr(&st->err_flags, 1u);
+      st->status = ST_TIMEOUT;
+    }
   }
   x.bar.leave();
   if (x.warp == 1) {
@@ -204,22 +237,21 @@ __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st) {
 // All in line, so that what they carry stays in registers: the grid barrier's acquire empties L1, and a
 // context kept in local memory for calls was read back from L2 at the start of every product.
 
-// mbt: the mirrored (K-major) map of B for SYM, whose upper triangle alone is stored.
-template <int TN, bool A_MN, bool SYM>
-__device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, const CUtensorMap* ma, const CUtensorMap* mb,
-                                         const CUtensorMap* mbt, CoTiles ct, int K, int withhold) {
-  using C = CoCfg<TN>;
+// SYM: B is symmetric and only its upper triangle is stored.
+template <int TN, int P, bool A_MN, bool SYM, class Src>
+__device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src, int withhold) {
+  using C = CoCfg<TN, P>;
   if (withhold) return;   // test hook: no copies are issued, the consumers' bounded waits expire
   co_fence_proxy();
   int stage = pp.stage;
   uint32_t phase = pp.phase;
   bool ok = true;
   uint32_t armed = 0, armed_phase = 0;
-  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
-    int bi, bj;
-    co_coords<TN>(ct, t, bi, bj);
-    const int m0 = bi * BM, n0 = bj * TN;
+  CoTile c;
+  while (ok && src.next(c)) {
+    const int m0 = c.bi * BM, n0 = c.bj * TN, K = c.K;
     const int km = SYM ? co_mirror_from<TN>(n0) : 0x7fffffff;
+    const CUtensorMap *ma = c.ma, *mb = c.mb, *mbt = c.mbt;
     for (int k0 = 0; k0 < K; k0 += C::BKS) {
       if (!mbar_wait(x.br.empty0 + 8 * stage, phase ^ 1u, x.abort_flag)) { ok = false; break; }
       const uint32_t fb = x.br.full0 + 8 * stage;
@@ -233,18 +265,19 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, const CU
         const uint32_t a_dst = x.smem_base + stage * C::STAGE_BYTES + s * C::KB_BYTES, b_dst = a_dst + C::A_BYTES;
         if (A_MN) {
 #pragma unroll
-          for (int cc = 0; cc < BM / 64; ++cc) tma_load_3d(a_dst + cc * CO_P * MN_CHUNK, ma, fb, m0 + 64 * cc, k, 0);
+          for (int cc = 0; cc < BM / 64; ++cc) tma_load_3d(a_dst + cc * P * MN_CHUNK, ma, fb, m0 + 64 * cc, k, 0);
         } else {
           tma_load_3d(a_dst, ma, fb, k, m0, 0);
         }
         if (k < km) {
 #pragma unroll
-          for (int cc = 0; cc < TN / 64; ++cc) tma_load_3d(b_dst + cc * CO_P * MN_CHUNK, mb, fb, n0 + 64 * cc, k, 0);
+          for (int cc = 0; cc < TN / 64; ++cc) tma_load_3d(b_dst + cc * P * MN_CHUNK, mb, fb, n0 + 64 * cc, k, 0);
         } else {
           tma_load_3d(b_dst, mbt, fb, k, n0, 0);
         }
       }
       if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+      if (k0 == 0) src.poke(true);
     }
   }
   pp.stage = stage;
@@ -256,13 +289,13 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, const CU
 
 // The whole warp runs the loop and one elected lane issues, a stage's waits between the halves of the stage
 // before it (see role_mma; with four slice buffers the wait for one is rarely a real one).
-template <int TN, bool A_MN, bool SYM>
-__device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, CoTiles ct, int K) {
-  using C = CoCfg<TN>;
+template <int TN, int P, bool A_MN, bool SYM, class Src>
+__device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, Src src) {
+  using C = CoCfg<TN, P>;
   const bool issuer = elect_one();
-  const uint64_t a0 = A_MN ? smem_desc(x.smem_base, CO_P * MN_CHUNK, 1024, 2)
+  const uint64_t a0 = A_MN ? smem_desc(x.smem_base, P * MN_CHUNK, 1024, 2)
                            : smem_desc(x.smem_base, 16, KM_SBO, KM_SWZ);
-  const uint64_t bm0 = smem_desc(x.smem_base + C::A_BYTES, CO_P * MN_CHUNK, 1024, 2);
+  const uint64_t bm0 = smem_desc(x.smem_base + C::A_BYTES, P * MN_CHUNK, 1024, 2);
   const uint64_t bk0 = smem_desc(x.smem_base + C::A_BYTES, 16, KM_SBO, KM_SWZ);
   const Bars br = x.br;
   volatile int* abort_flag = x.abort_flag;
@@ -270,15 +303,15 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, CoTiles ct, i
   int stage = pp.stage, buf = pp.buf;
   uint32_t phase = pp.phase, buf_phase = pp.buf_phase;
   bool ok = true;
-  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
-    int bi, bj;
-    co_coords<TN>(ct, t, bi, bj);
-    const int km = SYM ? co_mirror_from<TN>(bj * TN) : 0x7fffffff;
+  CoTile c;
+  while (ok && src.next(c)) {
+    const int K = c.K, kin_last = Src::TABLE ? c.slice / C::SUB - 1 : C::SLICE - 1;
+    const int km = SYM ? co_mirror_from<TN>(c.bj * TN) : 0x7fffffff;
     int kin = 0;
     ok = mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag) &&
          mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag);
     for (int k0 = 0; k0 < K && ok; k0 += C::BKS) {
-      const bool last = kin == C::SLICE - 1 || k0 + C::BKS >= K;
+      const bool last = kin == kin_last || k0 + C::BKS >= K;
       const uint32_t d = tmem + (uint32_t)(buf * TN), acc = kin == 0 ? 0u : 1u;
       const uint64_t so = (uint64_t)((stage * C::STAGE_BYTES) >> 4);
       const int this_stage = stage, this_buf = buf;
@@ -287,13 +320,14 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, CoTiles ct, i
       if (issuer) {
         // km and the stages are multiples of 64: a stage lies on one side of it
         if (k0 < km) {
-          issue_half<CO_P, A_MN, true, CO_P, TN, 1, 0>(d, a0 + so, bm0 + so, acc);
-          if (two) issue_half<CO_P, A_MN, true, CO_P, TN, 1, 1>(d, a0 + so, bm0 + so, 1u);
+          issue_half<P, A_MN, true, P, TN, 1, 0>(d, a0 + so, bm0 + so, acc);
+          if (two) issue_half<P, A_MN, true, P, TN, 1, 1>(d, a0 + so, bm0 + so, 1u);
         } else {
-          issue_half<CO_P, A_MN, false, CO_P, TN, 1, 0>(d, a0 + so, bk0 + so, acc);
-          if (two) issue_half<CO_P, A_MN, false, CO_P, TN, 1, 1>(d, a0 + so, bk0 + so, 1u);
+          issue_half<P, A_MN, false, P, TN, 1, 0>(d, a0 + so, bk0 + so, acc);
+          if (two) issue_half<P, A_MN, false, P, TN, 1, 1>(d, a0 + so, bk0 + so, 1u);
         }
       }
+      if (k0 == 0) src.poke(false);
       if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       if (last) {
         if (++buf == C::NBUF) { buf = 0; buf_phase ^= 1u; }
@@ -307,11 +341,11 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, CoTiles ct, i
       if (issuer) {
         const uint64_t so2 = so + (two ? (uint64_t)(C::KB_BYTES >> 4) : 0u);
         if (k0 < km) {
-          if (two) issue_half<CO_P, A_MN, true, CO_P, TN, 1, 0>(d, a0 + so2, bm0 + so2, 1u);
-          issue_half<CO_P, A_MN, true, CO_P, TN, 1, 1>(d, a0 + so2, bm0 + so2, 1u);
+          if (two) issue_half<P, A_MN, true, P, TN, 1, 0>(d, a0 + so2, bm0 + so2, 1u);
+          issue_half<P, A_MN, true, P, TN, 1, 1>(d, a0 + so2, bm0 + so2, 1u);
         } else {
-          if (two) issue_half<CO_P, A_MN, false, CO_P, TN, 1, 0>(d, a0 + so2, bk0 + so2, 1u);
-          issue_half<CO_P, A_MN, false, CO_P, TN, 1, 1>(d, a0 + so2, bk0 + so2, 1u);
+          if (two) issue_half<P, A_MN, false, P, TN, 1, 0>(d, a0 + so2, bk0 + so2, 1u);
+          issue_half<P, A_MN, false, P, TN, 1, 1>(d, a0 + so2, bk0 + so2, 1u);
         }
         tc_commit(br.empty0 + 8 * this_stage);
         if (last) tc_commit(br.tfull0 + 8 * this_buf);
@@ -338,27 +372,28 @@ struct CoEpi {
   float diag;
   float2* part;              // GRAM: per epilogue warp of every block; NS_STEP: two each
   double* norm;              // NORM: per epilogue warp of every block
+  double* tile_part;         // GRAM from a table: this tile's EPI_WARPS sums
 };
 
 // Sums over each warp's tiles, as unevaluated pairs hi + lo, go to e.part: GRAM ||G - I||_F^2; NS_STEP
 // ||X' - X||^2 and ||X'||^2. NORM's go to e.norm, in float64 (entries of any magnitude).
-template <int TN, int EPI>
-__device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const CoEpi& e, CoTiles ct, int K) {
+template <int TN, int EPI, class Src>
+__device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src) {
   using C = CoCfg<TN>;
   constexpr int CW = C::CW, NCH = CW / 32;
   constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP, STEP = EPI == TC_EPI_NS_STEP;
   constexpr bool READS_X = NS || EPI == TC_EPI_CLENSHAW;
   const int q = x.warp & 3, half = (x.warp - 2) >> 2, lane = x.lane, lq = lane & 3;
   const uint32_t t_lane = x.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * CW);
-  const int nslices = (K + 63) / 64;
   int buf = pp.buf;
   uint32_t buf_phase = pp.buf_phase;
   float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
   double norm = 0.0;
   bool ok = true;
-  for (int t = blockIdx.x; t < ct.ntiles && ok; t += gridDim.x) {
-    int bi, bj;
-    co_coords<TN>(ct, t, bi, bj);
+  CoTile ti;
+  while (ok && src.next(ti)) {
+    const CoEpi& e = src.epi(ti);
+    const int bi = ti.bi, bj = ti.bj, nslices = (ti.K + ti.slice * BK - 1) / (ti.slice * BK);
     const int r = bi * BM + q * 32 + lane, r4 = r - lq;
     const int cb = bj * TN + half * CW;
     unsigned rows4 = 0;
@@ -387,6 +422,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
       __syncwarp();
       if (lane == 0) mbar_arrive(x.br.tempty0 + 8 * buf);
       if (++buf == C::NBUF) { buf = 0; buf_phase ^= 1u; }
+      if (sl == 0) src.poke(false);
     }
     if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
     float d2 = 0.f, x2 = 0.f;
@@ -463,11 +499,17 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
           }
           if (rows4 & (1u << i)) store_planes8(pr + i * e.ldo, e.os, 3, v + 8 * i);
         }
-      } else {   // STORE (the pitch is a multiple of 4: whole 16-byte groups up to it)
+      } else {   // STORE: whole 16-byte groups up to a pitch that is a multiple of 4, else single entries
         float* cr = e.C + r4 * e.ldc + c0 + 8 * lq;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (!(rows4 & (1u << i))) continue;
+          if (Src::TABLE && (e.ldc & 3)) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (c0 + 8 * lq + j < e.N) cr[i * e.ldc + j] = v[8 * i + j];
+            continue;
+          }
           if (c0 + 8 * lq < e.ldc)
             *reinterpret_cast<float4*>(cr + i * e.ldc) = make_float4(v[8 * i], v[8 * i + 1], v[8 * i + 2], v[8 * i + 3]);
           if (c0 + 8 * lq + 4 < e.ldc)
@@ -475,6 +517,13 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
                 make_float4(v[8 * i + 4], v[8 * i + 5], v[8 * i + 6], v[8 * i + 7]);
         }
       }
+    }
+    if (Src::TABLE && EPI == TC_EPI_GRAM) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
+      if (lane == 0) e.tile_part[x.warp - 2] = (double)sum0.x + (double)sum0.y;
+      sum0 = make_float2(0.f, 0.f);
     }
     if (STEP) {
       two_sum(sum0, make_float2(d2, 0.f));
@@ -486,9 +535,10 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, const Co
   if (EPI == CO_EPI_NORM) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
-    if (lane == 0) __stcg(e.norm + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
+    if (lane == 0) __stcg(src.epi(ti).norm + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
   }
-  if (EPI == TC_EPI_GRAM || STEP) {
+  if (!Src::TABLE && (EPI == TC_EPI_GRAM || STEP)) {
+    const CoEpi& e = src.epi(ti);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
@@ -533,30 +583,6 @@ __device__ __forceinline__ double co_block_sum(CoCtx& x, double v) {
   if (threadIdx.x == 0)
     for (int w = 0; w < CO_WARPS; ++w) t += x.ctl->red[w];
   return t;
-}
-
-// 8 consecutive values of a float32 row, `n` of them existing (zeros beyond), 16-byte loads when vec.
-__device__ __forceinline__ void co_load8(const float* p, int n, bool vec, float (&v)[8]) {
-  if (vec && n >= 8) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = j < n ? __ldg(p + j) : 0.0f;
-  }
-}
-
-// The reverse for stores.
-__device__ __forceinline__ void co_store8(float* p, int n, bool vec, const float (&v)[8]) {
-  if (vec && n >= 8) {
-    reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (j < n) p[j] = v[j];
-  }
 }
 
 }  // namespace

@@ -65,15 +65,14 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
   bool run = true;
   // ---- ||A||_F, float64 sums in a fixed order
   {
-    double acc = 0.0;
+    SquareSum acc;
     for (int u = gtid; u < m * c8n; u += gthr) {
       const int r = u / c8n, c = (u - r * c8n) * 8;
       float v[8];
-      co_load8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc = fma((double)v[j], (double)v[j], acc);
+      load_row8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
+      acc.add8(v);
     }
-    const double t = co_block_sum(x, acc);
+    const double t = co_block_sum(x, acc.value());
     if (tid == 0) p.partials[blockIdx.x] = t;
     run = co_grid_sync(x);
   }
@@ -98,7 +97,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
       for (int u = gtid; u < m * c8n; u += gthr) {
         const int r = u / c8n, c = (u - r * c8n) * 8;
         float v[8], y[8];
-        co_load8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
+        load_row8(p.A + (int64_t)r * p.lda + c, n - c, vec_a, v);
 #pragma unroll
         for (int j = 0; j < 8; ++j) y[j] = __fdiv_rn(v[j], s);
         const int64_t o = (int64_t)r * p.ldp + c;
@@ -116,24 +115,26 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
     const int b = k & 1;
     // Gram of X_k: the upper triangle's tiles, and this block's part of ||G - I||_F^2
     if (x.warp == 0) {
-      if (x.lane == 0) co_producer<TN, true, false>(x, pipe, &p.xmn[b], &p.xmn[b], nullptr, tg, m, p.withhold);
+      if (x.lane == 0)
+        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.xmn[b], &p.xmn[b], nullptr, tg, m), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, true, false>(x, pipe, tg, m);
+      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tg, m));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = n; e.N = n;
       e.out = p.gp; e.ldo = p.ldp; e.os = p.gps;
       e.part = p.part2;
-      co_epilogue<TN, TC_EPI_GRAM>(x, pipe, e, tg, m);
+      co_epilogue<TN, TC_EPI_GRAM>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tg, m, &e));
     }
     run = co_grid_sync(x);
     if (!run) break;
     // the update, and beside it the stop test of X_k and its record
     if (k < p.max_iter) {
       if (x.warp == 0) {
-        if (x.lane == 0) co_producer<TN, false, true>(x, pipe, &p.xk[b], &p.gmn, &p.gk, tu, n, p.withhold);
+        if (x.lane == 0)
+        co_producer<TN, CO_P, false, true>(x, pipe, CoChainSrc<TN>(&p.xk[b], &p.gmn, &p.gk, tu, n), p.withhold);
       } else if (x.warp == 1) {
-        co_mma<TN, false, true>(x, pipe, tu, n);
+        co_mma<TN, CO_P, false, true>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, n));
       } else if (x.warp < CO_CTL_WARP) {
         CoEpi e{};
         e.M = m; e.N = n;
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
         e.out = p.xp[b ^ 1]; e.ldo = p.ldp; e.os = p.xps;
         e.c1 = k < p.n_pre ? p.pre_c1 : 1.5f;
         e.c3 = k < p.n_pre ? p.pre_c3 : -0.5f;
-        co_epilogue<TN, TC_EPI_NS>(x, pipe, e, tu, n);
+        co_epilogue<TN, TC_EPI_NS>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, n, &e));
       }
     }
     if (x.warp == CO_CTL_WARP) {
@@ -170,14 +171,15 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
   if (run && (status == ST_CONVERGED || status == ST_NOT_CONVERGED)) {
     const CoTiles th = co_tiles<TN>(n, n, false);
     if (x.warp == 0) {
-      if (x.lane == 0) co_producer<TN, true, false>(x, pipe, &p.xmn[it & 1], &p.amn, nullptr, th, m, p.withhold);
+      if (x.lane == 0)
+        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.xmn[it & 1], &p.amn, nullptr, th, m), p.withhold);
     } else if (x.warp == 1) {
-      co_mma<TN, true, false>(x, pipe, th, m);
+      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, th, m));
     } else if (x.warp < CO_CTL_WARP) {
       CoEpi e{};
       e.M = n; e.N = n;
       e.C = p.C; e.ldc = p.ldc;
-      co_epilogue<TN, TC_EPI_STORE>(x, pipe, e, th, m);
+      co_epilogue<TN, TC_EPI_STORE>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, th, m, &e));
     }
     run = co_grid_sync(x);
     if (run) {
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
         const int r = u / c8n, c = (u - r * c8n) * 8;
         float v[8];
         sum_planes8(load_planes8(X + (int64_t)r * p.ldp + c, p.xps, true), v);
-        co_store8(p.U + (int64_t)r * p.ldu + c, n - c, vec_u, v);
+        store_row8(p.U + (int64_t)r * p.ldu + c, n - c, vec_u, v);
       }
       // H by pairs of 32 x 32 tiles (bi <= bj) through shared memory (the stages are idle)
       float* ta = reinterpret_cast<float*>(x.smem);

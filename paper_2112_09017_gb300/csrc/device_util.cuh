@@ -28,6 +28,108 @@ __device__ __forceinline__ void split_planes_dev(float x, uint16_t (&planes)[3])
   }
 }
 
+// s + e = a + b exactly (Knuth's two-sum), accumulated into the unevaluated pair s.x + s.y.
+__device__ __forceinline__ void two_sum(float2& s, float2 b) {
+  const float t = s.x + b.x, bb = t - s.x;
+  const float e = (s.x - (t - bb)) + (b.x - bb);
+  s = make_float2(t, s.y + (b.y + e));
+}
+
+// A float64-grade sum of squares of float32 values. FP64 runs at 1/64 of the FP32 rate here (two FMAs a cycle
+// and SM), which made the norm of a batch take longer than reading it; so squares are split exactly into FP32
+// pairs (p = x x, e = fma(x, x, -p)) and added by two-sums, about 2^-44 relative, and only every eighth
+// group of eight goes through FP64. Groups whose largest magnitude is outside [2^-50, 2^60], where squares or
+// their errors could leave float32's range, are summed in FP64 as they are.
+struct SquareSum {
+  double total = 0.0;
+  float2 pair = {0.f, 0.f};
+  int held = 0;
+  __device__ __forceinline__ void add8(const float (&v)[8]) {
+    float top = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) top = fmaxf(top, fabsf(v[j]));
+    if (top <= 0x1p60f && (top >= 0x1p-50f || top == 0.f)) {   // a NaN among smaller values passes through the sums
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float q = v[j] * v[j];
+        two_sum(pair, make_float2(q, fmaf(v[j], v[j], -q)));
+      }
+      if (++held == 8) flush();
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) total = fma((double)v[j], (double)v[j], total);
+    }
+  }
+  __device__ __forceinline__ void flush() {
+    total += (double)pair.x + (double)pair.y;
+    pair = make_float2(0.f, 0.f);
+    held = 0;
+  }
+  __device__ __forceinline__ double value() {
+    flush();
+    return total;
+  }
+};
+
+// 8 consecutive values of a float32 row, `n` of them existing (zeros beyond), 16-byte loads when vec.
+__device__ __forceinline__ void load_row8(const float* p, int64_t n, bool vec, float (&v)[8]) {
+  if (vec && n >= 8) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = j < n ? __ldg(p + j) : 0.0f;
+  }
+}
+
+// The reverse for stores.
+__device__ __forceinline__ void store_row8(float* p, int64_t n, bool vec, const float (&v)[8]) {
+  if (vec && n >= 8) {
+    reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < n) p[j] = v[j];
+  }
+}
+
+// np planes of 8 consecutive values, one 16-byte store per plane (base 16-byte aligned, pstride a multiple of 8).
+// Each plane is the round-to-nearest-even BF16 of what the previous planes left.
+__device__ __forceinline__ void split_store8(uint16_t* base, int64_t pstride, int np, const float (&v)[8]) {
+  float r[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) r[j] = v[j];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (q >= np) break;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(r[2 * k + 1]), "f"(r[2 * k]));
+      r[2 * k] -= __uint_as_float(w[k] << 16);
+      r[2 * k + 1] -= __uint_as_float(w[k] & 0xffff0000u);
+    }
+    *reinterpret_cast<uint4*>(base + q * pstride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// The exact sum of three planes' 8 consecutive values.
+__device__ __forceinline__ void sum_row8(const uint16_t* p, int64_t pstride, float (&v)[8]) {
+  uint4 q[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) q[i] = *reinterpret_cast<const uint4*>(p + i * pstride);
+  const uint32_t h[4] = {q[0].x, q[0].y, q[0].z, q[0].w}, m[4] = {q[1].x, q[1].y, q[1].z, q[1].w},
+                 l[4] = {q[2].x, q[2].y, q[2].z, q[2].w};
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    v[2 * w] = (__uint_as_float(h[w] << 16) + __uint_as_float(m[w] << 16)) + __uint_as_float(l[w] << 16);
+    v[2 * w + 1] = (__uint_as_float(h[w] & 0xffff0000u) + __uint_as_float(m[w] & 0xffff0000u)) +
+                   __uint_as_float(l[w] & 0xffff0000u);
+  }
+}
+
 // The strictly lower triangle of a symmetric n x n matrix kept as three BF16 planes (pitch ldp,
 // plane stride ps) from its upper triangle: 64 x 64 blocks (bi <= bj) of the upper triangle, taken
 // t0, t0 + dt, ... in column order, read with 16-byte accesses into shared memory (`tile`, at least

@@ -245,27 +245,3 @@ cudaError_t launch_tc_gemm_fp8(const TcArgs& a_in, cudaStream_t s) {
 }
 
 }  // namespace polar
-
-// ---------------------------------------------------------------- grouped launches
-
-namespace polar {
-
-bool tc_make_entry_maps(TcGroupEntry* e) {
-  const TcArgs& a = e->args;
-  return make_map(reinterpret_cast<CUtensorMap*>(e->map_a), a.a, a.nplanes, !a.a.kmajor, BM) &&
-         make_map(reinterpret_cast<CUtensorMap*>(e->map_b), a.b, a.nplanes, !a.b.kmajor, BN);
-}
-
-cudaError_t launch_tc_gemm_grouped(const TcGroupLaunch& g_in, cudaStream_t s) {
-  TcGroupLaunch g = g_in;
-  if (g.nplanes < 1 || g.nplanes > 3 || !g.tiles || !g.entries) return cudaErrorInvalidValue;
-  if (g.slice_stages <= 0) g.slice_stages = default_slice_stages(g.nplanes);
-  g.withhold_tma = tc_withhold();
-  switch (g.nplanes) {
-    case 1: return tc_dispatch_grouped1(g, s);
-    case 2: return tc_dispatch_grouped2(g, s);
-    default: return tc_dispatch_grouped3(g, s);
-  }
-}
-
-}  // namespace polar

@@ -1,7 +1,8 @@
 // Split-BF16 GEMM / SYRK on the 5th-generation tensor cores (tcgen05, sm_103a): the kernels
 // and their launch templates. The host side (tensor maps, argument checks, the choice of
 // kernel) is gemm_tc.cu; the instantiations are spread over gemm_tc_*.cu so that they
-// compile in parallel.
+// compile in parallel. (Batched solves, and single ones of a few waves of small tiles, run in the
+// cooperative kernels of coop_kernel.cuh on the same pieces.)
 //
 // The products of the Newton-Schulz step (Eq. NewtonSchulz: G = X^T X and
 // X' = 1.5 X - 0.5 X G) and U^T A for H, with FP32 operands given as P BF16
@@ -83,9 +84,7 @@ constexpr uint32_t KM_SBO = 8 * BK * 2;
 constexpr uint32_t KM_SWZ = BK == 16 ? 6 : BK == 32 ? 4 : 2;   // descriptor codes: 32, 64, 128-byte swizzle
 constexpr uint32_t TMEM_COLS = 512;        // two 128 x 256 FP32 slice accumulators
 
-// Tile width TN: 256 (one epilogue group of eight warps, two 256-column TMEM slice buffers)
-// or 128 (two epilogue groups of four warps taking alternate tiles, two 128-column slice
-// buffers each, so that one group's output step overlaps the next tile's MMAs).
+// Tile width TN: 256 (one epilogue group of eight warps, two 256-column TMEM slice buffers).
 // CG = 2: CTA pairs; each CTA stages TN / 2 of the tile's B columns. P = FP8 (below): one plane of
 // FP8 E4M3 codes, 128-element (128-byte) k-stages, K-major operands only.
 constexpr int FP8 = 8;
@@ -95,9 +94,8 @@ struct Cfg {
   static constexpr int BKE = P == FP8 ? 128 : BK;         // elements of K per k-stage
   static constexpr int STAGES = P == FP8 ? 4
                               : CG == 2 ? (P == 3 ? 4 : (P == 2 ? 6 : 12))
-                              : TN == BN ? (P == 3 ? 6 : (P == 2 ? 9 : 16)) * 16 / BK : (P == 3 ? 4 : (P == 2 ? 6 : 12));
-  static constexpr int NBUF = TN == BN ? 2 : 4;          // TMEM slice buffers of TN columns
-  static constexpr int GROUP_WARPS = TN == BN ? EPI_WARPS : EPI_WARPS / 2;
+                                        : (P == 3 ? 6 : (P == 2 ? 9 : 16)) * 16 / BK;
+  static constexpr int NBUF = 2;                          // TMEM slice buffers of TN columns
   static constexpr uint32_t A_BYTES = P == FP8 ? BM * 128 : P * A_PLANE;
   static constexpr uint32_t B_BYTES = P == FP8 ? TNL * 128 : P * TNL * BK * 2;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
@@ -395,30 +393,6 @@ struct SingleSrc {
   }
 };
 
-// Many problems: tiles from a table; tiles of stopped problems are skipped (every
-// role reads the same status, which no launch-concurrent code changes).
-struct GroupSrc {
-  const TcTile* tiles;
-  const TcGroupEntry* entries;
-  int64_t ntiles;
-  int64_t t0, dt;
-  int sl_default;   // slice length of problems whose entry leaves it 0
-  __device__ __forceinline__ bool get(int64_t t, TileCtx& c) const {
-    const TcTile d = tiles[t];
-    const TcGroupEntry* e = entries + d.prob;
-    if (e->args.st && e->args.st->status != ST_RUNNING) return false;
-    c.ma = reinterpret_cast<const CUtensorMap*>(e->map_a);
-    c.mb = reinterpret_cast<const CUtensorMap*>(e->map_b);
-    c.bi = d.bi;
-    c.bj = d.bj;
-    c.nk = (e->args.K + BK - 1) / BK;
-    c.args = &e->args;
-    c.sl = e->args.slice_stages > 0 ? e->args.slice_stages : sl_default;
-    c.part = (int64_t)d.local * EPI_WARPS;
-    return true;
-  }
-};
-
 template <int P, bool A_MN, bool B_MN, int TN, int CG, class Src>
 __device__ __noinline__ void role_producer(const Src& src, uint32_t smem_base, Bars br, volatile int* abort_flag,
                                            int withhold) {
@@ -537,11 +511,8 @@ __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32
                                 : smem_desc(smem_base + C::A_BYTES, 16, KM_SBO, KM_SWZ);
   int stage = 0;
   uint32_t phase = 0;
-  // slice buffers: one pair for TN = 256; with TN = 128 a pair per epilogue group, the groups
-  // taking alternate tiles (each pair keeps its own position and phase)
-  int gbuf[2] = {0, 0};
-  uint32_t gphase[2] = {0u, 0u};
-  int64_t ntile = 0;
+  int buf = 0;   // of the two slice buffers
+  uint32_t buf_phase = 0;
   bool ok = true;
   auto half = [&](int h, uint32_t d_tmem, uint64_t soff, uint32_t first_acc) {
     if (!issuer) return;
@@ -560,16 +531,13 @@ __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32
   for (int64_t t = src.t0; t < src.ntiles && ok; t += src.dt) {
     TileCtx c;
     if (!src.get(t, c)) continue;
-    const int grp = TN == BN ? 0 : (int)(ntile++ & 1);
-    int buf = gbuf[grp];
-    uint32_t buf_phase = gphase[grp];
     int kin = 0;  // k-stage index within the current slice
     // c.sl k-stages into a fresh slice buffer, then published to the epilogue
-    ok = mbar_wait_warp(br.tempty0 + 8 * (2 * grp + buf), buf_phase ^ 1u, abort_flag) &&
+    ok = mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag) &&
          mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag);
     for (int64_t kb = 0; kb < c.nk && ok; ++kb) {
       const bool slice_end = kin == c.sl - 1 || kb == c.nk - 1;
-      const int bslot = 2 * grp + buf;
+      const int bslot = buf;
       const uint32_t d_tmem = tmem_base + (uint32_t)(bslot * TN);
       const uint64_t soff = (uint64_t)((stage * C::STAGE_BYTES) >> 4);
       const uint32_t first_acc = kin == 0 ? 0u : 1u;
@@ -585,7 +553,7 @@ __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32
         ++kin;
       }
       const bool more = kb + 1 < c.nk;
-      const uint32_t full = br.full0 + 8 * stage, tempty = br.tempty0 + 8 * (2 * grp + buf);
+      const uint32_t full = br.full0 + 8 * stage, tempty = br.tempty0 + 8 * buf;
       const bool full_ok = !more || mbar_peek_warp(full, phase);
       const bool tempty_ok = !more || !slice_end || mbar_peek_warp(tempty, buf_phase ^ 1u);
       half(1, d_tmem, soff, 1u);
@@ -602,8 +570,6 @@ __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32
       if (!full_ok) ok = mbar_wait_warp(full, phase, abort_flag);
       if (!tempty_ok) ok = ok && mbar_wait_warp(tempty, buf_phase ^ 1u, abort_flag);
     }
-    gbuf[grp] = buf;
-    gphase[grp] = buf_phase;
   }
   // every MMA issued so far completes before TMEM is released
   if (issuer) {
@@ -618,18 +584,15 @@ template <int EPI, int TN, int CG, class Src>
 __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, Bars br, volatile int* abort_flag,
                                            int warp, int lane) {
   const int q = warp & 3;                              // TMEM lane quarter this warp may access
-  const int half = TN == BN ? (warp - 2) >> 2 : 0;     // TN = 256: which 128 of the tile's columns
-  const int grp = TN == BN ? 0 : (warp - 2) >> 2;      // TN = 128: the group (alternate tiles)
-  const int gw = TN == BN ? warp - 2 : (warp - 2) & 3; // this warp's partials slot within the tile
+  const int half = (warp - 2) >> 2;                    // which 128 of the tile's columns
+  const int gw = warp - 2;                             // this warp's partials slot within the tile
   const int row_in_tile = q * 32 + lane;
   const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 128);
   int buf = 0;
   uint32_t buf_phase = 0;
-  int64_t ntile = 0;
   for (int64_t t = src.t0; t < src.ntiles; t += src.dt) {
     TileCtx ctx;
     if (!src.get(t, ctx)) continue;
-    if (TN != BN && (int)(ntile++ & 1) != grp) continue;   // the other group's tile
     const TcArgs& p = *ctx.args;
     const int64_t nslices = (ctx.nk + ctx.sl - 1) / ctx.sl;
     constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP;
@@ -641,7 +604,7 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
     int e_sum = 0;
     bool ok = true;
     for (int64_t sl = 0; sl < nslices; ++sl) {
-      const int bslot = 2 * grp + buf;
+      const int bslot = buf;
       if (!mbar_wait(br.tfull0 + 8 * bslot, buf_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       if (p.a_exp) {
@@ -743,7 +706,7 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
       } else if (EPI == TC_EPI_GRAM) {
         // planes of G for the chunks that reach the diagonal or lie above it, as whole 32-value rows;
         // the strictly lower triangle is written afterwards by the mirror pass from the upper one
-        // (launch_mirror_planes3, or the batched solves' own), which also overwrites what a chunk
+        // (launch_mirror_planes3), which also overwrites what a chunk
         // crossing the diagonal stores below it. Columns past N hold zeros (the operand maps stop at N)
         // and land in the pitch's padding, which no operand map reads.
         float s_off = 0.f, s_diag = 0.f;
@@ -845,7 +808,6 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
       for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
       if (lane == 0) {
         p.partials[ctx.part + gw] = part;
-        if (TN != BN) p.partials[ctx.part + 4 + gw] = 0.0;   // a 128-wide tile fills four of its eight slots
       }
     }
     if (STEP) {
@@ -858,10 +820,6 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
       if (lane == 0) {
         p.partials[2 * (ctx.part + gw)] = a;
         p.partials[2 * (ctx.part + gw) + 1] = b;
-        if (TN != BN) {
-          p.partials[2 * (ctx.part + 4 + gw)] = 0.0;
-          p.partials[2 * (ctx.part + 4 + gw) + 1] = 0.0;
-        }
       }
     }
   }
@@ -869,8 +827,8 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
 
 // Shared prologue/epilogue of both launch forms; `Src` supplies the tiles.
 template <int P, bool A_MN, bool B_MN, int EPI, int TN, int CG, class Src>
-__device__ __forceinline__ void tc_body(const Src& src, DevState* st, int* err_word, unsigned int* err_out,
-                                        const int* planes_dyn, int withhold) {
+__device__ __forceinline__ void tc_body(const Src& src, DevState* st, unsigned int* err_out, const int* planes_dyn,
+                                        int withhold) {
   using C = Cfg<P, TN, CG>;
   constexpr int S = C::STAGES;
   extern __shared__ uint8_t smem_raw[];
@@ -894,7 +852,7 @@ __device__ __forceinline__ void tc_body(const Src& src, DevState* st, int* err_w
     }
     for (int a = 0; a < C::NBUF; ++a) {
       mbar_init(br.tfull0 + 8 * a, 1);
-      mbar_init(br.tempty0 + 8 * a, C::GROUP_WARPS * CG);   // a pair: both CTAs' epilogue warps
+      mbar_init(br.tempty0 + 8 * a, EPI_WARPS * CG);   // a pair: both CTAs' epilogue warps
     }
     mbar_init(br.drain, 1);
     *abort_flag = 0;
@@ -937,7 +895,6 @@ __device__ __forceinline__ void tc_body(const Src& src, DevState* st, int* err_w
   // a pair: neither CTA leaves (or frees TMEM) while the other's MMAs, copies or arrives may still
   // touch its shared memory or TMEM
   if (CG == 2) cluster_sync_all();
-  if (*abort_flag && threadIdx.x == 0 && err_word) atomicOr(err_word, 1);
   if (*abort_flag && threadIdx.x == 0) {
     if (st) {
       atomicOr(&st->err_flags, 1u);
@@ -975,7 +932,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   src.dt = gridDim.x;
   src.rank = 0;
   src.tri = p.triangular != 0;
-  tc_body<P, A_MN, B_MN, EPI, BN, 1>(src, p.st, nullptr, p.err_out, p.planes_dyn, p.withhold_tma);
+  tc_body<P, A_MN, B_MN, EPI, BN, 1>(src, p.st, p.err_out, p.planes_dyn, p.withhold_tma);
 }
 
 // CTA pairs: clusters of two; pair tiles t0 = cluster index, dt = number of clusters. Both CTAs read
@@ -998,20 +955,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
   src.dt = gridDim.x / 2;
   src.rank = cluster_rank();
   src.tri = p.triangular != 0;
-  tc_body<P, A_MN, B_MN, EPI, BN, 2>(src, p.st, nullptr, p.err_out, p.planes_dyn, p.withhold_tma);
-}
-
-template <int P, bool A_MN, bool B_MN, int EPI, int TN>
-__global__ void __launch_bounds__(NTHREADS, 1) tc_gemm_grouped_kernel(const __grid_constant__ TcGroupLaunch g) {
-  if (g.done && *g.done) return;
-  GroupSrc src;
-  src.tiles = g.tiles;
-  src.entries = g.entries;
-  src.ntiles = g.ntiles;
-  src.t0 = blockIdx.x;
-  src.dt = gridDim.x;
-  src.sl_default = g.slice_stages > 0 ? g.slice_stages : 1;
-  tc_body<P, A_MN, B_MN, EPI, TN, 1>(src, nullptr, g.err, nullptr, g.planes_dyn, g.withhold_tma);
+  tc_body<P, A_MN, B_MN, EPI, BN, 2>(src, p.st, p.err_out, p.planes_dyn, p.withhold_tma);
 }
 
 inline int sm_count() {
@@ -1125,33 +1069,6 @@ cudaError_t dispatch_p(const CUtensorMap& ma, const CUtensorMap& mb, const TcArg
 }
 
 
-template <int P, bool A_MN, bool B_MN, int EPI, int TN>
-cudaError_t launch_grouped_t(const TcGroupLaunch& g, cudaStream_t s) {
-  auto k = tc_gemm_grouped_kernel<P, A_MN, B_MN, EPI, TN>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<P, TN>::SMEM);
-  if (e != cudaSuccess) return e;
-  int64_t grid = g.ntiles < sm_count() ? g.ntiles : sm_count();
-  if (grid < 1) return cudaSuccess;
-  k<<<(unsigned)grid, NTHREADS, Cfg<P, TN>::SMEM, s>>>(g);
-  return cudaGetLastError();
-}
-
-template <int P, int TN>
-cudaError_t dispatch_grouped_tn(const TcGroupLaunch& g, cudaStream_t s) {
-  if (g.epi == TC_EPI_NS && !g.a_mn && g.b_mn) return launch_grouped_t<P, false, true, TC_EPI_NS, TN>(g, s);
-  if (g.epi == TC_EPI_GRAM && g.a_mn && g.b_mn) return launch_grouped_t<P, true, true, TC_EPI_GRAM, TN>(g, s);
-  if (g.epi == TC_EPI_STORE && g.a_mn && g.b_mn) return launch_grouped_t<P, true, true, TC_EPI_STORE, TN>(g, s);
-  return cudaErrorInvalidValue;
-}
-
-template <int P>
-cudaError_t dispatch_grouped(const TcGroupLaunch& g, cudaStream_t s) {
-  if (g.tile_n == 128) return dispatch_grouped_tn<P, 128>(g, s);
-  if (g.tile_n == 0 || g.tile_n == BN) return dispatch_grouped_tn<P, BN>(g, s);
-  return cudaErrorInvalidValue;
-}
-
-
 }  // namespace
 
 // One function per translation unit that instantiates a group of the kernels above.
@@ -1165,8 +1082,5 @@ cudaError_t tc_dispatch_pair3(const CUtensorMap& ma, const CUtensorMap& mb, cons
                               int64_t ntiles, cudaStream_t s);
 cudaError_t tc_dispatch_fp8(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, int64_t tm, int64_t tn,
                             int64_t ntiles, cudaStream_t s);
-cudaError_t tc_dispatch_grouped1(const TcGroupLaunch& g, cudaStream_t s);
-cudaError_t tc_dispatch_grouped2(const TcGroupLaunch& g, cudaStream_t s);
-cudaError_t tc_dispatch_grouped3(const TcGroupLaunch& g, cudaStream_t s);
 
 }  // namespace polar

@@ -209,33 +209,6 @@ cudaError_t launch_tc_gemm_fp8(const TcArgs& a, cudaStream_t s);
 // timeout; waits for `s` and writes the old value to *out.
 cudaError_t tc_take_error(cudaStream_t s, unsigned int* out);
 
-// Grouped launch: many independent problems in one persistent launch. Each problem
-// has an entry (its TMA maps and its own TcArgs: sizes, epilogue pointers, status);
-// the tile table lists (problem, tile row, tile column, tile index within the problem)
-// in the order CTAs take them. Tiles of problems whose status is not RUNNING are skipped.
-struct TcGroupEntry {
-  alignas(128) unsigned char map_a[128];  // CUtensorMap
-  alignas(128) unsigned char map_b[128];
-  TcArgs args;                            // per problem: M, N, K, epilogue fields, st
-};
-struct TcTile {
-  int32_t prob, bi, bj, local;
-};
-struct TcGroupLaunch {
-  int nplanes, epi, a_mn, b_mn;           // shared by every problem of the launch
-  const TcTile* tiles;                    // device
-  int64_t ntiles;
-  const TcGroupEntry* entries;            // device
-  const int* done;                        // device flag: nonzero -> the launch returns at once
-  int* err;                               // device word: set to 1 when a bounded wait expired
-  const int* planes_dyn;
-  int slice_stages;
-  int withhold_tma;                       // test hook, as in TcArgs
-  int tile_n;                             // 256 (0 also) or 128: the tiles' width; the table must match
-};
-cudaError_t launch_tc_gemm_grouped(const TcGroupLaunch& g, cudaStream_t s);
-// Fills entry->map_a / map_b for the operands of entry->args (host side).
-bool tc_make_entry_maps(TcGroupEntry* entry);
 // Residual partial slots a GRAM launch of an n x n triangle with `planes` planes writes (the CTA-pair
 // and single-CTA forms tile it differently), and the largest of the two (for allocation).
 int tc_gram_partials(int64_t n, int planes);
