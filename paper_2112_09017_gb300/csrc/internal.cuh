@@ -89,6 +89,10 @@ cudaError_t launch_norm_finalize(const double* partials, int nparts, DevState* s
 cudaError_t launch_scale_split(const float* src, int64_t lds, int64_t m, int64_t n, const DevState* st,
                                bool scale, float* dst, int64_t ldd, uint16_t* planes, int64_t ldp,
                                int64_t plane_stride, int nplanes, cudaStream_t s);
+// BF16 planes of two matrices in one launch.
+cudaError_t launch_split2(const float* A, int64_t lda, int64_t ma, int64_t na, uint16_t* pa, int64_t lpa, int64_t sa,
+                          const float* B, int64_t ldb, int64_t mb, int64_t nb, uint16_t* pb, int64_t lpb, int64_t sb,
+                          int nplanes, cudaStream_t s);
 // Residual finalize: fixed-order sum of Gram partials, stop rule, schedule.
 cudaError_t launch_residual_finalize(const double* partials, int nparts, DevState* st, StopRule rule,
                                      int k, int planes_this, cudaStream_t s);

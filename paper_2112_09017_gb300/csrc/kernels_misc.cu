@@ -44,15 +44,15 @@ __device__ double block_sum(double v) {
 
 __global__ void frob_partials_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda,
                                      double* __restrict__ partials) {
-  double acc = 0.0;
-  for (int64_t r = blockIdx.x; r < m; r += gridDim.x) {
-    const float* row = A + r * lda;
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-      double v = (double)row[c];
-      acc = fma(v, v, acc);
+  const bool vec = (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && lda % 4 == 0;
+  SquareSum acc;
+  for (int64_t r = blockIdx.x; r < m; r += gridDim.x)
+    for (int64_t c = 8 * threadIdx.x; c < n; c += 8 * blockDim.x) {
+      float v[8];
+      load_row8(A + r * lda + c, n - c, vec, v);
+      acc.add8(v);
     }
-  }
-  double t = block_sum(acc);
+  double t = block_sum(acc.value());
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
@@ -78,24 +78,44 @@ __global__ void norm_finalize_kernel(const double* __restrict__ partials, int np
   }
 }
 
-// dst = src * (1/||A||_F as float32 divisor) and/or BF16 planes of the same values.
-__global__ void scale_split_kernel(const float* __restrict__ src, int64_t lds, int64_t m, int64_t n,
-                                   const DevState* __restrict__ st, int scale, float* __restrict__ dst,
-                                   int64_t ldd, uint16_t* __restrict__ planes, int64_t ldp,
-                                   int64_t plane_stride, int nplanes) {
+// dst = src (divided by ||A||_F as float32 with `scale`) and/or BF16 planes of the same values, 8 columns per
+// thread: 16-byte loads where the rows are aligned, 16-byte plane stores (planes 16-byte aligned, ldp and the
+// plane stride multiples of 8; the columns from n to the next multiple of 8 are zeros). Grid (blocks, jobs).
+struct SplitJob {
+  const float* src;
+  int64_t lds, m, n;
+  uint16_t* planes;
+  int64_t ldp, ps;
+};
+struct SplitJobs {
+  SplitJob j[2];
+};
+
+__global__ void scale_split_kernel(const __grid_constant__ SplitJobs jobs, const DevState* __restrict__ st, int scale,
+                                   float* __restrict__ dst, int64_t ldd, int nplanes) {
   if (st && st->status != ST_RUNNING) return;
-  float s = scale ? (float)st->normA : 1.0f;
-  for (int64_t r = blockIdx.x; r < m; r += gridDim.x) {
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-      float x = src[r * lds + c];
-      if (scale) x = __fdiv_rn(x, s);
-      if (dst) dst[r * ldd + c] = x;
-      float rem = x;
-      for (int p = 0; p < nplanes; ++p) {
-        uint16_t b = bf16_rne_bits(rem);
-        planes[p * plane_stride + r * ldp + c] = b;
-        rem = rem - bf16_bits_to_float(b);
-      }
+  const SplitJob& q = jobs.j[blockIdx.y];
+  const float s = scale ? (float)st->normA : 1.0f;
+  const bool vec = (reinterpret_cast<uintptr_t>(q.src) & 15u) == 0 && q.lds % 4 == 0;
+  const bool vec_d = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && ldd % 4 == 0;
+  const int64_t c8 = (q.n + 7) / 8, units = q.m * c8, step = (int64_t)gridDim.x * blockDim.x;
+  int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t r = u / c8, c = u - r * c8;
+  const int64_t dr = step / c8, dc = step - dr * c8;   // a step in rows and units: no division per unit
+  for (; u < units; u += step) {
+    float v[8];
+    load_row8(q.src + r * q.lds + 8 * c, q.n - 8 * c, vec, v);
+    if (scale) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = __fdiv_rn(v[j], s);
+    }
+    if (dst) store_row8(dst + r * ldd + 8 * c, q.n - 8 * c, vec_d, v);
+    if (nplanes) split_store8(q.planes + r * q.ldp + 8 * c, q.ps, nplanes, v);
+    r += dr;
+    c += dc;
+    if (c >= c8) {
+      c -= c8;
+      ++r;
     }
   }
 }
@@ -252,10 +272,12 @@ __global__ void mirror_planes3_kernel(uint16_t* __restrict__ P, int64_t ldp, int
 // hi + mid has at most 16 significant bits and (hi + mid) + lo at most 24.
 __global__ void planes_to_f32_kernel(const uint16_t* __restrict__ P, int64_t ldp, int64_t ps, int64_t m, int64_t n,
                                      float* __restrict__ dst, int64_t ldd) {
+  const bool vec = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && ldd % 4 == 0;
   for (int64_t r = blockIdx.x; r < m; r += gridDim.x)
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-      const int64_t i = r * ldp + c;
-      dst[r * ldd + c] = (bf16_bits_to_float(P[i]) + bf16_bits_to_float(P[ps + i])) + bf16_bits_to_float(P[2 * ps + i]);
+    for (int64_t c = 8 * threadIdx.x; c < n; c += 8 * blockDim.x) {
+      float v[8];
+      sum_row8(P + r * ldp + c, ps, v);
+      store_row8(dst + r * ldd + c, n - c, vec, v);
     }
 }
 
@@ -456,11 +478,29 @@ cudaError_t launch_norm_finalize(const double* partials, int nparts, DevState* s
   return cudaGetLastError();
 }
 
+static int split_blocks(int64_t units) {
+  const int64_t b = (units + kThreads - 1) / kThreads;
+  return (int)(b < 1 ? 1 : b < 4096 ? b : 4096);
+}
+
 cudaError_t launch_scale_split(const float* src, int64_t lds, int64_t m, int64_t n, const DevState* st, bool scale,
                                float* dst, int64_t ldd, uint16_t* planes, int64_t ldp, int64_t plane_stride,
                                int nplanes, cudaStream_t s) {
-  scale_split_kernel<<<grid_rows(m), kThreads, 0, s>>>(src, lds, m, n, st, scale ? 1 : 0, dst, ldd, planes, ldp,
-                                                        plane_stride, nplanes);
+  SplitJobs jobs{};
+  jobs.j[0] = {src, lds, m, n, planes, ldp, plane_stride};
+  scale_split_kernel<<<split_blocks(m * ((n + 7) / 8)), kThreads, 0, s>>>(jobs, st, scale ? 1 : 0, dst, ldd, nplanes);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_split2(const float* A, int64_t lda, int64_t ma, int64_t na, uint16_t* pa, int64_t lpa, int64_t sa,
+                          const float* B, int64_t ldb, int64_t mb, int64_t nb, uint16_t* pb, int64_t lpb, int64_t sb,
+                          int nplanes, cudaStream_t s) {
+  SplitJobs jobs{};
+  jobs.j[0] = {A, lda, ma, na, pa, lpa, sa};
+  jobs.j[1] = {B, ldb, mb, nb, pb, lpb, sb};
+  const int64_t ua = ma * ((na + 7) / 8), ub = mb * ((nb + 7) / 8);
+  scale_split_kernel<<<dim3(split_blocks(ua > ub ? ua : ub), 2), kThreads, 0, s>>>(jobs, nullptr, 0, nullptr, 0,
+                                                                                  nplanes);
   return cudaGetLastError();
 }
 

@@ -92,8 +92,7 @@ extern "C" polar_status_t polar_gemm_noalloc(int transA, int transB, int64_t M, 
   if (r != POLAR_OK) return r;
   uint16_t* pa = static_cast<uint16_t*>(base);
   uint16_t* pb = pa + P * sa;
-  if (launch_scale_split(A, lda, a_rows, a_cols, nullptr, false, nullptr, 0, pa, lpa, sa, P, s) != cudaSuccess ||
-      launch_scale_split(B, ldb, b_rows, b_cols, nullptr, false, nullptr, 0, pb, lpb, sb, P, s) != cudaSuccess)
+  if (launch_split2(A, lda, a_rows, a_cols, pa, lpa, sa, B, ldb, b_rows, b_cols, pb, lpb, sb, P, s) != cudaSuccess)
     return POLAR_ECUDA;
   TcArgs g{};
   g.M = M; g.N = N; g.K = K;

@@ -971,9 +971,7 @@ polar_status_t polar_gemm(int transA, int transB, int64_t M, int64_t N, int64_t 
   if (r != POLAR_OK) return r;
   uint16_t* pa = (uint16_t*)scr;
   uint16_t* pb = pa + P * sa;
-  CK(cudaMemsetAsync(scr, 0, (size_t)P * (sa + sb) * 2, s));
-  CK(launch_scale_split(A, lda, a_rows, a_cols, nullptr, false, nullptr, 0, pa, lpa, sa, P, s));
-  CK(launch_scale_split(B, ldb, b_rows, b_cols, nullptr, false, nullptr, 0, pb, lpb, sb, P, s));
+  CK(launch_split2(A, lda, a_rows, a_cols, pa, lpa, sa, B, ldb, b_rows, b_cols, pb, lpb, sb, P, s));
   TcArgs g{};
   g.M = M; g.N = N; g.K = K;
   g.a = op_planes(pa, a_rows, a_cols, lpa, sa, transA ? 0 : 1);
@@ -1064,7 +1062,6 @@ polar_status_t polar_syrk(int64_t n, int64_t k, float alpha, const float* A, int
   polar_status_t r = scratch_get((size_t)P * sa * 2, &scr);
   if (r != POLAR_OK) return r;
   uint16_t* pa = (uint16_t*)scr;
-  CK(cudaMemsetAsync(scr, 0, (size_t)P * sa * 2, s));
   CK(launch_scale_split(A, lda, k, n, nullptr, false, nullptr, 0, pa, lp, sa, P, s));
   TcArgs g{};
   g.M = n; g.N = n; g.K = k;
