@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) co_fp32_kernel(const __grid_con
           const int rr = r0t + 16 * h, r = bi * SS_T + rr, c = bj * SS_T + ct;
           if (r < m && c < n) {
             const int64_t o = (int64_t)r * p.ldx + c;
-            xn[o] = c1 * __ldcg(xo + o) + c3 * ss_sum(sm, rr, ct);
+            xn[o] = fmaf(c1, __ldcg(xo + o), c3 * ss_sum(sm, rr, ct));   // c3 = -0.5: one rounding
           }
         }
         __syncthreads();

@@ -485,7 +485,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             if (NS) {
-              const float xn = e.c1 * xo[j] + e.c3 * v[8 * i + j];
+              const float xn = fmaf(e.c1, xo[j], e.c3 * v[8 * i + j]);   // c3 = -0.5, -1: one rounding
               if (STEP) {
                 d2 = fmaf(xn - xo[j], xn - xo[j], d2);
                 x2 = fmaf(xn, xn, x2);

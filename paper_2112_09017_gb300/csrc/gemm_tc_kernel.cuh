@@ -694,7 +694,7 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
           if (i < 3) xv = load_planes8(xr + (i + 1) * p.ldxp, p.x_plane_stride, (rows4 & (2u << i)) != 0);
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float xn = c1 * x[e] + c3 * v[8 * i + e];
+            const float xn = fmaf(c1, x[e], c3 * v[8 * i + e]);   // c3 = -0.5: one rounding
             if (STEP) {
               d2 = fmaf(xn - x[e], xn - x[e], d2);
               x2 = fmaf(xn, xn, x2);

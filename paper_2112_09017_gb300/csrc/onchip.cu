@@ -66,7 +66,7 @@ struct OcCtl {
   uint32_t tmem_base;
   int pad;
   float c1, c3;
-  double red[OC_WARPS];
+  float2 red[OC_WARPS];    // the warps' sums, unevaluated pairs hi + lo
 };
 
 __host__ __device__ __forceinline__ uint32_t oc_rows(int64_t m) { return (uint32_t)((m + 15) / 16 * 16); }
@@ -216,8 +216,9 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
   const bool issuer = tid == 0 && !withhold;
   if (issuer) iss.init(xbase, ch, mp, np, tmem, br.full);
   bool issued = false;
-  const double inv_sqrt_n = tid == 32 ? st->inv_sqrt_n : 0.0;
-  double v_km1 = 0.0, v_km2 = 0.0;                                 // thread 0: sums of squares of steps k-1, k-2
+  const double inv_sqrt_n = tid == 64 ? st->inv_sqrt_n : 0.0;
+  double v_km1 = 0.0, v_stag = 0.0;                                // warp 1: the last sum of squares, and the one
+                                                                   // before it times stagnation^2
   uint32_t use0 = 0, use1 = 0;                                     // completions awaited on full[0], full[1]
   const uint32_t nslices = (mp / 16 + 3) / 4;
   const uint32_t gch = np / 16, uch = mp / 16;                     // 16-wide chunks of G's columns, X's rows
@@ -304,26 +305,38 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
       }
     }
     if (stored) tmem_st_wait();
-    double part = (double)part32;
+    // sums of pairs in FP32 (a chain of FP64 additions takes as long as the products of a small problem)
+    float2 part = make_float2(part32, 0.0f);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-    if (lane == 0) ctl->red[warp] = part;
+    for (int o = 16; o > 0; o >>= 1)
+      two_sum(part, make_float2(__shfl_xor_sync(0xffffffffu, part.x, o), __shfl_xor_sync(0xffffffffu, part.y, o)));
+    if (lane == 0) {
+      ctl->red[warp].x = part.x;
+      ctl->red[warp].y = part.y;
+    }
     tc_fence_before();
     oc_sync_workers();
-    // ---- the stop rule: warp 0 sums the warps' partials in a fixed order and thread 0
-    // decides on the sum of squares v = n r^2 against squared thresholds, then issues the
-    // update at once; thread 32 records r and the outcome while the update runs
-    if (warp == 0) {
-      double v = lane < OC_WARPS ? ctl->red[lane] : 0.0;
+    // ---- the update starts at once, whatever the stop rule will say (its result is not used after a stop);
+    // meanwhile warp 1 sums the warps' pairs in a fixed order and decides on the sum of squares v = n r^2
+    // against squared thresholds; thread 64 records r and the outcome while the update runs
+    if (issuer && !*abort_flag) {
+      tc_fence_after();
+      iss.update();
+    }
+    if (warp == 1) {
+      const int wl = lane & (OC_WARPS - 1);
+      float2 t = make_float2(ctl->red[wl].x, ctl->red[wl].y);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      for (int o = OC_WARPS / 2; o > 0; o >>= 1)
+        two_sum(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
       if (lane == 0) {
+        const double v = (double)t.x + (double)t.y;
         int dec = 2, status = ST_TIMEOUT;
         if (!*abort_flag) {
           const bool testing = k >= ctl->dr.n_pre;
-          if (!isfinite(v)) status = ST_NONFINITE;
+          if (!isfinite(t.x + t.y)) status = ST_NONFINITE;
           else if (testing && v <= ctl->dr.v_tol) status = ST_CONVERGED;
-          else if (testing && k >= ctl->dr.n_pre + 2 && v > ctl->dr.stag2 * v_km2 && v < ctl->dr.v_floor) status = ST_NOT_CONVERGED;
+          else if (testing && k >= ctl->dr.n_pre + 2 && v > v_stag && v < ctl->dr.v_floor) status = ST_NOT_CONVERGED;
           else if (k >= ctl->dr.max_iter) status = ST_NOT_CONVERGED;
           else status = ST_RUNNING;
           dec = status == ST_RUNNING ? 0 : 1;
@@ -333,16 +346,12 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
           ctl->v = v;
         }
         ctl->decision = dec;
-        v_km2 = v_km1;
+        v_stag = ctl->dr.stag2 * v_km1;
         v_km1 = v;
-        if (dec == 0 && issuer) {
-          tc_fence_after();
-          iss.update();
-        }
       }
     }
     oc_sync_workers();
-    if (tid == 32 && ctl->decision != 2) {
+    if (tid == 64 && ctl->decision != 2) {
       // the record of step k, as the batched finalize keeps it
       const double r = sqrt(ctl->v) * inv_sqrt_n;
       if (k < POLAR_HIST) {
@@ -392,8 +401,8 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
               x1 = (bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1)) +
                     bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1 + 2 * ch))) +
                    bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1 + 4 * ch));
-            const float xn0 = c1 * x0 + c3 * __uint_as_float(cur[e]);
-            const float xn1 = c1 * x1 + c3 * __uint_as_float(cur[e + 1]);
+            const float xn0 = fmaf(c1, x0, c3 * __uint_as_float(cur[e]));
+            const float xn1 = fmaf(c1, x1, c3 * __uint_as_float(cur[e + 1]));
             uint32_t w[3];
             oc_split2(xn0, xn1, w);
             if (v0) {
