@@ -8,7 +8,7 @@
 // X' = 1.5 X - 0.5 X G) and U^T A for H, with FP32 operands given as P BF16
 // planes (x = x_0 + x_1 + x_2). Each k-slice of every plane of both operands is
 // staged once in shared memory and all plane-pair passes are issued on it
-// (P = 3: hi*hi, hi*mid, mid*hi, hi*lo, lo*hi, mid*mid), accumulating into one
+// (P = 3: mid*mid, mid*hi, lo*hi, hi*lo, hi*mid, hi*hi), accumulating into one
 // FP32 TMEM accumulator, so the split costs tensor-pipe time but not extra
 // global or L2 traffic per pass.
 //
@@ -115,18 +115,25 @@ __host__ __device__ constexpr uint32_t make_idesc_f8(int tn = BN) {
   return (1u << 4) | ((uint32_t)(tn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-// Plane pairs of the split product in issue order for `np` planes: the smallest
-// terms first, hi*hi last (6 passes: (1,1) (0,2) (2,0) (0,1) (1,0) (0,0)).
-__host__ __device__ constexpr int pass_a(int np, int i) {
-  return ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 0 ? 1
-       : ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 2 ? 2
-       : ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 4 ? 1 : 0;
+// The MMAs of one k-stage (two K = 16 steps) of the split product with `np` planes in issue order: step, plane
+// of A, plane of B, and the use of the tensor core's collector, which keeps one A operand between
+// consecutive MMAs (0: not used, 1: filled, 2: used again, 3: used for the last time). hi*hi comes last, so
+// that the truncations of the small terms happen at 2^-8 of the result's scale; among the small terms those
+// that share an A plane are neighbours. Reading A seven times per stage instead of twelve matters because the
+// shared memory serves the MMAs' operands and the copies of later stages: 128 bytes a cycle, of which a stage
+// of 128 x 64 tiles needed 864 cycles for 595 of products, of 128 x 128 tiles 1152 for 786. Alone, a 64-wide
+// stage took 593 cycles and takes 494.
+struct MmaStep {
+  int kk, a, b, keep;
+};
+__host__ __device__ constexpr MmaStep mma_step(int np, int i) {
+  constexpr MmaStep s3[12] = {{0, 1, 1, 1}, {0, 1, 0, 3}, {0, 2, 0, 0}, {0, 0, 2, 1}, {0, 0, 1, 3}, {1, 1, 1, 1},
+                              {1, 1, 0, 3}, {1, 2, 0, 0}, {1, 0, 2, 1}, {1, 0, 1, 2}, {1, 0, 0, 3}, {0, 0, 0, 0}};
+  constexpr MmaStep s2[6] = {{0, 1, 0, 0}, {0, 0, 1, 0}, {1, 1, 0, 0}, {1, 0, 1, 1}, {1, 0, 0, 3}, {0, 0, 0, 0}};
+  constexpr MmaStep s1[2] = {{0, 0, 0, 0}, {1, 0, 0, 0}};
+  return np == 3 ? s3[i] : np == 2 ? s2[i] : s1[i];
 }
-__host__ __device__ constexpr int pass_b(int np, int i) {
-  return ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 0 ? 1
-       : ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 1 ? 2
-       : ((np == 1 ? 5 : np == 2 ? 3 : 0) + i) == 3 ? 1 : 0;
-}
+static_assert(BK == 32, "the issue order is that of two K = 16 steps per stage");
 
 __host__ __device__ constexpr int passes_for(int planes) { return planes == 1 ? 1 : (planes == 2 ? 3 : 6); }
 
@@ -458,7 +465,7 @@ __device__ __noinline__ void role_producer(const Src& src, uint32_t smem_base, B
     if (armed & (1u << s2)) mbar_drain(br.full0 + 8 * s2, (armed_phase >> s2) & 1u);
 }
 
-// MMAs LO .. HI-1 of one k-stage's NP-plane passes (two K = 16 MMAs per pass): descriptors are the stage-0
+// MMAs LO .. HI-1 of one k-stage (mma_step): descriptors are the stage-0
 // bases plus compile-time offsets (the start-address field is the low 14 bits, address / 16).
 template <int P, bool A_MN, bool B_MN, int NP, int TN, int CG, int LO, int HI>
 __device__ __forceinline__ void issue_range(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t first_acc) {
@@ -466,12 +473,10 @@ __device__ __forceinline__ void issue_range(uint32_t d_tmem, uint64_t a_desc, ui
   constexpr uint32_t B_PL = (TN / CG) * BK * 2;
 #pragma unroll
   for (int i = LO; i < HI; ++i) {
-    const int ps = i / (BK / 16), kk = i % (BK / 16);
-    const uint32_t aoff = A_MN ? pass_a(NP, ps) * MN_CHUNK + kk * 2048 : pass_a(NP, ps) * A_PLANE + kk * 32;
-    const uint32_t boff = B_MN ? pass_b(NP, ps) * MN_CHUNK + kk * 2048 : pass_b(NP, ps) * B_PL + kk * 32;
-    const uint32_t acc = i == 0 ? first_acc : 1u;
-    if (CG == 2) tc_mma_pair(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
-    else tc_mma(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, acc);
+    const MmaStep m = mma_step(NP, i);
+    const uint32_t aoff = A_MN ? m.a * MN_CHUNK + m.kk * 2048 : m.a * A_PLANE + m.kk * 32;
+    const uint32_t boff = B_MN ? m.b * MN_CHUNK + m.kk * 2048 : m.b * B_PL + m.kk * 32;
+    tc_mma_step<CG>(d_tmem, a_desc + (aoff >> 4), b_desc + (boff >> 4), idesc, i == 0 ? first_acc : 1u, m.keep);
   }
 }
 

@@ -247,17 +247,32 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       : "memory");
 }
 
-// One pair MMA (issued by one thread of the even CTA): A's rows 0..127 from the even CTA's shared
-// memory and 128..255 from the odd one's (same descriptor address), B's columns split the same way,
-// D at the same TMEM address in both CTAs.
-__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// An MMA of a sequence whose neighbours share A (keep: 0 as tc_mma, 1 A stays in the collector, 2 A comes from
+// it and stays, 3 A comes from it). CG = 2: a pair MMA (issued by one thread of the even CTA), A's rows 0..127
+// from the even CTA's shared memory and 128..255 from the odd one's (same descriptor address), B's columns
+// split the same way, D at the same TMEM address in both CTAs.
+template <int CG>
+__device__ __forceinline__ void tc_mma_step(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate, int keep) {
+#define POLAR_MMA(GROUP, COLLECTOR)                                                                  \
+  asm volatile(                                                                                      \
+      "{\n\t.reg .pred p;\n\t"                                                                        \
+      "setp.ne.b32 p, %4, 0;\n\t"                                                                    \
+      "tcgen05.mma.cta_group::" GROUP ".kind::f16" COLLECTOR " [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), \
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                                            \
+      : "memory")
+  if (CG == 1) {
+    if (keep == 1) POLAR_MMA("1", ".collector::a::fill");
+    else if (keep == 2) POLAR_MMA("1", ".collector::a::use");
+    else if (keep == 3) POLAR_MMA("1", ".collector::a::lastuse");
+    else POLAR_MMA("1", "");
+  } else {
+    if (keep == 1) POLAR_MMA("2", ".collector::a::fill");
+    else if (keep == 2) POLAR_MMA("2", ".collector::a::use");
+    else if (keep == 3) POLAR_MMA("2", ".collector::a::lastuse");
+    else POLAR_MMA("2", "");
+  }
+#undef POLAR_MMA
 }
 
 // Arrives (once) on the mbarrier at shared offset `bar` of every CTA in `mask` when the pair MMAs
