@@ -23,7 +23,7 @@ enum : int { CB_GRAM = 0, CB_UPDATE = 1, CB_H = 2 };
 // status on their way while a tile is worked on; no status changes during a product.
 template <int KIND>
 struct CoTableSrc {
-  static constexpr bool TABLE = true;
+  static constexpr bool TABLE = true, SPLIT = false;
   const CoBatch& p;
   const TcTile* tiles;
   int n, par, t;
@@ -66,6 +66,7 @@ struct CoTableSrc {
       c.mbt = KIND == CB_UPDATE ? reinterpret_cast<const CUtensorMap*>(p.gram_m[0][prob].b) : nullptr;
       c.bi = r.y & 0xfffff;
       c.bj = (int)((uint32_t)r.y >> 20);
+      c.kbeg = 0;
       c.K = r.w;
       c.slice = __ldg(&p.meta[prob].slice);
       return true;

@@ -28,13 +28,15 @@ constexpr int CO_WARPS = CO_THREADS / 32;
 constexpr int CO_CTL_WARP = CO_WARPS - 1;
 constexpr int CO_EPI_NORM = 16;             // beside the TcEpi kinds: no output, ||C||_F^2 of a symmetric product
 
-template <int TN, int P = CO_P>
+template <int TN, int P = CO_P, bool SPLIT = false>
 struct CoCfg {
   // A stage holds SUB k-blocks of 32: with 64-wide tiles two, because the twelve short MMAs of one do not
-  // cover the waits and commits of a stage (measured at 512 x 512: about 940 cycles per k-block against 595
-  // of products).
-  static constexpr int SUB = TN == 64 ? 2 : 1;
-  static constexpr int STAGES = TN == 64 ? 3 : 4;          // 72 or 48 KiB each
+  // cover the waits and commits of a stage (1024 x 1024: 766 us per solve against 824 with six stages of one).
+  // A split chain has 34 KiB less (the exchange of partial tiles) and takes five stages of one: two of two
+  // are too few in flight (1000 x 700: 684 against 537 us).
+  static constexpr int SUB = TN == 64 && !SPLIT ? 2 : 1;
+  // 72, 48 or (split) 36 KiB each
+  static constexpr int STAGES = TN == 64 ? (SPLIT ? 5 : 3) : 4;
   static constexpr uint32_t A_BYTES = P * A_PLANE;         // of one k-block
   static constexpr uint32_t B_BYTES = P * TN * BK * 2;
   static constexpr uint32_t KB_BYTES = A_BYTES + B_BYTES;
@@ -46,18 +48,23 @@ struct CoCfg {
   static constexpr int SLICE = 64 / BKS;                   // stages per promoted slice
 };
 
-// Shared control block, behind the stages.
+// Clusters of a split chain, and floats per row of the exchange buffer: [source][row][columns].
+constexpr int CO_CLUSTER = 4;
+constexpr int CO_XLD = 64 + 4;
+constexpr size_t CO_XBUF = (size_t)128 * CO_XLD * 4;
+
+// Shared control block, behind the stages (and the exchange buffer).
 struct CoCtl {
-  uint64_t bars[2 * 6 + 2 * 4 + 1];
+  uint64_t bars[2 * 5 + 2 * 4 + 2];
   double red[CO_WARPS];
   uint32_t tmem;
   int abort;
   int status;              // of the last stop test
 };
 
-template <int TN, int P = CO_P>
+template <int TN, int P = CO_P, bool SPLIT = false>
 constexpr size_t co_smem() {
-  return (size_t)CoCfg<TN, P>::STAGES * CoCfg<TN, P>::STAGE_BYTES + sizeof(CoCtl) + 1024;
+  return (size_t)CoCfg<TN, P, SPLIT>::STAGES * CoCfg<TN, P, SPLIT>::STAGE_BYTES + (SPLIT ? CO_XBUF : 0) + sizeof(CoCtl) + 1024;
 }
 
 // What a role carries from one product to the next.
@@ -72,6 +79,8 @@ struct CoCtx {
   CoCtl* ctl;
   uint8_t* smem;             // 1024-byte aligned, the stages
   uint32_t smem_base, tmem;
+  uint32_t xbuf, xfull;      // split chains: the exchange buffer and its barrier (shared addresses)
+  uint32_t xphase;
   Bars br;
   GridBarrier bar;
   int warp, lane;
@@ -121,29 +130,41 @@ struct CoTile {
   const CUtensorMap* ma;
   const CUtensorMap* mb;
   const CUtensorMap* mbt;    // the mirrored (K-major) map of a B whose upper triangle alone is stored
-  int bi, bj, K;
+  int bi, bj;
+  int kbeg, K;               // from kbeg to below K
   int slice;                 // k-blocks of 32 per promoted slice
 };
 
 struct CoEpi;
 
-// Tiles of one product of a chain: this block's are blockIdx.x, blockIdx.x + gridDim.x, ...
-template <int TN>
+// Tiles of one product of a chain: this block's are blockIdx.x, blockIdx.x + gridDim.x, ... With S > 1 (split
+// chains) S neighbouring blocks of a cluster share a tile, each taking a part of K, and there are at least as
+// many such groups as tiles.
+template <int TN, bool SPLIT_ = false>
 struct CoChainSrc {
-  static constexpr bool TABLE = false;
+  static constexpr bool TABLE = false, SPLIT = SPLIT_;
   const CUtensorMap *ma, *mb, *mbt;
   CoTiles ct;
-  int K;
+  int K, kbeg;
   const CoEpi* e;
-  int t;
+  int t, dt;
   __device__ __forceinline__ CoChainSrc(const CUtensorMap* a, const CUtensorMap* b, const CUtensorMap* bt, CoTiles c,
-                                        int k, const CoEpi* ep = nullptr)
-      : ma(a), mb(b), mbt(bt), ct(c), K(k), e(ep), t((int)blockIdx.x) {}
+                                        int k, const CoEpi* ep = nullptr, int S = 1)
+      : ma(a), mb(b), mbt(bt), ct(c), K(k), kbeg(0), e(ep), t((int)blockIdx.x), dt((int)gridDim.x) {
+    if (SPLIT && S > 1) {
+      const int sub = t % S, kc = ((k + S - 1) / S + 63) / 64 * 64;
+      t /= S;
+      dt /= S;
+      kbeg = sub * kc;
+      K = min(k, kbeg + kc);
+    }
+  }
   __device__ __forceinline__ bool next(CoTile& c) {
     if (t >= ct.ntiles) return false;
     co_coords<TN>(ct, t, c.bi, c.bj);
-    t += (int)gridDim.x;
+    t += dt;
     c.ma = ma; c.mb = mb; c.mbt = mbt;
+    c.kbeg = kbeg;
     c.K = K;
     c.slice = 64 / BK;
     return true;
@@ -159,18 +180,20 @@ __device__ __forceinline__ int co_mirror_from(int n0) { return 128 * ((n0 + TN -
 
 // ------------------------------------------------------------------ set-up, grid barrier, teardown
 
-template <int TN, int P = CO_P>
+template <int TN, int P = CO_P, bool SPLIT = false>
 __device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
-  using C = CoCfg<TN, P>;
+  using C = CoCfg<TN, P, SPLIT>;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  CoCtl* ctl = reinterpret_cast<CoCtl*>(smem + C::STAGES * C::STAGE_BYTES);
-  CoCtx x{ctl, smem, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort)};
+  CoCtl* ctl = reinterpret_cast<CoCtl*>(smem + C::STAGES * C::STAGE_BYTES + (SPLIT ? CO_XBUF : 0));
+  CoCtx x{ctl, smem, 0, 0, 0, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort)};
   x.smem_base = smem_u32(x.smem);
   x.br.full0 = smem_u32(&x.ctl->bars[0]);
   x.br.empty0 = smem_u32(&x.ctl->bars[C::STAGES]);
   x.br.tfull0 = smem_u32(&x.ctl->bars[2 * C::STAGES]);
   x.br.tempty0 = smem_u32(&x.ctl->bars[2 * C::STAGES + C::NBUF]);
   x.br.drain = smem_u32(&x.ctl->bars[2 * C::STAGES + 2 * C::NBUF]);
+  x.xfull = smem_u32(&x.ctl->bars[2 * C::STAGES + 2 * C::NBUF + 1]);
+  x.xbuf = x.smem_base + C::STAGES * C::STAGE_BYTES;
   x.warp = threadIdx.x >> 5;
   x.lane = threadIdx.x & 31;
   x.abort_flag = reinterpret_cast<volatile int*>(&x.ctl->abort);
@@ -184,6 +207,7 @@ __device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
       mbar_init(x.br.tempty0 + 8 * b, EPI_WARPS);
     }
     mbar_init(x.br.drain, 1);
+    mbar_init(x.xfull, EPI_WARPS);
     x.ctl->abort = 0;
     x.ctl->status = ST_RUNNING;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -197,6 +221,7 @@ __device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
   }
   tc_fence_before();
   __syncthreads();
+  if (SPLIT) cluster_sync_all();   // the cluster's barriers are initialised before anyone arrives on them
   tc_fence_after();
   x.tmem = *reinterpret_cast<volatile uint32_t*>(&x.ctl->tmem);
   return x;
@@ -209,7 +234,7 @@ __device__ __forceinline__ void co_fence_proxy() { asm volatile("fence.proxy.asy
 __device__ __forceinline__ bool co_grid_sync(CoCtx& x) { return x.bar.sync(); }
 
 // Leaves the kernel: every thread of the block, after its last product. Reports an expired wait.
-template <int TN>
+template <int TN, bool SPLIT = false>
 __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st, int* err_word = nullptr) {
   if (x.warp == 1 && x.lane == 0) {   // every MMA issued has completed before TMEM is released
     tc_commit(x.br.drain);
@@ -217,6 +242,7 @@ __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st, int* err_wor
   }
   tc_fence_before();
   __syncthreads();
+  if (SPLIT) cluster_sync_all();   // no block leaves while another may still write into its exchange buffer
   if (threadIdx.x == 0 && *x.abort_flag) {
     if (err_word) atomicOr(err_word, 1);
     if (st) {
@@ -240,7 +266,7 @@ __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st, int* err_wor
 // SYM: B is symmetric and only its upper triangle is stored.
 template <int TN, int P, bool A_MN, bool SYM, class Src>
 __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src, int withhold) {
-  using C = CoCfg<TN, P>;
+  using C = CoCfg<TN, P, Src::SPLIT>;
   if (withhold) return;   // test hook: no copies are issued, the consumers' bounded waits expire
   co_fence_proxy();
   int stage = pp.stage;
@@ -252,7 +278,7 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src,
     const int m0 = c.bi * BM, n0 = c.bj * TN, K = c.K;
     const int km = SYM ? co_mirror_from<TN>(n0) : 0x7fffffff;
     const CUtensorMap *ma = c.ma, *mb = c.mb, *mbt = c.mbt;
-    for (int k0 = 0; k0 < K; k0 += C::BKS) {
+    for (int k0 = c.kbeg; k0 < K; k0 += C::BKS) {
       if (!mbar_wait(x.br.empty0 + 8 * stage, phase ^ 1u, x.abort_flag)) { ok = false; break; }
       const uint32_t fb = x.br.full0 + 8 * stage;
       mbar_expect_tx(fb, C::SUB == 2 && k0 + BK < K ? 2 * C::KB_BYTES : C::KB_BYTES);
@@ -277,7 +303,7 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src,
         }
       }
       if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
-      if (k0 == 0) src.poke(true);
+      if (k0 == c.kbeg) src.poke(true);
     }
   }
   pp.stage = stage;
@@ -291,7 +317,7 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src,
 // before it (see role_mma; with four slice buffers the wait for one is rarely a real one).
 template <int TN, int P, bool A_MN, bool SYM, class Src>
 __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, Src src) {
-  using C = CoCfg<TN, P>;
+  using C = CoCfg<TN, P, Src::SPLIT>;
   const bool issuer = elect_one();
   const uint64_t a0 = A_MN ? smem_desc(x.smem_base, P * MN_CHUNK, 1024, 2)
                            : smem_desc(x.smem_base, 16, KM_SBO, KM_SWZ);
@@ -308,9 +334,10 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, Src src) {
     const int K = c.K, kin_last = Src::TABLE ? c.slice / C::SUB - 1 : C::SLICE - 1;
     const int km = SYM ? co_mirror_from<TN>(c.bj * TN) : 0x7fffffff;
     int kin = 0;
+    if (Src::SPLIT && c.kbeg >= K) continue;   // no part of K for this block
     ok = mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag) &&
          mbar_wait_warp(br.full0 + 8 * stage, phase, abort_flag);
-    for (int k0 = 0; k0 < K && ok; k0 += C::BKS) {
+    for (int k0 = c.kbeg; k0 < K && ok; k0 += C::BKS) {
       const bool last = kin == kin_last || k0 + C::BKS >= K;
       const uint32_t d = tmem + (uint32_t)(buf * TN), acc = kin == 0 ? 0u : 1u;
       const uint64_t so = (uint64_t)((stage * C::STAGE_BYTES) >> 4);
@@ -327,7 +354,7 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, Src src) {
           if (two) issue_half<P, A_MN, false, P, TN, 1, 1>(d, a0 + so, bk0 + so, 1u);
         }
       }
-      if (k0 == 0) src.poke(false);
+      if (k0 == c.kbeg) src.poke(false);
       if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       if (last) {
         if (++buf == C::NBUF) { buf = 0; buf_phase ^= 1u; }
@@ -393,7 +420,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
   CoTile ti;
   while (ok && src.next(ti)) {
     const CoEpi& e = src.epi(ti);
-    const int bi = ti.bi, bj = ti.bj, nslices = (ti.K + ti.slice * BK - 1) / (ti.slice * BK);
+    const int bi = ti.bi, bj = ti.bj, nslices = (ti.K - ti.kbeg + ti.slice * BK - 1) / (ti.slice * BK);
     const int r = bi * BM + q * 32 + lane, r4 = r - lq;
     const int cb = bj * TN + half * CW;
     unsigned rows4 = 0;
@@ -550,6 +577,135 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
       __stcg(dst, sum0);
       if (STEP) __stcg(dst + 1, sum1);
     }
+  }
+}
+
+// mbar_wait on a barrier that other blocks of the cluster arrive on after writing into this block's shared
+// memory.
+__device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  const uint64_t t0 = gtime();
+  for (uint32_t i = 1;; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((i & 63u) == 0) {
+      if (*abort_flag) return false;
+      if (gtime() - t0 > WAIT_LIMIT_NS) {
+        *abort_flag = 1;
+        return false;
+      }
+    }
+  }
+}
+
+// The epilogue of a product whose tiles are shared by S blocks (2 or 4), each with its part of K: every warp
+// sends its 32 x 32 partial to the block that finishes those rows (rows 128 / S * sub of the tile belong to the
+// group's block `sub`), which adds the S partials in a fixed order and runs the output step on 128 / S rows,
+// 8 columns per lane. At most one tile per group.
+template <int EPI, class Src>
+__device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src, int S) {
+  using C = CoCfg<64, CO_P, true>;
+  const int q = x.warp & 3, half = (x.warp - 2) >> 2, lane = x.lane, w = x.warp - 2;
+  const int sub = (int)blockIdx.x % S, rows = 128 / S, units = 4 / S;
+  CoTile ti;
+  float2 sum0 = make_float2(0.f, 0.f);
+  const bool have = src.next(ti);        // the same in every block of the group
+  const CoEpi& e = src.epi(ti);
+  if (have) {
+    const int nslices = (ti.K - ti.kbeg + 63) / 64;
+    const int col = ti.bj * 64 + 8 * (lane & 7);
+    Planes8 pre[2];
+    if (EPI == TC_EPI_NS) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = ti.bi * BM + sub * rows + (u * EPI_WARPS + w) * 4 + (lane >> 3);
+        if (u < units) pre[u] = load_planes8(e.x + r * e.ldx + col, e.xs, r < e.M && col < e.N);
+      }
+    }
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+    bool ok = true;
+    for (int sl = 0; sl < nslices; ++sl) {
+      if (!mbar_wait(x.br.tfull0 + 8 * pp.buf, pp.buf_phase, x.abort_flag)) { ok = false; break; }
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float v[16];
+        tmem_ld16(x.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(pp.buf * 64 + half * 32 + c * 16), v);
+        add16_packed(&acc[c * 16], v);   // round-to-nearest promotion
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(x.br.tempty0 + 8 * pp.buf);
+      if (++pp.buf == C::NBUF) { pp.buf = 0; pp.buf_phase ^= 1u; }
+    }
+    if (__all_sync(0xffffffffu, ok)) {
+      // to the block that finishes these rows: [sub][row][column] of its exchange buffer
+      const uint32_t dst_rank = cluster_rank() - sub + q * S / 4;
+      const uint32_t row = (uint32_t)((q % units) * 32 + lane);
+      const uint32_t dst = mapa_shared(x.xbuf, dst_rank) + (((uint32_t)sub * rows + row) * CO_XLD + half * 32) * 4;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + 16 * i), "f"(acc[4 * i]),
+                     "f"(acc[4 * i + 1]), "f"(acc[4 * i + 2]), "f"(acc[4 * i + 3])
+                     : "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(mapa_shared(x.xfull, dst_rank));
+      ok = mbar_wait_cluster(x.xfull, x.xphase, x.abort_flag);
+      x.xphase ^= 1u;
+    }
+    if (__all_sync(0xffffffffu, ok)) {
+      const float* xb = reinterpret_cast<const float*>(x.smem + C::STAGES * C::STAGE_BYTES);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (u >= units) break;
+        const int lr = (u * EPI_WARPS + w) * 4 + (lane >> 3), r = ti.bi * BM + sub * rows + lr;
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+        for (int s = 0; s < S; ++s) {
+          const float4* src4 = reinterpret_cast<const float4*>(xb + (s * rows + lr) * CO_XLD + 8 * (lane & 7));
+          const float4 a = src4[0], b = src4[1];
+          v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+          v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+        }
+        if (r >= e.M || col >= e.N) continue;
+        if (EPI == TC_EPI_GRAM) {
+          float t = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int d = col + j - r;   // above the diagonal twice, on it (g - 1)^2 (columns past N hold zeros)
+            const float g = d == 0 ? v[j] - 1.0f : v[j], wt = d < 0 ? 0.0f : d == 0 ? 1.0f : 2.0f;
+            t = fmaf(wt * g, g, t);
+          }
+          two_sum(sum0, make_float2(t, 0.f));
+          store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
+        } else if (EPI == TC_EPI_NS) {
+          float xo[8];
+          sum_planes8(pre[u], xo);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = fmaf(e.c1, xo[j], e.c3 * v[j]);   // c3 = -0.5: one rounding
+          store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
+        } else {   // STORE (a pitch that is a multiple of 4)
+          float* cr = e.C + r * e.ldc + col;
+          if (col < e.ldc) *reinterpret_cast<float4*>(cr) = make_float4(v[0], v[1], v[2], v[3]);
+          if (col + 4 < e.ldc) *reinterpret_cast<float4*>(cr + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        }
+      }
+    }
+  }
+  if (EPI == TC_EPI_GRAM) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
+    if (lane == 0) __stcg(e.part + blockIdx.x * EPI_WARPS + w, sum0);
   }
 }
 

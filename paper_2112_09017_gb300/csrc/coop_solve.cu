@@ -1,6 +1,9 @@
 // One polar solve in one cooperative launch (Sec. III.D, Eq. NewtonSchulz, Algorithm 1), for matrices whose
 // products are a few waves of 128 x 64 or 128 x 128 tiles; the pieces are in coop_kernel.cuh.
 //
+// Where the products have so few 128 x 64 tiles that most SMs would idle, clusters of four blocks share tiles
+// along K (co_epilogue_split).
+//
 //   ||A||_F | X_0 = A / ||A||_F and the planes of A | per step: Gram | update | ... | U^T A | U, H
 //
 // with a grid barrier at every bar. The update of step k runs before its stop test is known (each block
@@ -9,6 +12,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 
 #include "coop_kernel.cuh"
@@ -38,6 +42,7 @@ struct CoSolve {
   float pre_c1, pre_c3;                      // update coefficients of the first n_pre steps
   double inv_sqrt_n;
   int withhold;
+  int sg, su, sh;                            // split chains: blocks per tile of the Gram, the update and U^T A
 };
 
 // The stop rule of step k on v = ||G - I||_F^2 = n r^2 against squared thresholds: r <= tol is
@@ -51,10 +56,30 @@ __device__ __forceinline__ int co_stop_status(const CoSolve& p, int k, double v,
   return ST_RUNNING;
 }
 
-template <int TN>
-__global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_constant__ CoSolve p) {
-  extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
+// One product of the solve by all its roles.
+template <int TN, bool SPLIT, bool A_MN, bool SYM, int EPI>
+__device__ __forceinline__ void co_product(CoCtx& x, CoPipe& pipe, const CUtensorMap* ma, const CUtensorMap* mb,
+                                           const CUtensorMap* mbt, CoTiles t, int K, const CoEpi& e, int S,
+                                           int withhold) {
+  using Src = CoChainSrc<TN, SPLIT>;
+  if (x.warp == 0) {
+    if (x.lane == 0) co_producer<TN, CO_P, A_MN, SYM>(x, pipe, Src(ma, mb, mbt, t, K, nullptr, S), withhold);
+  } else if (x.warp == 1) {
+    co_mma<TN, CO_P, A_MN, SYM>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, nullptr, S));
+  } else if (x.warp < CO_CTL_WARP) {
+    if constexpr (SPLIT) {
+      if (S > 1) {
+        co_epilogue_split<EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e, S), S);
+        return;
+      }
+    }
+    co_epilogue<TN, EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e));
+  }
+}
+
+template <int TN, bool SPLIT>
+__device__ __forceinline__ void co_solve(const CoSolve& p, uint8_t* co_raw) {
+  CoCtx x = co_setup<TN, CO_P, SPLIT>(co_raw, &p.st->bar);
   const int m = p.m, n = p.n, tid = threadIdx.x, nthr = CO_THREADS;
   const int gtid = blockIdx.x * nthr + tid, gthr = gridDim.x * nthr;
   const bool vec_a = (reinterpret_cast<uintptr_t>(p.A) & 15u) == 0 && p.lda % 4 == 0;
@@ -114,36 +139,25 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
   for (int k = 0; run; ++k) {
     const int b = k & 1;
     // Gram of X_k: the upper triangle's tiles, and this block's part of ||G - I||_F^2
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.xmn[b], &p.xmn[b], nullptr, tg, m), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tg, m));
-    } else if (x.warp < CO_CTL_WARP) {
+    {
       CoEpi e{};
       e.M = n; e.N = n;
       e.out = p.gp; e.ldo = p.ldp; e.os = p.gps;
       e.part = p.part2;
-      co_epilogue<TN, TC_EPI_GRAM>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tg, m, &e));
+      co_product<TN, SPLIT, true, false, TC_EPI_GRAM>(x, pipe, &p.xmn[b], &p.xmn[b], nullptr, tg, m, e, p.sg,
+                                                      p.withhold);
     }
     run = co_grid_sync(x);
     if (!run) break;
     // the update, and beside it the stop test of X_k and its record
     if (k < p.max_iter) {
-      if (x.warp == 0) {
-        if (x.lane == 0)
-        co_producer<TN, CO_P, false, true>(x, pipe, CoChainSrc<TN>(&p.xk[b], &p.gmn, &p.gk, tu, n), p.withhold);
-      } else if (x.warp == 1) {
-        co_mma<TN, CO_P, false, true>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, n));
-      } else if (x.warp < CO_CTL_WARP) {
-        CoEpi e{};
-        e.M = m; e.N = n;
-        e.x = p.xp[b]; e.ldx = p.ldp; e.xs = p.xps;
-        e.out = p.xp[b ^ 1]; e.ldo = p.ldp; e.os = p.xps;
-        e.c1 = k < p.n_pre ? p.pre_c1 : 1.5f;
-        e.c3 = k < p.n_pre ? p.pre_c3 : -0.5f;
-        co_epilogue<TN, TC_EPI_NS>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, n, &e));
-      }
+      CoEpi e{};
+      e.M = m; e.N = n;
+      e.x = p.xp[b]; e.ldx = p.ldp; e.xs = p.xps;
+      e.out = p.xp[b ^ 1]; e.ldo = p.ldp; e.os = p.xps;
+      e.c1 = k < p.n_pre ? p.pre_c1 : 1.5f;
+      e.c3 = k < p.n_pre ? p.pre_c3 : -0.5f;
+      co_product<TN, SPLIT, false, true, TC_EPI_NS>(x, pipe, &p.xk[b], &p.gmn, &p.gk, tu, n, e, p.su, p.withhold);
     }
     if (x.warp == CO_CTL_WARP) {
       const double v = co_warp_sum2(p.part2, gridDim.x * EPI_WARPS, 1, x.lane);
@@ -170,16 +184,12 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
   // ---- C = U^T A, then U and H = (C + C^T) / 2
   if (run && (status == ST_CONVERGED || status == ST_NOT_CONVERGED)) {
     const CoTiles th = co_tiles<TN>(n, n, false);
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.xmn[it & 1], &p.amn, nullptr, th, m), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, th, m));
-    } else if (x.warp < CO_CTL_WARP) {
+    {
       CoEpi e{};
       e.M = n; e.N = n;
       e.C = p.C; e.ldc = p.ldc;
-      co_epilogue<TN, TC_EPI_STORE>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, th, m, &e));
+      co_product<TN, SPLIT, true, false, TC_EPI_STORE>(x, pipe, &p.xmn[it & 1], &p.amn, nullptr, th, m, e, p.sh,
+                                                       p.withhold);
     }
     run = co_grid_sync(x);
     if (run) {
@@ -235,12 +245,73 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_co
       }
     }
   }
-  co_teardown<TN>(x, st);
+  co_teardown<TN, SPLIT>(x, st);
+}
+
+template <int TN>
+__global__ void __launch_bounds__(CO_THREADS, 1) co_solve_kernel(const __grid_constant__ CoSolve p) {
+  extern __shared__ uint8_t co_raw[];
+  co_solve<TN, false>(p, co_raw);
+}
+
+// Clusters whose blocks share tiles along K: products with few 128 x 64 tiles.
+__global__ void __cluster_dims__(CO_CLUSTER, 1, 1) __launch_bounds__(CO_THREADS, 1)
+    co_solve_split_kernel(const __grid_constant__ CoSolve p) {
+  extern __shared__ uint8_t co_raw[];
+  co_solve<64, true>(p, co_raw);
 }
 
 template <int TN>
 cudaError_t co_prepare() {
   return cudaFuncSetAttribute(co_solve_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)co_smem<TN>());
+}
+
+cudaError_t co_launch_split(const CoSolve& p, int grid, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(CO_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = co_smem<64, CO_P, true>();
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  void* args[] = {const_cast<CoSolve*>(&p)};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(co_solve_split_kernel), args);
+}
+
+// Clusters of the split form that can be resident at once; 0 when it cannot run. Asked once per device.
+int co_split_clusters_now(int sms) {
+  const int smem = (int)co_smem<64, CO_P, true>();
+  int n = 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(sms / CO_CLUSTER * CO_CLUSTER), 1, 1);
+  cfg.blockDim = dim3(CO_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = CO_CLUSTER;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(co_solve_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(co_solve_split_kernel), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+int co_split_clusters(int sms) {
+  static std::mutex mu;
+  static int known[64];   // clusters + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!known[dev]) known[dev] = co_split_clusters_now(sms) + 1;
+  return known[dev] - 1;
 }
 
 template <int TN>
@@ -255,10 +326,11 @@ cudaError_t co_launch(const CoSolve& p, int grid, cudaStream_t s) {
 struct CoopSolve {
   CoSolve p;
   int tn, grid;
+  bool split;
 };
 
-// Cycles of a chain's products with tiles of one width: whole waves, a k-block of 32 costing about 820 cycles
-// with 64-wide tiles and 950 with 128-wide ones (measured inside the solve; the MMAs alone take 595 and 790),
+// Cycles of a chain's products with tiles of one width: whole waves, a k-block of 32 costing about 750 cycles
+// with 64-wide tiles and 870 with 128-wide ones (measured inside the solve; the MMAs alone take 494 and 786),
 // a tile's output step about 4000 and 7000. Waves: the most of any product.
 template <int TN>
 static double co_cost(const CoopProduct* p, int count, int sms, int64_t* waves) {
@@ -266,7 +338,7 @@ static double co_cost(const CoopProduct* p, int count, int sms, int64_t* waves) 
   *waves = 0;
   for (int i = 0; i < count; ++i) {
     const int64_t w = ((int64_t)co_tiles<TN>(p[i].M, p[i].N, p[i].tri).ntiles + sms - 1) / sms;
-    c += (double)w * ((double)((p[i].K + BK - 1) / BK) * (TN == 64 ? 820.0 : 950.0) + (TN == 64 ? 4000.0 : 7000.0));
+    c += (double)w * ((double)((p[i].K + BK - 1) / BK) * (TN == 64 ? 750.0 : 870.0) + (TN == 64 ? 4000.0 : 7000.0));
     *waves = std::max(*waves, w);
   }
   return c;
@@ -283,6 +355,25 @@ int coop_tile_n(const CoopProduct* p, int count, int sms) {
   return c64 <= c128 ? 64 : 128;
 }
 
+// Blocks per 128 x 64 tile of one product on `blocks` blocks (1, 2 or 4), and its cycles (co_cost's measure). A
+// split tile's exchange costs a little more than its smaller output step saves; k-blocks cost a little more than
+// in the other form, whose stages hold two.
+static int co_split_of(const CoopProduct& q, int blocks, double* cycles) {
+  const int64_t tiles = co_tiles<64>(q.M, q.N, q.tri).ntiles;
+  int best = 1;
+  *cycles = (double)((tiles + blocks - 1) / blocks) * ((double)((q.K + 31) / 32) * 850.0 + 4000.0);
+  for (int S = 2; S <= CO_CLUSTER; S *= 2) {
+    if (tiles * S > blocks) break;
+    const int64_t kc = ((q.K + S - 1) / S + 63) / 64 * 64;
+    const double c = (double)((std::min(kc, q.K) + 31) / 32) * 800.0 + 5000.0;
+    if (c < *cycles) {
+      *cycles = c;
+      best = S;
+    }
+  }
+  return best;
+}
+
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {
   const CoopProduct prod[2] = {{n, n, m, true}, {m, n, n, false}};
   const int tn = coop_tile_n(prod, 2, sms);
@@ -290,12 +381,40 @@ CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms
   CoopSolve* c = new (std::nothrow) CoopSolve();
   if (!c) return nullptr;
   c->tn = tn;
+  // few tiles: share each between blocks along K, where that shortens a step by a tenth
+  const int blocks = CO_CLUSTER * co_split_clusters(sms);
+  c->split = false;
+  c->p.sg = c->p.su = c->p.sh = 1;
+  if (blocks > 0 && blocks <= b.nparts / 2) {
+    int64_t waves;
+    double cg, cu, ch;
+    const double whole = co_cost<64>(prod, 2, sms, &waves), wide = co_cost<128>(prod, 2, sms, &waves);
+    const int sg = co_split_of(prod[0], blocks, &cg), su = co_split_of(prod[1], blocks, &cu);
+    const CoopProduct h = {n, n, m, false};
+    if (cg + cu < 0.9 * std::min(whole, wide)) {
+      c->split = true;
+      c->tn = 64;
+      c->p.sg = sg;
+      c->p.su = su;
+      c->p.sh = co_split_of(h, blocks, &ch);
+    }
+  }
   // enough blocks for the larger product's tiles, and for the passes over A
-  const int64_t tiles = tn == 64 ? co_tiles<64>(m, n, false).ntiles : co_tiles<128>(m, n, false).ntiles;
+  const int64_t tiles = c->tn == 64 ? co_tiles<64>(m, n, false).ntiles : co_tiles<128>(m, n, false).ntiles;
   int64_t grid = std::max<int64_t>(tiles, (m * n + 8191) / 8192);
   grid = std::min<int64_t>(grid, std::min<int64_t>(sms, b.nparts / 2));
+  if (c->split) {
+    const int64_t t = std::max<int64_t>(std::max<int64_t>((int64_t)co_tiles<64>(n, n, true).ntiles * c->p.sg, tiles * c->p.su),
+                                        std::max<int64_t>((int64_t)co_tiles<64>(n, n, false).ntiles * c->p.sh, (m * n + 8191) / 8192));
+    grid = std::min<int64_t>(blocks, (t + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER);
+  }
+  if (!c->split && tiles <= 2) grid = 1;   // a second tile takes less time than two grid barriers
   c->grid = (int)std::max<int64_t>(grid, 1);
-  if (8 * c->grid > b.nparts && (size_t)8 * c->grid * 8 > (size_t)n * b.ldc * 4) c->grid = std::max(1, b.nparts / 8);
+  if (8 * c->grid > b.nparts && (size_t)8 * c->grid * 8 > (size_t)n * b.ldc * 4) {
+    c->split = false;   // no room for a sum per block and warp
+    c->p.sg = c->p.su = c->p.sh = 1;
+    c->grid = std::max(1, b.nparts / 8);
+  }
   CoSolve& p = c->p;
   TcOperand x[2], g, a;
   for (int i = 0; i < 2; ++i) {
@@ -306,11 +425,11 @@ CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms
   g.planes = b.gp; g.rows = n; g.plane_stride = b.gps;
   a = x[0];
   a.planes = b.ap;
-  bool ok = tc_make_map(&p.gmn, g, CO_P, true, 0) && tc_make_map(&p.gk, g, CO_P, false, tn) &&
+  bool ok = tc_make_map(&p.gmn, g, CO_P, true, 0) && tc_make_map(&p.gk, g, CO_P, false, c->tn) &&
             tc_make_map(&p.amn, a, CO_P, true, 0);
   for (int i = 0; i < 2; ++i)
     ok = ok && tc_make_map(&p.xmn[i], x[i], CO_P, true, 0) && tc_make_map(&p.xk[i], x[i], CO_P, false, BM);
-  ok = ok && (tn == 64 ? co_prepare<64>() : co_prepare<128>()) == cudaSuccess;
+  ok = ok && (c->tn == 64 ? co_prepare<64>() : co_prepare<128>()) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     delete c;
@@ -338,6 +457,7 @@ cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* 
   p.max_iter = rule.max_iter;
   update_coeffs(rule, 0, p.pre_c1, p.pre_c3);   // of the preconditioning steps, where there are any
   p.withhold = tc_withhold();
+  if (c->split) return co_launch_split(p, c->grid, s);
   return c->tn == 64 ? co_launch<64>(p, c->grid, s) : co_launch<128>(p, c->grid, s);
 }
 

@@ -24,10 +24,11 @@ def _solve(lib, a, prec="bf16x6", **kw):
 
 
 # one tile, tile edges in rows (128) and columns (64 and 128), an odd and an even number of 64-wide columns
-# (the triangle's pairs), k-block remainders, tall and narrow, more tiles than SMs (the 128-wide tiles), the
+# (the triangle's pairs), k-block remainders, tall and narrow, tiles shared by four and by two blocks and by
+# none (parts of K that are empty among them), more tiles than SMs (the 128-wide tiles), the
 # largest sizes below the separate launches and the smallest above
 SIZES = [(1, 1), (32, 31), (64, 64), (128, 65), (129, 128), (130, 129), (192, 192), (257, 200), (384, 320),
-         (2500, 33), (1000, 996), (1300, 1290), (2100, 2050), (2400, 2304)]
+         (2500, 33), (700, 700), (1000, 700), (1000, 996), (1300, 1290), (2100, 2050), (2400, 2304)]
 
 
 # the plain form's 32 x 32 tiles: edges, remainders of the 64-deep chunks, the largest of its dispatch
