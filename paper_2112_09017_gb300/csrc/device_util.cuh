@@ -28,6 +28,30 @@ __device__ __forceinline__ void split_planes_dev(float x, uint16_t (&planes)[3])
   }
 }
 
+// Two FP32 operations per instruction (round-to-nearest each): a + b, a b + c, a - b.
+__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 c, a, b;\n\t"
+      "mov.b64 {%0, %1}, c;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 a, a, b, c;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 sub_x2(float2 a, float2 b) { return fma_x2(b, make_float2(-1.0f, -1.0f), a); }
+
+// The two BF16 values of a word as floats.
+__device__ __forceinline__ float2 bf16_pair(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
 // s + e = a + b exactly (Knuth's two-sum), accumulated into the unevaluated pair s.x + s.y.
 __device__ __forceinline__ void two_sum(float2& s, float2 b) {
   const float t = s.x + b.x, bb = t - s.x;

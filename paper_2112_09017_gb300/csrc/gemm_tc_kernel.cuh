@@ -265,22 +265,6 @@ __device__ __forceinline__ void quad_rows(float* x, int c) {
   }
 }
 
-// Two FP32 operations per instruction (round-to-nearest each).
-__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 c, a, b;\n\t"
-      "mov.b64 {%0, %1}, c;\n\t}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
-__device__ __forceinline__ float2 sub_x2(float2 a, float2 b) { return add_x2(a, make_float2(-b.x, -b.y)); }
-
-// The two BF16 values of a word as floats.
-__device__ __forceinline__ float2 bf16_pair(uint32_t w) {
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
 // The planes of 8 consecutive values, one 16-byte store per plane. Each plane is the round-to-nearest-even
 // BF16 of what the previous planes left.
 __device__ __forceinline__ void store_planes8(uint16_t* base, int64_t pstride, int np, const float* x) {

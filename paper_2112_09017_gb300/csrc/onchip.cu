@@ -18,11 +18,11 @@
 //                  columns of X), B = X, N = the rows of X; then
 //                  X_{k+1}(r, i) = c1 X_k(r, i) + c3 P^T(i, r), split back into the
 //                  planes in place
-// Sixteen warps, four per TMEM lane quarter taking 16-wide chunks of columns or rows in
-// turn, load X_0, promote accumulators, evaluate the residual and the stop rule, write
-// G into TMEM and X back into shared memory; warp 0 allocates TMEM and thread 0 issues
-// the MMAs once a barrier has published their operands. Every mbarrier wait is bounded (about one second); on expiry the
-// problem reports a timeout, the MMAs in flight drain and TMEM is freed.
+// Sixteen worker warps, four per TMEM lane quarter taking 16-wide chunks of columns or rows in turn, load X_0,
+// promote accumulators, sum the residual, write G into TMEM and X back into shared memory; a warp of its own
+// issues the MMAs once the workers have handed over their operands and decides (warp 0 allocates TMEM). Every
+// mbarrier wait is bounded (about one second); on expiry the problem reports a timeout, the MMAs in flight
+// drain and TMEM is freed.
 #include <cuda.h>
 #include <math.h>
 #include <stdint.h>
@@ -35,8 +35,11 @@
 namespace polar {
 namespace {
 
-constexpr int OC_WARPS = 16;          // four per TMEM lane quarter
-constexpr int OC_THREADS = OC_WARPS * 32;
+constexpr int OC_WARPS = 16;          // workers (12 and 8, with more registers each, measured 6 and 15 % slower)
+constexpr int OC_SUB = OC_WARPS / 4;  // per TMEM lane quarter
+constexpr int OC_GT = (128 / 16 + OC_SUB - 1) / OC_SUB;   // 16-wide chunks of G per worker, at most
+constexpr int OC_WORKERS = OC_WARPS * 32;
+constexpr int OC_THREADS = OC_WORKERS + 32;   // and one warp that issues the MMAs and decides
 constexpr uint32_t OC_TMEM_COLS = 512;
 constexpr uint32_t OC_G_COL = 256;          // first TMEM column of G's planes
 constexpr int64_t OC_MAX_M = 256, OC_MAX_N = 128;
@@ -57,11 +60,10 @@ struct OcRule {
 
 struct OcCtl {
   uint64_t full[2];    // tcgen05.commit -> all warps: accumulator ready
+  uint64_t empty[2];   // the workers' warps have read a Gram accumulator that another slice takes
   uint64_t drain;
   int abort;           // a bounded wait expired
   int decision;        // 0: keep iterating, 1: stop, 2: abort
-  int status;          // the problem's status after the step
-  double v;            // ||G - I||_F^2 of the step
   OcRule dr;
   uint32_t tmem_base;
   int pad;
@@ -80,7 +82,12 @@ __device__ __forceinline__ uint32_t oc_off(uint32_t r, uint32_t c, uint32_t ch) 
   return (c >> 6) * ch + r * 128u + ((((c & 63u) >> 3) ^ (r & 7u)) << 4) + ((c & 7u) << 1);
 }
 
-__device__ __forceinline__ void oc_sync_workers() { asm volatile("bar.sync 1, %0;" ::"n"(OC_THREADS) : "memory"); }
+// Workers hand over to the issuing warp (X_k complete: 2, G's planes stored: 3) without waiting; the whole
+// block meets once per step (4), so that no hand-over can overtake another, whatever a wait that expired skips.
+template <int ID>
+__device__ __forceinline__ void oc_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(OC_THREADS) : "memory"); }
+template <int ID>
+__device__ __forceinline__ void oc_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(OC_THREADS) : "memory"); }
 
 // 8 consecutive 32-bit columns of this thread's TMEM lane (completed by tmem_st_wait).
 __device__ __forceinline__ void oc_st8(uint32_t taddr, const uint32_t (&r)[8]) {
@@ -98,7 +105,7 @@ __device__ __forceinline__ uint32_t oc_idesc(bool a_mn, bool b_mn, uint32_t n) {
 }
 
 struct OcBars {
-  uint32_t full, drain;
+  uint32_t full, empty, drain;
 };
 
 // TMEM loads without the wait, and the wait tied to the loaded registers so that no use
@@ -125,119 +132,173 @@ __device__ __forceinline__ uint32_t oc_bf16x2(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
   return d;
 }
-__device__ __forceinline__ float oc_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float oc_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
-// The three-plane split of a pair (each value the sum of its planes exactly): planes of
-// x0 in the low halves of w[0..2], of x1 in the high halves.
-__device__ __forceinline__ void oc_split2(float x0, float x1, uint32_t (&w)[3]) {
+// The issuing warp: the Gram's 64-row slices of X_k into accumulators s % 2, the update P^T = G X^T into columns
+// 0 .. mp, each completed on its full barrier, and the stop test between. Plane q of X is read through
+// MN-major descriptors (chunk stride ch, 8-row groups of 1024 bytes) and K-major ones (rows of 128 bytes).
+//
+// A warp of its own, every lane of it in the loops and one elected lane issuing, keeps the descriptors in uniform
+// registers; as thread 0 of a worker warp the MMAs took 85 to 115 cycles each to issue instead of about 55, and
+// the stop test stood between the Gram and the update.
+template <int P>
+__device__ __noinline__ void oc_issue(const OcTask& tk, uint32_t xbase, uint32_t ch, uint32_t mp, uint32_t np,
+                                      uint32_t tmem, OcBars br, volatile OcCtl* ctl, int lane, int withhold) {
+  // descriptor high word: stride between 8-row groups 1024 bytes, version 1, 128-byte swizzle
+  constexpr uint64_t HI = (uint64_t)((1024u >> 4) | (1u << 14) | (2u << 29)) << 32;
+  volatile int* abort_flag = &ctl->abort;
+  xbase = __shfl_sync(0xffffffffu, xbase, 0);
+  ch = __shfl_sync(0xffffffffu, ch, 0);
+  mp = __shfl_sync(0xffffffffu, mp, 0);
+  np = __shfl_sync(0xffffffffu, np, 0);
+  tmem = __shfl_sync(0xffffffffu, tmem, 0);
+  const bool issuer = elect_one();
+  const uint32_t idesc_g = oc_idesc(true, true, np), idesc_u = oc_idesc(false, false, mp);
+  const uint32_t ks_g = mp / 16, ks_u = np / 16, nslices = (ks_g + 3) / 4;
+  const uint64_t mn0 = HI | ((uint64_t)((ch >> 4) & 0x3FFFu) << 16) | ((xbase >> 4) & 0x3FFFu);   // plane 0, MN-major
+  const uint64_t km0 = HI | (1u << 16) | ((xbase >> 4) & 0x3FFFu);                                // plane 0, K-major
+  const uint64_t pl = (2 * ch) >> 4;   // from one plane to the next
+  DevState* st = tk.st;
+  const double inv_sqrt_n = st->inv_sqrt_n;
+  double v_km1 = 0.0, v_stag = 0.0;    // the last sum of squares, and the one before it times stagnation^2
+  uint32_t ephase = 0;                 // completions awaited on empty[0], empty[1] (one bit each)
+  bool issued = false;
+  for (int k = 0;; ++k) {
+    oc_sync<2>();
+    bool go = !withhold && __all_sync(0xffffffffu, !*abort_flag);
+    for (uint32_t s = 0; s < nslices && go; ++s) {
+      const uint32_t bsl = s & 1u, d = tmem + 128 * bsl, nkk = min(4u, ks_g - 4 * s);
+      if (s >= 2) {
+        go = mbar_wait_warp(br.empty + 8 * bsl, (ephase >> bsl) & 1u, abort_flag);
+        ephase ^= 1u << bsl;
+        if (!go) break;
+      }
+      tc_fence_after();
+      issued = true;
+      // small terms first, hi*hi last; neighbours share A (see mma_step of the tiled products)
+      for (uint32_t kk = 0; kk < nkk; ++kk) {
+        const uint64_t x = mn0 + (4 * s + kk) * 128;   // 16 rows of X: 2048 bytes
+        const uint32_t first = kk == 0 ? 0u : 1u;
+        if (issuer) {
+          if (P == 3) {
+            tc_mma_step<1>(d, x + pl, x + pl, idesc_g, first, 1);
+            tc_mma_step<1>(d, x + pl, x, idesc_g, 1u, 3);
+            tc_mma_step<1>(d, x + 2 * pl, x, idesc_g, 1u, 0);
+            tc_mma_step<1>(d, x, x + 2 * pl, idesc_g, 1u, 1);
+            tc_mma_step<1>(d, x, x + pl, idesc_g, 1u, 3);
+          } else if (P == 2) {
+            tc_mma(d, x + pl, x, idesc_g, first);
+            tc_mma(d, x, x + pl, idesc_g, 1u);
+          }
+        }
+        __syncwarp();
+      }
+      for (uint32_t kk = 0; kk < nkk; ++kk) {
+        const uint64_t x = mn0 + (4 * s + kk) * 128;
+        if (issuer) tc_mma(d, x, x, idesc_g, P == 1 && kk == 0 ? 0u : 1u);
+        __syncwarp();
+      }
+      if (issuer) tc_commit(br.full + 8 * bsl);
+      __syncwarp();
+    }
+    oc_sync<3>();
+    // the update starts at once, whatever the stop rule will say (its result is not used after a stop)
+    go = go && __all_sync(0xffffffffu, !*abort_flag);
+    if (go) {
+      tc_fence_after();
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    w[q] = oc_bf16x2(x0, x1);
-    x0 -= oc_lo(w[q]);
-    x1 -= oc_hi(w[q]);
+      for (int ps = P == 3 ? 0 : P == 2 ? 3 : 5; ps < 6; ++ps) {
+        const uint64_t b0 = km0 + oc_pass_b(ps) * pl;
+        const uint32_t a0 = tmem + OC_G_COL + 64 * oc_pass_a(ps);
+        for (uint32_t kk = 0; kk < ks_u; ++kk) {   // 16 columns of X: 32 bytes within its 64-column chunk
+          const uint64_t b = b0 + (kk >> 2) * (ch >> 4) + (kk & 3u) * 2;
+          const uint32_t first = ps == (P == 3 ? 0 : P == 2 ? 3 : 5) && kk == 0 ? 0u : 1u;
+          if (issuer) tc_mma_ts(tmem, a0 + 8 * kk, b, idesc_u, first);
+          __syncwarp();
+        }
+      }
+      if (issuer) {
+        tc_commit(br.full);
+        tc_commit(br.full + 8);
+      }
+      __syncwarp();
+    }
+    // the stop test: the workers' pairs summed in a fixed order, v = n r^2 against squared thresholds
+    float2 t = make_float2(0.f, 0.f);
+    if (lane < OC_WARPS) t = make_float2(ctl->red[lane].x, ctl->red[lane].y);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)   // at most 16 of them; lane 0 has the sum
+      two_sum(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
+    t.x = __shfl_sync(0xffffffffu, t.x, 0);
+    t.y = __shfl_sync(0xffffffffu, t.y, 0);
+    const double v = (double)t.x + (double)t.y;
+    int dec = 2, status = ST_TIMEOUT;
+    if (go) {
+      const bool testing = k >= ctl->dr.n_pre;
+      if (!isfinite(t.x + t.y)) status = ST_NONFINITE;
+      else if (testing && v <= ctl->dr.v_tol) status = ST_CONVERGED;
+      else if (testing && k >= ctl->dr.n_pre + 2 && v > v_stag && v < ctl->dr.v_floor) status = ST_NOT_CONVERGED;
+      else if (k >= ctl->dr.max_iter) status = ST_NOT_CONVERGED;
+      else status = ST_RUNNING;
+      dec = status == ST_RUNNING ? 0 : 1;
+    }
+    const float c1 = k < ctl->dr.n_pre ? ctl->dr.pre_c1 : 1.5f, c3 = k < ctl->dr.n_pre ? ctl->dr.pre_c3 : -0.5f;
+    if (lane == 0) {
+      ctl->c1 = c1;
+      ctl->c3 = c3;
+      ctl->decision = dec;
+    }
+    v_stag = ctl->dr.stag2 * v_km1;
+    v_km1 = v;
+    oc_sync<4>();
+    if (lane == 0 && dec != 2) {
+      // the record of step k, as the batched finalize keeps it
+      const double r = sqrt(v) * inv_sqrt_n;
+      if (k < POLAR_HIST) {
+        st->res_hist[k] = r;
+        st->planes_hist[k] = (unsigned char)P;
+        st->hist_len = k + 1;
+      }
+      st->ring[k & 3] = r;
+      st->iters = k;
+      if (status != ST_RUNNING) st->status = status;
+      else {
+        st->upd_c1 = c1;
+        st->upd_c3 = c3;
+      }
+    }
+    if (dec != 0) break;
+  }
+  // everything issued has completed before the CTA frees TMEM
+  if (issued) {
+    if (issuer) tc_commit(br.drain);
+    __syncwarp();
+    mbar_drain(br.drain, 0);
   }
 }
 
-// MMA issue, by one thread: the Gram's 64-row slice s of X into accumulator s % 2, and the
-// update P^T = G X^T into columns 0 .. mp, each completed on its full barrier. Plane q of
-// X is read through MN-major descriptors (chunk stride ch, 8-row groups of 1024 bytes)
-// and K-major ones (rows of 128 bytes), built per MMA from the plane's address.
+// The whole loop for one problem by the workers. The four warps of a TMEM lane quarter take 16-wide chunks in
+// turn: chunk c of the Gram's columns and of the update's rows belongs to warp sub = c % 4 of the quarter.
 template <int P>
-struct OcIssuer {
-  static constexpr int NPASS = P == 3 ? 6 : (P == 2 ? 3 : 1);
-  static constexpr int P0 = 6 - NPASS;
-  // descriptor high word: stride between 8-row groups 1024 bytes, version 1, 128-byte swizzle
-  static constexpr uint32_t HI = (1024u >> 4) | (1u << 14) | (2u << 29);
-  uint32_t xbase, ch, tmem, full, idesc_g, idesc_u, ks_g, ks_u;
-
-  __device__ __forceinline__ void init(uint32_t xbase_, uint32_t ch_, uint32_t mp, uint32_t np, uint32_t tmem_,
-                                       uint32_t full_) {
-    xbase = xbase_;
-    ch = ch_;
-    tmem = tmem_;
-    full = full_;
-    idesc_g = oc_idesc(true, true, np);
-    idesc_u = oc_idesc(false, false, mp);
-    ks_g = mp / 16;
-    ks_u = np / 16;
-  }
-
-  __device__ __forceinline__ static uint64_t desc(uint32_t addr, uint32_t lbo) {
-    return ((uint64_t)HI << 32) | ((addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
-  }
-
-  __device__ __forceinline__ void gram_slice(uint32_t s) {
-    const uint32_t b = s & 1u;
-    const uint32_t k_end = 4 * s + 4 < ks_g ? 4 * s + 4 : ks_g;
-#pragma unroll
-    for (int ps = 0; ps < NPASS; ++ps) {
-      const uint32_t a0 = xbase + 2 * oc_pass_a(P0 + ps) * ch, b0 = xbase + 2 * oc_pass_b(P0 + ps) * ch;
-      for (uint32_t kk = 4 * s; kk < k_end; ++kk)   // 16 rows of X: 2048 bytes
-        tc_mma(tmem + 128 * b, desc(a0 + kk * 2048, ch), desc(b0 + kk * 2048, ch), idesc_g,
-               (ps == 0 && kk == 4 * s) ? 0u : 1u);
-    }
-    tc_commit(full + 8 * b);
-  }
-
-  __device__ __forceinline__ void update() {
-#pragma unroll
-    for (int ps = 0; ps < NPASS; ++ps) {
-      const uint32_t b0 = xbase + 2 * oc_pass_b(P0 + ps) * ch;
-      for (uint32_t kk = 0; kk < ks_u; ++kk)   // 16 columns of X: 32 bytes within its 64-column chunk
-        tc_mma_ts(tmem, tmem + OC_G_COL + 64 * oc_pass_a(P0 + ps) + 8 * kk, desc(b0 + (kk >> 2) * ch + (kk & 3u) * 32, 16),
-                  idesc_u, (ps == 0 && kk == 0) ? 0u : 1u);
-    }
-    tc_commit(full);
-    tc_commit(full + 8);
-  }
-};
-
-// The whole loop for one problem, all warps. The four warps of a TMEM lane quarter take
-// 16-wide chunks in turn: chunk c of the Gram's columns and of the update's rows belongs
-// to warp sub = c % 4 of the quarter. Thread 0 issues the MMAs as soon as a barrier has
-// published their operands (X_k in shared memory, G in TMEM, an accumulator read).
-template <int P>
-__device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xbase, uint32_t ch, uint32_t mp,
-                                      uint32_t np, uint32_t tmem, OcBars br, volatile OcCtl* ctl,
-                                      int warp, int lane, int withhold) {
+__device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t ch, uint32_t mp, uint32_t np,
+                                      uint32_t tmem, OcBars br, volatile OcCtl* ctl, int warp, int lane) {
   const int tid = warp * 32 + lane;
   const uint32_t sub = (uint32_t)warp >> 2;
   const uint32_t i = (uint32_t)((warp & 3) * 32 + lane);           // TMEM lane: a row of G, a column of X
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const int64_t m = tk.m, n = tk.n;
-  DevState* st = tk.st;
   volatile int* abort_flag = &ctl->abort;
-  // byte offset of column i in a plane for each of the 8 row phases of the swizzle
-  uint32_t colo[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) colo[e] = (i >> 6) * ch + ((((i & 63u) >> 3) ^ (uint32_t)e) << 4) + ((i & 7u) << 1);
-  OcIssuer<P> iss;
-  const bool issuer = tid == 0 && !withhold;
-  if (issuer) iss.init(xbase, ch, mp, np, tmem, br.full);
-  bool issued = false;
-  const double inv_sqrt_n = tid == 64 ? st->inv_sqrt_n : 0.0;
-  double v_km1 = 0.0, v_stag = 0.0;                                // warp 1: the last sum of squares, and the one
-                                                                   // before it times stagnation^2
   uint32_t use0 = 0, use1 = 0;                                     // completions awaited on full[0], full[1]
   const uint32_t nslices = (mp / 16 + 3) / 4;
   const uint32_t gch = np / 16, uch = mp / 16;                     // 16-wide chunks of G's columns, X's rows
   int k = 0;
   for (;; ++k) {
-    // X_k complete in shared memory (and the last accumulator read): the first two Gram slices
+    // X_k complete in shared memory (and the last accumulator read)
     oc_fence_async();
     tc_fence_before();
-    oc_sync_workers();
-    if (issuer && !*abort_flag) {
-      tc_fence_after();
-      iss.gram_slice(0);
-      if (nslices > 1) iss.gram_slice(1);
-      issued = true;
-    }
+    oc_arrive<2>();
     // ---- Gram: promote this warp's chunks (at most two) of every slice
-    float g[2][16];
+    float g[OC_GT][16];
 #pragma unroll
-    for (int t = 0; t < 2; ++t)
+    for (int t = 0; t < OC_GT; ++t)
 #pragma unroll
       for (int e = 0; e < 16; ++e) g[t][e] = 0.0f;
     for (uint32_t s = 0; s < nslices; ++s) {
@@ -246,30 +307,20 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
       ok = __all_sync(0xffffffffu, ok);
       if (ok) {
         tc_fence_after();
-        uint32_t v[2][16];
 #pragma unroll
-        for (int t = 0; t < 2; ++t)
-          if (sub + 4 * t < gch) oc_ld16(tmem + lane_addr + 128u * b + 16u * (sub + 4 * t), v[t]);
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          if (sub + 4 * t < gch) {
-            oc_wait16(v[t]);
+        for (int t = 0; t < OC_GT; ++t) {
+          if (sub + OC_SUB * t < gch) {
             float f[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) f[e] = __uint_as_float(v[t][e]);
+            tmem_ld16(tmem + lane_addr + 128u * b + 16u * (sub + OC_SUB * t), f);
             add16_packed(g[t], f);
           }
         }
       }
       if (b) ++use1; else ++use0;
-      if (s + 2 < nslices) {
-        // every warp has read slice s: its accumulator takes slice s + 2
+      if (s + 2 < nslices) {   // this accumulator takes slice s + 2
         tc_fence_before();
-        oc_sync_workers();
-        if (issuer && !*abort_flag) {
-          tc_fence_after();
-          iss.gram_slice(s + 2);
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(br.empty + 8 * b);
       }
     }
     // ---- residual ||G - I||_F^2 over the n x n block (float per thread, at most 32 terms;
@@ -278,8 +329,8 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
     float part32 = 0.0f;
     bool stored = false;
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const uint32_t c = sub + 4 * t;
+    for (int t = 0; t < OC_GT; ++t) {
+      const uint32_t c = sub + OC_SUB * t;
       if (c < gch) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
@@ -296,8 +347,9 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             w[j] = oc_bf16x2(g[t][2 * j], g[t][2 * j + 1]);
-            g[t][2 * j] -= oc_lo(w[j]);
-            g[t][2 * j + 1] -= oc_hi(w[j]);
+            const float2 rest = sub_x2(make_float2(g[t][2 * j], g[t][2 * j + 1]), bf16_pair(w[j]));
+            g[t][2 * j] = rest.x;
+            g[t][2 * j + 1] = rest.y;
           }
           oc_st8(tmem + lane_addr + OC_G_COL + 64u * qp + 8u * c, w);
         }
@@ -315,58 +367,8 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
       ctl->red[warp].y = part.y;
     }
     tc_fence_before();
-    oc_sync_workers();
-    // ---- the update starts at once, whatever the stop rule will say (its result is not used after a stop);
-    // meanwhile warp 1 sums the warps' pairs in a fixed order and decides on the sum of squares v = n r^2
-    // against squared thresholds; thread 64 records r and the outcome while the update runs
-    if (issuer && !*abort_flag) {
-      tc_fence_after();
-      iss.update();
-    }
-    if (warp == 1) {
-      const int wl = lane & (OC_WARPS - 1);
-      float2 t = make_float2(ctl->red[wl].x, ctl->red[wl].y);
-#pragma unroll
-      for (int o = OC_WARPS / 2; o > 0; o >>= 1)
-        two_sum(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
-      if (lane == 0) {
-        const double v = (double)t.x + (double)t.y;
-        int dec = 2, status = ST_TIMEOUT;
-        if (!*abort_flag) {
-          const bool testing = k >= ctl->dr.n_pre;
-          if (!isfinite(t.x + t.y)) status = ST_NONFINITE;
-          else if (testing && v <= ctl->dr.v_tol) status = ST_CONVERGED;
-          else if (testing && k >= ctl->dr.n_pre + 2 && v > v_stag && v < ctl->dr.v_floor) status = ST_NOT_CONVERGED;
-          else if (k >= ctl->dr.max_iter) status = ST_NOT_CONVERGED;
-          else status = ST_RUNNING;
-          dec = status == ST_RUNNING ? 0 : 1;
-          ctl->c1 = k < ctl->dr.n_pre ? ctl->dr.pre_c1 : 1.5f;
-          ctl->c3 = k < ctl->dr.n_pre ? ctl->dr.pre_c3 : -0.5f;
-          ctl->status = status;
-          ctl->v = v;
-        }
-        ctl->decision = dec;
-        v_stag = ctl->dr.stag2 * v_km1;
-        v_km1 = v;
-      }
-    }
-    oc_sync_workers();
-    if (tid == 64 && ctl->decision != 2) {
-      // the record of step k, as the batched finalize keeps it
-      const double r = sqrt(ctl->v) * inv_sqrt_n;
-      if (k < POLAR_HIST) {
-        st->res_hist[k] = r;
-        st->planes_hist[k] = (unsigned char)P;
-        st->hist_len = k + 1;
-      }
-      st->ring[k & 3] = r;
-      st->iters = k;
-      if (ctl->status != ST_RUNNING) st->status = ctl->status;
-      else {
-        st->upd_c1 = ctl->c1;
-        st->upd_c3 = ctl->c3;
-      }
-    }
+    oc_arrive<3>();
+    oc_sync<4>();   // the decision
     if (ctl->decision != 0) break;
     // ---- update: P^T = G X^T, then X_{k+1} = c1 X_k + c3 P in place, this warp's 16-row
     // chunks one at a time from TMEM with the next in flight
@@ -377,41 +379,38 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
     if (ok && sub < uch) {
       tc_fence_after();
       const float c1 = ctl->c1, c3 = ctl->c3;
-      const bool active = (int64_t)i < n;
+      // Lanes 2j and 2j + 1 share columns 2j and 2j + 1: the even lane takes rows 0..3 and 8..11 of a chunk of
+      // 16, the odd lane rows 4..7 and 12..15, both columns of each, so that X moves as 32-bit words and the
+      // arithmetic as FP32 pairs (rows four apart lie in different halves of the swizzled 128 bytes: no bank
+      // conflicts). Columns past n are zeros in X and in the product and stay so.
+      const uint32_t odd = i & 1u, i2 = i & ~1u;
+      const bool active = (int64_t)i2 < n;
+      const uint32_t cb = (i2 >> 6) * ch + ((i2 & 7u) << 1), unit = (i2 & 63u) >> 3;
       uint32_t cur[16], nxt[16];
       oc_ld16(tmem + lane_addr + 16u * sub, cur);
       oc_wait16(cur);
-      for (uint32_t c = sub; c < uch; c += 4) {
-        const bool more = c + 4 < uch;
-        if (more) oc_ld16(tmem + lane_addr + 16u * (c + 4), nxt);
+      for (uint32_t c = sub; c < uch; c += OC_SUB) {
+        const bool more = c + OC_SUB < uch;
+        if (more) oc_ld16(tmem + lane_addr + 16u * (c + OC_SUB), nxt);
         const uint32_t rb = 16u * c;
-        if (active && rb < (uint32_t)m) {
-          uint8_t* row = xs + rb * 128u;
 #pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            uint8_t* a0 = row + e * 128 + colo[e & 7];
-            uint8_t* a1 = row + (e + 1) * 128 + colo[(e + 1) & 7];
-            const bool v0 = rb + e < (uint32_t)m, v1 = rb + e + 1 < (uint32_t)m;
-            float x0 = 0.0f, x1 = 0.0f;
-            if (v0)
-              x0 = (bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a0)) +
-                    bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a0 + 2 * ch))) +
-                   bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a0 + 4 * ch));
-            if (v1)
-              x1 = (bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1)) +
-                    bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1 + 2 * ch))) +
-                   bf16_to_f32_dev(*reinterpret_cast<uint16_t*>(a1 + 4 * ch));
-            const float xn0 = fmaf(c1, x0, c3 * __uint_as_float(cur[e]));
-            const float xn1 = fmaf(c1, x1, c3 * __uint_as_float(cur[e + 1]));
-            uint32_t w[3];
-            oc_split2(xn0, xn1, w);
-            if (v0) {
+        for (int t = 0; t < 8; ++t) {
+          const int re = (t & 3) + 8 * (t >> 2), ro = re + 4;   // the even and the odd lane's row
+          const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? cur[re] : cur[ro], 1);
+          const float2 pr = make_float2(__uint_as_float(odd ? got : cur[re]), __uint_as_float(odd ? cur[ro] : got));
+          const uint32_t row = rb + (uint32_t)(odd ? ro : re);
+          if (active && row < (uint32_t)m) {
+            uint8_t* a = xs + row * 128u + ((unit ^ (row & 7u)) << 4) + cb;
+            const uint32_t h = *reinterpret_cast<uint32_t*>(a), md = *reinterpret_cast<uint32_t*>(a + 2 * ch),
+                           l = *reinterpret_cast<uint32_t*>(a + 4 * ch);
+            const float2 x = add_x2(add_x2(bf16_pair(h), bf16_pair(md)), bf16_pair(l));
+            // c1 X + (c3 P), the product with c3 = -0.5 exact
+            float2 r = fma_x2(make_float2(c1, c1), x, make_float2(c3 * pr.x, c3 * pr.y));
 #pragma unroll
-              for (int q = 0; q < 3; ++q) *reinterpret_cast<uint16_t*>(a0 + 2 * q * ch) = (uint16_t)w[q];
-            }
-            if (v1) {
-#pragma unroll
-              for (int q = 0; q < 3; ++q) *reinterpret_cast<uint16_t*>(a1 + 2 * q * ch) = (uint16_t)(w[q] >> 16);
+            for (int q = 0; q < 3; ++q) {
+              const uint32_t w = oc_bf16x2(r.x, r.y);
+              r = sub_x2(r, bf16_pair(w));
+              *reinterpret_cast<uint32_t*>(a + 2 * q * ch) = w;
             }
           }
         }
@@ -423,15 +422,10 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t xb
       }
     }
   }
-  // everything issued has completed before the CTA frees TMEM
-  if (tid == 0 && issued) {
-    tc_commit(br.drain);
-    mbar_drain(br.drain, 0);
-  }
   if (ctl->decision != 1) return;
   // ---- the final iterate's planes to global memory, where the H product and U read them
   uint16_t* dst = tk.xp[k & 1];
-  for (uint32_t u = (uint32_t)tid; u < 3u * (uint32_t)m * 16u; u += OC_THREADS) {
+  for (uint32_t u = (uint32_t)tid; u < 3u * (uint32_t)m * 16u; u += OC_WORKERS) {
     const uint32_t q = u / ((uint32_t)m * 16u), rem = u % ((uint32_t)m * 16u), r = rem >> 4, c8 = (rem & 15u) * 8u;
     if (c8 >= n) continue;
     const uint4 v = *reinterpret_cast<const uint4*>(xs + 2 * q * ch + oc_off(r, c8, ch));
@@ -461,10 +455,13 @@ __global__ void __launch_bounds__(OC_THREADS, 1)
   volatile OcCtl* ctl = reinterpret_cast<volatile OcCtl*>(xs + 6 * ch);
   OcBars br;
   br.full = smem_u32((const void*)&ctl->full[0]);
+  br.empty = smem_u32((const void*)&ctl->empty[0]);
   br.drain = smem_u32((const void*)&ctl->drain);
   if (threadIdx.x == 0) {
     mbar_init(br.full, 1);
     mbar_init(br.full + 8, 1);
+    mbar_init(br.empty, OC_WARPS);
+    mbar_init(br.empty + 8, OC_WARPS);
     mbar_init(br.drain, 1);
     ctl->abort = 0;
     ctl->decision = 0;
@@ -509,7 +506,8 @@ __global__ void __launch_bounds__(OC_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
-  oc_solve<P>(tk, xs, xbase, ch, mp, np, tmem, br, ctl, warp, lane, withhold);
+  if (warp < OC_WARPS) oc_solve<P>(tk, xs, ch, mp, np, tmem, br, ctl, warp, lane);
+  else oc_issue<P>(tk, xbase, ch, mp, np, tmem, br, ctl, lane, withhold);
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && ctl->decision == 2) {
