@@ -28,12 +28,12 @@ struct CoInverse {
   float2* part;                              // 2 EPI_WARPS per block
   DevState* st;
   int rows, cols, max_iter, withhold;
+  int sa2, su;                               // split chains: blocks per tile of A X and of the update
 };
 
-template <int TN>
-__global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_constant__ CoInverse p) {
-  extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
+template <int TN, bool SPLIT>
+__device__ __forceinline__ void co_inverse(const CoInverse& p, uint8_t* co_raw) {
+  CoCtx x = co_setup<TN, CO_P, SPLIT>(co_raw, &p.st->bar);
   const int N = p.rows, M = p.cols, tid = threadIdx.x;
   const int gtid = blockIdx.x * CO_THREADS + tid, gthr = gridDim.x * CO_THREADS;
   DevState* st = p.st;
@@ -61,17 +61,10 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
   // ---- a = ||A A^T||_F = ||A^T A||_F, from the upper triangle of A^T A
   if (run) {
     const CoTiles t = co_tiles<TN>(M, M, true);
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(&p.amn, &p.amn, nullptr, t, N), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, true, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, t, N));
-    } else if (x.warp < CO_CTL_WARP) {
-      CoEpi e{};
-      e.M = M; e.N = M;
-      e.norm = p.norm;
-      co_epilogue<TN, CO_EPI_NORM>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, t, N, &e));
-    }
+    CoEpi e{};
+    e.M = M; e.N = M;
+    e.norm = p.norm;
+    co_product<TN, SPLIT, true, false, CO_EPI_NORM>(x, pipe, &p.amn, &p.amn, nullptr, t, N, e, 1, p.withhold);
     run = co_grid_sync(x);
   }
   int status = ST_TIMEOUT;
@@ -116,17 +109,14 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
   int k = 0;
   for (; run; ++k) {
     const int b = k & 1;
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(&p.ak, &p.xmn[b], nullptr, ta, M), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, ta, M));
-    } else if (x.warp < CO_CTL_WARP) {
+    {
       CoEpi e{};
       e.M = N; e.N = N;
       e.out = p.pp; e.ldo = p.lpx; e.os = p.sp;
-      co_epilogue<TN, TC_EPI_PLANES>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, ta, M, &e));
-    } else if (k > 0) {
+      co_product<TN, SPLIT, false, false, TC_EPI_PLANES>(x, pipe, &p.ak, &p.xmn[b], nullptr, ta, M, e, p.sa2,
+                                                         p.withhold);
+    }
+    if (x.warp == CO_CTL_WARP && k > 0) {
       // Algorithm 2's test after update k - 1: ||X' - X||_F / ||X'||_F against u 2^(k-1), u = 2^-24
       const double sd = co_warp_sum2(p.part, gridDim.x * EPI_WARPS, 2, x.lane);
       const double sx = co_warp_sum2(p.part + 1, gridDim.x * EPI_WARPS, 2, x.lane);
@@ -152,20 +142,14 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
     if (k > 0) status = *reinterpret_cast<volatile int*>(&x.ctl->status);
     else status = ST_RUNNING;
     if (status != ST_RUNNING) break;
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(&p.xk[b], &p.pmn, nullptr, tu, N), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, false, false>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, N));
-    } else if (x.warp < CO_CTL_WARP) {
-      CoEpi e{};
-      e.M = M; e.N = N;
-      e.x = p.xp[b]; e.ldx = p.lpx; e.xs = p.sx;
-      e.out = p.xp[b ^ 1]; e.ldo = p.lpx; e.os = p.sx;
-      e.c1 = 2.0f; e.c3 = -1.0f;
-      e.part = p.part;
-      co_epilogue<TN, TC_EPI_NS_STEP>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tu, N, &e));
-    }
+    CoEpi e{};
+    e.M = M; e.N = N;
+    e.x = p.xp[b]; e.ldx = p.lpx; e.xs = p.sx;
+    e.out = p.xp[b ^ 1]; e.ldo = p.lpx; e.os = p.sx;
+    e.c1 = 2.0f; e.c3 = -1.0f;
+    e.part = p.part;
+    co_product<TN, SPLIT, false, false, TC_EPI_NS_STEP>(x, pipe, &p.xk[b], &p.pmn, nullptr, tu, N, e, p.su,
+                                                        p.withhold);
     run = co_grid_sync(x);
   }
   if (run && (status == ST_CONVERGED || status == ST_NOT_CONVERGED)) {
@@ -179,7 +163,18 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_
       store_row8(p.X + (int64_t)r * p.ldx + c, N - c, vec, v);
     }
   }
-  co_teardown<TN>(x, st);
+  co_teardown<TN, SPLIT>(x, st);
+}
+
+template <int TN>
+__global__ void __launch_bounds__(CO_THREADS, 1) co_inverse_kernel(const __grid_constant__ CoInverse p) {
+  extern __shared__ uint8_t co_raw[];
+  co_inverse<TN, false>(p, co_raw);
+}
+__global__ void __cluster_dims__(CO_CLUSTER, 1, 1) __launch_bounds__(CO_THREADS, 1)
+    co_inverse_split_kernel(const __grid_constant__ CoInverse p) {
+  extern __shared__ uint8_t co_raw[];
+  co_inverse<64, true>(p, co_raw);
 }
 
 // ------------------------------------------------------------------ Chebyshev
@@ -196,6 +191,7 @@ struct CoCheb {
   double am, bm, cd, cd1;                    // T = am A + bm I; c_d and c_{d-1}
   DevState* st;
   int n, degree, withhold;
+  int S;                                     // split chains: blocks per tile
   float coef[COOP_MAX_DEGREE + 1];
 };
 
@@ -208,10 +204,9 @@ __device__ __forceinline__ void co_put(uint16_t* P, int64_t ld, int64_t ps, int 
   for (int s = 0; s < 3; ++s) d[s * ps] = q[s];
 }
 
-template <int TN>
-__global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_constant__ CoCheb p) {
-  extern __shared__ uint8_t co_raw[];
-  CoCtx x = co_setup<TN>(co_raw, &p.st->bar);
+template <int TN, bool SPLIT>
+__device__ __forceinline__ void co_cheb(const CoCheb& p, uint8_t* co_raw) {
+  CoCtx x = co_setup<TN, CO_P, SPLIT>(co_raw, &p.st->bar);
   const int n = p.n, d = p.degree, tid = threadIdx.x;
   const int nt = (n + 31) / 32, npair = nt * (nt + 1) / 2;
   CoPipe pipe;
@@ -255,21 +250,15 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_con
   // ---- B_k = 2 T B_{k+1} - B_{k+2} + c_k I for k = d-2 .. 1, F = T B_1 - B_2 + c_0 I
   const CoTiles tt = co_tiles<TN>(n, n, true);
   for (int k = d - 2; k >= 0 && run; --k) {
-    if (x.warp == 0) {
-      if (x.lane == 0)
-        co_producer<TN, CO_P, true, true>(x, pipe, CoChainSrc<TN>(&p.tmn, &p.bmn[(k + 1) % 3], &p.bk[(k + 1) % 3], tt, n), p.withhold);
-    } else if (x.warp == 1) {
-      co_mma<TN, CO_P, true, true>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tt, n));
-    } else if (x.warp < CO_CTL_WARP) {
-      CoEpi e{};
-      e.M = n; e.N = n;
-      e.x = p.bp[(k + 2) % 3]; e.ldx = p.ldp; e.xs = p.sp;
-      e.out = p.bp[k % 3]; e.ldo = p.ldp; e.os = p.sp;
-      e.c1 = -1.0f;
-      e.c3 = k > 0 ? 2.0f : 1.0f;
-      e.diag = p.coef[k];
-      co_epilogue<TN, TC_EPI_CLENSHAW>(x, pipe, CoChainSrc<TN>(nullptr, nullptr, nullptr, tt, n, &e));
-    }
+    CoEpi e{};
+    e.M = n; e.N = n;
+    e.x = p.bp[(k + 2) % 3]; e.ldx = p.ldp; e.xs = p.sp;
+    e.out = p.bp[k % 3]; e.ldo = p.ldp; e.os = p.sp;
+    e.c1 = -1.0f;
+    e.c3 = k > 0 ? 2.0f : 1.0f;
+    e.diag = p.coef[k];
+    co_product<TN, SPLIT, true, true, TC_EPI_CLENSHAW>(x, pipe, &p.tmn, &p.bmn[(k + 1) % 3], &p.bk[(k + 1) % 3], tt, n,
+                                                       e, p.S, p.withhold);
     run = co_grid_sync(x);
   }
   // ---- F from the upper triangle
@@ -297,7 +286,18 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_con
       }
     }
   }
-  co_teardown<TN>(x, p.st);
+  co_teardown<TN, SPLIT>(x, p.st);
+}
+
+template <int TN>
+__global__ void __launch_bounds__(CO_THREADS, 1) co_cheb_kernel(const __grid_constant__ CoCheb p) {
+  extern __shared__ uint8_t co_raw[];
+  co_cheb<TN, false>(p, co_raw);
+}
+__global__ void __cluster_dims__(CO_CLUSTER, 1, 1) __launch_bounds__(CO_THREADS, 1)
+    co_cheb_split_kernel(const __grid_constant__ CoCheb p) {
+  extern __shared__ uint8_t co_raw[];
+  co_cheb<64, true>(p, co_raw);
 }
 
 // ------------------------------------------------------------------ host
@@ -306,9 +306,18 @@ template <class Params>
 cudaError_t co_run(void (*kernel)(Params), const Params& p, size_t smem, int grid, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(CO_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   void* args[] = {const_cast<Params*>(&p)};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)grid), dim3(CO_THREADS),
-                                     args, smem, s);
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), args);
 }
 
 TcOperand co_operand(const uint16_t* planes, int64_t rows, int64_t cols, int64_t ld, int64_t stride) {
@@ -341,12 +350,18 @@ cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaS
   p.A = a.A; p.lda = a.lda; p.X = a.X; p.ldx = a.ldx;
   p.ap = a.ap; p.pp = a.pp;
   p.lpa = a.lpa; p.sa = a.sa; p.lpx = a.lpx; p.sx = a.sx; p.sp = a.sp;
+  const CoopProduct prod[2] = {{a.rows, a.rows, a.cols, false}, {a.cols, a.rows, a.rows, false}};
+  int S[2] = {1, 1}, blocks = 0;
+  const bool split = coop_split_plan(prod, 2, sms, S, &blocks);
   const int grid = co_grid(a.rows, a.rows, tn, sms);
+  p.sa2 = S[0];
+  p.su = S[1];
   p.norm = a.sums;
   p.part = reinterpret_cast<float2*>(a.sums + (size_t)sms * EPI_WARPS);
   p.st = a.st;
   p.rows = (int)a.rows; p.cols = (int)a.cols; p.max_iter = a.max_iter;
   p.withhold = tc_withhold();
+  if (split) return co_run(co_inverse_split_kernel, p, co_smem<64, CO_P, true>(), blocks, s);
   return tn == 64 ? co_run(co_inverse_kernel<64>, p, co_smem<64>(), grid, s)
                   : co_run(co_inverse_kernel<128>, p, co_smem<128>(), grid, s);
 }
@@ -354,6 +369,10 @@ cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaS
 cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_t s) {
   CoCheb p{};
   if (a.degree < 2 || a.degree > COOP_MAX_DEGREE) return cudaErrorInvalidValue;
+  const CoopProduct prod = {a.n, a.n, a.n, true};
+  int blocks = 0;
+  const bool split = coop_split_plan(&prod, 1, sms, &p.S, &blocks);
+  if (split) tn = 64;
   bool ok = tc_make_map(&p.tmn, co_operand(a.tp, a.n, a.n, a.ldp, a.sp), CO_P, true, 0);
   for (int i = 0; i < 3; ++i) {
     const TcOperand B = co_operand(a.bp[i], a.n, a.n, a.ldp, a.sp);
@@ -369,6 +388,7 @@ cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_
   p.n = (int)a.n; p.degree = a.degree;
   p.withhold = tc_withhold();
   const int grid = co_grid(a.n, a.n, tn, sms);
+  if (split) return co_run(co_cheb_split_kernel, p, co_smem<64, CO_P, true>(), blocks, s);
   return tn == 64 ? co_run(co_cheb_kernel<64>, p, co_smem<64>(), grid, s)
                   : co_run(co_cheb_kernel<128>, p, co_smem<128>(), grid, s);
 }

@@ -613,15 +613,18 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
   using C = CoCfg<64, CO_P, true>;
   const int q = x.warp & 3, half = (x.warp - 2) >> 2, lane = x.lane, w = x.warp - 2;
   const int sub = (int)blockIdx.x % S, rows = 128 / S, units = 4 / S;
+  constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP, STEP = EPI == TC_EPI_NS_STEP;
+  constexpr bool READS_X = NS || EPI == TC_EPI_CLENSHAW;
   CoTile ti;
-  float2 sum0 = make_float2(0.f, 0.f);
+  float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
+  double norm = 0.0;
   const bool have = src.next(ti);        // the same in every block of the group
   const CoEpi& e = src.epi(ti);
   if (have) {
     const int nslices = (ti.K - ti.kbeg + 63) / 64;
     const int col = ti.bj * 64 + 8 * (lane & 7);
     Planes8 pre[2];
-    if (EPI == TC_EPI_NS) {
+    if (READS_X) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int r = ti.bi * BM + sub * rows + (u * EPI_WARPS + w) * 4 + (lane >> 3);
@@ -687,12 +690,35 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           }
           two_sum(sum0, make_float2(t, 0.f));
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
-        } else if (EPI == TC_EPI_NS) {
-          float xo[8];
+        } else if (READS_X) {
+          float xo[8], d2 = 0.0f, x2 = 0.0f;
           sum_planes8(pre[u], xo);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = fmaf(e.c1, xo[j], e.c3 * v[j]);   // c3 = -0.5: one rounding
+          for (int j = 0; j < 8; ++j) {
+            if (NS) {
+              v[j] = fmaf(e.c1, xo[j], e.c3 * v[j]);   // c3 = -0.5, -1: one rounding
+              if (STEP) {
+                d2 = fmaf(v[j] - xo[j], v[j] - xo[j], d2);
+                x2 = fmaf(v[j], v[j], x2);
+              }
+            } else {
+              v[j] = fmaf(e.c3, v[j], e.c1 * xo[j]);
+              if (r == col + j) v[j] += e.diag;
+            }
+          }
+          if (STEP) {
+            two_sum(sum0, make_float2(d2, 0.f));
+            two_sum(sum1, make_float2(x2, 0.f));
+          }
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
+        } else if (EPI == TC_EPI_PLANES) {
+          store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
+        } else if (EPI == CO_EPI_NORM) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const double g = (double)v[j], wt = col + j < r ? 0.0 : col + j == r ? 1.0 : 2.0;
+            norm = fma(wt * g, g, norm);
+          }
         } else {   // STORE (a pitch that is a multiple of 4)
           float* cr = e.C + r * e.ldc + col;
           if (col < e.ldc) *reinterpret_cast<float4*>(cr) = make_float4(v[0], v[1], v[2], v[3]);
@@ -701,11 +727,45 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
       }
     }
   }
-  if (EPI == TC_EPI_GRAM) {
+  if (EPI == CO_EPI_NORM) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
+    if (lane == 0) __stcg(e.norm + blockIdx.x * EPI_WARPS + w, norm);
+  }
+  if (EPI == TC_EPI_GRAM || STEP) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
       two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-    if (lane == 0) __stcg(e.part + blockIdx.x * EPI_WARPS + w, sum0);
+      if (STEP)
+        two_sum(sum1, make_float2(__shfl_xor_sync(0xffffffffu, sum1.x, o), __shfl_xor_sync(0xffffffffu, sum1.y, o)));
+    }
+    if (lane == 0) {
+      float2* dst = e.part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + w);
+      __stcg(dst, sum0);
+      if (STEP) __stcg(dst + 1, sum1);
+    }
+  }
+}
+
+
+// One product of a chain by all its roles, its tiles shared by S blocks.
+template <int TN, bool SPLIT, bool A_MN, bool SYM, int EPI>
+__device__ __forceinline__ void co_product(CoCtx& x, CoPipe& pipe, const CUtensorMap* ma, const CUtensorMap* mb,
+                                           const CUtensorMap* mbt, CoTiles t, int K, const CoEpi& e, int S,
+                                           int withhold) {
+  using Src = CoChainSrc<TN, SPLIT>;
+  if (x.warp == 0) {
+    if (x.lane == 0) co_producer<TN, CO_P, A_MN, SYM>(x, pipe, Src(ma, mb, mbt, t, K, nullptr, S), withhold);
+  } else if (x.warp == 1) {
+    co_mma<TN, CO_P, A_MN, SYM>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, nullptr, S));
+  } else if (x.warp < CO_CTL_WARP) {
+    if constexpr (SPLIT) {
+      if (S > 1) {
+        co_epilogue_split<EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e, S), S);
+        return;
+      }
+    }
+    co_epilogue<TN, EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e));
   }
 }
 

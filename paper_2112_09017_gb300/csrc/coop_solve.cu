@@ -56,27 +56,6 @@ __device__ __forceinline__ int co_stop_status(const CoSolve& p, int k, double v,
   return ST_RUNNING;
 }
 
-// One product of the solve by all its roles.
-template <int TN, bool SPLIT, bool A_MN, bool SYM, int EPI>
-__device__ __forceinline__ void co_product(CoCtx& x, CoPipe& pipe, const CUtensorMap* ma, const CUtensorMap* mb,
-                                           const CUtensorMap* mbt, CoTiles t, int K, const CoEpi& e, int S,
-                                           int withhold) {
-  using Src = CoChainSrc<TN, SPLIT>;
-  if (x.warp == 0) {
-    if (x.lane == 0) co_producer<TN, CO_P, A_MN, SYM>(x, pipe, Src(ma, mb, mbt, t, K, nullptr, S), withhold);
-  } else if (x.warp == 1) {
-    co_mma<TN, CO_P, A_MN, SYM>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, nullptr, S));
-  } else if (x.warp < CO_CTL_WARP) {
-    if constexpr (SPLIT) {
-      if (S > 1) {
-        co_epilogue_split<EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e, S), S);
-        return;
-      }
-    }
-    co_epilogue<TN, EPI>(x, pipe, Src(nullptr, nullptr, nullptr, t, K, &e));
-  }
-}
-
 template <int TN, bool SPLIT>
 __device__ __forceinline__ void co_solve(const CoSolve& p, uint8_t* co_raw) {
   CoCtx x = co_setup<TN, CO_P, SPLIT>(co_raw, &p.st->bar);
@@ -374,6 +353,23 @@ static int co_split_of(const CoopProduct& q, int blocks, double* cycles) {
   return best;
 }
 
+bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks) {
+  *blocks = CO_CLUSTER * co_split_clusters(sms);
+  if (*blocks <= 0) return false;
+  int64_t waves;
+  const double whole = co_cost<64>(p, count, sms, &waves), wide = co_cost<128>(p, count, sms, &waves);
+  double split = 0.0, c;
+  int64_t want = CO_CLUSTER;
+  for (int i = 0; i < count; ++i) {
+    S[i] = co_split_of(p[i], *blocks, &c);
+    split += c;
+    want = std::max<int64_t>(want, (int64_t)co_tiles<64>(p[i].M, p[i].N, p[i].tri).ntiles * S[i]);
+    want = std::max<int64_t>(want, (p[i].M * p[i].N + 8191) / 8192);
+  }
+  *blocks = (int)std::min<int64_t>(*blocks, (want + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER);
+  return split < 0.9 * std::min(whole, wide);
+}
+
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {
   const CoopProduct prod[2] = {{n, n, m, true}, {m, n, n, false}};
   const int tn = coop_tile_n(prod, 2, sms);
@@ -382,32 +378,21 @@ CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms
   if (!c) return nullptr;
   c->tn = tn;
   // few tiles: share each between blocks along K, where that shortens a step by a tenth
-  const int blocks = CO_CLUSTER * co_split_clusters(sms);
-  c->split = false;
+  int S[2], blocks;
+  c->split = coop_split_plan(prod, 2, sms, S, &blocks) && blocks <= b.nparts / 2;
   c->p.sg = c->p.su = c->p.sh = 1;
-  if (blocks > 0 && blocks <= b.nparts / 2) {
-    int64_t waves;
-    double cg, cu, ch;
-    const double whole = co_cost<64>(prod, 2, sms, &waves), wide = co_cost<128>(prod, 2, sms, &waves);
-    const int sg = co_split_of(prod[0], blocks, &cg), su = co_split_of(prod[1], blocks, &cu);
-    const CoopProduct h = {n, n, m, false};
-    if (cg + cu < 0.9 * std::min(whole, wide)) {
-      c->split = true;
-      c->tn = 64;
-      c->p.sg = sg;
-      c->p.su = su;
-      c->p.sh = co_split_of(h, blocks, &ch);
-    }
+  if (c->split) {
+    double ch;
+    c->tn = 64;
+    c->p.sg = S[0];
+    c->p.su = S[1];
+    c->p.sh = co_split_of({n, n, m, false}, blocks, &ch);
   }
   // enough blocks for the larger product's tiles, and for the passes over A
   const int64_t tiles = c->tn == 64 ? co_tiles<64>(m, n, false).ntiles : co_tiles<128>(m, n, false).ntiles;
   int64_t grid = std::max<int64_t>(tiles, (m * n + 8191) / 8192);
   grid = std::min<int64_t>(grid, std::min<int64_t>(sms, b.nparts / 2));
-  if (c->split) {
-    const int64_t t = std::max<int64_t>(std::max<int64_t>((int64_t)co_tiles<64>(n, n, true).ntiles * c->p.sg, tiles * c->p.su),
-                                        std::max<int64_t>((int64_t)co_tiles<64>(n, n, false).ntiles * c->p.sh, (m * n + 8191) / 8192));
-    grid = std::min<int64_t>(blocks, (t + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER);
-  }
+  if (c->split) grid = blocks;
   if (!c->split && tiles <= 2) grid = 1;   // a second tile takes less time than two grid barriers
   c->grid = (int)std::max<int64_t>(grid, 1);
   if (8 * c->grid > b.nparts && (size_t)8 * c->grid * 8 > (size_t)n * b.ldc * 4) {

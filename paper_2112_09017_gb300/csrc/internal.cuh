@@ -267,6 +267,9 @@ struct CoopProduct {
   bool tri;                                       // only the upper triangle's tiles
 };
 int coop_tile_n(const CoopProduct* p, int count, int sms);   // tile width of a chain; 0: not for these sizes
+// Whether the chain is better run with blocks of a cluster sharing 128 x 64 tiles along K: S[i] blocks (1, 2 or
+// 4) per tile of product i, on *blocks blocks.
+bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks);
 constexpr int COOP_MAX_DEGREE = 511;
 struct CoopInverseArgs {
   const float* A; int64_t rows, cols, lda;
