@@ -77,14 +77,14 @@ typedef void* polar_stream_t;
 typedef struct polar_plan_s* polar_plan_t;
 
 /* One entry of a batched plan's tuning table: the problems with n_lo <= n <= n_hi and
- * aspect_lo <= m / n <= aspect_hi use the tile width and slice length given here (the first
- * matching entry wins; problems no entry matches use the plan's options). Written by the
- * library's autotuner (paper_2112_09017_gb300/autotune.py), which times the choices per size
- * bucket and keeps the fastest whose orthogonality and backward errors stay within 5e-6. */
+ * aspect_lo <= m / n <= aspect_hi use the slice length given here (the first matching entry
+ * wins; problems no entry matches use the library's). Written by the library's autotuner
+ * (paper_2112_09017_gb300/autotune.py), which times the choices per size bucket and keeps the
+ * fastest whose orthogonality and backward errors stay within 5e-6. */
 typedef struct {
   int64_t n_lo, n_hi;
   double aspect_lo, aspect_hi;
-  int tile_n;        /* width of the grouped launches' output tiles: 128 or 256 (0: the plan's) */
+  int tile_n;        /* accepted, without effect: the batched loop's tiles are 128 wide */
   int slice_stages;  /* 32-element k-stages accumulated per promoted slice, 1..8 (0: the library's) */
 } polar_tune_entry_t;
 
@@ -103,14 +103,11 @@ typedef struct {
   double s_minus;          /* preconditioning threshold; <= 0 means 0.1 */
   double s0;               /* estimate of the smallest singular value of A / ||A||_F; <= 0 means 2^-23 */
   double fp8_switch_residual; /* SCHED_FP8_BF16_X3: residual below which the FP8 phase ends; <= 0 means 0.5 */
-  int batched_tile_n;      /* batched plans: width of the grouped launches' output tiles, 256 (0 means 256:
-                              one epilogue group, as in the single solve) or 128 (two epilogue groups on
-                              alternate tiles, so that one tile's output step can overlap the next tile's
-                              products; measured no faster on the 4096-problem configuration) */
+  int batched_tile_n;      /* batched plans: accepted, without effect (the loop's tiles are 128 wide) */
   int small_onchip;        /* batched plans with a fixed plane count: nonzero (the default) solves every
                               problem with n <= 128 and m <= 256 in one CTA that keeps X, G and the
                               accumulators on its SM for the whole loop; 0 sends them through the
-                              grouped tile kernels like the others */
+                              tiled loop like the others */
   const polar_tune_entry_t* tune; /* batched plans: a tuning table of n_tune entries (host memory, read
                               only during plan creation), or NULL */
   int n_tune;
@@ -127,7 +124,8 @@ typedef struct {
   double normA_F;             /* ||A||_F (float64 accumulation) */
   double sym_err;             /* ||skew(U^T A)||_F / ||U^T A||_F */
   float ms_total;             /* device time of the whole solve (CUDA events), milliseconds */
-  int launches;               /* kernels this run enqueued (including ones that found the run stopped) */
+  int launches;               /* kernels this run enqueued (including ones that found the run stopped); 1 when
+                                 the whole solve is one cooperative launch */
   int n_gram, n_update;       /* profile: Gram and update launches that did work */
   int n_precond;              /* preconditioning steps among the iters updates (0 without preconditioning) */
   float ms_gram, ms_update;   /* profile: their summed device time (CUDA events), milliseconds */
@@ -252,8 +250,8 @@ POLAR_API polar_status_t polar_split_bf16(const float* X, int64_t count, int pla
  * ill-conditioned A (kappa >~ 1e2) the result is an approximate inverse. prec: BF16X6, BF16X3 or BF16
  * (products on the tensor cores with the same promotion as polar_run); FP32 -> ENOTSUP. Device pointers.
  * Its workspace is a library-owned block of at most 512 MiB kept between calls (one per device; concurrent
- * calls get their own), or, when that does not fit, allocated for the call; returns after the result is in X. *iters (updates applied)
- * and *delta (the last relative change) may be NULL. Returns OK, NOT_CONVERGED (max_iter reached),
+ * calls get their own), or, when that does not fit, allocated for the call; returns after the result is in X.
+ * *iters (updates applied) and *delta (the last relative change) may be NULL. Returns OK, NOT_CONVERGED (max_iter reached),
  * ENONFINITE (A zero or non-finite), EINVAL, ENOMEM, ENOTSUP or ECUDA.
  * Paper: Sec. III.D, Algorithm 2. */
 POLAR_API polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t cols, int64_t lda, float* X,

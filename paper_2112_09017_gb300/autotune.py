@@ -1,16 +1,13 @@
-"""Autotuner of batched plans: per size bucket, the tile width of the grouped launches and the
-slice length of the promotion, chosen by timing.
+"""Autotuner of batched plans: per size bucket, the slice length of the promotion, chosen by timing.
 
-The grouped Gram and update launches of a batched plan (polar_batched_plan_create) take two
-choices per problem: the width of the output tiles (256, one epilogue group; or 128, two groups on
-alternate tiles, less padding for n just above a multiple of 128) and the number of 32-element
-k-stages accumulated in TMEM before each round-to-nearest promotion (2 or 4: 64 or 128 of K; longer
-slices issue fewer promotions but let the accumulator's round-toward-zero drift longer, so they
-can cost accuracy). For every bucket of problem sizes (n in a range, m = n or m = 2n) the tuner
-times each candidate on a synthetic batch of that bucket and keeps the fastest whose worst
-orthogonality ||U^T U - I||_F / sqrt(n) and backward error ||A - U H||_F / ||A||_F over the batch
-stay within 5e-6. Problems with n <= 128 and m <= 256 are solved one SM each (no tiles) and are not
-tuned.
+The batched loop's products (polar_batched_plan_create) take one choice per problem: the number of
+32-element k-stages accumulated in TMEM before each round-to-nearest promotion (2 or 4: 64 or 128 of K;
+longer slices issue fewer promotions but let the accumulator's round-toward-zero drift longer, so they
+can cost accuracy). Entries also name a tile width, which the library accepts and ignores: its batched
+tiles are 128 wide. For every bucket of problem sizes (n in a range, m = n or m = 2n) the tuner times
+each candidate on a synthetic batch of that bucket and keeps the fastest whose worst orthogonality
+||U^T U - I||_F / sqrt(n) and backward error ||A - U H||_F / ||A||_F over the batch stay within 5e-6.
+Problems with n <= 128 and m <= 256 are solved one SM each (no tiles) and are not tuned.
 
 The result is cached as JSON under ``tuning/`` keyed by the GPU's name and the plane count, and
 ``load()`` returns its entries in the form polar_batched_plan_create(..., tune=...) takes (the
@@ -32,7 +29,7 @@ TUNING_DIR = os.path.join(HERE, "tuning")
 # (n_lo, n_hi) buckets beyond the on-chip sizes, and the two aspect classes m = n and m = 2n
 BUCKETS = [(129, 256), (257, 384), (385, 512), (513, 768), (769, 1024)]
 ASPECTS = [(1, 0.0, 1.5), (2, 1.5, 1.0e9)]          # (m / n drawn, aspect_lo, aspect_hi)
-CANDIDATES = [(256, 2), (256, 4), (128, 2), (128, 4)]  # (tile_n, slice_stages)
+CANDIDATES = [(128, 2), (128, 4)]  # (tile_n, slice_stages)
 BOUND = 5e-6
 
 
