@@ -44,7 +44,7 @@ struct GridBarrier {
 
   // After the block's last sync: the last block out clears the words for the next launch.
   __device__ __forceinline__ void leave() {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && w) {   // no words: a launch without barriers
       __threadfence();
       if (atomicAdd(&w->left, 1u) == gridDim.x - 1) {
         w->count = 0;

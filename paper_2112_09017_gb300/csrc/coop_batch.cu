@@ -23,7 +23,7 @@ enum : int { CB_GRAM = 0, CB_UPDATE = 1, CB_H = 2 };
 // status on their way while a tile is worked on; no status changes during a product.
 template <int KIND>
 struct CoTableSrc {
-  static constexpr bool TABLE = true, SPLIT = false;
+  static constexpr bool TABLE = true, SPLIT = false, BKM = false;
   const CoBatch& p;
   const TcTile* tiles;
   int n, par, t;

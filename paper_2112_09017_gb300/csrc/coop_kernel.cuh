@@ -26,7 +26,8 @@ constexpr int CO_P = 3;                     // planes of the chains (the batched
 constexpr int CO_THREADS = NTHREADS + 32;   // one warp more, for what must not hold up the products: the stop test
 constexpr int CO_WARPS = CO_THREADS / 32;
 constexpr int CO_CTL_WARP = CO_WARPS - 1;
-constexpr int CO_EPI_NORM = 16;             // beside the TcEpi kinds: no output, ||C||_F^2 of a symmetric product
+// beside the TcEpi kinds: no output, ||C||_F^2 of a symmetric product; C = c3 acc + c1 C, any pitch and alignment
+constexpr int CO_EPI_NORM = 16, CO_EPI_GEMM = 17;
 
 template <int TN, int P = CO_P, bool SPLIT = false>
 struct CoCfg {
@@ -140,9 +141,10 @@ struct CoEpi;
 // Tiles of one product of a chain: this block's are blockIdx.x, blockIdx.x + gridDim.x, ... With S > 1 (split
 // chains) S neighbouring blocks of a cluster share a tile, each taking a part of K, and there are at least as
 // many such groups as tiles.
-template <int TN, bool SPLIT_ = false>
+template <int TN, bool SPLIT_ = false, bool BKM_ = false>
 struct CoChainSrc {
   static constexpr bool TABLE = false, SPLIT = SPLIT_;
+  static constexpr bool BKM = BKM_;          // B is a K-major operand (its map is mbt)
   const CUtensorMap *ma, *mb, *mbt;
   CoTiles ct;
   int K, kbeg;
@@ -276,7 +278,7 @@ __device__ __forceinline__ void co_producer(const CoCtx& x, CoPipe& pp, Src src,
   CoTile c;
   while (ok && src.next(c)) {
     const int m0 = c.bi * BM, n0 = c.bj * TN, K = c.K;
-    const int km = SYM ? co_mirror_from<TN>(n0) : 0x7fffffff;
+    const int km = Src::BKM ? 0 : SYM ? co_mirror_from<TN>(n0) : 0x7fffffff;
     const CUtensorMap *ma = c.ma, *mb = c.mb, *mbt = c.mbt;
     for (int k0 = c.kbeg; k0 < K; k0 += C::BKS) {
       if (!mbar_wait(x.br.empty0 + 8 * stage, phase ^ 1u, x.abort_flag)) { ok = false; break; }
@@ -332,7 +334,7 @@ __device__ __forceinline__ void co_mma(const CoCtx& x, CoPipe& pp, Src src) {
   CoTile c;
   while (ok && src.next(c)) {
     const int K = c.K, kin_last = Src::TABLE ? c.slice / C::SUB - 1 : C::SLICE - 1;
-    const int km = SYM ? co_mirror_from<TN>(c.bj * TN) : 0x7fffffff;
+    const int km = Src::BKM ? 0 : SYM ? co_mirror_from<TN>(c.bj * TN) : 0x7fffffff;
     int kin = 0;
     if (Src::SPLIT && c.kbeg >= K) continue;   // no part of K for this block
     ok = mbar_wait_warp(br.tempty0 + 8 * buf, buf_phase ^ 1u, abort_flag) &&
@@ -401,6 +403,25 @@ struct CoEpi {
   double* norm;              // NORM: per epilogue warp of every block
   double* tile_part;         // GRAM from a table: this tile's EPI_WARPS sums
 };
+
+// 8 consecutive entries of a row of C = c3 v + c1 C (C is not read for c1 = 0), `n` of them existing.
+__device__ __forceinline__ void co_gemm_store8(float* c, int n, bool vec, float c1, float c3, const float* v) {
+  if (vec && n >= 8) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4 o = make_float4(c3 * v[4 * h], c3 * v[4 * h + 1], c3 * v[4 * h + 2], c3 * v[4 * h + 3]);
+      if (c1 != 0.0f) {
+        const float4 x = reinterpret_cast<const float4*>(c)[h];
+        o = make_float4(fmaf(c1, x.x, o.x), fmaf(c1, x.y, o.y), fmaf(c1, x.z, o.z), fmaf(c1, x.w, o.w));
+      }
+      reinterpret_cast<float4*>(c)[h] = o;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < n) c[j] = c1 != 0.0f ? fmaf(c1, c[j], c3 * v[j]) : c3 * v[j];
+  }
+}
 
 // Sums over each warp's tiles, as unevaluated pairs hi + lo, go to e.part: GRAM ||G - I||_F^2; NS_STEP
 // ||X' - X||^2 and ||X'||^2. NORM's go to e.norm, in float64 (entries of any magnitude).
@@ -526,6 +547,12 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
           }
           if (rows4 & (1u << i)) store_planes8(pr + i * e.ldo, e.os, 3, v + 8 * i);
         }
+      } else if (EPI == CO_EPI_GEMM) {
+        const bool vec = (reinterpret_cast<uintptr_t>(e.C) & 15u) == 0 && (e.ldc & 3) == 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (rows4 & (1u << i))
+            co_gemm_store8(e.C + (r4 + i) * e.ldc + c0 + 8 * lq, e.N - c0 - 8 * lq, vec, e.c1, e.c3, v + 8 * i);
       } else {   // STORE: whole 16-byte groups up to a pitch that is a multiple of 4, else single entries
         float* cr = e.C + r4 * e.ldc + c0 + 8 * lq;
 #pragma unroll
@@ -713,6 +740,9 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
         } else if (EPI == TC_EPI_PLANES) {
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
+        } else if (EPI == CO_EPI_GEMM) {
+          co_gemm_store8(e.C + r * e.ldc + col, e.N - col,
+                         (reinterpret_cast<uintptr_t>(e.C) & 15u) == 0 && (e.ldc & 3) == 0, e.c1, e.c3, v);
         } else if (EPI == CO_EPI_NORM) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -749,11 +779,11 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
 
 
 // One product of a chain by all its roles, its tiles shared by S blocks.
-template <int TN, bool SPLIT, bool A_MN, bool SYM, int EPI>
+template <int TN, bool SPLIT, bool A_MN, bool SYM, int EPI, bool BKM = false>
 __device__ __forceinline__ void co_product(CoCtx& x, CoPipe& pipe, const CUtensorMap* ma, const CUtensorMap* mb,
                                            const CUtensorMap* mbt, CoTiles t, int K, const CoEpi& e, int S,
                                            int withhold) {
-  using Src = CoChainSrc<TN, SPLIT>;
+  using Src = CoChainSrc<TN, SPLIT, BKM>;
   if (x.warp == 0) {
     if (x.lane == 0) co_producer<TN, CO_P, A_MN, SYM>(x, pipe, Src(ma, mb, mbt, t, K, nullptr, S), withhold);
   } else if (x.warp == 1) {

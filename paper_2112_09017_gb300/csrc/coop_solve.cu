@@ -353,11 +353,12 @@ static int co_split_of(const CoopProduct& q, int blocks, double* cycles) {
   return best;
 }
 
-bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks) {
-  *blocks = CO_CLUSTER * co_split_clusters(sms);
-  if (*blocks <= 0) return false;
+bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks, double* cycles) {
   int64_t waves;
   const double whole = co_cost<64>(p, count, sms, &waves), wide = co_cost<128>(p, count, sms, &waves);
+  if (cycles) *cycles = whole;
+  *blocks = CO_CLUSTER * co_split_clusters(sms);
+  if (*blocks <= 0) return false;
   double split = 0.0, c;
   int64_t want = CO_CLUSTER;
   for (int i = 0; i < count; ++i) {
@@ -367,7 +368,9 @@ bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* bloc
     want = std::max<int64_t>(want, (p[i].M * p[i].N + 8191) / 8192);
   }
   *blocks = (int)std::min<int64_t>(*blocks, (want + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER);
-  return split < 0.9 * std::min(whole, wide);
+  if (split >= 0.9 * std::min(whole, wide)) return false;
+  if (cycles) *cycles = split;
+  return true;
 }
 
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {

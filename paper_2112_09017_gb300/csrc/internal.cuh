@@ -269,7 +269,10 @@ struct CoopProduct {
 int coop_tile_n(const CoopProduct* p, int count, int sms);   // tile width of a chain; 0: not for these sizes
 // Whether the chain is better run with blocks of a cluster sharing 128 x 64 tiles along K: S[i] blocks (1, 2 or
 // 4) per tile of product i, on *blocks blocks.
-bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks);
+bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks, double* cycles = nullptr);
+// One product C = alpha op(A) op(B) + beta C of a STORE launch in 128 x 64 tiles (coop_gemm.cu), three planes.
+bool co_gemm_better(const TcArgs& a);             // whether that is faster than 128 x 256 tiles
+cudaError_t launch_co_gemm(const TcArgs& a, cudaStream_t s);
 constexpr int COOP_MAX_DEGREE = 511;
 struct CoopInverseArgs {
   const float* A; int64_t rows, cols, lda;

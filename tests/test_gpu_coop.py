@@ -120,6 +120,33 @@ def test_fp32_products_in_small_tiles(lib, ta, tb, M, N, K, off):
     assert np.all(err <= gemm_bound(np.abs(A64), np.abs(B64), K, np.abs(c), 0.75, -1.25))
 
 
+# tiles shared by four blocks and by two, whole tiles in one wave and in several; C's rows aligned and not (a
+# view one element into a wider matrix)
+@pytest.mark.parametrize("ta", [False, True])
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("M,N,K,off", [(48, 70, 6000, 0), (129, 65, 200, 1), (700, 500, 260, 1), (1000, 1001, 97, 0),
+                                       (2000, 1500, 131, 1)], ids=lambda v: str(v))
+def test_bf16x6_products_in_narrow_tiles(lib, ta, tb, M, N, K, off):
+    import torch
+
+    from .gpu_util import gemm_bound
+    rng = np.random.default_rng(M + N + K)
+    a = rng.standard_normal((K, M) if ta else (M, K)).astype(np.float32)
+    b = rng.standard_normal((N, K) if tb else (K, N)).astype(np.float32)
+    c = rng.standard_normal((M, N)).astype(np.float32)
+    big = torch.full((M + 1, N + 3 * off), 7.0, device="cuda")
+    C = big[:M, off:off + N]
+    for beta in (-1.25, 0.0):
+        C.copy_(torch.from_numpy(c) if beta else torch.full((M, N), float("nan")))
+        lib.polar_gemm(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda(), C, ta, tb, 0.75, beta, lib.POLAR_BF16X6)
+        A64 = (a.T if ta else a).astype(np.float64)
+        B64 = (b.T if tb else b).astype(np.float64)
+        err = np.abs(to_np(C).astype(np.float64) - (0.75 * A64 @ B64 + beta * c.astype(np.float64)))
+        assert np.all(err <= gemm_bound(np.abs(A64), np.abs(B64), K, np.abs(c), 0.75, beta, 3))
+        C.fill_(7.0)
+        assert bool((big == 7.0).all())   # nothing beside C was written
+
+
 # sizes of the inverse's and the Chebyshev function's dispatch and tiles that their own tests do not reach:
 # 64- and 128-wide tiles over the whole chip, two waves, the separate launches beyond
 @pytest.mark.parametrize("m,n", [(1001, 1001), (1300, 1250), (2100, 700), (2400, 2300)], ids=lambda v: str(v))
