@@ -512,6 +512,10 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
         }
         continue;
       }
+      if (EPI == CO_EPI_GEMM) {
+        store_c32(e.C + (r - lane) * e.ldc + c0, e.ldc, e.M - (r - lane), lane < e.N - c0 ? 31 : -1, lane, e.c3, e.c1, v);
+        continue;
+      }
       quad_rows(v, lq);
       if (EPI == TC_EPI_GRAM || EPI == TC_EPI_PLANES) {
         // columns past N hold zeros (the operand maps stop at N) and land in the pitch's padding
@@ -547,12 +551,6 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
           }
           if (rows4 & (1u << i)) store_planes8(pr + i * e.ldo, e.os, 3, v + 8 * i);
         }
-      } else if (EPI == CO_EPI_GEMM) {
-        const bool vec = (reinterpret_cast<uintptr_t>(e.C) & 15u) == 0 && (e.ldc & 3) == 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (rows4 & (1u << i))
-            co_gemm_store8(e.C + (r4 + i) * e.ldc + c0 + 8 * lq, e.N - c0 - 8 * lq, vec, e.c1, e.c3, v + 8 * i);
       } else {   // STORE: whole 16-byte groups up to a pitch that is a multiple of 4, else single entries
         float* cr = e.C + r4 * e.ldc + c0 + 8 * lq;
 #pragma unroll

@@ -293,6 +293,36 @@ __device__ __forceinline__ void store_chunk(uint16_t* base, int64_t ld, int64_t 
     if (mask & (1u << i)) store_planes8(base + i * ld, pstride, np, x + 8 * i);
 }
 
+// C = alpha V + beta C (C is not read for beta = 0) on a 32 x 32 block of a row-major FP32 matrix, lane l holding
+// row l of V. The block is transposed across the warp first (80 exchanges), so that every access is 128
+// contiguous bytes whatever C's alignment; with a lane on its own row each touched 32 lines, which took longer
+// than the products of a tile with a short K. rows: how many of the block's rows exist; last: the last row that
+// this lane's column takes (-1: none).
+__device__ __forceinline__ void store_c32(float* c, int64_t ldc, int rows, int last, int lane, float alpha, float beta,
+                                          float* x) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const bool hi = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (!(i & s)) {
+        const float r = __shfl_xor_sync(0xffffffffu, hi ? x[i] : x[i + s], s);
+        if (hi) x[i] = r; else x[i + s] = r;
+      }
+  }
+  last = min(last, rows - 1);
+  c += lane;
+#pragma unroll
+  for (int i0 = 0; i0 < 32; i0 += 8) {
+    float o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o[i] = beta != 0.0f && i0 + i <= last ? c[(i0 + i) * ldc] : 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i0 + i <= last) c[(i0 + i) * ldc] = beta != 0.0f ? fmaf(beta, o[i], alpha * x[i0 + i]) : alpha * x[i0 + i];
+  }
+}
+
 // Three planes of 8 values as loaded (16 bytes each) and their exact sum.
 struct Planes8 {
   uint4 q[3];
@@ -766,30 +796,9 @@ __device__ __noinline__ void role_epilogue(const Src& src, uint32_t tmem_base, B
         quad_rows(v, lq);
         store_chunk(p.out_planes + r4 * p.ldo + c0 + 8 * lq, p.ldo, p.out_plane_stride, p.out_nplanes, v, rows4);
       } else {  // STORE
-        if (!row_ok) continue;
-        float* cr = p.C + r * p.ldc + c0;
-        if (full_chunk && !(tri && r > c0) && (reinterpret_cast<uintptr_t>(cr) & 15u) == 0) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            float4 o = make_float4(p.alpha * v[4 * i], p.alpha * v[4 * i + 1], p.alpha * v[4 * i + 2],
-                                   p.alpha * v[4 * i + 3]);
-            if (p.beta != 0.0f) {
-              const float4 c = reinterpret_cast<const float4*>(cr)[i];
-              o = make_float4(fmaf(p.beta, c.x, o.x), fmaf(p.beta, c.y, o.y), fmaf(p.beta, c.z, o.z),
-                              fmaf(p.beta, c.w, o.w));
-            }
-            reinterpret_cast<float4*>(cr)[i] = o;
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (c0 + j < p.N && !(tri && r > c0 + j)) {
-              float o = p.alpha * v[j];
-              if (p.beta != 0.0f) o = fmaf(p.beta, cr[j], o);
-              cr[j] = o;
-            }
-          }
-        }
+        const int64_t r0 = r - lane, cols = p.N - c0;
+        const int last = lane >= cols ? -1 : tri && c0 + lane - r0 < 31 ? (int)(c0 + lane - r0) : 31;
+        store_c32(p.C + r0 * p.ldc + c0, p.ldc, (int)(p.M - r0 < 32 ? p.M - r0 : 32), last, lane, p.alpha, p.beta, v);
       }
     }
     if (EPI == TC_EPI_GRAM) {
