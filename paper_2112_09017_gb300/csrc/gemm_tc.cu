@@ -148,6 +148,14 @@ int tc_gram_partials(int64_t n, int planes) {
   return (int)(tri_tiles(tm, tn) * EPI_WARPS);
 }
 
+// Pairs of residual sums of an M x N update: one per epilogue warp of every 128 x 256 tile; in CTA pairs of both
+// halves of every 256 x 256 one, also of a half whose rows all lie past M.
+int tc_step_partials(int64_t M, int64_t N, int planes) {
+  const int64_t tn = (N + BN - 1) / BN;
+  const int64_t tm = use_pair(planes, M, N, false) ? (M + 2 * BM - 1) / (2 * BM) * 2 : (M + BM - 1) / BM;
+  return (int)(tm * tn * EPI_WARPS);
+}
+
 int tc_gram_partials_max(int64_t n) {
   const int64_t tm = (n + BM - 1) / BM, tn = (n + BN - 1) / BN;
   const int64_t a = tri_tiles(tm, tn) * EPI_WARPS, b = pair_tri_tiles(tn) * 2 * EPI_WARPS;

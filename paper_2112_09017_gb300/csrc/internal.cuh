@@ -217,6 +217,7 @@ cudaError_t tc_take_error(cudaStream_t s, unsigned int* out);
 // and single-CTA forms tile it differently), and the largest of the two (for allocation).
 int tc_gram_partials(int64_t n, int planes);
 int tc_gram_partials_max(int64_t n);
+int tc_step_partials(int64_t M, int64_t N, int planes);   // pairs of NS_STEP sums; at most 2 ceil(M/256) ceil(N/256) 8
 bool tc_available();
 
 // Tensor map of one stage's box of an operand's planes: 64 columns x 32 rows for MN-major operands, 32

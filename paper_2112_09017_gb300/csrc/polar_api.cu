@@ -1099,14 +1099,13 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   const int64_t lpa = round_up(M, 64), lpx = round_up(N, 64);
   const int64_t sa = round_up(N * lpa, 64), sx = round_up(M * lpx, 64), sp = round_up(N * lpx, 64);
   const int64_t ldc = round_up(M, 4);
-  const int64_t tiles_ns = ((M + 127) / 128) * ((N + 255) / 256);
-  const int64_t npairs = tiles_ns * 8;
+  const int64_t npairs = tc_step_partials(M, N, P), npairs_max = 2 * ((M + 255) / 256) * ((N + 255) / 256) * 8;
   const int fb = frob_partials_blocks(M, M);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
   const size_t o_a = take((size_t)P * sa * 2), o_x0 = take((size_t)3 * sx * 2), o_x1 = take((size_t)3 * sx * 2),
                o_p = take((size_t)3 * sp * 2), o_c = take((size_t)M * ldc * 4),
-               o_part = take((size_t)std::max<int64_t>(2 * npairs, fb) * 8), o_st = take(sizeof(DevState));
+               o_part = take((size_t)std::max<int64_t>(2 * npairs_max, fb) * 8), o_st = take(sizeof(DevState));
   const size_t o_sums = take(coop_inverse_sums(sms));
   CallWorkspace call(s);
   polar_status_t wr = call.get(off);

@@ -169,6 +169,22 @@ def test_coop_inverse_matches_separate_launches(lib, monkeypatch, m, n):
     assert bool(torch.all(big == 9.0))
 
 
+@pytest.mark.parametrize("n", [100, 300, 640])
+def test_inverse_in_cta_pairs_with_an_odd_row_of_tiles(lib, monkeypatch, n):
+    """A pair whose second half lies past the last row still writes residual sums of its own; they have a
+    place in the workspace (they once landed in the state after it, and the call reported an expired wait)."""
+    import torch
+    a = torch.from_numpy(synth.matrix_with_spectrum(n, n, synth.logspace_spectrum(n, 0.2), n)).cuda()
+    out = []
+    for form in ("0", "1"):
+        monkeypatch.setenv("POLAR_TC_CTA_PAIR", form)
+        X = torch.empty((n, n), device="cuda")
+        out.append((lib.polar_ns_inverse(a, X), X))
+    (i0, X0), (i1, X1) = out
+    assert i0["status"] == i1["status"] == lib.POLAR_OK and i0["iters"] == i1["iters"]
+    assert float(torch.linalg.matrix_norm(X0 - X1) / torch.linalg.matrix_norm(X0)) <= 2e-6
+
+
 @pytest.mark.parametrize("n,d", [(1000, 9), (1450, 4), (1536, 3), (2300, 3)])
 def test_coop_chebyshev_matches_separate_launches(lib, monkeypatch, n, d):
     import torch
