@@ -145,12 +145,20 @@ __host__ __device__ __forceinline__ int64_t tri_tiles(int64_t tm, int64_t tn) {
 }
 
 __device__ __forceinline__ void tile_coords(int64_t t, int64_t tm, int64_t tn, bool tri, int64_t& bi, int64_t& bj) {
-  if (tri) {
-    int64_t j = (int64_t)((sqrt(4.0 * (double)t + 1.0) - 1.0) * 0.5);
-    while (j > 0 && j * (j + 1) > t) --j;
-    while ((j + 1) * (j + 2) <= t) ++j;
-    bj = j;
-    bi = t - j * (j + 1);
+  if (tri) {   // groups of 16 tile rows, from the diagonal to the last column, each column by column
+    int64_t j0 = 0;
+    for (; tn - j0 > 8 && t >= 72 + 16 * (tn - j0 - 8); j0 += 8) t -= 72 + 16 * (tn - j0 - 8);
+    if (tn - j0 > 8 && t >= 72) {
+      t -= 72;
+      bj = j0 + 8 + t / 16;
+      bi = 2 * j0 + t % 16;
+    } else {
+      int64_t j = (int64_t)((sqrtf(4.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+      while (j > 0 && j * (j + 1) > t) --j;
+      while ((j + 1) * (j + 2) <= t) ++j;
+      bj = j0 + j;
+      bi = 2 * j0 + t - j * (j + 1);
+    }
   } else {
     const int64_t G = 16;
     int64_t group = t / (G * tn);
@@ -169,11 +177,19 @@ __host__ __device__ __forceinline__ int64_t pair_tri_tiles(int64_t t) { return t
 __device__ __forceinline__ void pair_tile_coords(int64_t t, int64_t tm2, int64_t tn, bool tri, int64_t& bi2,
                                                  int64_t& bj) {
   if (tri) {
-    int64_t j = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-    while (j > 0 && j * (j + 1) / 2 > t) --j;
-    while ((j + 1) * (j + 2) / 2 <= t) ++j;
-    bj = j;
-    bi2 = t - j * (j + 1) / 2;
+    int64_t j0 = 0;
+    for (; tn - j0 > 8 && t >= 36 + 8 * (tn - j0 - 8); j0 += 8) t -= 36 + 8 * (tn - j0 - 8);
+    if (tn - j0 > 8 && t >= 36) {
+      t -= 36;
+      bj = j0 + 8 + t / 8;
+      bi2 = j0 + t % 8;
+    } else {
+      int64_t j = (int64_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+      while (j > 0 && j * (j + 1) / 2 > t) --j;
+      while ((j + 1) * (j + 2) / 2 <= t) ++j;
+      bj = j0 + j;
+      bi2 = j0 + t - j * (j + 1) / 2;
+    }
   } else {
     const int64_t G = 8;
     int64_t group = t / (G * tn);
