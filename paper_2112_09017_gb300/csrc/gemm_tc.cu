@@ -129,17 +129,18 @@ int forced_pair_mode() {
 
 bool tc_forced_form() { return forced_pair_mode() >= 0; }
 
-// Whether a launch of `planes`-plane products runs as CTA pairs: three planes (the pair kernels'
-// instantiations) and at least one 256 x 256 pair tile for every pair of SMs, so that the pairs'
-// halved shared-memory operand traffic is not paid for with idle SMs. POLAR_TC_CTA_PAIR in the
-// environment overrides the size rule: 0 never, 1 whenever the planes allow it.
-bool use_pair(int planes, int64_t M, int64_t N, bool tri) {
+// Whether a launch of `planes`-plane products runs as CTA pairs (instantiated for three planes): Grams of a solve
+// with at least four waves of 256 x 256 pair tiles. Gram and update, 128 x 256 tiles and CTA pairs (us): 4096^2 238
+// 245, 498 538; 6500^2 988 980, 1850 1953; 8192^2 1765 1713, 3640 3790; 10000^2 3426 3284, 6735 7195; 30000 x 3000
+// 1580 1665, 1820 1946. Pairs read half as much of B from shared memory, but a pair waits for the slower of its
+// two output steps, and a Gram's is the shortest. Products to C, Chebyshev
+// steps and syrk are 1 to 8 % slower in pairs at every size measured (8192 x 8192 x 4000 1770 against 1870).
+// POLAR_TC_CTA_PAIR in the environment overrides the rule: 0 never, 1 whenever the planes allow it.
+bool use_pair(int planes, int64_t M, int64_t N, bool gram) {
   if (planes != 3) return false;
   const int mode = forced_pair_mode();
   if (mode >= 0) return mode == 1;
-  const int64_t tm2 = (M + 2 * BM - 1) / (2 * BM), tn = (N + BN - 1) / BN;
-  const int64_t tiles = tri ? pair_tri_tiles(tn) : tm2 * tn;
-  return tiles >= sm_count() / 2;
+  return gram && pair_tri_tiles((N + BN - 1) / BN) >= 4 * (sm_count() / 2);
 }
 
 int tc_gram_partials(int64_t n, int planes) {
@@ -211,7 +212,7 @@ cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
       !tc_forced_form() && co_gemm_better(a))
     return launch_co_gemm(a, s);
   CUtensorMap ma, mb;
-  const bool pair = use_pair(a.nplanes, a.M, a.N, a.triangular != 0);
+  const bool pair = use_pair(a.nplanes, a.M, a.N, a.epi == TC_EPI_GRAM);
   if (!make_map(&ma, a.a, a.nplanes, !a.a.kmajor, BM)) return cudaErrorInvalidValue;
   if (!make_map(&mb, a.b, a.nplanes, !a.b.kmajor, pair ? BN / 2 : BN)) return cudaErrorInvalidValue;
   if (pair) {   // 256 x 256 pair tiles; each CTA stages 128 of the tile's columns of B
