@@ -325,8 +325,8 @@ static double co_cost(const CoopProduct* p, int count, int sms, int64_t* waves) 
 
 // One launch against separate ones, per step at kappa 100: 512^2 23 against 84 us, 1024^2 36 against 111, 2048^2
 // 113 against 174, 3072^2 326 against 445, 8192 x 2048 (7 waves of 128-wide tiles) 415 against 563, 4096^2 (7)
-// 805 against 838; 8192^2 (27 waves) 6782 against 5700, where the CTA pairs' 256 x 256 tiles read a third less
-// from L2. So the line lies at eight waves.
+// 798 against 796; 8192^2 (27 waves) 6782 against 5600, where wider tiles read less from L2. So the line lies at
+// eight waves.
 int coop_tile_n(const CoopProduct* p, int count, int sms) {
   int64_t w64, w128;
   const double c64 = co_cost<64>(p, count, sms, &w64), c128 = co_cost<128>(p, count, sms, &w128);

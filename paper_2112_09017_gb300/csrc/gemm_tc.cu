@@ -129,31 +129,36 @@ int forced_pair_mode() {
 
 bool tc_forced_form() { return forced_pair_mode() >= 0; }
 
-// Whether a launch of `planes`-plane products runs as CTA pairs (instantiated for three planes): Grams of a solve
-// with at least four waves of 256 x 256 pair tiles. Gram and update, 128 x 256 tiles and CTA pairs (us): 4096^2 238
-// 245, 498 538; 6500^2 988 980, 1850 1953; 8192^2 1765 1713, 3640 3790; 10000^2 3426 3284, 6735 7195; 30000 x 3000
-// 1580 1665, 1820 1946. Pairs read half as much of B from shared memory, but a pair waits for the slower of its
-// two output steps, and a Gram's is the shortest. Products to C, Chebyshev
-// steps and syrk are 1 to 8 % slower in pairs at every size measured (8192 x 8192 x 4000 1770 against 1870).
+// Whether a launch of `planes`-plane products runs as CTA pairs (instantiated for three planes): a solve's Grams of
+// at least four waves of 256 x 256 pair tiles, and products of at least 32 waves with K from 15000. Gram and update,
+// 128 x 256 tiles and CTA pairs (us): 4096^2 238 245, 498 538; 6500^2 988 980, 1850 1953; 8192^2 1765 1713, 3640
+// 3790; 10000^2 3426 3284, 6735 7195; 30000 x 3000 1580 1665, 1820 1946; 32768 x 8192 7290 6720, 14870 14930;
+// 13000^2 7560 6870, 14920 14790; 16384^2 15040 13680, 29420 29150; 32768^2 123600 109000, 260800 230800. Products
+// to C: 8192 x 8192 x 4000 1770 1870, 13000^3 14950 15020, 16384^3 30950 28200, 24000^3 98200 86900. A pair waits
+// for the slower of its two output steps, but it takes less power, and from about 8000^2 on the power limit sets the
+// clock: with a long K, where the output steps do not count, pairs then run at 1700 MHz and single CTAs at 1600.
+// Chebyshev steps are 3 to 6 % slower in pairs at every size measured (up to 24000^2): their output step is the longest.
 // POLAR_TC_CTA_PAIR in the environment overrides the rule: 0 never, 1 whenever the planes allow it.
-bool use_pair(int planes, int64_t M, int64_t N, bool gram) {
+bool use_pair(int planes, int64_t M, int64_t N, int64_t K, int epi, bool tri) {
   if (planes != 3) return false;
   const int mode = forced_pair_mode();
   if (mode >= 0) return mode == 1;
-  return gram && pair_tri_tiles((N + BN - 1) / BN) >= 4 * (sm_count() / 2);
+  if (epi == TC_EPI_CLENSHAW) return false;
+  const int64_t tn = (N + BN - 1) / BN, tiles = tri ? pair_tri_tiles(tn) : (M + 2 * BM - 1) / (2 * BM) * tn;
+  return tiles >= (epi == TC_EPI_GRAM ? 4 : K >= 15000 ? 32 : (int64_t)1 << 40) * (sm_count() / 2);
 }
 
 int tc_gram_partials(int64_t n, int planes) {
   const int64_t tm = (n + BM - 1) / BM, tn = (n + BN - 1) / BN;
-  if (use_pair(planes, n, n, true)) return (int)(pair_tri_tiles(tn) * 2 * EPI_WARPS);
+  if (use_pair(planes, n, n, 0, TC_EPI_GRAM, true)) return (int)(pair_tri_tiles(tn) * 2 * EPI_WARPS);
   return (int)(tri_tiles(tm, tn) * EPI_WARPS);
 }
 
-// Pairs of residual sums of an M x N update: one per epilogue warp of every 128 x 256 tile; in CTA pairs of both
+// Pairs of residual sums of an M x N update (K = N): one per epilogue warp of every 128 x 256 tile; in CTA pairs of both
 // halves of every 256 x 256 one, also of a half whose rows all lie past M.
 int tc_step_partials(int64_t M, int64_t N, int planes) {
   const int64_t tn = (N + BN - 1) / BN;
-  const int64_t tm = use_pair(planes, M, N, false) ? (M + 2 * BM - 1) / (2 * BM) * 2 : (M + BM - 1) / BM;
+  const int64_t tm = use_pair(planes, M, N, N, TC_EPI_NS_STEP, false) ? (M + 2 * BM - 1) / (2 * BM) * 2 : (M + BM - 1) / BM;
   return (int)(tm * tn * EPI_WARPS);
 }
 
@@ -212,7 +217,7 @@ cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
       !tc_forced_form() && co_gemm_better(a))
     return launch_co_gemm(a, s);
   CUtensorMap ma, mb;
-  const bool pair = use_pair(a.nplanes, a.M, a.N, a.epi == TC_EPI_GRAM);
+  const bool pair = use_pair(a.nplanes, a.M, a.N, a.K, a.epi, a.triangular != 0);
   if (!make_map(&ma, a.a, a.nplanes, !a.a.kmajor, BM)) return cudaErrorInvalidValue;
   if (!make_map(&mb, a.b, a.nplanes, !a.b.kmajor, pair ? BN / 2 : BN)) return cudaErrorInvalidValue;
   if (pair) {   // 256 x 256 pair tiles; each CTA stages 128 of the tile's columns of B

@@ -51,9 +51,9 @@
 // the even CTA. Each CTA stages its own 128 rows of A and its own 128 columns of B
 // (48 KiB stages instead of 72 KiB), the MMAs read the peer's half of B across the
 // pair, and each CTA's TMEM holds its 128 rows of the accumulator. Per SM this
-// halves the B operand's shared-memory reads and TMA writes, the limit of the
-// single-CTA form (about 90 % of the tensor pipe), and cuts the operand panels
-// read from L2 by a third. Both CTAs' copies complete on the even CTA's stage
+// halves the B operand's shared-memory reads and TMA writes and cuts the operand
+// panels read from L2 by a third, at the price of waiting for the slower CTA
+// (gemm_tc.cu: where it pays). Both CTAs' copies complete on the even CTA's stage
 // barriers; its MMA commits arrive on both CTAs' barriers (multicast); the odd
 // CTA's epilogue warps free an accumulator buffer by arriving on the even CTA's
 // barrier.

@@ -1,7 +1,7 @@
 """The CTA-pair form of the tensor-core products (cta_group::2: two CTAs of a cluster share a
 256 x 256 tile, each staging half of B) against the single-CTA form and float64.
 
-The pair form runs by default only for a solve's Grams over several waves of pair tiles; these
+The pair form runs by default only for large products (a solve's Grams, and long K); these
 tests force it (POLAR_TC_CTA_PAIR=1) on small and ragged shapes, where rows or columns of a pair
 tile fall outside the matrix, and check that every element equals the single-CTA result bit for
 bit (the same k-slices, passes and promotion order per element) and lies within the split
