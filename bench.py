@@ -220,7 +220,7 @@ def cpu_cores():
 def run_batched(lib, torch, count, steps, warmup, n_lo=64, n_hi=1024, onchip=1, As=None, tune=None):
     """The batched workload: `count` problems (n uniform on [n_lo, n_hi], m = n or 2n,
     sigma on [1e-3, 1]) in one polar_batched_run; solves/s and per-problem iterations.
-    onchip = 0 sends the problems that fit one SM through the grouped tile kernels too."""
+    onchip = 0 sends the problems that fit one SM through the tile loop too."""
     from paper_2112_09017_gb300 import synth
     t0 = time.perf_counter()
     if As is None:
