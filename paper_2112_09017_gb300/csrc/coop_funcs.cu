@@ -25,7 +25,7 @@ struct CoInverse {
   uint16_t* pp;
   int64_t lpa, sa, lpx, sx, sp;
   double* norm;                              // EPI_WARPS per block
-  float2* part;                              // 2 EPI_WARPS per block
+  double* step;                              // 2 EPI_WARPS per block
   DevState* st;
   int rows, cols, max_iter, withhold;
   int sa2, su;                               // split chains: blocks per tile of A X and of the update
@@ -118,8 +118,8 @@ __device__ __forceinline__ void co_inverse(const CoInverse& p, uint8_t* co_raw) 
     }
     if (x.warp == CO_CTL_WARP && k > 0) {
       // Algorithm 2's test after update k - 1: ||X' - X||_F / ||X'||_F against u 2^(k-1), u = 2^-24
-      const double sd = co_warp_sum2(p.part, gridDim.x * EPI_WARPS, 2, x.lane);
-      const double sx = co_warp_sum2(p.part + 1, gridDim.x * EPI_WARPS, 2, x.lane);
+      const double sd = co_warp_sum(p.step, gridDim.x * EPI_WARPS, 2, x.lane);
+      const double sx = co_warp_sum(p.step + 1, gridDim.x * EPI_WARPS, 2, x.lane);
       if (x.lane == 0) {
         const double delta = sx > 0.0 ? sqrt(sd / sx) : INFINITY;
         const int s = !isfinite(delta) ? ST_NONFINITE
@@ -147,7 +147,7 @@ __device__ __forceinline__ void co_inverse(const CoInverse& p, uint8_t* co_raw) 
     e.x = p.xp[b]; e.ldx = p.lpx; e.xs = p.sx;
     e.out = p.xp[b ^ 1]; e.ldo = p.lpx; e.os = p.sx;
     e.c1 = 2.0f; e.c3 = -1.0f;
-    e.part = p.part;
+    e.norm = p.step;
     co_product<TN, SPLIT, false, false, TC_EPI_NS_STEP>(x, pipe, &p.xk[b], &p.pmn, nullptr, tu, N, e, p.su,
                                                         p.withhold);
     run = co_grid_sync(x);
@@ -334,7 +334,7 @@ int co_grid(int64_t m, int64_t n, int tn, int sms) {
 
 }  // namespace
 
-size_t coop_inverse_sums(int sms) { return (size_t)sms * EPI_WARPS * (sizeof(double) + 2 * sizeof(float2)); }
+size_t coop_inverse_sums(int sms) { return (size_t)sms * EPI_WARPS * 3 * sizeof(double); }
 
 cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaStream_t s) {
   CoInverse p{};
@@ -357,7 +357,7 @@ cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaS
   p.sa2 = S[0];
   p.su = S[1];
   p.norm = a.sums;
-  p.part = reinterpret_cast<float2*>(a.sums + (size_t)sms * EPI_WARPS);
+  p.step = a.sums + (size_t)sms * EPI_WARPS;
   p.st = a.st;
   p.rows = (int)a.rows; p.cols = (int)a.cols; p.max_iter = a.max_iter;
   p.withhold = tc_withhold();

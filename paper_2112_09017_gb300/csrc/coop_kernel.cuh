@@ -399,8 +399,8 @@ struct CoEpi {
   int64_t ldc;
   float c1, c3;              // NS: c1 X + c3 acc; CLENSHAW: c3 acc + c1 Z + diag I
   float diag;
-  float2* part;              // GRAM: per epilogue warp of every block; NS_STEP: two each
-  double* norm;              // NORM: per epilogue warp of every block
+  float2* part;              // GRAM: per epilogue warp of every block
+  double* norm;              // NORM: per epilogue warp of every block; NS_STEP: two each
   double* tile_part;         // GRAM from a table: this tile's EPI_WARPS sums
 };
 
@@ -423,8 +423,8 @@ __device__ __forceinline__ void co_gemm_store8(float* c, int n, bool vec, float 
   }
 }
 
-// Sums over each warp's tiles, as unevaluated pairs hi + lo, go to e.part: GRAM ||G - I||_F^2; NS_STEP
-// ||X' - X||^2 and ||X'||^2. NORM's go to e.norm, in float64 (entries of any magnitude).
+// Sums over each warp's tiles: GRAM's ||G - I||_F^2 goes to e.part as an unevaluated pair hi + lo; NS_STEP's
+// ||X' - X||^2 and ||X'||^2 and NORM's go to e.norm, in float64 (entries of any magnitude).
 template <int TN, int EPI, class Src>
 __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src) {
   using C = CoCfg<TN>;
@@ -435,8 +435,8 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
   const uint32_t t_lane = x.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * CW);
   int buf = pp.buf;
   uint32_t buf_phase = pp.buf_phase;
-  float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
-  double norm = 0.0;
+  float2 sum0 = make_float2(0.f, 0.f);
+  double norm = 0.0, step0 = 0.0, step1 = 0.0;
   bool ok = true;
   CoTile ti;
   while (ok && src.next(ti)) {
@@ -578,8 +578,8 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
       sum0 = make_float2(0.f, 0.f);
     }
     if (STEP) {
-      two_sum(sum0, make_float2(d2, 0.f));
-      two_sum(sum1, make_float2(x2, 0.f));
+      step0 += warp_sum64(d2);
+      step1 += warp_sum64(x2);
     }
   }
   pp.buf = buf;
@@ -589,19 +589,16 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
     for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
     if (lane == 0) __stcg(src.epi(ti).norm + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
   }
-  if (!Src::TABLE && (EPI == TC_EPI_GRAM || STEP)) {
-    const CoEpi& e = src.epi(ti);
+  if (STEP && lane == 0) {
+    double* dst = src.epi(ti).norm + 2 * (blockIdx.x * EPI_WARPS + x.warp - 2);
+    __stcg(dst, step0);
+    __stcg(dst + 1, step1);
+  }
+  if (!Src::TABLE && EPI == TC_EPI_GRAM) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o > 0; o >>= 1)
       two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-      if (STEP)
-        two_sum(sum1, make_float2(__shfl_xor_sync(0xffffffffu, sum1.x, o), __shfl_xor_sync(0xffffffffu, sum1.y, o)));
-    }
-    if (lane == 0) {
-      float2* dst = e.part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + x.warp - 2);
-      __stcg(dst, sum0);
-      if (STEP) __stcg(dst + 1, sum1);
-    }
+    if (lane == 0) __stcg(src.epi(ti).part + blockIdx.x * EPI_WARPS + x.warp - 2, sum0);
   }
 }
 
@@ -641,8 +638,8 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
   constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP, STEP = EPI == TC_EPI_NS_STEP;
   constexpr bool READS_X = NS || EPI == TC_EPI_CLENSHAW;
   CoTile ti;
-  float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
-  double norm = 0.0;
+  float2 sum0 = make_float2(0.f, 0.f);
+  double norm = 0.0, step0 = 0.0, step1 = 0.0;
   const bool have = src.next(ti);        // the same in every block of the group
   const CoEpi& e = src.epi(ti);
   if (have) {
@@ -704,8 +701,10 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
           v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
         }
-        if (r >= e.M || col >= e.N) continue;
-        if (EPI == TC_EPI_GRAM) {
+        float d2 = 0.0f, x2 = 0.0f;
+        const bool in = r < e.M && col < e.N;
+        if (!in) {
+        } else if (EPI == TC_EPI_GRAM) {
           float t = 0.0f;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -716,7 +715,7 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           two_sum(sum0, make_float2(t, 0.f));
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
         } else if (READS_X) {
-          float xo[8], d2 = 0.0f, x2 = 0.0f;
+          float xo[8];
           sum_planes8(pre[u], xo);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -730,10 +729,6 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
               v[j] = fmaf(e.c3, v[j], e.c1 * xo[j]);
               if (r == col + j) v[j] += e.diag;
             }
-          }
-          if (STEP) {
-            two_sum(sum0, make_float2(d2, 0.f));
-            two_sum(sum1, make_float2(x2, 0.f));
           }
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
         } else if (EPI == TC_EPI_PLANES) {
@@ -752,6 +747,10 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           if (col < e.ldc) *reinterpret_cast<float4*>(cr) = make_float4(v[0], v[1], v[2], v[3]);
           if (col + 4 < e.ldc) *reinterpret_cast<float4*>(cr + 4) = make_float4(v[4], v[5], v[6], v[7]);
         }
+        if (STEP) {
+          step0 += warp_sum64(d2);
+          step1 += warp_sum64(x2);
+        }
       }
     }
   }
@@ -760,18 +759,16 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
     for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
     if (lane == 0) __stcg(e.norm + blockIdx.x * EPI_WARPS + w, norm);
   }
-  if (EPI == TC_EPI_GRAM || STEP) {
+  if (STEP && lane == 0) {
+    double* dst = e.norm + 2 * (blockIdx.x * EPI_WARPS + w);
+    __stcg(dst, step0);
+    __stcg(dst + 1, step1);
+  }
+  if (EPI == TC_EPI_GRAM) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o > 0; o >>= 1)
       two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-      if (STEP)
-        two_sum(sum1, make_float2(__shfl_xor_sync(0xffffffffu, sum1.x, o), __shfl_xor_sync(0xffffffffu, sum1.y, o)));
-    }
-    if (lane == 0) {
-      float2* dst = e.part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + w);
-      __stcg(dst, sum0);
-      if (STEP) __stcg(dst + 1, sum1);
-    }
+    if (lane == 0) __stcg(e.part + blockIdx.x * EPI_WARPS + w, sum0);
   }
 }
 

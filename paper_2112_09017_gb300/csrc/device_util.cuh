@@ -52,6 +52,27 @@ __device__ __forceinline__ float2 bf16_pair(uint32_t w) {
   return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
 
+// The sum of the lanes' non-negative floats as a float64, the same in every lane of a converged warp, whatever
+// their magnitudes: fixed point with 35 bits below the largest value's last one, so that what is cut off is no more
+// than a float64 sum's rounding, in integers because a chain of FP64 shuffles costs a step of a small
+// solve more than its warp-wide integer sums (FP64 runs at two operations a cycle and SM). An infinity or a NaN
+// among them is the result.
+__device__ __forceinline__ double warp_sum64(float v) {
+  const uint32_t b = __float_as_uint(v), top = __reduce_max_sync(0xffffffffu, b);
+  if (top >= 0x7f800000u) return (double)__uint_as_float(top);
+  const int ex = max((int)(top >> 23), 1), down = ex - max((int)(b >> 23), 1);
+  const uint64_t man = (b & 0x7fffffu) | (b >> 23 ? 0x800000u : 0u);
+  const uint64_t q = down < 59 ? (man << 35) >> down : 0u;   // v = q 2^(ex - 185), q < 2^59
+  const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)q & 0x1fffffu),
+                 s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(q >> 21) & 0x1fffffu),
+                 s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(q >> 42));
+  const uint64_t s = ((uint64_t)s2 << 42) + ((uint64_t)s1 << 21) + s0;
+  if (s == 0) return 0.0;
+  const int lz = __clzll((long long)s);
+  const uint64_t n = s << lz, r = (n >> 11) + ((n >> 10) & 1u);   // 53 bits, rounded; its top bit adds one to the exponent
+  return __longlong_as_double((long long)(((uint64_t)(1023 + 63 - lz + ex - 185 - 1) << 52) + r));
+}
+
 // s + e = a + b exactly (Knuth's two-sum), accumulated into the unevaluated pair s.x + s.y.
 __device__ __forceinline__ void two_sum(float2& s, float2 b) {
   const float t = s.x + b.x, bb = t - s.x;

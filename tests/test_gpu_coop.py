@@ -169,6 +169,25 @@ def test_coop_inverse_matches_separate_launches(lib, monkeypatch, m, n):
     assert bool(torch.all(big == 9.0))
 
 
+# tiles shared along K, whole tiles 64 and 128 wide in one launch, separate launches; the scales put ||X||_F between 3e19 and 5e19
+@pytest.mark.parametrize("m,n,e,form", [(300, 300, -59, ""), (1001, 1001, -58, ""), (2400, 2300, -57, ""),
+                                        (1001, 1001, -58, "0")], ids=lambda v: str(v))
+def test_inverse_of_a_matrix_of_very_small_norm(lib, monkeypatch, m, n, e, form):
+    """||X||_F^2 beyond float32's range, every entry's square and every sum of a row chunk well inside it: the
+    relative steps, the updates and the result are those of the same matrix at unit scale."""
+    import torch
+    monkeypatch.setenv("POLAR_TC_CTA_PAIR", form)
+    a = torch.from_numpy(synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 0.1), m)).cuda()
+    X, Y = torch.empty((n, m), device="cuda"), torch.empty((n, m), device="cuda")
+    one = lib.polar_ns_inverse(a, X)
+    tiny = lib.polar_ns_inverse(a * 2.0 ** e, Y, raw_status=True)
+    assert float(torch.linalg.matrix_norm(Y.double())) > 2.0 ** 64
+    assert tiny["status"] == one["status"] == lib.POLAR_OK
+    assert tiny["iters"] == one["iters"] and tiny["delta"] == pytest.approx(one["delta"], rel=1e-2, abs=1e-7)
+    # ||A^T A||_F of the tiny matrix is a sum of float32 denormals in part: another scale of X_0, another rounding
+    assert float(torch.linalg.matrix_norm(Y * 2.0 ** e - X) / torch.linalg.matrix_norm(X)) <= 1e-5
+
+
 @pytest.mark.parametrize("n", [100, 300, 640])
 def test_inverse_in_cta_pairs_with_an_odd_row_of_tiles(lib, monkeypatch, n):
     """A pair whose second half lies past the last row still writes residual sums of its own; they have a
