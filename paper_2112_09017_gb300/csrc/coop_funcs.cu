@@ -63,7 +63,7 @@ __device__ __forceinline__ void co_inverse(const CoInverse& p, uint8_t* co_raw) 
     const CoTiles t = co_tiles<TN>(M, M, true);
     CoEpi e{};
     e.M = M; e.N = M;
-    e.norm = p.norm;
+    e.part = p.norm;
     co_product<TN, SPLIT, true, false, CO_EPI_NORM>(x, pipe, &p.amn, &p.amn, nullptr, t, N, e, 1, p.withhold);
     run = co_grid_sync(x);
   }
@@ -147,7 +147,7 @@ __device__ __forceinline__ void co_inverse(const CoInverse& p, uint8_t* co_raw) 
     e.x = p.xp[b]; e.ldx = p.lpx; e.xs = p.sx;
     e.out = p.xp[b ^ 1]; e.ldo = p.lpx; e.os = p.sx;
     e.c1 = 2.0f; e.c3 = -1.0f;
-    e.norm = p.step;
+    e.part = p.step;
     co_product<TN, SPLIT, false, false, TC_EPI_NS_STEP>(x, pipe, &p.xk[b], &p.pmn, nullptr, tu, N, e, p.su,
                                                         p.withhold);
     run = co_grid_sync(x);

@@ -399,8 +399,7 @@ struct CoEpi {
   int64_t ldc;
   float c1, c3;              // NS: c1 X + c3 acc; CLENSHAW: c3 acc + c1 Z + diag I
   float diag;
-  float2* part;              // GRAM: per epilogue warp of every block
-  double* norm;              // NORM: per epilogue warp of every block; NS_STEP: two each
+  double* part;              // GRAM, NORM: per epilogue warp of every block; NS_STEP: two each
   double* tile_part;         // GRAM from a table: this tile's EPI_WARPS sums
 };
 
@@ -423,8 +422,8 @@ __device__ __forceinline__ void co_gemm_store8(float* c, int n, bool vec, float 
   }
 }
 
-// Sums over each warp's tiles: GRAM's ||G - I||_F^2 goes to e.part as an unevaluated pair hi + lo; NS_STEP's
-// ||X' - X||^2 and ||X'||^2 and NORM's go to e.norm, in float64 (entries of any magnitude).
+// Sums over each warp's tiles, in float64 from a warp's 32 row chunks on, go to e.part: GRAM ||G - I||_F^2,
+// NS_STEP ||X' - X||^2 and ||X'||^2, NORM ||C||_F^2.
 template <int TN, int EPI, class Src>
 __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src) {
   using C = CoCfg<TN>;
@@ -435,8 +434,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
   const uint32_t t_lane = x.tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * CW);
   int buf = pp.buf;
   uint32_t buf_phase = pp.buf_phase;
-  float2 sum0 = make_float2(0.f, 0.f);
-  double norm = 0.0, step0 = 0.0, step1 = 0.0;
+  double sum0 = 0.0, sum1 = 0.0, norm = 0.0;   // norm: this lane's
   bool ok = true;
   CoTile ti;
   while (ok && src.next(ti)) {
@@ -481,6 +479,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
       if (c0 >= e.N) continue;                       // the same for every lane of the warp
       if (EPI == TC_EPI_GRAM) {
         // residual terms: twice the squares above the diagonal, (g - 1)^2 on it (columns past N hold zeros)
+        float t = 0.0f;
         if (r < e.M && c0 + 31 >= r) {
           float s4[4] = {0.f, 0.f, 0.f, 0.f};
           if (c0 > r) {
@@ -496,8 +495,9 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
               s4[j & 3] = fmaf(w * g, g, s4[j & 3]);
             }
           }
-          two_sum(sum0, make_float2((s4[0] + s4[1]) + (s4[2] + s4[3]), 0.f));
+          t = (s4[0] + s4[1]) + (s4[2] + s4[3]);
         }
+        sum0 += warp_sum64(t);
       }
       if (EPI == CO_EPI_NORM) {   // twice the squares above the diagonal, the squares on it
         if (r < e.M && c0 + 31 >= r) {
@@ -571,15 +571,12 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
       }
     }
     if (Src::TABLE && EPI == TC_EPI_GRAM) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-      if (lane == 0) e.tile_part[x.warp - 2] = (double)sum0.x + (double)sum0.y;
-      sum0 = make_float2(0.f, 0.f);
+      if (lane == 0) e.tile_part[x.warp - 2] = sum0;
+      sum0 = 0.0;
     }
     if (STEP) {
-      step0 += warp_sum64(d2);
-      step1 += warp_sum64(x2);
+      sum0 += warp_sum64(d2);
+      sum1 += warp_sum64(x2);
     }
   }
   pp.buf = buf;
@@ -587,18 +584,12 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
   if (EPI == CO_EPI_NORM) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
-    if (lane == 0) __stcg(src.epi(ti).norm + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
+    if (lane == 0) __stcg(src.epi(ti).part + blockIdx.x * EPI_WARPS + x.warp - 2, norm);
   }
-  if (STEP && lane == 0) {
-    double* dst = src.epi(ti).norm + 2 * (blockIdx.x * EPI_WARPS + x.warp - 2);
-    __stcg(dst, step0);
-    __stcg(dst + 1, step1);
-  }
-  if (!Src::TABLE && EPI == TC_EPI_GRAM) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-    if (lane == 0) __stcg(src.epi(ti).part + blockIdx.x * EPI_WARPS + x.warp - 2, sum0);
+  if (!Src::TABLE && (EPI == TC_EPI_GRAM || STEP) && lane == 0) {
+    double* dst = src.epi(ti).part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + x.warp - 2);
+    __stcg(dst, sum0);
+    if (STEP) __stcg(dst + 1, sum1);
   }
 }
 
@@ -638,8 +629,7 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
   constexpr bool NS = EPI == TC_EPI_NS || EPI == TC_EPI_NS_STEP, STEP = EPI == TC_EPI_NS_STEP;
   constexpr bool READS_X = NS || EPI == TC_EPI_CLENSHAW;
   CoTile ti;
-  float2 sum0 = make_float2(0.f, 0.f);
-  double norm = 0.0, step0 = 0.0, step1 = 0.0;
+  double sum0 = 0.0, sum1 = 0.0, norm = 0.0;   // norm: this lane's
   const bool have = src.next(ti);        // the same in every block of the group
   const CoEpi& e = src.epi(ti);
   if (have) {
@@ -701,18 +691,15 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
           v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
         }
-        float d2 = 0.0f, x2 = 0.0f;
-        const bool in = r < e.M && col < e.N;
-        if (!in) {
+        float d2 = 0.0f, x2 = 0.0f;   // GRAM: the residual terms; STEP: the step's
+        if (r >= e.M || col >= e.N) {
         } else if (EPI == TC_EPI_GRAM) {
-          float t = 0.0f;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const int d = col + j - r;   // above the diagonal twice, on it (g - 1)^2 (columns past N hold zeros)
             const float g = d == 0 ? v[j] - 1.0f : v[j], wt = d < 0 ? 0.0f : d == 0 ? 1.0f : 2.0f;
-            t = fmaf(wt * g, g, t);
+            d2 = fmaf(wt * g, g, d2);
           }
-          two_sum(sum0, make_float2(t, 0.f));
           store_planes8(e.out + r * e.ldo + col, e.os, 3, v);
         } else if (READS_X) {
           float xo[8];
@@ -747,28 +734,20 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           if (col < e.ldc) *reinterpret_cast<float4*>(cr) = make_float4(v[0], v[1], v[2], v[3]);
           if (col + 4 < e.ldc) *reinterpret_cast<float4*>(cr + 4) = make_float4(v[4], v[5], v[6], v[7]);
         }
-        if (STEP) {
-          step0 += warp_sum64(d2);
-          step1 += warp_sum64(x2);
-        }
+        if (EPI == TC_EPI_GRAM || STEP) sum0 += warp_sum64(d2);
+        if (STEP) sum1 += warp_sum64(x2);
       }
     }
   }
   if (EPI == CO_EPI_NORM) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
-    if (lane == 0) __stcg(e.norm + blockIdx.x * EPI_WARPS + w, norm);
+    if (lane == 0) __stcg(e.part + blockIdx.x * EPI_WARPS + w, norm);
   }
-  if (STEP && lane == 0) {
-    double* dst = e.norm + 2 * (blockIdx.x * EPI_WARPS + w);
-    __stcg(dst, step0);
-    __stcg(dst + 1, step1);
-  }
-  if (EPI == TC_EPI_GRAM) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      two_sum(sum0, make_float2(__shfl_xor_sync(0xffffffffu, sum0.x, o), __shfl_xor_sync(0xffffffffu, sum0.y, o)));
-    if (lane == 0) __stcg(e.part + blockIdx.x * EPI_WARPS + w, sum0);
+  if ((EPI == TC_EPI_GRAM || STEP) && lane == 0) {
+    double* dst = e.part + (STEP ? 2 : 1) * (blockIdx.x * EPI_WARPS + w);
+    __stcg(dst, sum0);
+    if (STEP) __stcg(dst + 1, sum1);
   }
 }
 
@@ -801,16 +780,6 @@ __device__ __forceinline__ double co_warp_sum(const double* p, int n, int stride
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// The same of unevaluated pairs; the lanes' sums stay pairs until the end (see two_sum).
-__device__ __forceinline__ double co_warp_sum2(const float2* p, int n, int stride, int lane) {
-  float2 v = make_float2(0.f, 0.f);
-  for (int i = lane; i < n; i += 32) two_sum(v, __ldcg(p + (size_t)i * stride));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    two_sum(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)));
-  return (double)v.x + (double)v.y;
 }
 
 // Block sum of one double per thread (valid in thread 0).

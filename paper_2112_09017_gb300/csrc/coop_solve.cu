@@ -34,7 +34,7 @@ struct CoSolve {
   float* C;
   int64_t ldc, ldp, xps, gps;
   double* partials;                          // one per block, two per block at the end
-  float2* part2;                             // residual sums, EPI_WARPS per block
+  double* part2;                             // residual sums, EPI_WARPS per block
   DevState* st;
   int m, n;
   double v_tol, stag2, v_floor;              // the stop rule on squares: n tol^2, stagnation^2, n stag_floor^2
@@ -139,7 +139,7 @@ __device__ __forceinline__ void co_solve(const CoSolve& p, uint8_t* co_raw) {
       co_product<TN, SPLIT, false, true, TC_EPI_NS>(x, pipe, &p.xk[b], &p.gmn, &p.gk, tu, n, e, p.su, p.withhold);
     }
     if (x.warp == CO_CTL_WARP) {
-      const double v = co_warp_sum2(p.part2, gridDim.x * EPI_WARPS, 1, x.lane);
+      const double v = co_warp_sum(p.part2, gridDim.x * EPI_WARPS, 1, x.lane);
       const int s = co_stop_status(p, k, v, v_km2);
       v_km2 = v_km1;
       v_km1 = v;
@@ -426,7 +426,7 @@ CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms
   p.gp = b.gp; p.ap = b.ap; p.C = b.C; p.ldc = b.ldc; p.ldp = b.ldp; p.xps = b.xps; p.gps = b.gps;
   p.partials = b.partials; p.st = b.st;
   // the residual sums take C's place (written only after the iteration) where the partials are too few
-  p.part2 = 8 * c->grid <= b.nparts ? reinterpret_cast<float2*>(b.partials) : reinterpret_cast<float2*>(b.C);
+  p.part2 = 8 * c->grid <= b.nparts ? b.partials : reinterpret_cast<double*>(b.C);
   p.m = (int)m; p.n = (int)n;
   p.inv_sqrt_n = 1.0 / sqrt((double)n);
   return c;

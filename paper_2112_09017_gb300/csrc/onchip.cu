@@ -37,6 +37,7 @@ namespace {
 
 constexpr int OC_WARPS = 16;          // workers (12 and 8, with more registers each, measured 6 and 15 % slower)
 constexpr int OC_SUB = OC_WARPS / 4;  // per TMEM lane quarter
+static_assert(OC_WARPS == 16, "the stop test adds 16 sums");
 constexpr int OC_GT = (128 / 16 + OC_SUB - 1) / OC_SUB;   // 16-wide chunks of G per worker, at most
 constexpr int OC_WORKERS = OC_WARPS * 32;
 constexpr int OC_THREADS = OC_WORKERS + 32;   // and one warp that issues the MMAs and decides
@@ -68,7 +69,7 @@ struct OcCtl {
   uint32_t tmem_base;
   int pad;
   float c1, c3;
-  float2 red[OC_WARPS];    // the warps' sums, unevaluated pairs hi + lo
+  double red[OC_WARPS];    // the warps' sums
 };
 
 __host__ __device__ __forceinline__ uint32_t oc_rows(int64_t m) { return (uint32_t)((m + 15) / 16 * 16); }
@@ -221,19 +222,16 @@ __device__ __noinline__ void oc_issue(const OcTask& tk, uint32_t xbase, uint32_t
       }
       __syncwarp();
     }
-    // the stop test: the workers' pairs summed in a fixed order, v = n r^2 against squared thresholds
-    float2 t = make_float2(0.f, 0.f);
-    if (lane < OC_WARPS) t = make_float2(ctl->red[lane].x, ctl->red[lane].y);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1)   // at most 16 of them; lane 0 has the sum
-      two_sum(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
-    t.x = __shfl_sync(0xffffffffu, t.x, 0);
-    t.y = __shfl_sync(0xffffffffu, t.y, 0);
-    const double v = (double)t.x + (double)t.y;
+    // the stop test: the warps' sums added in a fixed order (every lane has the sum), v = n r^2 against squared
+    // thresholds
+    const volatile double* red = ctl->red + 4 * (lane & 3);
+    double v = (red[0] + red[1]) + (red[2] + red[3]);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
     int dec = 2, status = ST_TIMEOUT;
     if (go) {
       const bool testing = k >= ctl->dr.n_pre;
-      if (!isfinite(t.x + t.y)) status = ST_NONFINITE;
+      if (!isfinite(v)) status = ST_NONFINITE;
       else if (testing && v <= ctl->dr.v_tol) status = ST_CONVERGED;
       else if (testing && k >= ctl->dr.n_pre + 2 && v > v_stag && v < ctl->dr.v_floor) status = ST_NOT_CONVERGED;
       else if (k >= ctl->dr.max_iter) status = ST_NOT_CONVERGED;
@@ -357,15 +355,8 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t ch
       }
     }
     if (stored) tmem_st_wait();
-    // sums of pairs in FP32 (a chain of FP64 additions takes as long as the products of a small problem)
-    float2 part = make_float2(part32, 0.0f);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      two_sum(part, make_float2(__shfl_xor_sync(0xffffffffu, part.x, o), __shfl_xor_sync(0xffffffffu, part.y, o)));
-    if (lane == 0) {
-      ctl->red[warp].x = part.x;
-      ctl->red[warp].y = part.y;
-    }
+    const double part = warp_sum64(part32);
+    if (lane == 0) ctl->red[warp] = part;
     tc_fence_before();
     oc_arrive<3>();
     oc_sync<4>();   // the decision
