@@ -73,21 +73,21 @@ __device__ __forceinline__ double warp_sum64(float v) {
   return __longlong_as_double((long long)(((uint64_t)(1023 + 63 - lz + ex - 185 - 1) << 52) + r));
 }
 
-// s + e = a + b exactly (Knuth's two-sum), accumulated into the unevaluated pair s.x + s.y.
-__device__ __forceinline__ void two_sum(float2& s, float2 b) {
-  const float t = s.x + b.x, bb = t - s.x;
-  const float e = (s.x - (t - bb)) + (b.x - bb);
-  s = make_float2(t, s.y + (b.y + e));
+// s <- s + b rounded, and its rounding error, exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float& s, float b) {
+  const float t = s + b, bb = t - s, e = (s - (t - bb)) + (b - bb);
+  s = t;
+  return e;
 }
 
-// A float64-grade sum of squares of float32 values. FP64 runs at 1/64 of the FP32 rate here (two FMAs a cycle
-// and SM), which made the norm of a batch take longer than reading it; so squares are split exactly into FP32
-// pairs (p = x x, e = fma(x, x, -p)) and added by two-sums, about 2^-44 relative, and only every eighth
-// group of eight goes through FP64. Groups whose largest magnitude is outside [2^-50, 2^60], where squares or
-// their errors could leave float32's range, are summed in FP64 as they are.
+// A float64 sum of squares of float32 values. FP64 runs at 1/64 of the FP32 rate here (two FMAs a cycle and SM),
+// which made the norm of a batch take longer than reading it; so squares are split exactly into FP32 pairs
+// (p = x x, e = fma(x, x, -p)) and added by two-sums into three floats, the last of which alone rounds, at about
+// 2^-68 of the sum, and only every eighth group of eight goes through FP64. Groups whose largest magnitude is
+// outside [2^-50, 2^60], where squares or their errors could leave float32's range, are summed in FP64 as they are.
 struct SquareSum {
   double total = 0.0;
-  float2 pair = {0.f, 0.f};
+  float hi = 0.f, mid = 0.f, lo = 0.f;
   int held = 0;
   __device__ __forceinline__ void add8(const float (&v)[8]) {
     float top = 0.f;
@@ -96,8 +96,9 @@ struct SquareSum {
     if (top <= 0x1p60f && (top >= 0x1p-50f || top == 0.f)) {   // a NaN among smaller values passes through the sums
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float q = v[j] * v[j];
-        two_sum(pair, make_float2(q, fmaf(v[j], v[j], -q)));
+        const float p = v[j] * v[j];
+        lo += two_sum(mid, two_sum(hi, p));
+        lo += two_sum(mid, fmaf(v[j], v[j], -p));
       }
       if (++held == 8) flush();
     } else {
@@ -106,8 +107,8 @@ struct SquareSum {
     }
   }
   __device__ __forceinline__ void flush() {
-    total += (double)pair.x + (double)pair.y;
-    pair = make_float2(0.f, 0.f);
+    total += (double)hi + ((double)mid + (double)lo);
+    hi = mid = lo = 0.f;
     held = 0;
   }
   __device__ __forceinline__ double value() {

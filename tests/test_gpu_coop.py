@@ -163,6 +163,25 @@ def test_residuals_are_summed_in_float64(lib, n, k, how):
     assert np.sqrt(np.mean(np.square(errs))) <= 3e-16, errs
 
 
+@pytest.mark.parametrize("prec,m,n,seeds", [("bf16x6", 8, 8, 12), ("bf16x6", 96, 64, 12), ("fp32", 300, 200, 12),
+                                            ("bf16x6", 3000, 2900, 3), ("bf16x6", 5000, 4500, 2)], ids=lambda v: str(v))
+def test_norm_is_summed_in_float64(lib, prec, m, n, seeds):
+    """||A||_F against the exact sum of squares, entries over eleven binades. A float64 sum as the kernels order it
+    (at most some 40 additions one after another) is off by about 1e-16, as in the test of the residuals; pairs
+    of floats by 3e-16 to 7.6e-16."""
+    import torch
+    plan = lib.Plan(m, n, prec=prec, max_iter=1)
+    errs = []
+    for seed in range(seeds):
+        rng = np.random.default_rng(1000 * seed + m + n)
+        a = (rng.standard_normal((m, n)) * 2.0 ** rng.integers(-5, 6, (m, n))).astype(np.float32)
+        want = math.sqrt(math.fsum((a.astype(np.float64) ** 2).reshape(-1)))   # the squares are exact
+        _, _, info = plan(torch.from_numpy(a).cuda(), raw_status=True)
+        errs.append((info["normA_F"] - want) / want)
+    plan.close()
+    assert np.sqrt(np.mean(np.square(errs))) <= 2.5e-16, errs
+
+
 @pytest.mark.parametrize("ta", [False, True])
 @pytest.mark.parametrize("tb", [False, True])
 @pytest.mark.parametrize("M,N,K,off", [(31, 33, 1, 0), (32, 64, 64, 0), (100, 700, 130, 1), (700, 40, 129, 0),
