@@ -238,8 +238,9 @@ __device__ __forceinline__ bool co_grid_sync(CoCtx& x) { return x.bar.sync(); }
 // Leaves the kernel: every thread of the block, after its last product. Reports an expired wait.
 template <int TN, bool SPLIT = false>
 __device__ __forceinline__ void co_teardown(CoCtx& x, DevState* st, int* err_word = nullptr) {
-  if (x.warp == 1 && x.lane == 0) {   // every MMA issued has completed before TMEM is released
-    tc_commit(x.br.drain);
+  if (x.warp == 1) {   // every MMA issued has completed before TMEM is released; a commit covers its own thread's
+    if (elect_one()) tc_commit(x.br.drain);   // the lane that issued them (co_mma)
+    __syncwarp();
     mbar_drain(x.br.drain, 0);
   }
   tc_fence_before();

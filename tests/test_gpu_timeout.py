@@ -68,3 +68,74 @@ def test_product_timeouts_reach_the_caller(lib, monkeypatch):
         assert lib.polar_async_status() == lib.POLAR_OK, name
         err = (c.double() - want).abs().max().item()
         assert err <= 1e-4 * want.abs().max().item(), (name, err)
+
+
+# one block, tiles shared by four blocks, whole tiles 64 and 128 wide
+ONE_LAUNCH = [("solve", 96, 64), ("solve", 512, 512), ("solve", 1300, 1290), ("solve", 2304, 2304),
+              ("inverse", 300, 300), ("inverse", 1001, 1001), ("inverse", 2300, 2300),
+              ("chebyshev", 300, 300), ("chebyshev", 1450, 1450), ("chebyshev", 2300, 2300)]
+
+
+@pytest.mark.parametrize("kind,m,n", ONE_LAUNCH, ids=lambda v: str(v))
+def test_one_launch_forms_expire_and_the_next_call_is_correct(lib, monkeypatch, kind, m, n):
+    """The blocks of a one-launch kernel leave at different times, each after its own wait; the last one out clears
+    the grid barrier, and the buffers (a plan's, or the block kept between calls) serve the next call."""
+    import torch
+    a = synth.matrix_with_spectrum_on_device(m, n, synth.logspace_spectrum(n, 0.2), 5, "cuda", torch.float32)
+    if kind == "chebyshev":
+        a = 0.5 * (a + a.T)
+    plan = lib.Plan(m, n) if kind == "solve" else None
+
+    def call():
+        if kind == "solve":
+            U, H, info = plan(a, raw_status=True)
+            return info["status"], torch.cat([U, H])
+        X = torch.zeros((n, m), device="cuda")
+        if kind == "inverse":
+            return lib.polar_ns_inverse(a, X, raw_status=True)["status"], X
+        return lib.polar_chebyshev(a, X, -1.0, 1.0, [0.3, 1.0, 0.2, 0.1], raw_status=True), X
+
+    status, want = call()
+    assert status == lib.POLAR_OK
+    monkeypatch.setenv("POLAR_TEST_WITHHOLD_TMA", "1")
+    t0 = time.time()
+    status, _ = call()
+    monkeypatch.delenv("POLAR_TEST_WITHHOLD_TMA")
+    assert status == lib.POLAR_ETIMEOUT and time.time() - t0 < 30.0
+    status, got = call()
+    assert status == lib.POLAR_OK and torch.equal(got, want)
+    if plan:
+        plan.close()
+
+
+def test_batched_loop_expires_and_the_next_run_starts_afresh(lib, monkeypatch):
+    """A batched plan built while copies are withheld keeps withholding them: each of its runs reports a timeout for
+    every problem and leaves U alone, the second as the first (the barrier and the counts are clear again); a plan
+    built afterwards solves."""
+    import torch
+    sizes = [(300, 300), (520, 260), (96, 96), (1000, 700)]
+    As = [torch.from_numpy(synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 1e-2), 60 + i)).cuda()
+          for i, (m, n) in enumerate(sizes)]
+    ms, ns = [m for m, _ in sizes], [n for _, n in sizes]
+    it = torch.zeros(len(sizes), dtype=torch.int32, device="cuda")
+    monkeypatch.setenv("POLAR_TEST_WITHHOLD_TMA", "1")
+    plan = lib.polar_batched_plan_create(ms, ns)
+    monkeypatch.delenv("POLAR_TEST_WITHHOLD_TMA")
+    for rep in range(2):
+        Us = [torch.full_like(a, 7.0) for a in As]
+        Hs = [torch.full((n, n), 7.0, device="cuda") for n in ns]
+        t0 = time.time()
+        lib.polar_batched_run(plan, As, Us, Hs, 0.0, it, None)
+        torch.cuda.synchronize()
+        assert time.time() - t0 < 30.0
+        assert bool((it == torch.iinfo(torch.int32).min).all()), it
+        assert all(bool((u == 7.0).all()) for u in Us)
+    lib.polar_plan_destroy(plan)
+    plan = lib.polar_batched_plan_create(ms, ns)
+    lib.polar_batched_run(plan, As, Us, Hs, 0.0, it, None)
+    torch.cuda.synchronize()
+    lib.polar_plan_destroy(plan)
+    assert bool((it >= 0).all()), it
+    for u in Us:
+        g = u.double().T @ u.double()
+        assert float(torch.linalg.matrix_norm(g - torch.eye(len(g), dtype=torch.float64, device="cuda"))) < 1e-4
