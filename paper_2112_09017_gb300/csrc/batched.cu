@@ -201,6 +201,7 @@ struct BatchedPlan {
   TcMapPair* h_m = nullptr;
   TcTile *gram_t = nullptr, *upd_t = nullptr, *h_t = nullptr;
   int n_gram = 0, n_upd = 0, n_h = 0;
+  int64_t deepest = 0;             // most K of all tiles that one block takes in a product
   int sms = 0;
   OcTask* oc_tasks = nullptr;      // problems solved on one SM each (largest first)
   int n_oc = 0;
@@ -210,6 +211,7 @@ struct BatchedPlan {
   int32_t* iters_cap = nullptr;    // the graph writes results here; copied out per run
   double* resid_cap = nullptr;
   cudaEvent_t tab_ev = nullptr;    // the last upload of host_tab has been consumed
+  int grid() const { return std::max(1, std::min(sms, std::max(std::max(n_gram, n_upd), n_h))); }
 };
 
 namespace {
@@ -225,19 +227,29 @@ polar_status_t b_alloc(BatchedPlan* b, size_t bytes, void** out) {
 }
 
 
-// Tile table: problems by decreasing work, each problem's tiles contiguous (neighbouring blocks of a wave
-// share that problem's operand panels in L2). tri: the tiles that hold an entry on or above the diagonal.
+// Tiles of a rows x cols product; tri: those that hold an entry on or above the diagonal.
+int64_t tile_count(int64_t rows, int64_t cols, bool tri) {
+  const int64_t tm = (rows + kTile - 1) / kTile, tn = (cols + kTile - 1) / kTile;
+  return tri ? tn * (tn + 1) / 2 : tm * tn;
+}
+
+// Tile table: problems by decreasing work, each problem's tiles contiguous and column by column (neighbouring
+// blocks of a wave share that problem's operand panels in L2).
 void build_tiles(const std::vector<int>& order, const std::vector<int64_t>& rows, const std::vector<int64_t>& cols,
-                 const std::vector<int64_t>& depth, bool tri, std::vector<TcTile>& out, std::vector<int>* ntiles_of) {
+                 const std::vector<int64_t>& depth, bool tri, std::vector<TcTile>& out) {
   out.clear();
   for (int p : order) {
     const int64_t tm = (rows[p] + kTile - 1) / kTile, tn = (cols[p] + kTile - 1) / kTile;
-    int local = 0;
     for (int64_t j = 0; j < tn; ++j)
-      for (int64_t i = 0; i < (tri ? std::min(j + 1, tm) : tm); ++i)
-        out.push_back({p, (uint32_t)(i | (j << 20)), local++, (int32_t)depth[p]});
-    if (ntiles_of) (*ntiles_of)[p] = local;
+      for (int64_t i = 0; i < (tri ? j + 1 : tm); ++i) out.push_back({p, (int32_t)i, (int32_t)j, (int32_t)depth[p]});
   }
+}
+
+// Most K of all tiles that one of `grid` blocks takes from a table.
+int64_t deepest_block(const std::vector<TcTile>& t, int grid) {
+  std::vector<int64_t> sum(grid, 0);
+  for (size_t i = 0; i < t.size(); ++i) sum[i % grid] += t[i].K;
+  return *std::max_element(sum.begin(), sum.end());
 }
 
 TcOperand opnd(const uint16_t* planes, int64_t rows, int64_t cols, int64_t ld, int64_t stride, int kmajor) {
@@ -281,8 +293,9 @@ polar_status_t enqueue_all(BatchedPlan* b, cudaStream_t s) {
   c.rule = rule;
   update_coeffs(rule, 0, c.pre_c1, c.pre_c3);   // of the preconditioning steps, where there are any
   c.withhold = tc_withhold();
-  const int most = std::max(std::max(b->n_gram, b->n_upd), b->n_h);
-  BK_(launch_co_batch(c, std::max(1, std::min(b->sms, most)), s));
+  // a block may wait for one that has all its tiles to do: about 14 ns per unit of K and tile, four times that
+  c.wait_ns = 2000000000ull + 56ull * (uint64_t)b->deepest;
+  BK_(launch_co_batch(c, b->grid(), s));
   b_u_kernel<<<dim3(count, ys), kThreads, 0, s>>>(b->meta_d, b->st_d, b->U_tab, b->sh_d);
   BK_(cudaGetLastError());
   b_h_kernel<<<dim3(count, ys), kThreads, 0, s>>>(b->meta_d, b->st_d, b->H_tab, b->sh_d);
@@ -340,8 +353,6 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
     a_bytes += (size_t)b->P * mt.xps * 2;
     c_bytes += (size_t)up(n[p] * n[p], 64) * 4;
   }
-  for (int p = 0; p < count; ++p)   // a tile's place has 20 bits for its row and 12 for its column
-    if (m[p] > ((int64_t)kTile << 20) || n[p] > ((int64_t)kTile << 12)) return fail(POLAR_ENOTSUP);
   std::vector<int> order(count);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
@@ -349,12 +360,11 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
   // problems that fit one SM run their loop there; the rest go through the tiles, which all problems share for H
   std::vector<int> order_tc, order_oc;
   for (int p : order) (opt.small_onchip != 0 && onchip_fits(m[p], n[p]) ? order_oc : order_tc).push_back(p);
-  std::vector<TcTile> gram_t, upd_t, h_t;
-  build_tiles(order_tc, b->n, b->n, b->m, true, gram_t, &ntg);
-  build_tiles(order_tc, b->m, b->n, b->n, false, upd_t, nullptr);
-  build_tiles(order, b->n, b->n, b->m, false, h_t, nullptr);
   size_t part_count = 0;
-  for (int p = 0; p < count; ++p) part_count += (size_t)ntg[p] * kBatchEpiWarps;
+  for (int p : order_tc) {
+    ntg[p] = (int)tile_count(n[p], n[p], true);
+    part_count += (size_t)ntg[p] * kBatchEpiWarps;
+  }
 
   uint8_t *xb[2], *gb, *ab, *cb;
   for (int i = 0; i < 2; ++i) {
@@ -454,6 +464,10 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
   }
   if ((r = put(hm.data(), sizeof(TcMapPair) * hm.size(), &v)) != POLAR_OK) return fail(r);
   b->h_m = (TcMapPair*)v;
+  std::vector<TcTile> gram_t, upd_t, h_t;
+  build_tiles(order_tc, b->n, b->n, b->m, true, gram_t);
+  build_tiles(order_tc, b->m, b->n, b->n, false, upd_t);
+  build_tiles(order, b->n, b->n, b->m, false, h_t);
   if ((r = put(gram_t.data(), sizeof(TcTile) * gram_t.size(), &v)) != POLAR_OK) return fail(r);
   b->gram_t = (TcTile*)v;
   b->n_gram = (int)gram_t.size();
@@ -463,6 +477,7 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
   if ((r = put(h_t.data(), sizeof(TcTile) * h_t.size(), &v)) != POLAR_OK) return fail(r);
   b->h_t = (TcTile*)v;
   b->n_h = (int)h_t.size();
+  for (const auto* t : {&gram_t, &upd_t}) b->deepest = std::max(b->deepest, deepest_block(*t, b->grid()));
 
   // capture the whole sequence once; each run uploads its pointer tables and replays it
   if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) return fail(POLAR_ECUDA);

@@ -33,11 +33,9 @@ struct alignas(128) TcMapPair {
   unsigned char a[128], b[128];
 };
 
-// One 128 x 128 tile of one problem: its place, the tile's index within the problem, and the product's K.
+// One 128 x 128 tile of one problem: its row and column, and the product's K.
 struct TcTile {
-  int32_t prob;
-  uint32_t place;    // tile row | tile column << 20
-  int32_t local;
+  int32_t prob, bi, bj;
   int32_t K;
 };
 
@@ -54,6 +52,7 @@ struct CoBatch {
   StopRule rule;
   float pre_c1, pre_c3;
   int withhold;
+  uint64_t wait_ns;             // bound of a grid barrier's wait
 };
 
 // The loop of every problem in the tables, then U^T A of every finished problem, in one cooperative launch

@@ -17,11 +17,13 @@ struct GridBarrier {
   GridBarWords* w;
   volatile int* abort_flag;   // in shared memory, zero at the start
   unsigned int target;        // arrivals the next sync waits for
+  uint64_t limit_ns;          // bound of a wait: longer than any block's work between two barriers
 
-  __device__ __forceinline__ GridBarrier(GridBarWords* words, int* abort) : w(words), abort_flag(abort), target(0) {}
+  __device__ __forceinline__ GridBarrier(GridBarWords* words, int* abort, uint64_t limit = 2 * WAIT_LIMIT_NS)
+      : w(words), abort_flag(abort), target(0), limit_ns(limit) {}
 
-  // Every block's global writes before it are visible after it. False when the wait expired (two seconds) or
-  // the block had aborted before. Must be reached by all threads of the block.
+  // Every block's global writes before it are visible after it. False when the wait expired or the block had
+  // aborted before. Must be reached by all threads of the block.
   __device__ __forceinline__ bool sync() {
     __syncthreads();
     target += gridDim.x;
@@ -32,7 +34,7 @@ struct GridBarrier {
         unsigned int v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&w->count) : "memory");
         if (v >= target) break;
-        if ((i & 63u) == 0 && gtime() - t0 > 2 * WAIT_LIMIT_NS) {
+        if ((i & 63u) == 0 && gtime() - t0 > limit_ns) {
           *abort_flag = 1;
           break;
         }

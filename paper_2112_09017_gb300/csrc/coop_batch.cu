@@ -31,7 +31,7 @@ struct CoTableSrc {
   int4 rec;          // of tile t
   int2 stat;         // its problem's (status, iters), once `have`
   bool have;
-  int prob, local;   // of the tile given out last
+  int prob;          // of the tile given out last
   int cur_par;
   CoEpi e;
 
@@ -58,14 +58,13 @@ struct CoTableSrc {
       if (t < n) rec = __ldg(reinterpret_cast<const int4*>(tiles + t));
       if (KIND == CB_H ? !finished_ok(s.x) : s.x != ST_RUNNING) continue;
       prob = r.x;
-      local = r.z;
       cur_par = KIND == CB_H ? (s.y & 1) : par;
       const TcMapPair* mp = maps(prob, cur_par);
       c.ma = reinterpret_cast<const CUtensorMap*>(mp->a);
       c.mb = KIND == CB_GRAM ? c.ma : reinterpret_cast<const CUtensorMap*>(mp->b);
       c.mbt = KIND == CB_UPDATE ? reinterpret_cast<const CUtensorMap*>(p.gram_m[0][prob].b) : nullptr;
-      c.bi = r.y & 0xfffff;
-      c.bj = (int)((uint32_t)r.y >> 20);
+      c.bi = r.y;
+      c.bj = r.z;
       c.kbeg = 0;
       c.K = r.w;
       c.slice = __ldg(&p.meta[prob].slice);
@@ -84,7 +83,7 @@ struct CoTableSrc {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(mp->b)) : "memory");
     }
   }
-  __device__ __forceinline__ const CoEpi& epi(const CoTile&) {
+  __device__ __forceinline__ const CoEpi& epi(const CoTile& c) {
     const BMeta& m = p.meta[prob];
     e.N = (int)m.n;
     e.M = KIND == CB_UPDATE ? (int)m.m : (int)m.n;
@@ -95,7 +94,8 @@ struct CoTableSrc {
       e.ldo = m.ldp;
       e.out = KIND == CB_GRAM ? m.gp : m.xp[par ^ 1];
       e.os = KIND == CB_GRAM ? m.gps : m.xps;
-      if (KIND == CB_GRAM) e.tile_part = m.partials + (int64_t)local * EPI_WARPS;
+      // the triangle's tiles are counted column by column
+      if (KIND == CB_GRAM) e.tile_part = m.partials + ((int64_t)c.bj * (c.bj + 1) / 2 + c.bi) * EPI_WARPS;
       if (KIND == CB_UPDATE) {
         e.x = m.xp[par];
         e.ldx = m.ldp;
@@ -112,7 +112,7 @@ template <int P>
 __global__ void __launch_bounds__(CO_THREADS, 1) co_batch_kernel(const __grid_constant__ CoBatch p) {
   extern __shared__ uint8_t co_raw[];
   constexpr int TN = 128;
-  CoCtx x = co_setup<TN, P>(co_raw, p.sh->bar);
+  CoCtx x = co_setup<TN, P>(co_raw, p.sh->bar, p.wait_ns);
   CoPipe pipe;
   bool run = true;
   const double tol = p.sh->tol > 0 ? p.sh->tol : p.rule.tol;
@@ -181,10 +181,12 @@ cudaError_t launch_p(const CoBatch& b, int grid, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_co_batch(const CoBatch& b, int max_grid, cudaStream_t s) {
-  // Any number of blocks solves the batch: where fewer SMs are available than the device has, half as many.
+  // Any number of blocks solves the batch: where fewer SMs are available than the device has, half as many, each
+  // with twice the tiles.
   cudaError_t e = cudaSuccess;
-  for (int grid = max_grid; grid >= 1; grid /= 2) {
-    e = b.P == 1 ? launch_p<1>(b, grid, s) : b.P == 2 ? launch_p<2>(b, grid, s) : launch_p<3>(b, grid, s);
+  CoBatch c = b;
+  for (int grid = max_grid; grid >= 1; grid /= 2, c.wait_ns *= 2) {
+    e = c.P == 1 ? launch_p<1>(c, grid, s) : c.P == 2 ? launch_p<2>(c, grid, s) : launch_p<3>(c, grid, s);
     if (e != cudaErrorCooperativeLaunchTooLarge) return e;
     cudaGetLastError();
   }

@@ -183,11 +183,11 @@ __device__ __forceinline__ int co_mirror_from(int n0) { return 128 * ((n0 + TN -
 // ------------------------------------------------------------------ set-up, grid barrier, teardown
 
 template <int TN, int P = CO_P, bool SPLIT = false>
-__device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar) {
+__device__ __forceinline__ CoCtx co_setup(uint8_t* smem_raw, void* bar, uint64_t wait_ns = 2 * WAIT_LIMIT_NS) {
   using C = CoCfg<TN, P, SPLIT>;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   CoCtl* ctl = reinterpret_cast<CoCtl*>(smem + C::STAGES * C::STAGE_BYTES + (SPLIT ? CO_XBUF : 0));
-  CoCtx x{ctl, smem, 0, 0, 0, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort)};
+  CoCtx x{ctl, smem, 0, 0, 0, 0, 0, Bars(), GridBarrier(static_cast<GridBarWords*>(bar), &ctl->abort, wait_ns)};
   x.smem_base = smem_u32(x.smem);
   x.br.full0 = smem_u32(&x.ctl->bars[0]);
   x.br.empty0 = smem_u32(&x.ctl->bars[C::STAGES]);

@@ -157,3 +157,14 @@ def test_bound_buffers_match_the_list_call(lib, torch_cuda):
         lib.polar_batched_bind(plan, As[:-1], U2[:-1], H2[:-1])
     lib.polar_plan_destroy(other)
     lib.polar_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("m,n", [((1 << 27) + 1, 1), ((1 << 19) + 1, (1 << 19) + 1)], ids=["tall", "wide"])
+def test_no_size_is_refused_but_for_memory(lib, m, n):
+    """Problems of more than 2^20 tile rows or 2^12 tile columns are laid out like any other; what refuses them here
+    is the workspace limit."""
+    o = lib.polar_default_options()
+    o.ws_limit = 1 << 20
+    with pytest.raises(lib.PolarError) as e:
+        lib.polar_batched_plan_create([m], [n], o)
+    assert e.value.code == lib.POLAR_ENOMEM
