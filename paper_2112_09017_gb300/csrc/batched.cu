@@ -319,9 +319,9 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
   if (!device_is_sm103(&b->sms)) { delete b; return POLAR_ECUDA; }
   b->m.assign(m, m + count);
   b->n.assign(n, n + count);
-  // k-blocks of 32 per promoted slice: the first matching tuning entry's, else 64 of K for three planes, 128
-  // for two, 256 for one (entries' tile widths are accepted and have no effect: every tile is 128 wide)
-  std::vector<int> slice_of(count, (b->P == 3 ? 64 : b->P == 2 ? 128 : 256) / 32);
+  // k-blocks of 32 per promoted slice: the first matching tuning entry's, else the library's (entries' tile widths
+  // are accepted and have no effect: every tile is 128 wide)
+  std::vector<int> slice_of(count, tc_default_slice(b->P));
   for (int p = 0; p < count && opt.tune; ++p) {
     const double aspect = (double)m[p] / (double)n[p];
     for (int e = 0; e < opt.n_tune; ++e) {

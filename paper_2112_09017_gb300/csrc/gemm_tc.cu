@@ -127,8 +127,6 @@ int forced_pair_mode() {
   return (e && (e[0] == '0' || e[0] == '1')) ? e[0] - '0' : -1;
 }
 
-bool tc_forced_form() { return forced_pair_mode() >= 0; }
-
 // Whether a launch of `planes`-plane products runs as CTA pairs (instantiated for three planes): a solve's Grams of
 // at least four waves of 256 x 256 pair tiles, and products of at least 32 waves with K from 15000. Gram and update,
 // 128 x 256 tiles and CTA pairs (us): 4096^2 238 245, 498 538; 6500^2 988 980, 1850 1953; 8192^2 1765 1713, 3640
@@ -171,8 +169,9 @@ int tc_gram_partials_max(int64_t n) {
 // k-stages per promoted slice. Each slice accumulates passes x K/16 MMAs with
 // round-toward-zero before its round-to-nearest promotion; 64 of K for three
 // planes (24 MMAs), 128 for two and 256 for one keep the promotion work below the
-// MMA time of a slice. POLAR_TC_SLICE_STAGES (1..16) overrides it for tuning.
-int default_slice_stages(int planes) {
+// MMA time of a slice. POLAR_TC_SLICE_STAGES (1..16) overrides it for tuning in every product (and sends what
+// would run in one launch to separate ones, below) and in batched plans, for problems their table does not name.
+int tc_default_slice(int planes) {
   static int env = [] {
     const char* e = getenv("POLAR_TC_SLICE_STAGES");
     int x = e ? atoi(e) : 0;
@@ -182,6 +181,9 @@ int default_slice_stages(int planes) {
   static_assert(BK == 16 || BK == 32, "slice lengths are multiples of the k-stage width");
   return (planes == 3 ? 64 : planes == 2 ? 128 : 256) / BK;
 }
+
+// The one-launch forms promote slices of 64 of K.
+bool tc_forced_form() { return forced_pair_mode() >= 0 || tc_default_slice(3) != 64 / BK; }
 
 // Test hook for the bounded waits: with POLAR_TEST_WITHHOLD_TMA=1 in the environment
 // the producer issues no copies, so the consumers' waits expire after about one
@@ -193,7 +195,7 @@ int tc_withhold() {
 
 cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
   TcArgs a = a_in;
-  if (a.slice_stages <= 0) a.slice_stages = default_slice_stages(a.nplanes);
+  if (a.slice_stages <= 0) a.slice_stages = tc_default_slice(a.nplanes);
   a.withhold_tma = tc_withhold();
   if (!a.st && !a.err_out) a.err_out = default_error_word();
   if (a.nplanes < 1 || a.nplanes > 3 || a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;

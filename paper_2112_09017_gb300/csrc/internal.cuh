@@ -224,7 +224,8 @@ bool tc_available();
 // columns x mn_box rows for K-major ones.
 bool tc_make_map(void* map, const TcOperand& op, int nplanes, bool mn_major, int mn_box);
 int tc_withhold();                                // test hook: 1 when producers are to issue no copies
-bool tc_forced_form();                            // the environment names the single-CTA or the CTA-pair form
+int tc_default_slice(int planes);                 // 32-wide k-stages per promoted slice
+bool tc_forced_form();                            // the environment names a form that only separate launches have
 
 // ---------------------------------------------------------------------------------
 // One solve in one cooperative launch (coop_solve.cu), for sizes whose products are a few waves of small

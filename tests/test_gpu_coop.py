@@ -344,3 +344,51 @@ def test_kept_workspace_is_not_shared_between_threads(lib):
     for t in ts:
         t.join()
     assert not errs
+
+
+_SLICE_PROBE = """
+import hashlib, sys, torch
+from paper_2112_09017_gb300 import polar, synth
+tune = [{"n_lo": 1, "n_hi": 10 ** 6, "aspect_lo": 0.0, "aspect_hi": 1e9, "tile_n": 0, "slice_stages": int(sys.argv[1])}]
+def digest(*ts):
+    torch.cuda.synchronize()
+    return hashlib.sha256(b"".join(t.cpu().numpy().tobytes() for t in ts)).hexdigest()[:16]
+a = torch.from_numpy(synth.matrix_with_spectrum(300, 300, synth.logspace_spectrum(300, 0.1), 1)).cuda()
+out = []
+U, H, info = polar.Plan(300, 300)(a)
+out += [info["launches"] > 1, digest(U, H)]
+X = torch.empty_like(a)
+polar.polar_ns_inverse(a, X)
+out.append(digest(X))
+s = a + a.T
+polar.polar_chebyshev(s, X, -4.0, 4.0, [1.0, 0.5, 0.25, 0.125, 0.0625])
+out.append(digest(X))
+for t in (None, tune):
+    p = polar.polar_batched_plan_create([300], [300], None, tune=t)
+    polar.polar_batched_run(p, [a], [U], [H], 0.0, None, None)
+    out.append(digest(U, H))
+print(*out)
+"""
+
+
+def _slice_probe(stages, env):
+    import os
+    import subprocess
+    import sys
+    e = {k: v for k, v in os.environ.items() if not k.startswith("POLAR_TC_")}
+    e.update(env)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _SLICE_PROBE, str(stages)], cwd=root, env=e, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    return r.stdout.split()
+
+
+def test_slice_length_of_the_environment_reaches_every_product(lib):
+    """POLAR_TC_SLICE_STAGES: the solve, the inverse and the Chebyshev series leave their one-launch forms, whose slices
+    are 64 of K, and a batched plan takes it where no table says otherwise. Read once per process, so in others."""
+    multi0, solve0, inv0, cheb0, batch0, tuned0 = _slice_probe(4, {})
+    multi4, solve4, inv4, cheb4, batch4, tuned4 = _slice_probe(4, {"POLAR_TC_SLICE_STAGES": "4"})
+    assert (multi0, multi4) == ("False", "True")
+    assert solve4 != solve0 and inv4 != inv0 and cheb4 != cheb0
+    assert batch0 != tuned0 and batch4 == tuned4 == tuned0
