@@ -203,6 +203,12 @@ POLAR_API void polar_plan_destroy(polar_plan_t plan);
  * stream of the device. The paper has no counterpart: error reporting of this library. */
 POLAR_API polar_status_t polar_async_status(polar_stream_t stream);
 
+/* Frees the block that polar_ns_inverse and polar_chebyshev keep on the current device between calls (at most
+ * 512 MiB; the next such call allocates one again). A block in use by a call of another thread is not touched and
+ * goes back to being kept when that call ends. Returns POLAR_OK, also when nothing was kept, or POLAR_ECUDA without
+ * a device. The paper has no counterpart: memory management of this library. */
+POLAR_API polar_status_t polar_release_workspace(void);
+
 /* C = alpha * op(A) op(B) + beta * C, op(X) = X or X^T (trans != 0), with op(A) M x K and
  * op(B) K x N, in precision `prec` (FP32, BF16, BF16X3, BF16X6, AUTO: BF16X6 when min(M, N) >= 256,
  * else FP32; the schedules return EINVAL). beta == 0 does not read C. Stream-asynchronous: a
@@ -250,7 +256,8 @@ POLAR_API polar_status_t polar_split_bf16(const float* X, int64_t count, int pla
  * ill-conditioned A (kappa >~ 1e2) the result is an approximate inverse. prec: BF16X6, BF16X3 or BF16
  * (products on the tensor cores with the same promotion as polar_run); FP32 -> ENOTSUP. Device pointers.
  * Its workspace is a library-owned block of at most 512 MiB kept between calls (one per device; concurrent
- * calls get their own), or, when that does not fit, allocated for the call; returns after the result is in X.
+ * calls get their own; polar_release_workspace frees it, and so does an allocation of the library that fails), or,
+ * when that does not fit, allocated for the call; returns after the result is in X.
  * *iters (updates applied) and *delta (the last relative change) may be NULL. Returns OK, NOT_CONVERGED (max_iter reached),
  * ENONFINITE (A zero or non-finite), EINVAL, ENOMEM, ENOTSUP or ECUDA.
  * Paper: Sec. III.D, Algorithm 2. */

@@ -88,7 +88,8 @@ polar_status_t scratch_get(size_t bytes, void** out) {
 // per device is kept between calls, up to kKeepBytes, because cudaMalloc, cudaMallocHost and their frees
 // cost such a call 0.3 to 1 ms, as much as the work of a matrix of a few hundred rows. A call takes the
 // block out (another thread's call then allocates its own) and puts it back after its stream has been
-// waited for, so no two calls ever share it; an allocation that fails in this library frees it first.
+// waited for, so no two calls ever share it; an allocation that fails in this library frees it first, and
+// polar_release_workspace gives it back to the program.
 constexpr size_t kKeepBytes = (size_t)512 << 20;
 
 struct CallBlock {
@@ -878,6 +879,13 @@ polar_status_t polar_async_status(polar_stream_t stream) {
   unsigned int v = 0;
   if (tc_take_error((cudaStream_t)stream, &v) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
   return v ? POLAR_ETIMEOUT : POLAR_OK;
+}
+
+polar_status_t polar_release_workspace(void) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
+  kept_trim();
+  return POLAR_OK;
 }
 
 polar_status_t polar_batched_plan_create(polar_plan_t* plan, int count, const int64_t* m, const int64_t* n,

@@ -82,6 +82,7 @@ def load():
         "polar_run": (i32, [vp, vp, i64, vp, i64, vp, i64, f64, C.POINTER(polar_info_t), vp]),
         "polar_run_host": (i32, [vp, vp, i64, vp, i64, vp, i64, f64, C.POINTER(polar_info_t), vp]),
         "polar_async_status": (i32, [vp]),
+        "polar_release_workspace": (i32, []),
         "polar_batched_plan_create": (i32, [C.POINTER(vp), i32, C.POINTER(i64), C.POINTER(i64),
                                             C.POINTER(polar_options_t)]),
         "polar_batched_run": (i32, [vp, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), f64, vp, vp, vp]),
@@ -192,6 +193,13 @@ def polar_async_status(stream=None) -> int:
     """Waits for `stream` and returns (and clears) the device's timeout status of the
     stream-asynchronous products: POLAR_OK, POLAR_ETIMEOUT or POLAR_ECUDA."""
     return load().polar_async_status(_stream(stream))
+
+
+def polar_release_workspace():
+    """Frees the block that polar_ns_inverse and polar_chebyshev keep on the current device between calls."""
+    r = load().polar_release_workspace()
+    if r != POLAR_OK:
+        raise PolarError(r, "polar_release_workspace")
 
 
 class BatchedPlan:

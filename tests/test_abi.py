@@ -166,6 +166,7 @@ def test_new_entry_points_check_arguments_without_gpu(built_lib):
     assert lib.polar_run_host(None, None, 1, None, 1, None, 1, 0.0, None, None) == polar.POLAR_EINVAL
     if not torch.cuda.is_available():
         assert lib.polar_async_status(None) == polar.POLAR_ECUDA
+        assert lib.polar_release_workspace() == polar.POLAR_ECUDA
         assert lib.polar_gemm_noalloc(0, 0, 4, 4, 4, 1.0, None, 4, None, 4, 0.0, None, 4,
                                       polar.POLAR_AUTO, None) == polar.POLAR_EINVAL   # null C first
     with pytest.raises(ValueError):

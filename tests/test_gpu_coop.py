@@ -346,6 +346,21 @@ def test_kept_workspace_is_not_shared_between_threads(lib):
     assert not errs
 
 
+def test_kept_workspace_is_given_back(lib):
+    import torch
+    a = torch.from_numpy(synth.matrix_with_spectrum(1500, 1500, synth.logspace_spectrum(1500, 0.3), 9)).cuda()
+    X, Y = torch.empty_like(a), torch.empty_like(a)
+    lib.polar_ns_inverse(a, X)
+    torch.cuda.synchronize()
+    held = torch.cuda.mem_get_info()[0]
+    lib.polar_release_workspace()
+    # planes of A, of X twice and of A X, and C = A^T A
+    assert torch.cuda.mem_get_info()[0] - held >= (4 * 3 * 2 + 4) * 1500 * 1500
+    lib.polar_release_workspace()                   # nothing is kept now
+    lib.polar_ns_inverse(a, Y)
+    assert torch.equal(X, Y)
+
+
 _SLICE_PROBE = """
 import hashlib, sys, torch
 from paper_2112_09017_gb300 import polar, synth
