@@ -57,3 +57,9 @@ def test_committed_cache_covers_the_tiled_sizes():
                 assert e["tile_n"] in (128, 256) and 1 <= e["slice_stages"] <= 8
         for b in d["measured"]:
             assert any(c["ok"] for c in b["candidates"])
+
+
+def test_committed_cache_keeps_the_short_slices_of_the_smallest_square_problems():
+    """Where 128 of K per slice gains about as much as two runs differ, the table keeps 64 and half the error."""
+    for n in (129, 200, 256):
+        assert autotune.choice_for(autotune.load("NVIDIA GB300"), n, n)["slice_stages"] == 2
