@@ -301,6 +301,8 @@ CoopFp32* coop_fp32_create(const CoopFp32Buffers& b, int64_t m, int64_t n, int s
 
 void coop_fp32_destroy(CoopFp32* c) { delete c; }
 
+int coop_fp32_blocks(const CoopFp32* c) { return c->grid; }
+
 cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                              const StopRule& rule, cudaStream_t s) {
   Co32& p = c->p;

@@ -336,7 +336,7 @@ int co_grid(int64_t m, int64_t n, int tn, int sms) {
 
 size_t coop_inverse_sums(int sms) { return (size_t)sms * EPI_WARPS * 3 * sizeof(double); }
 
-cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaStream_t s) {
+cudaError_t coop_inverse_launch(const CoopInverseArgs& a, const CoopForm& f, int sms, cudaStream_t s) {
   CoInverse p{};
   const TcOperand A = co_operand(a.ap, a.rows, a.cols, a.lpa, a.sa), P = co_operand(a.pp, a.rows, a.rows, a.lpx, a.sp);
   bool ok = tc_make_map(&p.amn, A, CO_P, true, 0) && tc_make_map(&p.ak, A, CO_P, false, BM) &&
@@ -350,33 +350,26 @@ cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaS
   p.A = a.A; p.lda = a.lda; p.X = a.X; p.ldx = a.ldx;
   p.ap = a.ap; p.pp = a.pp;
   p.lpa = a.lpa; p.sa = a.sa; p.lpx = a.lpx; p.sx = a.sx; p.sp = a.sp;
-  const CoopProduct prod[2] = {{a.rows, a.rows, a.cols, false}, {a.cols, a.rows, a.rows, false}};
-  int S[2] = {1, 1}, blocks = 0;
-  const bool split = coop_split_plan(prod, 2, sms, S, &blocks);
-  const int grid = co_grid(a.rows, a.rows, tn, sms);
-  p.sa2 = S[0];
-  p.su = S[1];
+  const int grid = co_grid(a.rows, a.rows, f.tn, sms);
+  p.sa2 = f.S[0];
+  p.su = f.S[1];
   p.norm = a.sums;
   p.step = a.sums + (size_t)sms * EPI_WARPS;
   p.st = a.st;
   p.rows = (int)a.rows; p.cols = (int)a.cols; p.max_iter = a.max_iter;
   p.withhold = tc_withhold();
-  if (split) return co_run(co_inverse_split_kernel, p, co_smem<64, CO_P, true>(), blocks, s);
-  return tn == 64 ? co_run(co_inverse_kernel<64>, p, co_smem<64>(), grid, s)
-                  : co_run(co_inverse_kernel<128>, p, co_smem<128>(), grid, s);
+  if (f.split) return co_run(co_inverse_split_kernel, p, co_smem<64, CO_P, true>(), f.blocks, s);
+  return f.tn == 64 ? co_run(co_inverse_kernel<64>, p, co_smem<64>(), grid, s)
+                    : co_run(co_inverse_kernel<128>, p, co_smem<128>(), grid, s);
 }
 
-cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_t s) {
+cudaError_t coop_cheb_launch(const CoopChebArgs& a, const CoopForm& f, int sms, cudaStream_t s) {
   CoCheb p{};
   if (a.degree < 2 || a.degree > COOP_MAX_DEGREE) return cudaErrorInvalidValue;
-  const CoopProduct prod = {a.n, a.n, a.n, true};
-  int blocks = 0;
-  const bool split = coop_split_plan(&prod, 1, sms, &p.S, &blocks);
-  if (split) tn = 64;
   bool ok = tc_make_map(&p.tmn, co_operand(a.tp, a.n, a.n, a.ldp, a.sp), CO_P, true, 0);
   for (int i = 0; i < 3; ++i) {
     const TcOperand B = co_operand(a.bp[i], a.n, a.n, a.ldp, a.sp);
-    ok = ok && tc_make_map(&p.bmn[i], B, CO_P, true, 0) && tc_make_map(&p.bk[i], B, CO_P, false, tn);
+    ok = ok && tc_make_map(&p.bmn[i], B, CO_P, true, 0) && tc_make_map(&p.bk[i], B, CO_P, false, f.tn);
     p.bp[i] = a.bp[i];
   }
   if (!ok) return cudaErrorInvalidValue;
@@ -386,11 +379,12 @@ cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_
   for (int k = 0; k <= a.degree; ++k) p.coef[k] = (float)a.coef[k];
   p.st = a.st;
   p.n = (int)a.n; p.degree = a.degree;
+  p.S = f.S[0];
   p.withhold = tc_withhold();
-  const int grid = co_grid(a.n, a.n, tn, sms);
-  if (split) return co_run(co_cheb_split_kernel, p, co_smem<64, CO_P, true>(), blocks, s);
-  return tn == 64 ? co_run(co_cheb_kernel<64>, p, co_smem<64>(), grid, s)
-                  : co_run(co_cheb_kernel<128>, p, co_smem<128>(), grid, s);
+  const int grid = co_grid(a.n, a.n, f.tn, sms);
+  if (f.split) return co_run(co_cheb_split_kernel, p, co_smem<64, CO_P, true>(), f.blocks, s);
+  return f.tn == 64 ? co_run(co_cheb_kernel<64>, p, co_smem<64>(), grid, s)
+                    : co_run(co_cheb_kernel<128>, p, co_smem<128>(), grid, s);
 }
 
 }  // namespace polar

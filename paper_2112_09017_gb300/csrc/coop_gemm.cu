@@ -1,6 +1,6 @@
 // One split-BF16 product C = alpha op(A) op(B) + beta C (three planes) in 128 x 64 tiles, for shapes with few
 // 128 x 256 tiles; the pieces are in coop_kernel.cuh (no grid barrier here: an ordinary launch). A 48 x 48 x 6000
-// product was one tile of 180 us. Where even the narrow tiles are few, clusters of four blocks share them
+// product was one tile of 165 us. Where even the narrow tiles are few, clusters of four blocks share them
 // along K.
 #include <algorithm>
 
@@ -67,36 +67,32 @@ int gemm_sms() {
 // 128 x 256 tiles take about 1600 cycles per k-block of 32 and 17000 for set-up and output step, in whole waves
 // (co_cost's measure; narrow ones about 750). Whole calls (splits and product) on 128 x 256 tiles and on narrow
 // ones: 48 x 48 x 6000 165 and 36 us, 128 x 128 x 512 31 and 17, 512^3 35 and 17, 1024^3 52 and 27, 100 x 5000 x
-// 500 38 and 25, 5000 x 100 x 5000 183 and 120, 1500^3 68 and 56, 971 x 1725 x 2232 109 and 76. Beyond one wave
-// of wide tiles the rule keeps those (2048^3 88, 3000 x 2500 x 500 60): twice the operand traffic per product is
-// what bounds narrow tiles there.
-bool co_gemm_better(const TcArgs& a) {
+// 500 38 and 25, 5000 x 100 x 5000 183 and 120, 1500^3 68 and 56, 971 x 1725 x 2232 109 and 76. From about one wave
+// of wide tiles on the costs decide for those (2048^3, 128 of them, 88 us; 3000 x 2500 x 500, 240, 60 us): twice the
+// operand traffic per product is what bounds narrow tiles there; past two waves they are not asked.
+CoopForm co_gemm_form(int64_t M, int64_t N, int64_t K, bool tri) {
+  CoopForm f;
   const int64_t lim = (int64_t)1 << 30;
-  if (a.M > lim || a.N > lim || a.K > lim) return false;
+  if (M > lim || N > lim || K > lim) return f;
   const int sms = gemm_sms();
-  const int64_t tm = (a.M + 127) / 128, tn = (a.N + 255) / 256;
-  const int64_t wide = a.triangular ? tri_tiles(tm, tn) : tm * tn;
-  if (wide > 2 * sms) return false;
-  const CoopProduct p = {a.M, a.N, a.K, a.triangular != 0};
-  int S, blocks;
+  const int64_t tm = (M + 127) / 128, tn = (N + 255) / 256;
+  const int64_t wide = tri ? tri_tiles(tm, tn) : tm * tn;
+  if (wide > 2 * sms) return f;
+  const CoopProduct p = {M, N, K, tri};
   double narrow;
-  coop_split_plan(&p, 1, sms, &S, &blocks, &narrow);
-  const double big = (double)((wide + sms - 1) / sms) * ((double)((a.K + 31) / 32) * 1600.0 + 17000.0);
-  return narrow + 4000.0 < big;
+  f.split = coop_split_plan(&p, 1, sms, f.S, &f.blocks, &narrow);
+  const double big = (double)((wide + sms - 1) / sms) * ((double)((K + 31) / 32) * 1600.0 + 17000.0);
+  if (narrow + 4000.0 >= big) return CoopForm();
+  f.tn = 64;
+  const int tiles = co_tiles<64>(M, N, tri).ntiles;
+  if (!f.split) f.S[0] = 1;
+  f.blocks = f.split ? (tiles * f.S[0] + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER : std::min(sms, tiles);
+  return f;
 }
 
-cudaError_t launch_co_gemm(const TcArgs& a, cudaStream_t s) {
+cudaError_t launch_co_gemm(const TcArgs& a, const CoopForm& f, cudaStream_t s) {
   CoGemm p{};
-  const int sms = gemm_sms();
-  const CoopProduct q = {a.M, a.N, a.K, a.triangular != 0};
-  int blocks = 0;
-  const bool split = coop_split_plan(&q, 1, sms, &p.S, &blocks);
-  if (!split) {
-    p.S = 1;
-    blocks = std::min(sms, co_tiles<64>(a.M, a.N, a.triangular != 0).ntiles);
-  } else {
-    blocks = (co_tiles<64>(a.M, a.N, a.triangular != 0).ntiles * p.S + CO_CLUSTER - 1) / CO_CLUSTER * CO_CLUSTER;
-  }
+  p.S = f.S[0];
   if (!tc_make_map(&p.a, a.a, CO_P, !a.a.kmajor, BM) || !tc_make_map(&p.b, a.b, CO_P, !a.b.kmajor, 64))
     return cudaErrorInvalidValue;
   p.C = a.C; p.ldc = a.ldc;
@@ -104,8 +100,8 @@ cudaError_t launch_co_gemm(const TcArgs& a, cudaStream_t s) {
   p.alpha = a.alpha; p.beta = a.beta;
   p.err = a.err_out;
   p.withhold = a.withhold_tma;
-  if (a.a.kmajor) return a.b.kmajor ? launch_t<false, true>(p, split, blocks, s) : launch_t<false, false>(p, split, blocks, s);
-  return a.b.kmajor ? launch_t<true, true>(p, split, blocks, s) : launch_t<true, false>(p, split, blocks, s);
+  if (a.a.kmajor) return a.b.kmajor ? launch_t<false, true>(p, f.split, f.blocks, s) : launch_t<false, false>(p, f.split, f.blocks, s);
+  return a.b.kmajor ? launch_t<true, true>(p, f.split, f.blocks, s) : launch_t<true, false>(p, f.split, f.blocks, s);
 }
 
 }  // namespace polar

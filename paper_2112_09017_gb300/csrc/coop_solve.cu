@@ -327,11 +327,16 @@ static double co_cost(const CoopProduct* p, int count, int sms, int64_t* waves) 
 // 113 against 174, 3072^2 326 against 445, 8192 x 2048 (7 waves of 128-wide tiles) 415 against 563, 4096^2 (7)
 // 798 against 796; 8192^2 (27 waves) 6782 against 5600, where wider tiles read less from L2. So the line lies at
 // eight waves.
-int coop_tile_n(const CoopProduct* p, int count, int sms) {
+CoopForm coop_form(const CoopProduct* p, int count, int sms) {
   int64_t w64, w128;
   const double c64 = co_cost<64>(p, count, sms, &w64), c128 = co_cost<128>(p, count, sms, &w128);
-  if (w128 > 8) return 0;
-  return c64 <= c128 ? 64 : 128;
+  CoopForm f;
+  if (w128 > 8) return f;
+  // few tiles: share each between blocks along K, where that shortens a step by a tenth
+  f.split = coop_split_plan(p, count, sms, f.S, &f.blocks);
+  if (!f.split) f.S[0] = f.S[1] = 1, f.blocks = 0;
+  f.tn = f.split || c64 <= c128 ? 64 : 128;
+  return f;
 }
 
 // Blocks per 128 x 64 tile of one product on `blocks` blocks (1, 2 or 4), and its cycles (co_cost's measure). A
@@ -375,27 +380,24 @@ bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* bloc
 
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms) {
   const CoopProduct prod[2] = {{n, n, m, true}, {m, n, n, false}};
-  const int tn = coop_tile_n(prod, 2, sms);
-  if (!tn) return nullptr;
+  const CoopForm f = coop_form(prod, 2, sms);
+  if (!f.tn) return nullptr;
   CoopSolve* c = new (std::nothrow) CoopSolve();
   if (!c) return nullptr;
-  c->tn = tn;
-  // few tiles: share each between blocks along K, where that shortens a step by a tenth
-  int S[2], blocks;
-  c->split = coop_split_plan(prod, 2, sms, S, &blocks) && blocks <= b.nparts / 2;
+  c->tn = f.tn;
+  c->split = f.split && f.blocks <= b.nparts / 2;
   c->p.sg = c->p.su = c->p.sh = 1;
   if (c->split) {
     double ch;
-    c->tn = 64;
-    c->p.sg = S[0];
-    c->p.su = S[1];
-    c->p.sh = co_split_of({n, n, m, false}, blocks, &ch);
+    c->p.sg = f.S[0];
+    c->p.su = f.S[1];
+    c->p.sh = co_split_of({n, n, m, false}, f.blocks, &ch);
   }
   // enough blocks for the larger product's tiles, and for the passes over A
   const int64_t tiles = c->tn == 64 ? co_tiles<64>(m, n, false).ntiles : co_tiles<128>(m, n, false).ntiles;
   int64_t grid = std::max<int64_t>(tiles, (m * n + 8191) / 8192);
   grid = std::min<int64_t>(grid, std::min<int64_t>(sms, b.nparts / 2));
-  if (c->split) grid = blocks;
+  if (c->split) grid = f.blocks;
   if (!c->split && tiles <= 2) grid = 1;   // a second tile takes less time than two grid barriers
   c->grid = (int)std::max<int64_t>(grid, 1);
   if (8 * c->grid > b.nparts && (size_t)8 * c->grid * 8 > (size_t)n * b.ldc * 4) {
@@ -433,6 +435,16 @@ CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms
 }
 
 void coop_solve_destroy(CoopSolve* c) { delete c; }
+
+CoopForm coop_solve_form(const CoopSolve* c) {
+  CoopForm f;
+  f.tn = c->tn;
+  f.blocks = c->grid;
+  f.S[0] = c->p.sg;
+  f.S[1] = c->p.su;
+  f.split = c->split;
+  return f;
+}
 
 cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                               const StopRule& rule, cudaStream_t s) {

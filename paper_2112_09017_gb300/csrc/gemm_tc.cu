@@ -216,8 +216,10 @@ cudaError_t launch_tc_gemm(const TcArgs& a_in, cudaStream_t s) {
   if (a.triangular && a.M != a.N) return cudaErrorInvalidValue;
   // few 128 x 256 tiles: 128 x 64 ones, shared between blocks along K where they are few too
   if (a.epi == TC_EPI_STORE && a.nplanes == 3 && a.slice_stages == 64 / BK && !a.st && !a.planes_dyn &&
-      !tc_forced_form() && co_gemm_better(a))
-    return launch_co_gemm(a, s);
+      !tc_forced_form()) {
+    const CoopForm f = co_gemm_form(a.M, a.N, a.K, a.triangular != 0);
+    if (f.tn) return launch_co_gemm(a, f, s);
+  }
   CUtensorMap ma, mb;
   const bool pair = use_pair(a.nplanes, a.M, a.N, a.K, a.epi, a.triangular != 0);
   if (!make_map(&ma, a.a, a.nplanes, !a.a.kmajor, BM)) return cudaErrorInvalidValue;

@@ -227,6 +227,20 @@ int tc_withhold();                                // test hook: 1 when producers
 int tc_default_slice(int planes);                 // 32-wide k-stages per promoted slice
 bool tc_forced_form();                            // the environment names a form that only separate launches have
 
+struct CoopProduct {
+  int64_t M, N, K;
+  bool tri;                                       // only the upper triangle's tiles
+};
+// How a chain of one or two products runs in one launch: tiles of 128 x tn (0: not for these sizes), each shared along
+// K by S[i] blocks (2 or 4) of a cluster in product i, on `blocks` blocks; unshared (split false) the launch chooses
+// the blocks.
+struct CoopForm {
+  int tn = 0, blocks = 0;
+  int S[2] = {1, 1};
+  bool split = false;
+};
+CoopForm coop_form(const CoopProduct* p, int count, int sms);
+
 // ---------------------------------------------------------------------------------
 // One solve in one cooperative launch (coop_solve.cu), for sizes whose products are a few waves of small
 // tiles, three planes. The buffers are the plan's.
@@ -243,6 +257,7 @@ struct CoopBuffers {
 struct CoopSolve;
 CoopSolve* coop_solve_create(const CoopBuffers& b, int64_t m, int64_t n, int sms);   // null: not for this size
 void coop_solve_destroy(CoopSolve* c);
+CoopForm coop_solve_form(const CoopSolve* c);
 cudaError_t coop_solve_launch(CoopSolve* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                               const StopRule& rule, cudaStream_t s);
 
@@ -259,22 +274,18 @@ struct CoopFp32Buffers {
 struct CoopFp32;
 CoopFp32* coop_fp32_create(const CoopFp32Buffers& b, int64_t m, int64_t n, int sms);
 void coop_fp32_destroy(CoopFp32* c);
+int coop_fp32_blocks(const CoopFp32* c);
 cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                              const StopRule& rule, cudaStream_t s);
 
 // The inverse and the Chebyshev function in one cooperative launch (coop_funcs.cu), three planes. The
 // caller provides the plane buffers (no initial contents needed) and a state whose barrier words are zero.
-struct CoopProduct {
-  int64_t M, N, K;
-  bool tri;                                       // only the upper triangle's tiles
-};
-int coop_tile_n(const CoopProduct* p, int count, int sms);   // tile width of a chain; 0: not for these sizes
 // Whether the chain is better run with blocks of a cluster sharing 128 x 64 tiles along K: S[i] blocks (1, 2 or
 // 4) per tile of product i, on *blocks blocks.
 bool coop_split_plan(const CoopProduct* p, int count, int sms, int* S, int* blocks, double* cycles = nullptr);
 // One product C = alpha op(A) op(B) + beta C of a STORE launch in 128 x 64 tiles (coop_gemm.cu), three planes.
-bool co_gemm_better(const TcArgs& a);             // whether that is faster than 128 x 256 tiles
-cudaError_t launch_co_gemm(const TcArgs& a, cudaStream_t s);
+CoopForm co_gemm_form(int64_t M, int64_t N, int64_t K, bool tri);   // tn 0: 128 x 256 tiles are faster
+cudaError_t launch_co_gemm(const TcArgs& a, const CoopForm& f, cudaStream_t s);
 constexpr int COOP_MAX_DEGREE = 511;
 struct CoopInverseArgs {
   const float* A; int64_t rows, cols, lda;
@@ -287,7 +298,7 @@ struct CoopInverseArgs {
   int max_iter;
 };
 size_t coop_inverse_sums(int sms);
-cudaError_t coop_inverse_launch(const CoopInverseArgs& a, int tn, int sms, cudaStream_t s);
+cudaError_t coop_inverse_launch(const CoopInverseArgs& a, const CoopForm& f, int sms, cudaStream_t s);
 struct CoopChebArgs {
   const float* A; int64_t n, lda;
   float* F; int64_t ldf;
@@ -297,7 +308,7 @@ struct CoopChebArgs {
   int degree;                                     // 2 .. COOP_MAX_DEGREE
   DevState* st;
 };
-cudaError_t coop_cheb_launch(const CoopChebArgs& a, int tn, int sms, cudaStream_t s);
+cudaError_t coop_cheb_launch(const CoopChebArgs& a, const CoopForm& f, int sms, cudaStream_t s);
 
 // Host helpers defined in polar_api.cu and shared with the other entry points.
 cudaError_t device_alloc(void** p, size_t bytes); // cudaMalloc; when it fails, again without the block kept

@@ -881,6 +881,37 @@ polar_status_t polar_async_status(polar_stream_t stream) {
   return v ? POLAR_ETIMEOUT : POLAR_OK;
 }
 
+polar_status_t polar_query_form(polar_plan_t plan, int what, int64_t m, int64_t n, int64_t k, polar_form_t* form) {
+  if (!form || (plan && plan->batched)) return POLAR_EINVAL;
+  if (!plan && (m < 1 || n < 1 || k < 1)) return POLAR_EINVAL;
+  int sms = 0;
+  if (!device_ok(&sms)) { cudaGetLastError(); return POLAR_ECUDA; }
+  CoopForm f;
+  if (plan) {
+    if (plan->coop) f = coop_solve_form(plan->coop);
+    if (plan->coop32) {
+      f.tn = 32;
+      f.blocks = coop_fp32_blocks(plan->coop32);
+    }
+  } else if (what == POLAR_FORM_INVERSE) {
+    const CoopProduct prod[2] = {{m, m, n, false}, {n, m, m, false}};
+    f = coop_form(prod, 2, sms);
+  } else if (what == POLAR_FORM_CHEBYSHEV) {
+    const CoopProduct prod = {n, n, n, true};
+    f = coop_form(&prod, 1, sms);
+  } else if (what == POLAR_FORM_GEMM) {
+    f = co_gemm_form(m, n, k, false);
+  } else {
+    return POLAR_EINVAL;
+  }
+  if (!plan && tc_forced_form()) f = CoopForm();
+  form->tile_n = f.tn;
+  form->blocks = f.blocks;
+  form->split[0] = f.S[0];
+  form->split[1] = f.S[1];
+  return POLAR_OK;
+}
+
 polar_status_t polar_release_workspace(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
@@ -1121,8 +1152,8 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
   uint8_t* w = call.dev();
   // small and medium matrices: the whole iteration in one cooperative launch
   const CoopProduct prod[2] = {{N, N, M, false}, {M, N, N, false}};
-  const int tn = prec == POLAR_BF16X6 && !tc_forced_form() ? coop_tile_n(prod, 2, sms) : 0;
-  if (tn) {
+  const CoopForm form = prec == POLAR_BF16X6 && !tc_forced_form() ? coop_form(prod, 2, sms) : CoopForm();
+  if (form.tn) {
     DevState* st = (DevState*)(w + o_st);
     if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
     CoopInverseArgs c{};
@@ -1133,7 +1164,7 @@ extern "C" polar_status_t polar_ns_inverse(const float* A, int64_t rows, int64_t
     c.sums = (double*)(w + o_sums);
     c.st = st;
     c.max_iter = max_iter;
-    const cudaError_t e = coop_inverse_launch(c, tn, sms, s);
+    const cudaError_t e = coop_inverse_launch(c, form, sms, s);
     if (e == cudaSuccess) {
       if (cudaMemcpyAsync(call.host(), st, sizeof(DevState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {
@@ -1297,9 +1328,9 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
   DevState* st = (DevState*)(w + o_st);
   // small and medium matrices: every step in one cooperative launch
   const CoopProduct prod = {n, n, n, true};
-  const int tn = prec == POLAR_BF16X6 && degree >= 2 && degree <= COOP_MAX_DEGREE && !tc_forced_form()
-                     ? coop_tile_n(&prod, 1, sms) : 0;
-  if (tn) {
+  const CoopForm form = prec == POLAR_BF16X6 && degree >= 2 && degree <= COOP_MAX_DEGREE && !tc_forced_form()
+                            ? coop_form(&prod, 1, sms) : CoopForm();
+  if (form.tn) {
     if (cudaMemsetAsync(st, 0, sizeof(DevState), s) != cudaSuccess) { cudaGetLastError(); return POLAR_ECUDA; }
     CoopChebArgs c{};
     c.A = A; c.n = n; c.lda = lda; c.F = F; c.ldf = ldf;
@@ -1307,7 +1338,7 @@ extern "C" polar_status_t polar_chebyshev(const float* A, int64_t n, int64_t lda
     for (int i = 0; i < 3; ++i) c.bp[i] = bk[i];
     c.am = am; c.bm = bm; c.coef = coef; c.degree = degree;
     c.st = st;
-    const cudaError_t e = coop_cheb_launch(c, tn, sms, s);
+    const cudaError_t e = coop_cheb_launch(c, form, sms, s);
     if (e == cudaSuccess) {
       if (cudaMemcpyAsync(call.host(), st, sizeof(DevState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess) {

@@ -17,6 +17,7 @@ POLAR_EINVAL, POLAR_ENOMEM, POLAR_ECUDA, POLAR_ENONFINITE, POLAR_ETIMEOUT, POLAR
 POLAR_FP32, POLAR_BF16X6, POLAR_TF32X3, POLAR_BF16X3 = 0, 1, 2, 3
 POLAR_SCHED_BF16_THEN_X3, POLAR_SCHED_FP8_BF16_X3, POLAR_AUTO, POLAR_BF16 = 4, 5, 6, 7
 POLAR_HIST = 128
+POLAR_FORM_INVERSE, POLAR_FORM_CHEBYSHEV, POLAR_FORM_GEMM = 0, 1, 2
 
 PREC = {"fp32": POLAR_FP32, "bf16x6": POLAR_BF16X6, "tf32x3": POLAR_TF32X3, "bf16x3": POLAR_BF16X3,
         "bf16_then_x3": POLAR_SCHED_BF16_THEN_X3, "fp8_bf16_x3": POLAR_SCHED_FP8_BF16_X3, "auto": POLAR_AUTO,
@@ -36,6 +37,10 @@ class polar_options_t(C.Structure):
                 ("precondition", C.c_int), ("s_minus", C.c_double), ("s0", C.c_double),
                 ("fp8_switch_residual", C.c_double), ("batched_tile_n", C.c_int), ("small_onchip", C.c_int),
                 ("tune", C.POINTER(polar_tune_entry_t)), ("n_tune", C.c_int)]
+
+
+class polar_form_t(C.Structure):
+    _fields_ = [("tile_n", C.c_int), ("blocks", C.c_int), ("split", C.c_int * 2)]
 
 
 class polar_info_t(C.Structure):
@@ -83,6 +88,7 @@ def load():
         "polar_run_host": (i32, [vp, vp, i64, vp, i64, vp, i64, f64, C.POINTER(polar_info_t), vp]),
         "polar_async_status": (i32, [vp]),
         "polar_release_workspace": (i32, []),
+        "polar_query_form": (i32, [vp, i32, i64, i64, i64, C.POINTER(polar_form_t)]),
         "polar_batched_plan_create": (i32, [C.POINTER(vp), i32, C.POINTER(i64), C.POINTER(i64),
                                             C.POINTER(polar_options_t)]),
         "polar_batched_run": (i32, [vp, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), f64, vp, vp, vp]),
@@ -193,6 +199,16 @@ def polar_async_status(stream=None) -> int:
     """Waits for `stream` and returns (and clears) the device's timeout status of the
     stream-asynchronous products: POLAR_OK, POLAR_ETIMEOUT or POLAR_ECUDA."""
     return load().polar_async_status(_stream(stream))
+
+
+def polar_query_form(plan=None, what=0, m=1, n=1, k=1):
+    """(tile_n, blocks, (split_0, split_1)) of a plan's solves, or of an inverse (POLAR_FORM_INVERSE, m x n), a
+    Chebyshev series (POLAR_FORM_CHEBYSHEV, n) or a product (POLAR_FORM_GEMM, m, n, k)."""
+    f = polar_form_t()
+    r = load().polar_query_form(plan, int(what), int(m), int(n), int(k), C.byref(f))
+    if r != POLAR_OK:
+        raise PolarError(r, "polar_query_form")
+    return f.tile_n, f.blocks, tuple(f.split)
 
 
 def polar_release_workspace():

@@ -65,6 +65,9 @@ def test_host_argument_checks_without_gpu(built_lib):
     assert lib.polar_plan_create(None, 4, 4, None) == polar.POLAR_EINVAL
     assert lib.polar_run(None, None, 1, None, 1, None, 1, 0.0, None, None) == polar.POLAR_EINVAL
     assert lib.polar_split_bf16(None, 10, 4, None, None) == polar.POLAR_EINVAL
+    f = polar.polar_form_t()
+    assert lib.polar_query_form(None, polar.POLAR_FORM_GEMM, 4, 4, 4, None) == polar.POLAR_EINVAL
+    assert lib.polar_query_form(None, polar.POLAR_FORM_GEMM, 4, 0, 4, ctypes.byref(f)) == polar.POLAR_EINVAL
     assert lib.polar_gemm(0, 0, -1, 1, 1, 1.0, None, 1, None, 1, 0.0, None, 1, 0, None) == polar.POLAR_EINVAL
     m = (ctypes.c_int64 * 2)(4, 2)
     n = (ctypes.c_int64 * 2)(4, 3)
@@ -113,7 +116,7 @@ def test_binding_structs_match_the_header_layout(tmp_path):
         pytest.skip("no C compiler")
     from paper_2112_09017_gb300 import polar
     lines = ["#include <stdio.h>", "#include <stddef.h>", '#include "polar.h"', "int main(void) {"]
-    for struct in (polar.polar_options_t, polar.polar_info_t):
+    for struct in (polar.polar_options_t, polar.polar_info_t, polar.polar_form_t):
         name = struct.__name__
         lines.append(f'  printf("{name} size %zu\\n", sizeof({name}));')
         for field, _ in struct._fields_:
@@ -125,7 +128,7 @@ def test_binding_structs_match_the_header_layout(tmp_path):
     subprocess.run([cc, "-I", os.path.join(ROOT, "include"), str(src), "-o", str(exe)], check=True)
     got = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n")
     want = []
-    for struct in (polar.polar_options_t, polar.polar_info_t):
+    for struct in (polar.polar_options_t, polar.polar_info_t, polar.polar_form_t):
         name = struct.__name__
         want.append(f"{name} size {ctypes.sizeof(struct)}")
         want += [f"{name} {field} {getattr(struct, field).offset}" for field, _ in struct._fields_]

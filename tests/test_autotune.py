@@ -42,7 +42,7 @@ def test_ctypes_table_matches_entries():
 
 
 def test_committed_cache_covers_the_tiled_sizes():
-    """Every committed table assigns a legal choice to every size the grouped launches see (n from
+    """Every committed table assigns a legal choice to every size the tiled loop sees (n from
     129 to 1024, m = n or 2n) and records the candidates it measured."""
     files = [f for f in os.listdir(autotune.TUNING_DIR) if f.endswith(".json")] if os.path.isdir(
         autotune.TUNING_DIR) else []

@@ -1,6 +1,5 @@
-"""Batched plans with tuning tables: per-problem tile widths and slice lengths (two grouped launches
-per product when both widths are in use) give the oracle's parity, like the default plan; and the
-autotuner's timing loop returns a legal choice."""
+"""Batched plans with tuning tables: per-problem slice lengths (and tile widths, which are accepted and have no
+effect) give the oracle's parity, like the default plan; and the autotuner's timing loop returns a legal choice."""
 import numpy as np
 import pytest
 
@@ -44,7 +43,7 @@ def test_tuned_plan_matches_oracle_like_default(lib):
             assert its[i] >= 0 and abs(int(its[i]) - ref["iters_at"]) <= 1, (SIZES[i], its[i], ref["iters_at"])
             met = metrics(a, Us[i], Hs[i], ref["U"])
             assert met["orth"] <= 5e-6 and met["bwd"] <= 5e-6 and met["fwd"] <= 1e-7 * KAPPA[i], (SIZES[i], met)
-        # the first two entries change the tiles of the n <= 300 problems; the results stay within the
+        # the first and the last entry change the slices of their problems; the results stay within the
         # forward bound of each other
         n = SIZES[i][1]
         diff = np.linalg.norm(tuned[0][i].astype(np.float64) - default[0][i]) / np.sqrt(n)
@@ -54,8 +53,8 @@ def test_tuned_plan_matches_oracle_like_default(lib):
 def test_tuner_returns_a_legal_choice(lib):
     import torch
     res = autotune.tune(lib, torch, count=8, reps=1, buckets=[(129, 256)], aspects=[(1, 0.0, 1.5)],
-                        candidates=[(256, 2), (128, 4)])
+                        candidates=[(128, 2), (128, 4)])
     (e,) = res["entries"]
-    assert (e["tile_n"], e["slice_stages"]) in ((256, 2), (128, 4))
+    assert (e["tile_n"], e["slice_stages"]) in ((128, 2), (128, 4))
     rows = res["measured"][0]["candidates"]
     assert all(r["ms"] > 0 for r in rows) and any(r["ok"] for r in rows)

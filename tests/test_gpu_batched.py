@@ -1,4 +1,4 @@
-"""GPU parity of polar_batched_run (grouped tensor-core launches, CUDA graph) against
+"""GPU parity of polar_batched_run (cooperative loop, CUDA graph) against
 the CPU oracle, problem by problem."""
 import math
 

@@ -1,6 +1,6 @@
 """GPU parity of the on-chip small-problem path of polar_batched_run (n <= 128,
 m <= 256: the whole Newton-Schulz loop in one CTA, X in shared memory, G and the
-accumulators in TMEM) against the CPU oracle, and against the grouped tile path."""
+accumulators in TMEM) against the CPU oracle, and against the tiled loop."""
 import math
 import time
 
@@ -61,7 +61,7 @@ def test_onchip_matches_oracle(lib):
         assert np.array_equal(Hs[i], Hs[i].T) or met["hsym"] <= 1e-6
 
 
-def test_onchip_agrees_with_grouped_path_and_is_deterministic(lib):
+def test_onchip_agrees_with_tiled_loop_and_is_deterministic(lib):
     mats = _mats(SMALL, KAPPA, 400)
     a_out = _run(lib, mats, onchip=1, reps=2)
     (Ua, Ha, ita, ra), (Ua2, Ha2, ita2, _) = a_out
@@ -135,29 +135,31 @@ def test_onchip_bounded_wait_expires_and_context_survives(lib, monkeypatch):
     assert metrics(mats[1], Us[1], Hs[1])["orth"] <= 5e-6
 
 
-@pytest.mark.parametrize("tile_n", [128, 256])
-def test_grouped_tile_widths_match_oracle(lib, tile_n):
-    """The grouped launches with 128-wide tiles (two epilogue groups on alternate tiles) and
-    with 256-wide tiles: parity with the oracle on uneven problems beyond the on-chip sizes."""
+@pytest.mark.parametrize("slice_stages", [1, 2, 4])
+def test_tiled_loop_matches_oracle(lib, slice_stages):
+    """The batched loop of 128-wide tiles with slices of 32, 64 and 128 of K between promotions: parity with the oracle on
+    uneven problems beyond the on-chip sizes, the same bits twice whatever width the options and the table name."""
     import torch
     sizes = [(300, 300), (520, 260), (257, 129), (400, 200), (1000, 500), (129, 129), (640, 640)]
     kap = [1e3, 1e2, 1e2, 1e2, 1e3, 10.0, 1e2]
     mats = _mats(sizes, kap, 1000)
     ms = [a.shape[0] for a in mats]
     ns = [a.shape[1] for a in mats]
-    o = lib.polar_default_options()
-    o.batched_tile_n = tile_n
-    plan = lib.polar_batched_plan_create(ms, ns, o)
     As = [torch.from_numpy(a).cuda() for a in mats]
     outs = []
-    for _ in range(2):
+    for tile_n in (128, 256):
+        o = lib.polar_default_options()
+        o.batched_tile_n = tile_n
+        plan = lib.polar_batched_plan_create(ms, ns, o, tune=[
+            {"n_lo": 1, "n_hi": 4096, "aspect_lo": 0.0, "aspect_hi": 1e9, "tile_n": 384 - tile_n,
+             "slice_stages": slice_stages}])
         Us = [torch.full((m, n), 7.0, device="cuda") for m, n in zip(ms, ns)]
         Hs = [torch.full((n, n), 7.0, device="cuda") for n in ns]
         it = torch.zeros(len(mats), dtype=torch.int32, device="cuda")
         lib.polar_batched_run(plan, As, Us, Hs, 0.0, it, None)
         torch.cuda.synchronize()
         outs.append(([to_np(u) for u in Us], [to_np(h) for h in Hs], it.cpu().numpy()))
-    lib.polar_plan_destroy(plan)
+        lib.polar_plan_destroy(plan)
     (Us, Hs, iters), (Us2, Hs2, iters2) = outs
     assert np.array_equal(iters, iters2)
     for i, a in enumerate(mats):

@@ -52,7 +52,7 @@ def test_polar_strided_views_and_guard_bands(lib, prec):
 
 def test_batched_outputs_stay_inside_their_problems(lib):
     """Batched outputs packed into one sentinel-filled buffer with gaps between the
-    problems (on-chip and grouped members alike): every gap keeps its sentinel and
+    problems (on-chip and tiled members alike): every gap keeps its sentinel and
     each problem's factors meet the bounds."""
     import torch
     sizes = [(64, 32), (300, 150), (96, 96), (520, 260), (256, 128), (129, 129)]

@@ -71,7 +71,7 @@ def test_product_timeouts_reach_the_caller(lib, monkeypatch):
 
 
 # one block, tiles shared by four blocks, whole tiles 64 and 128 wide
-ONE_LAUNCH = [("solve", 96, 64), ("solve", 512, 512), ("solve", 1300, 1290), ("solve", 2304, 2304),
+ONE_LAUNCH = [("solve", 96, 64), ("solve", 512, 512), ("solve", 1744, 1312), ("solve", 2304, 2304),
               ("inverse", 300, 300), ("inverse", 1001, 1001), ("inverse", 2300, 2300),
               ("chebyshev", 300, 300), ("chebyshev", 1450, 1450), ("chebyshev", 2300, 2300)]
 
