@@ -31,6 +31,7 @@ struct Co32 {
   int n_pre, max_iter;
   float pre_c1, pre_c3;
   double inv_sqrt_n;
+  int withhold;             // test hook: the first block leaves at once, the others' waits expire
 };
 
 struct Co32Ctl {
@@ -79,7 +80,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) co_fp32_kernel(const __grid_con
   const int tm = (m + SS_T - 1) / SS_T, tn = (n + SS_T - 1) / SS_T, ntri = tn * (tn + 1) / 2;
   DevState* st = p.st;
   GridBarrier bar(reinterpret_cast<GridBarWords*>(&st->bar), &ctl.abort);
-  if (tid == 0) ctl.abort = 0;
+  if (tid == 0) ctl.abort = p.withhold && blockIdx.x == 0 ? 1 : 0;
   __syncthreads();
   // ---- ||A||_F
   double acc = 0.0;
@@ -313,6 +314,7 @@ cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U,
   p.n_pre = rule.n_pre;
   p.max_iter = rule.max_iter;
   update_coeffs(rule, 0, p.pre_c1, p.pre_c3);   // of the preconditioning steps, where there are any
+  p.withhold = tc_withhold();
   void* args[] = {&p};
   return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(co_fp32_kernel), dim3((unsigned)c->grid),
                                      dim3(SS_THREADS), args, c32_smem(), s);

@@ -187,7 +187,8 @@ bool tc_forced_form() { return forced_pair_mode() >= 0 || tc_default_slice(3) !=
 
 // Test hook for the bounded waits: with POLAR_TEST_WITHHOLD_TMA=1 in the environment
 // the producer issues no copies, so the consumers' waits expire after about one
-// second and the launch reports a timeout instead of computing.
+// second and the launch reports a timeout instead of computing (the plain one-launch solve, which copies
+// nothing, leaves a block out of its grid barrier).
 int tc_withhold() {
   const char* e = getenv("POLAR_TEST_WITHHOLD_TMA");
   return (e && e[0] == '1') ? 1 : 0;
