@@ -33,7 +33,7 @@ struct GridBarrier {
       for (uint32_t i = 1;; ++i) {
         unsigned int v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&w->count) : "memory");
-        if (v >= target) break;
+        if ((int)(v - target) >= 0) break;   // arrivals count on past 2^32 in a very long loop
         if ((i & 63u) == 0 && gtime() - t0 > limit_ns) {
           *abort_flag = 1;
           break;
