@@ -323,18 +323,18 @@ POLAR_API polar_status_t polar_gemm_noalloc(int transA, int transB, int64_t M, i
                                             const float* A, int64_t lda, const float* B, int64_t ldb, float beta,
                                             float* C, int64_t ldc, int prec, polar_stream_t stream);
 
-/* Which form of its kernels a BF16X6 call takes on the current device, for tests and measurements: of `plan`'s solves
- * (`what` and the sizes are not read), or of polar_ns_inverse (m = rows, n = cols), polar_chebyshev (n) and polar_gemm
- * (m = M, n = N, k = K); sizes that are not read must be positive all the same. EINVAL for a null form, a
- * batched plan, a size below one or another `what`; ECUDA without an sm_103 device. */
+/* Which form of its kernels a call takes on the current device, for tests and measurements: of `plan`'s solves
+ * (`what` and the sizes are not read), or, in BF16X6, of polar_ns_inverse (m = rows, n = cols), polar_chebyshev (n)
+ * and polar_gemm (m = M, n = N, k = K), or of polar_gemm in FP32; sizes that are not read must be positive all the
+ * same. EINVAL for a null form, a batched plan, a size below one or another `what`; ECUDA without an sm_103 device. */
 typedef struct {
   int tile_n;    /* 64 or 128: one launch on tiles of that width (32: the plain form's); 0: separate launches, or
-                    for a product tiles of 128 x 256 */
+                    for a product tiles of 128 x 256 (FP32: 128 x 128) */
   int blocks;    /* of the launch, where the form names them, else 0 */
   int split[2];  /* blocks that share a tile along K: of the Gram and the update, of A X and the update, or of the
                     only product */
 } polar_form_t;
-enum { POLAR_FORM_INVERSE = 0, POLAR_FORM_CHEBYSHEV = 1, POLAR_FORM_GEMM = 2 };
+enum { POLAR_FORM_INVERSE = 0, POLAR_FORM_CHEBYSHEV = 1, POLAR_FORM_GEMM = 2, POLAR_FORM_GEMM_FP32 = 3 };
 POLAR_API polar_status_t polar_query_form(polar_plan_t plan, int what, int64_t m, int64_t n, int64_t k,
                                           polar_form_t* form);
 

@@ -270,12 +270,18 @@ struct CoopFp32 {
   int grid;
 };
 
-// Taken while the 32 x 32 tiles, at about 60 of the 128 FMAs a cycle an SM can do, finish before the 128 x 128
-// tiles, at about 80, whose last wave leaves SMs idle.
+// Taken where a step finishes first. In SM cycles, fitted to the steps of 45 solves of up to 2^24 entries (5 % off): a
+// wave of 32 x 32 tiles takes 26 per K, a step's barriers and stop test 21000; in separate launches a wave of 128 x
+// 128 tiles 236 per K, a step's launches 64000. One launch against separate ones, us per step: 300 x 200 18 and 98,
+// 1024^2 167 and 245, 1256^2 291 and 323, 1580^2 524 and 562; 1755^2 708 and 630, 2108^2 1143 and 972, 3159 x 1757
+// 1222 and 981.
 bool coop_fp32_fits(int64_t m, int64_t n, int sms) {
-  const int64_t t = ((m + 127) / 128) * ((n + 127) / 128), g = ((n + 127) / 128) * ((n + 127) / 128 + 1) / 2;
-  const double big = (double)((t + sms - 1) / sms * n + (g + sms - 1) / sms * m) * 128 * 128 / 80.0;
-  const double small = (1.0 * m * n * n + 0.5 * m * n * n) / sms / 60.0;
+  auto tri = [](int64_t t) { return t * (t + 1) / 2; };
+  auto waves = [](int64_t t, int64_t on) { return (double)((t + on - 1) / on); };
+  const int64_t um = (m + 127) / 128, un = (n + 127) / 128;
+  const double big = 236.0 * (waves(tri(un), sms) * (double)m + waves(um * un, sms) * (double)n) + 64000.0;
+  const int64_t tm = (m + SS_T - 1) / SS_T, tn = (n + SS_T - 1) / SS_T, grid = std::min<int64_t>(tm * tn, sms);
+  const double small = 26.0 * (waves(tri(tn), grid) * (double)m + waves(tm * tn, grid) * (double)n) + 21000.0;
   return m * n <= (int64_t)1 << 24 && small < big;
 }
 

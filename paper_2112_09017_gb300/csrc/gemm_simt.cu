@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(NT) simt_gemm_kernel(SimtArgs p, bool vec_a, b
   }
 }
 
-// C = alpha op(A) op(B) + beta C in 32 x 32 tiles, one per block (simt_small.cuh).
+// C = alpha op(A) op(B) + beta C in 32 x 32 tiles, one per block (simt_small.cuh): see simt_small_better.
 template <bool AK, bool BK_>
 __global__ void __launch_bounds__(SS_THREADS) simt_small_kernel(SimtArgs p, bool vec_a, bool vec_b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -286,20 +286,6 @@ int simt_sms() {
   return n > 0 ? n : 1;
 }
 
-// 32 x 32 tiles where they finish first: an SM does about 60 of its 128 FMAs a cycle on them and 80 on 128 x
-// 128 tiles, but those come in whole waves of one tile per SM.
-bool use_small(const SimtArgs& a, int64_t tiles128) {
-  const int64_t lim = (int64_t)1 << 30;
-  if (a.K < 1 || a.M > lim || a.N > lim || a.K > lim) return false;
-  const int64_t tm = (a.M + SS_T - 1) / SS_T, tn = (a.N + SS_T - 1) / SS_T;
-  const int64_t t32 = a.triangular ? tn * (tn + 1) / 2 : tm * tn;
-  if (t32 > lim) return false;
-  const int64_t sms = simt_sms();
-  const double big = (double)((tiles128 + sms - 1) / sms) * BM * BN / 80.0;
-  const double small = std::max(1.0, (double)t32 / sms) * SS_T * SS_T / 60.0;
-  return small < big;
-}
-
 cudaError_t launch_small(const SimtArgs& a, bool vec_a, bool vec_b, cudaStream_t s) {
   const int64_t tm = (a.M + SS_T - 1) / SS_T, tn = (a.N + SS_T - 1) / SS_T;
   const unsigned grid = (unsigned)(a.triangular ? tn * (tn + 1) / 2 : tm * tn);
@@ -315,6 +301,23 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 }  // namespace
 
+// 32 x 32 tiles where they finish first. In SM cycles, fitted to 230 products of 32 to 6000: a 32 x 32 tile takes 30
+// per K (34 FMAs a cycle) and 2500, a wave of 128 x 128 tiles 205 per K (80 FMAs a cycle) and 7000. Small against
+// large tiles, us: 52 x 77 x 3360 47 and 375, 634 x 161 x 1509 32 and 176, 4163 x 74 x 240 18 and 33, 911 x 625 x 774
+// 65 and 96, 1883 x 539 x 3684 337 and 410; 448 x 5480 x 1629 402 and 366, 1279 x 887 x 115 28 and 22, 2936 x 641 x
+// 580 114 and 73, 515 x 5211 x 27 48 and 19, 1890 x 2072 x 4561 2180 and 1037.
+bool simt_small_better(int64_t M, int64_t N, int64_t K, bool tri) {
+  const int64_t lim = (int64_t)1 << 30;
+  if (K < 1 || M > lim || N > lim || K > lim) return false;
+  const int64_t tm = (M + SS_T - 1) / SS_T, tn = (N + SS_T - 1) / SS_T;
+  const int64_t t32 = tri ? tn * (tn + 1) / 2 : tm * tn;
+  if (t32 > lim) return false;
+  const int64_t um = (M + BM - 1) / BM, un = (N + BN - 1) / BN, t128 = tri ? un * (un + 1) / 2 : um * un;
+  const int64_t sms = simt_sms();
+  const double big = (double)((t128 + sms - 1) / sms) * (205.0 * (double)K + 7000.0);
+  return std::max(1.0, (double)t32 / sms) * (30.0 * (double)K + 2500.0) < big;
+}
+
 int simt_gram_tiles(int64_t n) {
   int64_t t = (n + BN - 1) / BN;
   return (int)(t * (t + 1) / 2);
@@ -328,7 +331,8 @@ cudaError_t launch_simt_gemm(const SimtArgs& a, int epi, cudaStream_t s) {
   const bool vec_b = aligned16(a.B) && (a.ldb % 4 == 0);
   const bool vec_c = aligned16(a.C) && (a.ldc % 4 == 0) &&
                      (epi != SIMT_EPI_NS || (aligned16(a.Xold) && a.ldx % 4 == 0));
-  if (epi == SIMT_EPI_STORE && !a.st && use_small(a, tiles)) return launch_small(a, vec_a, vec_b, s);
+  if (epi == SIMT_EPI_STORE && !a.st && simt_small_better(a.M, a.N, a.K, a.triangular != 0))
+    return launch_small(a, vec_a, vec_b, s);
   const size_t smem = sizeof(Smem);
   cudaError_t e = cudaSuccess;
   switch (epi) {

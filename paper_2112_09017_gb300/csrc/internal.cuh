@@ -275,6 +275,7 @@ struct CoopFp32;
 CoopFp32* coop_fp32_create(const CoopFp32Buffers& b, int64_t m, int64_t n, int sms);
 void coop_fp32_destroy(CoopFp32* c);
 int coop_fp32_blocks(const CoopFp32* c);
+bool simt_small_better(int64_t M, int64_t N, int64_t K, bool tri);   // 32 x 32 tiles for a plain product (gemm_simt.cu)
 cudaError_t coop_fp32_launch(CoopFp32* c, const float* A, int64_t lda, float* U, int64_t ldu, float* H, int64_t ldh,
                              const StopRule& rule, cudaStream_t s);
 

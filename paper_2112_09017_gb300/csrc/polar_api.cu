@@ -901,10 +901,12 @@ polar_status_t polar_query_form(polar_plan_t plan, int what, int64_t m, int64_t 
     f = coop_form(&prod, 1, sms);
   } else if (what == POLAR_FORM_GEMM) {
     f = co_gemm_form(m, n, k, false);
+  } else if (what == POLAR_FORM_GEMM_FP32) {
+    f.tn = simt_small_better(m, n, k, false) ? 32 : 0;
   } else {
     return POLAR_EINVAL;
   }
-  if (!plan && tc_forced_form()) f = CoopForm();
+  if (!plan && what != POLAR_FORM_GEMM_FP32 && tc_forced_form()) f = CoopForm();
   form->tile_n = f.tn;
   form->blocks = f.blocks;
   form->split[0] = f.S[0];

@@ -17,7 +17,7 @@ POLAR_EINVAL, POLAR_ENOMEM, POLAR_ECUDA, POLAR_ENONFINITE, POLAR_ETIMEOUT, POLAR
 POLAR_FP32, POLAR_BF16X6, POLAR_TF32X3, POLAR_BF16X3 = 0, 1, 2, 3
 POLAR_SCHED_BF16_THEN_X3, POLAR_SCHED_FP8_BF16_X3, POLAR_AUTO, POLAR_BF16 = 4, 5, 6, 7
 POLAR_HIST = 128
-POLAR_FORM_INVERSE, POLAR_FORM_CHEBYSHEV, POLAR_FORM_GEMM = 0, 1, 2
+POLAR_FORM_INVERSE, POLAR_FORM_CHEBYSHEV, POLAR_FORM_GEMM, POLAR_FORM_GEMM_FP32 = 0, 1, 2, 3
 
 PREC = {"fp32": POLAR_FP32, "bf16x6": POLAR_BF16X6, "tf32x3": POLAR_TF32X3, "bf16x3": POLAR_BF16X3,
         "bf16_then_x3": POLAR_SCHED_BF16_THEN_X3, "fp8_bf16_x3": POLAR_SCHED_FP8_BF16_X3, "auto": POLAR_AUTO,
@@ -203,7 +203,7 @@ def polar_async_status(stream=None) -> int:
 
 def polar_query_form(plan=None, what=0, m=1, n=1, k=1):
     """(tile_n, blocks, (split_0, split_1)) of a plan's solves, or of an inverse (POLAR_FORM_INVERSE, m x n), a
-    Chebyshev series (POLAR_FORM_CHEBYSHEV, n) or a product (POLAR_FORM_GEMM, m, n, k)."""
+    Chebyshev series (POLAR_FORM_CHEBYSHEV, n) or a product (POLAR_FORM_GEMM, POLAR_FORM_GEMM_FP32, m, n, k)."""
     f = polar_form_t()
     r = load().polar_query_form(plan, int(what), int(m), int(n), int(k), C.byref(f))
     if r != POLAR_OK:

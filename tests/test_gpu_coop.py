@@ -34,8 +34,8 @@ SIZES = [(1, 1), (32, 31), (64, 64), (128, 65), (129, 128), (130, 129), (192, 19
 
 # the plain form's 32 x 32 tiles: edges, remainders of the 64-deep chunks, near the largest square one, and beyond it
 SIZES32 = [(1, 1), (31, 31), (33, 32), (64, 33), (65, 64), (300, 200), (130, 129), (3000, 40), (1000, 990),
-           (1700, 1650), (2000, 2000)]
-SEPARATE = [("bf16x6", 155649, 33), ("fp32", 2000, 2000)]
+           (1640, 1640), (1700, 1650), (2000, 2000)]
+SEPARATE = [("bf16x6", 155649, 33), ("fp32", 1700, 1650), ("fp32", 2000, 2000)]
 
 
 @pytest.mark.parametrize("prec,m,n", [("bf16x6", *s) for s in SIZES] + [("fp32", *s) for s in SIZES32],
@@ -185,10 +185,12 @@ def test_norm_is_summed_in_float64(lib, prec, m, n, seeds):
     assert np.sqrt(np.mean(np.square(errs))) <= 2.5e-16, errs
 
 
+PLAIN = [(31, 33, 1, 0), (32, 64, 64, 0), (100, 700, 130, 1), (700, 40, 129, 0), (900, 600, 520, 1)]
+
+
 @pytest.mark.parametrize("ta", [False, True])
 @pytest.mark.parametrize("tb", [False, True])
-@pytest.mark.parametrize("M,N,K,off", [(31, 33, 1, 0), (32, 64, 64, 0), (100, 700, 130, 1), (700, 40, 129, 0),
-                                       (1100, 1000, 65, 1)], ids=lambda v: str(v))
+@pytest.mark.parametrize("M,N,K,off", PLAIN, ids=lambda v: str(v))
 def test_fp32_products_in_small_tiles(lib, ta, tb, M, N, K, off):
     """Both storage orders of both operands, tile and chunk remainders, aligned rows and rows that are not
     (a view one element into a wider matrix), with C read and written in place."""
@@ -331,6 +333,11 @@ def test_these_sizes_reach_every_form(lib):
     assert forms(lib.POLAR_FORM_CHEBYSHEV, [(n, n) for n, _ in CHEBYSHEVS]) == {(64, 4, 1), (64, 2, 1), (64, 1, 1),
                                                                                (128, 1, 1)}
     assert forms(lib.POLAR_FORM_GEMM, [s[:3] for s in GEMMS]) == {(64, 4, 1), (64, 2, 1), (64, 1, 1), (0, 1, 1)}
+    # plain products and solves that were measured faster on 128 x 128 tiles, and on 32 x 32 ones
+    assert forms(lib.POLAR_FORM_GEMM_FP32, [(448, 5480, 1629), (1279, 887, 115), (2936, 641, 580), (515, 5211, 27),
+                                            (718, 2215, 806), (1656, 1757, 478)]) == {(0, 1, 1)}
+    assert forms(lib.POLAR_FORM_GEMM_FP32, [(52, 77, 3360), (634, 161, 1509), (4163, 74, 240), (911, 625, 774),
+                                            (1883, 539, 3684)] + [s[:3] for s in PLAIN]) == {(32, 1, 1)}
     assert forms(lib.POLAR_FORM_INVERSE, [(4500, 4400)]) == {(0, 1, 1)}
     assert forms(lib.POLAR_FORM_CHEBYSHEV, [(7000, 7000)]) == {(0, 1, 1)}
 
