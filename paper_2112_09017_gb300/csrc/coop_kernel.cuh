@@ -473,6 +473,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
     }
     if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
     float d2 = 0.f, x2 = 0.f;
+    float t[NCH] = {};   // GRAM: the chunks' residual terms
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const int c0 = cb + 32 * c;
@@ -480,7 +481,6 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
       if (c0 >= e.N) continue;                       // the same for every lane of the warp
       if (EPI == TC_EPI_GRAM) {
         // residual terms: twice the squares above the diagonal, (g - 1)^2 on it (columns past N hold zeros)
-        float t = 0.0f;
         if (r < e.M && c0 + 31 >= r) {
           float s4[4] = {0.f, 0.f, 0.f, 0.f};
           if (c0 > r) {
@@ -496,9 +496,8 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
               s4[j & 3] = fmaf(w * g, g, s4[j & 3]);
             }
           }
-          t = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+          t[c] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
         }
-        sum0 += warp_sum64(t);
       }
       if (EPI == CO_EPI_NORM) {   // twice the squares above the diagonal, the squares on it
         if (r < e.M && c0 + 31 >= r) {
@@ -571,6 +570,7 @@ __device__ __forceinline__ void co_epilogue(const CoCtx& x, CoPipe& pp, Src src)
         }
       }
     }
+    if (EPI == TC_EPI_GRAM) sum0 += warp_sum64<NCH>(t);
     if (Src::TABLE && EPI == TC_EPI_GRAM) {
       if (lane == 0) e.tile_part[x.warp - 2] = sum0;
       sum0 = 0.0;

@@ -52,25 +52,64 @@ __device__ __forceinline__ float2 bf16_pair(uint32_t w) {
   return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
 
-// The sum of the lanes' non-negative floats as a float64, the same in every lane of a converged warp, whatever
-// their magnitudes: fixed point with 35 bits below the largest value's last one, so that what is cut off is no more
-// than a float64 sum's rounding, in integers because a chain of FP64 shuffles costs a step of a small
-// solve more than its warp-wide integer sums (FP64 runs at two operations a cycle and SM). An infinity or a NaN
-// among them is the result.
-__device__ __forceinline__ double warp_sum64(float v) {
-  const uint32_t b = __float_as_uint(v), top = __reduce_max_sync(0xffffffffu, b);
-  if (top >= 0x7f800000u) return (double)__uint_as_float(top);
-  const int ex = max((int)(top >> 23), 1), down = ex - max((int)(b >> 23), 1);
-  const uint64_t man = (b & 0x7fffffu) | (b >> 23 ? 0x800000u : 0u);
-  const uint64_t q = down < 59 ? (man << 35) >> down : 0u;   // v = q 2^(ex - 185), q < 2^59
+// A non-negative number s 2^e; e = FIXED_BAD for one that is not finite.
+struct Fixed {
+  uint64_t s;
+  int e;
+};
+constexpr int FIXED_BAD = 1024;
+
+__device__ __forceinline__ double fixed_double(Fixed f) {   // rounded to nearest; for -900 < e
+  if (f.e == FIXED_BAD) return __longlong_as_double(0x7ff8000000000000ll);
+  if (f.s == 0) return 0.0;
+  const int lz = __clzll((long long)f.s);
+  const uint64_t n = f.s << lz, r = (n >> 11) + ((n >> 10) & 1u);   // 53 bits; the top one adds one to the exponent
+  return __longlong_as_double((long long)(((uint64_t)(1023 + 63 - 1 - lz + f.e) << 52) + r));
+}
+
+// The sum of the lanes' q, each below 2^59 (2^60 in half of the lanes, the others zero).
+__device__ __forceinline__ uint64_t warp_add59(uint64_t q) {
   const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)q & 0x1fffffu),
                  s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(q >> 21) & 0x1fffffu),
                  s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(q >> 42));
-  const uint64_t s = ((uint64_t)s2 << 42) + ((uint64_t)s1 << 21) + s0;
-  if (s == 0) return 0.0;
-  const int lz = __clzll((long long)s);
-  const uint64_t n = s << lz, r = (n >> 11) + ((n >> 10) & 1u);   // 53 bits, rounded; its top bit adds one to the exponent
-  return __longlong_as_double((long long)(((uint64_t)(1023 + 63 - lz + ex - 185 - 1) << 52) + r));
+  return ((uint64_t)s2 << 42) + ((uint64_t)s1 << 21) + s0;
+}
+
+// The sum of N non-negative floats of every lane, the same in every lane of a converged warp, whatever their
+// magnitudes: fixed point with 36 - N bits below the largest value's last one, so that what is cut off is no more
+// than a float64 sum's rounding, in integers because a chain of FP64 shuffles costs a step of a small solve more
+// than the warp-wide integer sums (FP64 runs at two operations a cycle and SM).
+template <int N>
+__device__ __forceinline__ Fixed warp_fixed(const float (&v)[N]) {
+  static_assert(N == 1 || N == 2, "a lane's values add up to less than 2^59");
+  uint32_t top = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) top = max(top, __float_as_uint(v[i]));
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (top >= 0x7f800000u) return {0, FIXED_BAD};
+  const int ex = max((int)(top >> 23), 1);
+  uint64_t q = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint32_t b = __float_as_uint(v[i]);
+    const int down = ex - max((int)(b >> 23), 1);
+    const uint64_t man = (b & 0x7fffffu) | (b >> 23 ? 0x800000u : 0u);
+    q += down < 60 - N ? (man << (36 - N)) >> down : 0u;
+  }
+  return {warp_add59(q), ex - 186 + N};
+}
+template <int N>
+__device__ __forceinline__ double warp_sum64(const float (&v)[N]) {
+  return fixed_double(warp_fixed<N>(v));
+}
+__device__ __forceinline__ double warp_sum64(float v) { return warp_sum64<1>({v}); }
+
+// The sum of 16 of them, in lanes 0 to 15.
+__device__ __forceinline__ double warp_sum16(Fixed f, int lane) {
+  const int top = (int)__reduce_max_sync(0xffffffffu, (uint32_t)(f.e + FIXED_BAD)) - FIXED_BAD;
+  if (top == FIXED_BAD) return fixed_double({0, FIXED_BAD});
+  const int down = top - f.e;
+  return fixed_double({warp_add59(lane < 16 && down < 60 ? (f.s >> 4) >> down : 0u), top + 4});
 }
 
 // s <- s + b rounded, and its rounding error, exactly (Knuth's two-sum).

@@ -69,7 +69,8 @@ struct OcCtl {
   uint32_t tmem_base;
   int pad;
   float c1, c3;
-  double red[OC_WARPS];    // the warps' sums
+  uint64_t red_s[OC_WARPS];   // the warps' sums
+  int red_e[OC_WARPS];
 };
 
 __host__ __device__ __forceinline__ uint32_t oc_rows(int64_t m) { return (uint32_t)((m + 15) / 16 * 16); }
@@ -222,12 +223,8 @@ __device__ __noinline__ void oc_issue(const OcTask& tk, uint32_t xbase, uint32_t
       }
       __syncwarp();
     }
-    // the stop test: the warps' sums added in a fixed order (every lane has the sum), v = n r^2 against squared
-    // thresholds
-    const volatile double* red = ctl->red + 4 * (lane & 3);
-    double v = (red[0] + red[1]) + (red[2] + red[3]);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    // the stop test: the warps' sums added up (every lane has the sum), v = n r^2 against squared thresholds
+    const double v = warp_sum16({ctl->red_s[lane & 15], ctl->red_e[lane & 15]}, lane);
     int dec = 2, status = ST_TIMEOUT;
     if (go) {
       const bool testing = k >= ctl->dr.n_pre;
@@ -355,8 +352,11 @@ __device__ __noinline__ void oc_solve(const OcTask& tk, uint8_t* xs, uint32_t ch
       }
     }
     if (stored) tmem_st_wait();
-    const double part = warp_sum64(part32);
-    if (lane == 0) ctl->red[warp] = part;
+    const Fixed part = warp_fixed<1>({part32});
+    if (lane == 0) {
+      ctl->red_s[warp] = part.s;
+      ctl->red_e[warp] = part.e;
+    }
     tc_fence_before();
     oc_arrive<3>();
     oc_sync<4>();   // the decision
