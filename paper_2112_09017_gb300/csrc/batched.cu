@@ -271,8 +271,12 @@ polar_status_t enqueue_all(BatchedPlan* b, cudaStream_t s) {
   rule.n_pre = b->opt.precondition ? precond_steps(b->opt.s_minus, b->opt.s0) : 0;
   rule.pre_a = 1.5 * sqrt(3.0) - b->opt.s_minus;
 #define BK_(x) do { if ((x) != cudaSuccess) return POLAR_ECUDA; } while (0)
-  // blocks per problem of the passes over A, U and H: about 8192 in all, so that a few large problems spread too
-  const int ys = std::max(8, std::min(kMaxSplit, 8192 / count));
+  // blocks per problem of the passes over A, U and H: about 8192 in all, so that a few large problems spread too, but
+  // no more than the largest problem has work for (123 problems of 30 x 30: 174 us with 64 blocks each, 120 with one)
+  int64_t units = 1;
+  for (int p = 0; p < count; ++p) units = std::max(units, b->m[p] * ((b->n[p] + 7) / 8));
+  const int most = std::max(8, std::min(kMaxSplit, 8192 / count));
+  const int ys = (int)std::min<int64_t>(most, (units + kThreads - 1) / kThreads);
   b_norm_kernel<<<dim3(count, ys), kThreads, 0, s>>>(b->A_tab, b->meta_d, b->st_d, b->sh_d);
   BK_(cudaGetLastError());
   b_scale_split_kernel<<<dim3(count, ys), kThreads, 0, s>>>(b->A_tab, b->meta_d, b->st_d, b->P, ys);
