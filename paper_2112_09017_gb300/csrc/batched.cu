@@ -483,6 +483,9 @@ polar_status_t batched_create(BatchedPlan** out, int count, const int64_t* m, co
   b->n_h = (int)h_t.size();
   for (const auto* t : {&gram_t, &upd_t}) b->deepest = std::max(b->deepest, deepest_block(*t, b->grid()));
 
+  // the buffers are cleared and filled on the default stream, which a run's stream need not wait for
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return fail(POLAR_ECUDA);
+
   // capture the whole sequence once; each run uploads its pointer tables and replays it
   if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) return fail(POLAR_ECUDA);
   if (cudaEventCreateWithFlags(&b->tab_ev, cudaEventDisableTiming) != cudaSuccess) return fail(POLAR_ECUDA);

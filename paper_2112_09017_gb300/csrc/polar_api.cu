@@ -429,6 +429,8 @@ polar_status_t plan_setup(polar_plan_s* p) {
     b.partials = p->partials; b.nparts = p->nparts; b.st = p->st;
     p->coop = coop_solve_create(b, m, n, p->sms);
   }
+  // the buffers are cleared on the default stream, which a run's stream need not wait for
+  CK(cudaStreamSynchronize(cudaStreamLegacy));
   return POLAR_OK;
 }
 

@@ -454,3 +454,32 @@ def test_slice_length_of_the_environment_reaches_every_product(lib):
     assert (multi0, multi4) == ("False", "True")
     assert solve4 != solve0 and inv4 != inv0 and cheb4 != cheb0
     assert batch0 != tuned0 and batch4 == tuned4 == tuned0
+
+
+@pytest.mark.parametrize("kind", ["solve", "fp32", "batch"])
+def test_a_plan_is_ready_for_any_stream(lib, kind):
+    """A plan made while the default stream is busy, run at once on a stream that does not wait for it: the clearing
+    of the plan's buffers is over when the plan is returned."""
+    import torch
+    n = 700
+    a = torch.from_numpy(synth.matrix_with_spectrum(n, n, synth.logspace_spectrum(n, 0.1), 21)).cuda()
+    outs = []
+    U, H = torch.empty_like(a), torch.empty_like(a)
+    for busy in (False, True):
+        s = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        if busy:
+            torch.cuda._sleep(400_000_000)            # about 0.2 s of the default stream
+        if kind == "batch":
+            plan = lib.polar_batched_plan_create([n], [n])
+            lib.polar_batched_run(plan, [a], [U], [H], 0.0, None, None, stream=s)
+        else:
+            plan = lib.Plan(n, n, prec="bf16x6" if kind == "solve" else "fp32")
+            plan(a, U=U, H=H, stream=s)
+        torch.cuda.synchronize()
+        outs.append((U.clone(), H.clone()))
+        if kind == "batch":
+            lib.polar_plan_destroy(plan)
+        else:
+            plan.close()
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
