@@ -90,13 +90,15 @@ typedef struct {
 
 typedef struct {
   double tol;              /* stop when ||X^T X - I||_F / sqrt(n) <= tol; <= 0 means 1e-6 */
-  int max_iter;            /* maximum number of updates; <= 0 means 100 */
+  int max_iter;            /* maximum number of updates; <= 0 means 100. POLAR_HIST or more: a small or medium single
+                              solve leaves its one-launch form, several times faster there, for separate launches */
   int prec;                /* a polar_precision_t */
   double stagnation;       /* stop (NOT_CONVERGED) when r_k > stagnation * r_{k-2} ... ; <= 0 means 0.7 */
   double stag_floor;       /* ... and r_k < stag_floor; <= 0 means 1e-4 */
   double switch_residual;  /* schedules: residual below which the finer precision is used; <= 0 means 1e-2 */
   size_t ws_limit;         /* maximum workspace bytes a plan may allocate; 0 = no limit */
-  int profile;             /* nonzero: time every Gram and update launch with CUDA events (info) */
+  int profile;             /* nonzero: time every Gram and update launch with CUDA events (info), which takes separate
+                              launches at every size */
   int precondition;        /* nonzero: Algorithm 1 - first the steps X <- a X (I - 4/27 a^2 X^T X),
                               a = 3 sqrt(3)/2 - s_minus (Eqs. a_def, RogueMatrix), as many as lift s0 to
                               s_minus under Eq. RogueScalar; then Newton-Schulz. Stop tests start after them */

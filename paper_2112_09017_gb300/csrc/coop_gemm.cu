@@ -100,8 +100,9 @@ cudaError_t launch_co_gemm(const TcArgs& a, const CoopForm& f, cudaStream_t s) {
   p.alpha = a.alpha; p.beta = a.beta;
   p.err = a.err_out;
   p.withhold = a.withhold_tma;
-  if (a.a.kmajor) return a.b.kmajor ? launch_t<false, true>(p, f.split, f.blocks, s) : launch_t<false, false>(p, f.split, f.blocks, s);
-  return a.b.kmajor ? launch_t<true, true>(p, f.split, f.blocks, s) : launch_t<true, false>(p, f.split, f.blocks, s);
+  auto launch = a.a.kmajor ? (a.b.kmajor ? launch_t<false, true> : launch_t<false, false>)
+                           : (a.b.kmajor ? launch_t<true, true> : launch_t<true, false>);
+  return launch(p, f.split, f.blocks, s);
 }
 
 }  // namespace polar

@@ -693,7 +693,7 @@ __device__ __forceinline__ void co_epilogue_split(CoCtx& x, CoPipe& pp, Src src,
           v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
         }
         float d2 = 0.0f, x2 = 0.0f;   // GRAM: the residual terms; STEP: the step's
-        if (r >= e.M || col >= e.N) {
+        if (r >= e.M || col >= e.N) {   // past the matrix: nothing but zeros to the sums
         } else if (EPI == TC_EPI_GRAM) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {

@@ -334,7 +334,10 @@ CoopForm coop_form(const CoopProduct* p, int count, int sms) {
   if (w128 > 8) return f;
   // few tiles: share each between blocks along K, where that shortens a step by a tenth
   f.split = coop_split_plan(p, count, sms, f.S, &f.blocks);
-  if (!f.split) f.S[0] = f.S[1] = 1, f.blocks = 0;
+  if (!f.split) {
+    f.S[0] = f.S[1] = 1;
+    f.blocks = 0;
+  }
   f.tn = f.split || c64 <= c128 ? 64 : 128;
   return f;
 }

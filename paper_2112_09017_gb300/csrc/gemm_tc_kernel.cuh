@@ -117,8 +117,9 @@ __host__ __device__ constexpr uint32_t make_idesc_f8(int tn = BN) {
 
 // The MMAs of one k-stage (two K = 16 steps) of the split product with `np` planes in issue order: step, plane
 // of A, plane of B, and the use of the tensor core's collector, which keeps one A operand between
-// consecutive MMAs (0: not used, 1: filled, 2: used again, 3: used for the last time). hi*hi comes last, so
-// that the truncations of the small terms happen at 2^-8 of the result's scale; among the small terms those
+// consecutive MMAs (0: not used, 1: filled, 2: used again, 3: used for the last time). hi*hi comes last in each
+// stage: in the first stage of a slice the small terms are truncated at 2^-8 of the result's scale, in the others
+// (one of two with slices of 64 of K) at the scale of the hi*hi sums already there. Among the small terms those
 // that share an A plane are neighbours. Reading A seven times per stage instead of twelve matters because the
 // shared memory serves the MMAs' operands and the copies of later stages: 128 bytes a cycle, of which a stage
 // of 128 x 64 tiles needed 864 cycles for 595 of products, of 128 x 128 tiles 1152 for 786. Alone, a 64-wide
@@ -528,9 +529,10 @@ __device__ __forceinline__ void issue_half(uint32_t d_tmem, uint64_t a_desc, uin
 // The whole warp runs the loop and one elected lane issues: the descriptors then stay in uniform registers.
 // A wait costs about 250 cycles even when its phase has completed, because it cannot pass the MMAs queued
 // before it, and only about three MMAs queue up; so a stage's barriers are tested between the halves of the
-// stage before it, and waited for after it where they were not complete. Measured alone (a stage of twelve MMAs with both waits and commits, one SM): 1735 cycles with
-// one lane waiting ahead of every stage and 1562 in this form for 256-wide tiles, whose MMAs take 1560;
-// 1212 and 839 for 128-wide ones (790); 1202 and 681 for 64-wide ones (595).
+// stage before it, and waited for after it where they were not complete. Measured alone (a stage of twelve MMAs
+// with both waits and commits, one SM): 1735 cycles with one lane waiting ahead of every stage and 1562 in this
+// form for 256-wide tiles, whose MMAs take 1560;
+// 1212 and 839 for 128-wide ones (790); 1202 and 681 for 64-wide ones (595, which mma_step's order made 494).
 template <int P, bool A_MN, bool B_MN, int TN, int CG, class Src>
 __device__ __noinline__ void role_mma(const Src& src, uint32_t smem_base, uint32_t tmem_base, Bars br,
                                       volatile int* abort_flag, int pu) {
