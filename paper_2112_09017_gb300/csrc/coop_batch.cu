@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(CO_THREADS, 1) co_batch_kernel(const __grid_co
       DevState& s = p.st[q];
       if (__ldcg(&s.status) != ST_RUNNING) continue;
       const BMeta& mt = p.meta[q];
-      const double v = co_warp_sum(mt.partials, mt.ntiles_gram * EPI_WARPS, 1, x.lane);
+      const double v = co_warp_sum<1>(mt.partials, mt.ntiles_gram * EPI_WARPS, 1, x.lane);
       if (x.lane == 0) {
         const double r = sqrt(v) * s.inv_sqrt_n;
         float c1, c3;

@@ -774,10 +774,22 @@ __device__ __forceinline__ void co_product(CoCtx& x, CoPipe& pipe, const CUtenso
   }
 }
 
-// Sum of n doubles in device memory in a fixed order, by one warp (every lane gets it).
+// Sum of n doubles in device memory in a fixed order, by one warp (every lane gets it). AHEAD loads in flight and
+// their sums as a tree: at 512^2 the stop test adds 36 per lane, and one at a time they took longer than the
+// products beside which it runs.
+template <int AHEAD = 8>
 __device__ __forceinline__ double co_warp_sum(const double* p, int n, int stride, int lane) {
   double v = 0.0;
-  for (int i = lane; i < n; i += 32) v += __ldcg(p + (size_t)i * stride);
+  for (int i = lane; i < n; i += 32 * AHEAD) {
+    double a[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) a[j] = i + 32 * j < n ? __ldcg(p + (size_t)(i + 32 * j) * stride) : 0.0;
+#pragma unroll
+    for (int o = AHEAD / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < o; ++j) a[j] += a[j + o];
+    v += a[0];
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

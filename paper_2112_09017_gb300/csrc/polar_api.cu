@@ -231,6 +231,7 @@ struct polar_plan_s {
   struct Prof { cudaEvent_t a, b; int kind, k; };  // kind 0: Gram, 1: update
   std::vector<Prof> prof;
   size_t prof_used = 0;
+  bool cleared = false;                  // a run has waited for the clearing of the buffers (ev_stop until then)
   CoopSolve* coop = nullptr;             // the whole solve in one cooperative launch (chosen at creation),
   CoopFp32* coop32 = nullptr;            // or its plain form
   // batched
@@ -429,8 +430,8 @@ polar_status_t plan_setup(polar_plan_s* p) {
     b.partials = p->partials; b.nparts = p->nparts; b.st = p->st;
     p->coop = coop_solve_create(b, m, n, p->sms);
   }
-  // the buffers are cleared on the default stream, which a run's stream need not wait for
-  CK(cudaStreamSynchronize(cudaStreamLegacy));
+  // the buffers are cleared on the default stream, which a run's stream need not wait for: the first run does
+  CK(cudaEventRecord(p->ev_stop, cudaStreamLegacy));
   return POLAR_OK;
 }
 
@@ -674,6 +675,10 @@ polar_status_t run_single(polar_plan_s* p, const float* A, int64_t lda, float* U
   StopRule rule = make_rule(p, tol);
   p->launches = 0;
   p->prof_used = 0;
+  if (!p->cleared) {
+    CK(cudaStreamWaitEvent(s, p->ev_stop, 0));
+    p->cleared = true;
+  }
   CK(cudaEventRecord(p->ev_start, s));
   if (p->coop || p->coop32) return run_coop(p, A, lda, U, ldu, H, ldh, rule, info, s);
   // ||A||_F and X_0 = A / ||A||_F (+ planes of X_0)
