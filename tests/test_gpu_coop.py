@@ -483,3 +483,54 @@ def test_a_plan_is_ready_for_any_stream(lib, kind):
         else:
             plan.close()
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("kind,m,n,count", [("bf16x6", 400, 300, 4), ("bf16x6", 1000, 700, 3), ("bf16x6", 2100, 2050, 2),
+                                            ("fp32", 300, 200, 4), ("batch", 500, 400, 3)], ids=lambda v: str(v))
+def test_one_launch_kernels_on_streams_of_their_own(lib, kind, m, n, count):
+    """Plans run at the same time from threads, each on its own stream, together more blocks than the GPU holds: a
+    cooperative launch starts when all of its blocks fit, so none waits for blocks that cannot start, and each
+    returns what it returns alone."""
+    import threading
+
+    import torch
+    mats = [torch.from_numpy(synth.matrix_with_spectrum(m, n, synth.logspace_spectrum(n, 0.1), 70 + i)).cuda()
+            for i in range(count)]
+    streams = [torch.cuda.Stream() for _ in range(count)]
+    outs = [[(torch.empty_like(a), torch.empty((n, n), device="cuda")) for _ in range(2)] for a in mats]
+    if kind == "batch":
+        plans = [lib.polar_batched_plan_create([m], [n]) for _ in mats]
+    else:
+        plans = [lib.Plan(m, n, prec=kind) for _ in mats]
+    torch.cuda.synchronize()                 # the inputs are there for every stream
+
+    def run(i, rep):
+        U, H = outs[i][rep]
+        if kind == "batch":
+            lib.polar_batched_run(plans[i], [mats[i]], [U], [H], 0.0, None, None, stream=streams[i])
+            streams[i].synchronize()
+        else:
+            plans[i](mats[i], U=U, H=H, stream=streams[i])
+
+    for i in range(count):
+        run(i, 0)
+    errs = []
+
+    def work(i):
+        try:
+            for _ in range(5):
+                run(i, 1)
+        except Exception as e:               # a timeout's status, for the assertion below
+            errs.append(e)
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(count)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errs
+    for (U, H), (U2, H2) in outs:
+        assert torch.equal(U, U2) and torch.equal(H, H2)
+    for p in plans:
+        lib.polar_plan_destroy(p) if kind == "batch" else p.close()
